@@ -445,34 +445,102 @@ __global__ void k_pp_ksk_finish(SfPpRing R, const u64 *prod, const u64 *e_res, c
     }
 }
 
-// RNS digits of ta = tau_h(a): d_i = [ta_i (Q/q_i)^-1]_{q_i} (an integer below
-// q_i), written as residues modulo every q_j: D[i][j][e]
-__global__ void k_pp_digits(SfPpRing R, const u64 *ta, u64 *D)
+// ---- key switch after tau_h, fused ------------------------------------------
+// Bound by the integer multiplier: 2 L^2 key transforms once per call, then
+// L + 2 length-M transforms per (ciphertext, limb).  One block per (limb j,
+// ciphertext): the digits of tau_h(a) are gathered from global memory as the
+// first stage of each forward transform reads them (the automorphism and the
+// Phi_M fold are two loads), the products with the transformed key stay in
+// registers, and the two inverse transforms write the result.  The launches
+// this replaces ran five kernels per ciphertext, each on L^2 blocks or fewer,
+// and transformed the key again for every ciphertext: M = 5^5, 3 limbs, 333
+// ciphertexts took 170 ms.
+
+// coefficient e of tau_h(x) mod Phi_M gathered from x (length N, canonical):
+// x_k sits at k h mod M of the unreduced image, and position e < N receives the
+// image at e minus the image at N + (e mod m); hinv = h^-1 mod M
+__device__ __forceinline__ u64 pp_auto_at(const u64 *x, int e, const SfPpRing &R, int hinv, u64 q)
 {
-    const size_t per = (size_t)R.L * R.N, total = (size_t)R.L * per;
-    for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < total; k += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(k / per);
-        const size_t r = k - (size_t)i * per;
-        const int j = (int)(r / R.N), e = (int)(r % R.N);
-        const SfPpMod &Pi = R.mod[i];
-        const u64 d = sf_mul_shoup(ta[(size_t)i * R.N + e], Pi.qh_inv, Pi.qh_inv_p, Pi.q);
-        D[k] = j == i ? d : sf_reduce(d, R.mod[j].q, R.mod[j].one_p);
+    const int k0 = (int)(((long long)e * hinv) % R.M);
+    const int k1 = (int)(((long long)(R.N + e % R.m) * hinv) % R.M);
+    return sf_sub(k0 < R.N ? x[k0] : 0, k1 < R.N ? x[k1] : 0, q);
+}
+
+// The key in the form the key switch reads: polynomial p = 2 i + part (digit
+// i, ka or kb) modulo limb j, transformed: key[p][j][M], then the Shoup
+// companions in the same order.  grid (L, 2 L).
+template <int T, int ALPHA>
+__global__ void __launch_bounds__(SfPpShape<T, ALPHA>::NT) k_pp_key_ntt(SfPpRing R, const u64 *ka, const u64 *kb, u64 *key)
+{
+    constexpr int NT = SfPpShape<T, ALPHA>::NT;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    u64 *s = (u64 *)smem_raw;
+    const int j = blockIdx.x, p = blockIdx.y, N = R.N;
+    const u64 *x = ((p & 1) ? kb : ka) + ((size_t)(p >> 1) * R.L + j) * N;
+    pp_block_forward_ld<T, ALPHA>(s, [x, N](int e) -> u64 { return e < N ? x[e] : 0; }, R, j);
+    u64 *dst = key + ((size_t)p * R.L + j) * R.M;
+    const size_t comp = (size_t)2 * R.L * R.L * R.M;
+    for (int e = threadIdx.x; e < R.M; e += NT) {
+        dst[e] = s[e];
+        dst[comp + e] = pp_companion(s[e], R.mod[j]);
     }
 }
 
-// out = (-sum_i PA[i], tb - sum_i PB[i]) for one ciphertext
-__global__ void k_pp_ks_combine(SfPpRing R, const u64 *PA, const u64 *PB, const u64 *tb, u64 *out)
+// out = (-sum_i d_i ka_i, tau_h(b) - sum_i d_i kb_i), d_i = [tau_h(a)_i
+// (Q/q_i)^-1]_{q_i} read as an integer; grid (L, count), key from k_pp_key_ntt.
+template <int T, int ALPHA>
+__global__ void __launch_bounds__(SfPpShape<T, ALPHA>::NT, SfPpShape<T, ALPHA>::MINB)
+    k_pp_ks(SfPpRing R, const u64 *in, u64 *out, int hinv, const u64 *key)
 {
-    const size_t per = (size_t)R.L * R.N;
-    for (size_t r = (size_t)blockIdx.x * blockDim.x + threadIdx.x; r < per; r += (size_t)gridDim.x * blockDim.x) {
-        const u64 q = R.mod[(int)(r / R.N)].q;
-        u64 a = 0, b = tb[r];
-        for (int i = 0; i < R.L; ++i) {
-            a = sf_sub(a, PA[(size_t)i * per + r], q);
-            b = sf_sub(b, PB[(size_t)i * per + r], q);
+    constexpr int NT = SfPpShape<T, ALPHA>::NT, EPT = (SfPpShape<T, ALPHA>::MMAX + NT - 1) / NT;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    u64 *s = (u64 *)smem_raw;
+    const int j = blockIdx.x, N = R.N, M = R.M, L = R.L;
+    const SfPpMod &P = R.mod[j];
+    const size_t per = (size_t)L * N;
+    const u64 *a = in + (size_t)blockIdx.y * 2 * per, *b = a + per + (size_t)j * N;
+    const size_t comp = (size_t)2 * L * L * M;
+    u64 acc_a[EPT], acc_b[EPT];
+#pragma unroll
+    for (int x = 0; x < EPT; ++x) acc_a[x] = acc_b[x] = 0;
+    for (int i = 0; i < L; ++i) {
+        const SfPpMod &Pi = R.mod[i];
+        const u64 *ai = a + (size_t)i * N;
+        pp_block_forward_ld<T, ALPHA>(
+            s,
+            [&](int e) -> u64 {
+                if (e >= N) return 0;
+                const u64 d = sf_mul_shoup(pp_auto_at(ai, e, R, hinv, Pi.q), Pi.qh_inv, Pi.qh_inv_p, Pi.q);
+                return i == j ? d : sf_reduce(d, P.q, P.one_p);
+            },
+            R, j);
+        const u64 *ka = key + ((size_t)(2 * i) * L + j) * M, *kb = key + ((size_t)(2 * i + 1) * L + j) * M;
+#pragma unroll
+        for (int x = 0; x < EPT; ++x) {
+            const int e = threadIdx.x + x * NT;
+            if (e < M) {
+                // canonical sums: L products of up to 61-bit residues leave no lazy room
+                const u64 v = s[e];
+                acc_a[x] = sf_add(acc_a[x], sf_mul_shoup(v, __ldg(ka + e), __ldg(ka + comp + e), P.q), P.q);
+                acc_b[x] = sf_add(acc_b[x], sf_mul_shoup(v, __ldg(kb + e), __ldg(kb + comp + e), P.q), P.q);
+            }
         }
-        out[r] = a;
-        out[per + r] = b;
+        __syncthreads();
+    }
+    for (int part = 0; part < 2; ++part) {
+#pragma unroll
+        for (int x = 0; x < EPT; ++x) {
+            const int e = threadIdx.x + x * NT;
+            if (e < M) s[e] = part ? acc_b[x] : acc_a[x];
+        }
+        __syncthreads();
+        pp_block_inverse<T, ALPHA>(s, R, j);
+        u64 *o = out + (size_t)blockIdx.y * 2 * per + (size_t)part * per + (size_t)j * N;
+        for (int e = threadIdx.x; e < N; e += NT) {
+            const u64 v = sf_sub(s[e], s[N + e % R.m], P.q);   // the Phi_M fold
+            o[e] = sf_sub(part ? pp_auto_at(b, e, R, hinv, P.q) : 0, v, P.q);
+        }
+        __syncthreads();
     }
 }
 
@@ -552,21 +620,34 @@ extern "C" sf_status sf_pp_ksk(sf_pp_ring *r, const int64_t *d_s, int32_t h, con
     return SF_OK;
 }
 
-// tau_h then the key switch back to s, one ciphertext at a time; `in` and
-// `out` may not alias; work: 2 + 3 L polynomials of L limbs
-static sf_status pp_keyswitch(sf_pp_ring *r, const u64 *in, u64 *out, int count, int h, const u64 *ka, const u64 *kb,
-                              u64 *work, cudaStream_t st)
+static int pp_inverse_index(int h, int M)
 {
-    const SfPpRing &R = r->R;
-    const size_t per = (size_t)R.L * R.N;
-    u64 *T = work, *D = T + 2 * per, *PA = D + per * R.L, *PB = PA + per * R.L;
-    for (int c = 0; c < count; ++c) {
-        SF_TRY(pp_auto(r, in + 2 * per * c, T, 2, h, st));
-        k_pp_digits<<<pp_grid(per * R.L), 256, 0, st>>>(R, T, D);
-        k_pp_mul<<<dim3(R.L, R.L), SF_PP_THREADS, 2 * sizeof(u64) * R.M, st>>>(R, D, ka, PA, R.L);
-        k_pp_mul<<<dim3(R.L, R.L), SF_PP_THREADS, 2 * sizeof(u64) * R.M, st>>>(R, D, kb, PB, R.L);
-        k_pp_ks_combine<<<pp_grid(per), 256, 0, st>>>(R, PA, PB, T + per, out + 2 * per * c);
-    }
+    for (int x = 1; x < M; ++x)
+        if ((long long)x * h % M == 1) return x;
+    return 0;
+}
+
+// words of a transformed key (values and companions)
+static size_t pp_key_words(const SfPpRing &R) { return (size_t)4 * R.L * R.L * R.M; }
+
+static sf_status pp_key_ntt(const SfPpRing &R, const u64 *ka, const u64 *kb, u64 *key, cudaStream_t st)
+{
+    SF_PP_DISPATCH_ANY(R, {
+        k_pp_key_ntt<T, ALPHA><<<dim3(R.L, 2 * R.L), SfPpShape<T, ALPHA>::NT, sizeof(u64) * R.M, st>>>(R, ka, kb, key);
+    });
+    SF_CUDA_TRY(cudaGetLastError());
+    return SF_OK;
+}
+
+// tau_h then the key switch back to s for `count` ciphertexts in one launch;
+// `in` and `out` may not alias; h coprime to M; key: the transformed key of tau_h
+static sf_status pp_keyswitch(const SfPpRing &R, const u64 *in, u64 *out, int count, int h, const u64 *key,
+                              cudaStream_t st)
+{
+    const int hinv = pp_inverse_index(((h % R.M) + R.M) % R.M, R.M);
+    SF_PP_DISPATCH_ANY(R, {
+        k_pp_ks<T, ALPHA><<<dim3(R.L, count), SfPpShape<T, ALPHA>::NT, sizeof(u64) * R.M, st>>>(R, in, out, hinv, key);
+    });
     SF_CUDA_TRY(cudaGetLastError());
     return SF_OK;
 }
@@ -577,9 +658,12 @@ extern "C" sf_status sf_pp_keyswitch(sf_pp_ring *r, const uint64_t *d_ct, uint64
     SF_TRY(pp_check(r, d_ct, d_out, count));
     if (!d_ka || !d_kb || d_ct == d_out) return sf_set_error(SF_EINVAL, "sf_pp_keyswitch: bad key or aliasing");
     const SfPpRing &R = r->R;
-    u64 *work;
-    SF_TRY(pp_ks_buffer(r, (size_t)R.L * R.N * (2 + 3 * (size_t)R.L), &work));
-    return pp_keyswitch(r, d_ct, d_out, count, h, d_ka, d_kb, work, (cudaStream_t)stream);
+    if (h % R.t == 0) return sf_set_error(SF_EINVAL, "automorphism index %d not coprime to M = %d", h, R.M);
+    cudaStream_t st = (cudaStream_t)stream;
+    u64 *key;
+    SF_TRY(pp_ks_buffer(r, pp_key_words(R), &key));
+    SF_TRY(pp_key_ntt(R, d_ka, d_kb, key, st));
+    return pp_keyswitch(R, d_ct, d_out, count, h, key, st);
 }
 
 extern "C" sf_status sf_pp_hom_trace(sf_pp_ring *r, const uint64_t *d_ct, uint64_t *d_out, int32_t count,
@@ -610,15 +694,17 @@ extern "C" sf_status sf_pp_hom_trace(sf_pp_ring *r, const uint64_t *d_ct, uint64
         r->scratch_words = 2 * words;
     }
     u64 *work;
-    SF_TRY(pp_ks_buffer(r, (size_t)R.L * R.N * (2 + 3 * (size_t)R.L), &work));
+    SF_TRY(pp_ks_buffer(r, pp_key_words(R), &work));
     u64 *cur = r->d_scratch, *nxt = cur + words;
     SF_CUDA_TRY(cudaMemcpyAsync(d_out, d_ct, sizeof(u64) * words, cudaMemcpyDeviceToDevice, st));
     int ks = 0;
     const int grid = pp_grid(words);
     for (size_t k = 0; k < steps.size(); ++k) {
         SF_CUDA_TRY(cudaMemcpyAsync(cur, d_out, sizeof(u64) * words, cudaMemcpyDeviceToDevice, st));
+        // one key per step, transformed once for its key switches
+        SF_TRY(pp_key_ntt(R, d_kas[key_of[k]], d_kbs[key_of[k]], work, st));
         for (int x = 1; x < steps[k].second; ++x) {
-            SF_TRY(pp_keyswitch(r, cur, nxt, count, steps[k].first, d_kas[key_of[k]], d_kbs[key_of[k]], work, st));
+            SF_TRY(pp_keyswitch(R, cur, nxt, count, steps[k].first, work, st));
             std::swap(cur, nxt);
             k_pp_add<<<grid, 256, 0, st>>>(R, d_out, cur, words);
             SF_CUDA_TRY(cudaGetLastError());

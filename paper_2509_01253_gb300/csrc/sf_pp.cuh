@@ -303,6 +303,64 @@ __device__ __forceinline__ void ppt_inverse(u64 *s, const u64 *iw, const u64 *iw
     if constexpr (LEN * T <= M) ppt_inverse<T, M, LEN * T>(s, iw, iwp, dc, q, one_p, P);
 }
 
+// ---- one interface over the compiled and the generic transforms -------------
+// T = 0 stands for the generic ring (runtime t and alpha).  The fused key
+// switches of compiled rings are bounded to two blocks per SM: at M = 3^7 and
+// 5^5 that caps the torus kernel's registers at 40 and 48 (with a few spilled
+// words) and was measured 12 and 10 % faster than one block of 72 and 94
+// registers; three blocks spill more and lose again.
+template <int T, int ALPHA>
+struct SfPpShape {
+    static constexpr int NT = SfPpT<T, ALPHA>::THREADS, MMAX = SfPpT<T, ALPHA>::M, MINB = 2;
+};
+template <int ALPHA>
+struct SfPpShape<0, ALPHA> {
+    static constexpr int NT = SF_PP_THREADS, MMAX = SF_PP_MAX_M, MINB = 1;
+};
+
+// forward transform of the block's length-M vector modulo prime j, the first
+// stage reading its inputs through ld(index), index < M (each read once)
+template <int T, int ALPHA, class LD>
+__device__ __forceinline__ void pp_block_forward_ld(u64 *s, LD ld, const SfPpRing &R, int j)
+{
+    if constexpr (T == 0) {
+        for (int e = threadIdx.x; e < R.M; e += blockDim.x) s[e] = ld(e);
+        __syncthreads();
+        pp_forward(s, R, j);
+    } else {
+        constexpr int M = SfPpT<T, ALPHA>::M, H = (T - 1) / 2;
+        const SfPpMod &P = R.mod[j];
+        ppt_forward_ld<T, M>(s, ld, R.w + (size_t)j * M, R.w_p + (size_t)j * M, R.dftc + (size_t)j * H * H * 4, P.q,
+                             P.one_p, P);
+    }
+}
+
+// inverse transform, scaled by M^-1
+template <int T, int ALPHA>
+__device__ __forceinline__ void pp_block_inverse(u64 *s, const SfPpRing &R, int j)
+{
+    if constexpr (T == 0) {
+        pp_inverse(s, R, j);
+    } else {
+        constexpr int M = SfPpT<T, ALPHA>::M, H = (T - 1) / 2, NT = SfPpT<T, ALPHA>::THREADS;
+        const SfPpMod &P = R.mod[j];
+        ppt_inverse<T, M, T>(s, R.iw + (size_t)j * M, R.iw_p + (size_t)j * M, R.dftc + (size_t)j * H * H * 4, P.q,
+                             P.one_p, P);
+        for (int e = threadIdx.x; e < M; e += NT) s[e] = sf_mul_shoup(s[e], P.minv, P.minv_p, P.q);
+        __syncthreads();
+    }
+}
+
+// floor(x 2^64 / q) for x < q: 2^64 = one_p q + rm, and floor(x rm / q) by
+// Shoup's product with at most one correction
+__device__ __forceinline__ u64 pp_companion(u64 x, const SfPpMod &P)
+{
+    u64 h = sf_mulhi(x, P.rm_p);
+    const u64 rem = x * P.rm - h * P.q;
+    if (rem >= P.q) ++h;
+    return x * P.one_p + h;
+}
+
 // runs the statements with constexpr T, ALPHA when (t, alpha) is one of the
 // compiled rings; `done` tells whether it did
 #define SF_PPT_DISPATCH(t, alpha, done, ...)                                                 \
@@ -317,6 +375,17 @@ __device__ __forceinline__ void ppt_inverse(u64 *s, const u64 *iw, const u64 *iw
         else if ((t) == 7 && (alpha) == 4) { constexpr int T = 7, ALPHA = 4; __VA_ARGS__ }     \
         else if ((t) == 7 && (alpha) == 2) { constexpr int T = 7, ALPHA = 2; __VA_ARGS__ }     \
         else done = false;                                                                     \
+    } while (0)
+
+// the same with T = 0 for every other ring
+#define SF_PP_DISPATCH_ANY(R, ...)                             \
+    do {                                                       \
+        bool done_ = false;                                    \
+        SF_PPT_DISPATCH((R).t, (R).alpha, done_, __VA_ARGS__); \
+        if (!done_) {                                          \
+            constexpr int T = 0, ALPHA = 0;                    \
+            __VA_ARGS__                                        \
+        }                                                      \
     } while (0)
 
 // the automorphisms of the tower of Sec. 2.3: per step (h, length), the step

@@ -58,69 +58,12 @@ struct sf_tq_ring {
     size_t work_words = 0;
 };
 
-// compile-time shape: T = 0 is the generic ring (runtime t, alpha).  The key
-// switch of a compiled ring is bounded to two blocks per SM: at M = 3^7 and
-// 5^5 that caps its registers at 40 and 48 (with a few spilled words) and was
-// measured 12 and 10 % faster than one block of 72 and 94 registers; three
-// blocks spill more and lose again.
-template <int T, int ALPHA>
-struct SfTqShape {
-    static constexpr int NT = SfPpT<T, ALPHA>::THREADS, MMAX = SfPpT<T, ALPHA>::M, MINB = 2;
-};
-template <int ALPHA>
-struct SfTqShape<0, ALPHA> {
-    static constexpr int NT = SF_PP_THREADS, MMAX = SF_PP_MAX_M, MINB = 1;
-};
-
-// forward transform of the block's length-M vector modulo prime j, the first
-// stage reading its inputs through ld(index), index < M (each read once)
-template <int T, int ALPHA, class LD>
-__device__ __forceinline__ void tq_forward_ld(u64 *s, LD ld, const SfPpRing &R, int j)
-{
-    if constexpr (T == 0) {
-        for (int e = threadIdx.x; e < R.M; e += blockDim.x) s[e] = ld(e);
-        __syncthreads();
-        pp_forward(s, R, j);
-    } else {
-        constexpr int M = SfPpT<T, ALPHA>::M, H = (T - 1) / 2;
-        const SfPpMod &P = R.mod[j];
-        ppt_forward_ld<T, M>(s, ld, R.w + (size_t)j * M, R.w_p + (size_t)j * M, R.dftc + (size_t)j * H * H * 4, P.q,
-                             P.one_p, P);
-    }
-}
-
-// inverse transform, scaled by M^-1
-template <int T, int ALPHA>
-__device__ __forceinline__ void tq_inverse(u64 *s, const SfPpRing &R, int j)
-{
-    if constexpr (T == 0) {
-        pp_inverse(s, R, j);
-    } else {
-        constexpr int M = SfPpT<T, ALPHA>::M, H = (T - 1) / 2, NT = SfPpT<T, ALPHA>::THREADS;
-        const SfPpMod &P = R.mod[j];
-        ppt_inverse<T, M, T>(s, R.iw + (size_t)j * M, R.iw_p + (size_t)j * M, R.dftc + (size_t)j * H * H * 4, P.q,
-                             P.one_p, P);
-        for (int e = threadIdx.x; e < M; e += NT) s[e] = sf_mul_shoup(s[e], P.minv, P.minv_p, P.q);
-        __syncthreads();
-    }
-}
-
 // a signed integer as a residue modulo P.q
 __device__ __forceinline__ u64 tq_lift_signed(long long v, const SfPpMod &P)
 {
     const u64 mag = v >= 0 ? (u64)v : (u64)0 - (u64)v;
     const u64 r = sf_reduce(mag, P.q, P.one_p);
     return (v < 0 && r) ? P.q - r : r;
-}
-
-// floor(x 2^64 / q) for x < q: 2^64 = one_p q + rm, and floor(x rm / q) by
-// Shoup's product with at most one correction
-__device__ __forceinline__ u64 tq_companion(u64 x, const SfPpMod &P)
-{
-    u64 h = sf_mulhi(x, P.rm_p);
-    const u64 rem = x * P.rm - h * P.q;
-    if (rem >= P.q) ++h;
-    return x * P.one_p + h;
 }
 
 // round(x D^l / 2^53) mod D^l for x < 2^53 (halves rounded up)
@@ -194,10 +137,10 @@ static size_t tq_ks_smem(const SfPpRing &R, int l)
 // transformed key values (digit i, part a / b, prime j), then their Shoup
 // companions in the same order.
 template <int T, int ALPHA>
-__global__ void __launch_bounds__(SfTqShape<T, ALPHA>::NT, SfTqShape<T, ALPHA>::MINB)
+__global__ void __launch_bounds__(SfPpShape<T, ALPHA>::NT, SfPpShape<T, ALPHA>::MINB)
     k_tq_ks(SfPpRing R, SfTqGadget G, const u64 *ct, u64 *out, int h, int hinv, const u64 *key)
 {
-    constexpr int NT = SfTqShape<T, ALPHA>::NT, EPT = (SfTqShape<T, ALPHA>::MMAX + NT - 1) / NT;
+    constexpr int NT = SfPpShape<T, ALPHA>::NT, EPT = (SfPpShape<T, ALPHA>::MMAX + NT - 1) / NT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     u64 *vec = (u64 *)smem_raw;
     u64 *res0 = vec + R.M;                      // [2][N]
@@ -230,7 +173,7 @@ __global__ void __launch_bounds__(SfTqShape<T, ALPHA>::NT, SfTqShape<T, ALPHA>::
             // digit i lifted mod p_j as the first stage reads it
             const int16_t *di = dig + (size_t)i * N;
             const u64 pq = P.q;
-            tq_forward_ld<T, ALPHA>(
+            pp_block_forward_ld<T, ALPHA>(
                 vec,
                 [di, N, pq](int e) -> u64 {
                     const int d = e < N ? di[e] : 0;
@@ -257,7 +200,7 @@ __global__ void __launch_bounds__(SfTqShape<T, ALPHA>::NT, SfTqShape<T, ALPHA>::
                 if (e < M) vec[e] = sf_reduce(part ? acc_b[x] : acc_a[x], P.q, P.one_p);
             }
             __syncthreads();
-            tq_inverse<T, ALPHA>(vec, R, j);
+            pp_block_inverse<T, ALPHA>(vec, R, j);
             for (int e = threadIdx.x; e < m; e += NT) {
                 const u64 v = vec[N + e];
                 for (int k = 0; k < R.t - 1; ++k) vec[e + k * m] = sf_sub(vec[e + k * m], v, P.q);
@@ -280,22 +223,22 @@ __global__ void __launch_bounds__(SfTqShape<T, ALPHA>::NT, SfTqShape<T, ALPHA>::
 // out[c] = a[c] s mod 2^53: a [count] torus polynomials at stride sa words,
 // s a signed polynomial (|s_e| <= SF_TQ_SECRET_BOUND); one block per polynomial
 template <int T, int ALPHA>
-__global__ void __launch_bounds__(SfTqShape<T, ALPHA>::NT)
+__global__ void __launch_bounds__(SfPpShape<T, ALPHA>::NT)
     k_tq_prod(SfPpRing R, SfTqGadget G, const u64 *a, size_t sa, const int64_t *s, u64 *out)
 {
-    constexpr int NT = SfTqShape<T, ALPHA>::NT;
+    constexpr int NT = SfPpShape<T, ALPHA>::NT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     u64 *va = (u64 *)smem_raw, *vs = va + R.M, *res0 = vs + R.M;
     const int M = R.M, N = R.N, m = R.m;
     const u64 *x = a + blockIdx.x * sa;
     for (int j = 0; j < 2; ++j) {
         const SfPpMod &P = R.mod[j];
-        tq_forward_ld<T, ALPHA>(
+        pp_block_forward_ld<T, ALPHA>(
             va, [x, N, &P](int e) -> u64 { return e < N ? sf_reduce(x[e] & SF_TQ_MASK, P.q, P.one_p) : 0; }, R, j);
-        tq_forward_ld<T, ALPHA>(vs, [s, N, &P](int e) -> u64 { return e < N ? tq_lift_signed(s[e], P) : 0; }, R, j);
+        pp_block_forward_ld<T, ALPHA>(vs, [s, N, &P](int e) -> u64 { return e < N ? tq_lift_signed(s[e], P) : 0; }, R, j);
         for (int e = threadIdx.x; e < M; e += NT) va[e] = pp_mulmod(va[e], vs[e], P);
         __syncthreads();
-        tq_inverse<T, ALPHA>(va, R, j);
+        pp_block_inverse<T, ALPHA>(va, R, j);
         for (int e = threadIdx.x; e < m; e += NT) {
             const u64 v = va[N + e];
             for (int k = 0; k < R.t - 1; ++k) va[e + k * m] = sf_sub(va[e + k * m], v, P.q);
@@ -312,23 +255,23 @@ __global__ void __launch_bounds__(SfTqShape<T, ALPHA>::NT)
 // The prepared key: grid (2 primes, 2 l polynomials); polynomial p is digit
 // p / 2, part p % 2 (ka, kb), each [l][N] torus words.
 template <int T, int ALPHA>
-__global__ void __launch_bounds__(SfTqShape<T, ALPHA>::NT)
+__global__ void __launch_bounds__(SfPpShape<T, ALPHA>::NT)
     k_tq_key_ntt(SfPpRing R, int l, const u64 *ka, const u64 *kb, u64 *key)
 {
-    constexpr int NT = SfTqShape<T, ALPHA>::NT;
+    constexpr int NT = SfPpShape<T, ALPHA>::NT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     u64 *vec = (u64 *)smem_raw;
     const int j = blockIdx.x, p = blockIdx.y, i = p / 2, part = p % 2;
     const SfPpMod &P = R.mod[j];
     const u64 *x = (part ? kb : ka) + (size_t)i * R.N;
     const int N = R.N;
-    tq_forward_ld<T, ALPHA>(
+    pp_block_forward_ld<T, ALPHA>(
         vec, [x, N, &P](int e) -> u64 { return e < N ? sf_reduce(x[e] & SF_TQ_MASK, P.q, P.one_p) : 0; }, R, j);
     u64 *dst = key + ((size_t)(i * 2 + part) * 2 + j) * R.M;
     const size_t kw = (size_t)4 * l * R.M;
     for (int e = threadIdx.x; e < R.M; e += NT) {
         dst[e] = vec[e];
-        dst[kw + e] = tq_companion(vec[e], P);
+        dst[kw + e] = pp_companion(vec[e], P);
     }
 }
 
@@ -390,16 +333,6 @@ __global__ void k_tq_add(u64 *acc, const u64 *x, size_t total)
 }
 
 // ---------------------------------------------------------------- host ----
-
-#define SF_TQ_DISPATCH(R, ...)                               \
-    do {                                                     \
-        bool done_ = false;                                  \
-        SF_PPT_DISPATCH((R).t, (R).alpha, done_, __VA_ARGS__); \
-        if (!done_) {                                        \
-            constexpr int T = 0, ALPHA = 0;                  \
-            __VA_ARGS__                                      \
-        }                                                    \
-    } while (0)
 
 static int tq_grid(size_t total) { return (int)std::min<size_t>((total + 255) / 256, 8192); }
 
@@ -478,7 +411,7 @@ extern "C" sf_status sf_tq_ring_create(int32_t t, int32_t alpha, int32_t D, int3
     // that rings of other gadgets sharing the kernel keep launching
     const int mx = 227 * 1024;
     cudaError_t err = cudaSuccess;
-    SF_TQ_DISPATCH(R, {
+    SF_PP_DISPATCH_ANY(R, {
         err = cudaFuncSetAttribute(k_tq_ks<T, ALPHA>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
         if (err == cudaSuccess)
             err = cudaFuncSetAttribute(k_tq_prod<T, ALPHA>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
@@ -531,8 +464,8 @@ static sf_status tq_prod(sf_tq_ring *r, const u64 *a, size_t sa, const int64_t *
                          cudaStream_t st)
 {
     const SfPpRing &R = r->pp->R;
-    SF_TQ_DISPATCH(R, {
-        k_tq_prod<T, ALPHA><<<count, SfTqShape<T, ALPHA>::NT, tq_prod_smem(R), st>>>(R, r->G, a, sa, s, out);
+    SF_PP_DISPATCH_ANY(R, {
+        k_tq_prod<T, ALPHA><<<count, SfPpShape<T, ALPHA>::NT, tq_prod_smem(R), st>>>(R, r->G, a, sa, s, out);
     });
     SF_CUDA_TRY(cudaGetLastError());
     return SF_OK;
@@ -593,8 +526,8 @@ extern "C" sf_status sf_tq_key_prepare(sf_tq_ring *r, const uint64_t *d_ka, cons
     SF_TRY(tq_check(r, d_ka, d_kb, 1));
     if (!d_key) return sf_set_error(SF_EINVAL, "sf_tq_key_prepare: null key");
     const SfPpRing &R = r->pp->R;
-    SF_TQ_DISPATCH(R, {
-        k_tq_key_ntt<T, ALPHA><<<dim3(2, 2 * r->G.l), SfTqShape<T, ALPHA>::NT, sizeof(u64) * R.M, (cudaStream_t)stream>>>(
+    SF_PP_DISPATCH_ANY(R, {
+        k_tq_key_ntt<T, ALPHA><<<dim3(2, 2 * r->G.l), SfPpShape<T, ALPHA>::NT, sizeof(u64) * R.M, (cudaStream_t)stream>>>(
             R, r->G.l, d_ka, d_kb, d_key);
     });
     SF_CUDA_TRY(cudaGetLastError());
@@ -606,8 +539,8 @@ static sf_status tq_keyswitch(sf_tq_ring *r, const u64 *in, u64 *out, int count,
 {
     const SfPpRing &R = r->pp->R;
     const size_t sm = tq_ks_smem(R, r->G.l);
-    SF_TQ_DISPATCH(R, {
-        k_tq_ks<T, ALPHA><<<count, SfTqShape<T, ALPHA>::NT, sm, st>>>(R, r->G, in, out, h, hinv, key);
+    SF_PP_DISPATCH_ANY(R, {
+        k_tq_ks<T, ALPHA><<<count, SfPpShape<T, ALPHA>::NT, sm, st>>>(R, r->G, in, out, h, hinv, key);
     });
     SF_CUDA_TRY(cudaGetLastError());
     return SF_OK;
