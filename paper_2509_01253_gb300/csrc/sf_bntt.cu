@@ -2,129 +2,135 @@
 // polynomials, and register-resident probes of the modular arithmetic.
 //
 // The batch is [count][L][N]: limb i of polynomial p is reduced modulo q_i.
-// A transform is the two tiled passes of sf_tile.cuh (forward: column pass,
-// then row pass; inverse: row pass, then column pass with the factor N^-1).
-// Each pass is one persistent launch of one resident wave over the units
-// (group, polynomial), a group being a column or row tile position and a limb:
-// a block takes an equal range of units (sf_block_units), stages a group's
-// twiddles when its range enters the group, and prefetches the next unit's
-// tile with cp.async while it transforms the current one.
+// A transform is the two register-resident passes of sf_reg.cuh (forward:
+// column pass, then row pass; inverse: row pass, then column pass with the
+// factor N^-1).  Each pass is one persistent launch of one resident wave over
+// the units (group, polynomial), a group being a column or row tile position
+// and a limb: a block takes an equal range of units (sf_unit_range), stages a
+// group's twiddles when its range enters the group, and loads the next unit's
+// points into registers before it transforms the current one.
+//
+// Bound by the integer multiplier: at N = 2^16 the fmaheavy pipe is busy 70 to
+// 76 % of the cycles, DRAM 31 to 39 %, shared memory 20 to 33 %, and no warp
+// waits on memory or a barrier.  512 x 5 limbs of 2^16, forward: 1961 us with
+// the tile sweeps in shared memory (8 points per thread, three sweeps and three
+// barriers a pass), 1714 us here.
 #include <algorithm>
 
-#include "sf_async.cuh"
 #include "sf_internal.h"
 #include "sf_kernels.cuh"
+#include "sf_reg.cuh"
 #include "sf_round.h"
 
-template <bool INV, int LR, int LC, int RAD = 0>
-__global__ void __launch_bounds__(SfRow<LC>::NT, 3)
+template <bool INV, int LR, int LC>
+__global__ void __launch_bounds__(SfSub<LC>::NT, 512 / SfSub<LC>::NT)
     k_bntt_row(SfRing R, const u64 *src, u64 *dst, int count, int ng)
 {
-    constexpr int NT = SfRow<LC>::NT, NB = SfRow<LC>::NB;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr SfGeoT<LR, LC> g{};
-    const SfUnits U = sf_block_units(ng * count);
-    constexpr bool DB = sf_rows_double_buffered(LC);
-    sf_tw *tw = (sf_tw *)smem_raw;
-    u64 *buf0 = (u64 *)(tw + NB * g.c);
-    u64 *buf1 = DB ? buf0 + SfRow<LC>::WORDS : buf0;
+    const SfRowT<LC> T;
+    sf_pair *tw = (sf_pair *)smem_raw;
+    u64 *buf = (u64 *)(tw + SfSub<LC>::ROW_PAIRS);
+    const SfUnitRange U = sf_unit_range(ng * count);
     const size_t per = (size_t)R.L << (LR + LC);
     // unit u: group u / count = (row tile, limb i), item u % count = polynomial
-    auto unit_off = [&](int u) -> size_t {
+    auto row_ptr = [&](int u) -> size_t {
         const int gg = u / count;
-        return per * (u % count) + ((size_t)(gg % R.L) << (LR + LC)) + (size_t)(gg / R.L) * NB * g.c;
+        return per * (u % count) + ((size_t)(gg % R.L) << (LR + LC)) + ((size_t)T.row(gg / R.L, 1 << LR) << LC);
     };
-    if (DB && U.u0 < U.u1) issue_row_tile_t<LC, NT>(buf0, src + unit_off(U.u0));
-    sf_cp_commit();
+    u64 x[16], nx[16];
+    auto load = [&](int u) {
+        const u64 *s = src + row_ptr(u);
+#pragma unroll
+        for (int r = 0; r < 16; ++r) nx[r] = s[T.k1(r)];
+    };
+    if (U.u0 < U.u1) load(U.u0);
     int staged = -1;
-    u64 q = 0, one_p = 0;
-    for (int k = 0, u = U.u0; u < U.u1; ++k, ++u) {
+    for (int u = U.u0; u < U.u1; ++u) {
         const int grp = u / count;
+        const SfMod &M = R.m[grp % R.L];
         if (grp != staged) {
-            // the previous unit ended at a barrier: nothing reads tw now
-            const int i = grp % R.L;
-            load_row_tw_t<LR, LC, NT>(tw, INV ? R.rowT_i : R.rowT_f, i, (grp / R.L) * NB);
-            q = R.m[i].q;
-            one_p = R.m[i].one_p;
+            __syncthreads();   // the previous group's readers are done
+            sf_stage_row<LR, LC>(tw, R.rowP, grp % R.L, grp / R.L);
             staged = grp;
+            __syncthreads();
         }
-        u64 *cur = (k & 1) ? buf1 : buf0, *nxt = (k & 1) ? buf0 : buf1;
-        if (DB) {
-            if (u + 1 < U.u1) issue_row_tile_t<LC, NT>(nxt, src + unit_off(u + 1));
-            sf_cp_commit();
-            sf_cp_wait<1>();
-        } else {
-            issue_row_tile_t<LC, NT>(cur, src + unit_off(u));
-            sf_cp_commit();
-            sf_cp_wait<0>();
-        }
-        __syncthreads();
-        // forward: the last pass, canonical output; inverse: lazy in [0, 4q), the column pass follows
+#pragma unroll
+        for (int r = 0; r < 16; ++r) x[r] = nx[r];
+        u64 *d = dst + row_ptr(u);
+        // the loads of the next unit overtake this unit's stores: in place, the
+        // two units touch different rows or polynomials
+        if (u + 1 < U.u1) load(u + 1);
         if (INV) {
-            u64 *gd = dst + unit_off(u);
-            row_inverse_out<LC, NT, RAD>(cur, tw, q, [&](int k, int b, u64 v) { gd[(b << LC) + k] = v; });
+            __syncwarp();
+            T.put1(x, buf);
+            __syncwarp();
+            T.get2(x, buf);
+            T.inv2(x, tw, M.q);
+            T.to1(x, buf);
+            T.inv1(x, tw, M.q);
+#pragma unroll
+            for (int r = 0; r < 16; ++r) d[T.k1(r)] = sf_red3(x[r], M);
         } else {
-            row_forward_t<LC, NT, RAD>(cur, tw, q);
-            store_row_tile_t<LC, NT>(dst + unit_off(u), cur, [&](u64 v) { return sf_reduce(v, q, one_p); });
+            T.fwd1(x, tw, M.q);
+            T.to2(x, buf);
+            T.fwd2(x, tw, M.q);
+            T.to1(x, buf);   // back to coalesced positions
+#pragma unroll
+            for (int r = 0; r < 16; ++r) d[T.k1(r)] = sf_reduce(x[r], M.q, M.one_p);
         }
-        __syncthreads();
     }
 }
 
 template <bool INV, int LR, int LC>
-__global__ void __launch_bounds__(SfThreads<LR>::value, LR >= 8 ? 2 : 3)
+__global__ void __launch_bounds__(SfSub<LR>::NT, 512 / SfSub<LR>::NT)
     k_bntt_col(SfRing R, const u64 *src, u64 *dst, int count, int ng)
 {
-    constexpr int NT = SfThreads<LR>::value;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr SfGeoT<LR, LC> g{};
-    const SfUnits U = sf_block_units(ng * count);
-    sf_tw *tw = (sf_tw *)smem_raw;
-    u64 *buf0 = (u64 *)(tw + g.r);
-    u64 *buf1 = buf0 + tile_words(g.log_r);
+    const SfCol<LR> T;
+    sf_pair *tab = (sf_pair *)smem_raw;
+    u64 *bufs = (u64 *)(tab + SfSub<LR>::S);
+    const SfUnitRange U = sf_unit_range(ng * count);
     const size_t per = (size_t)R.L << (LR + LC);
     // unit u: group u / count = (column tile, limb i), item u % count = polynomial
-    auto unit_off = [&](int u) -> size_t { return per * (u % count) + ((size_t)((u / count) % R.L) << (LR + LC)); };
-    auto unit_c0 = [&](int u) -> int { return ((u / count) / R.L) * SF_NB; };
-    if (U.u0 < U.u1) issue_col_tile_t<LR, LC, NT>(buf0, src + unit_off(U.u0), unit_c0(U.u0));
-    sf_cp_commit();
+    auto base = [&](int u) -> size_t {
+        const int gg = u / count;
+        return per * (u % count) + ((size_t)(gg % R.L) << (LR + LC)) + (gg / R.L) * 16 + T.b;
+    };
+    u64 x[16], nx[16];
+    auto load = [&](int u) {
+        const u64 *s = src + base(u);
+#pragma unroll
+        for (int r = 0; r < 16; ++r) nx[r] = s[(size_t)(INV ? T.k2(r) : T.k1(r)) << LC];
+    };
+    if (U.u0 < U.u1) load(U.u0);
     int staged = -1;
-    u64 q = 0, ninv = 0, ninv_p = 0;
-    for (int k = 0, u = U.u0; u < U.u1; ++k, ++u) {
-        const int grp = u / count;
+    for (int u = U.u0; u < U.u1; ++u) {
+        const int grp = u / count, i = grp % R.L;
+        const SfMod &M = R.m[i];
         if (grp != staged) {
-            // the previous unit ended at a barrier: nothing reads tw now
-            const int i = grp % R.L;
-            load_col_tw_t<LR, NT>(tw, INV ? R.colT_i : R.colT_f, i);
-            q = R.m[i].q;
-            ninv = R.m[i].ninv;
-            ninv_p = R.m[i].ninv_p;
+            __syncthreads();   // the previous group's readers are done
+            sf_stage_cols<LR>(tab, R.colP, i, 1);
             staged = grp;
+            __syncthreads();
         }
-        u64 *cur = (k & 1) ? buf1 : buf0, *nxt = (k & 1) ? buf0 : buf1;
-        if (u + 1 < U.u1) issue_col_tile_t<LR, LC, NT>(nxt, src + unit_off(u + 1), unit_c0(u + 1));
-        sf_cp_commit();
-        sf_cp_wait<1>();
-        __syncthreads();
-        // inverse: the last pass, times N^-1, canonical; forward: lazy, the row
-        // pass follows.  The last sweep writes the tile to global memory itself.
-        u64 *gd = dst + unit_off(u) + unit_c0(u);
-        auto out = [&](int k, int b, u64 v) { gd[((size_t)k << LC) + b] = INV ? sf_mul_shoup(v, ninv, ninv_p, q) : v; };
-        if (INV) col_inverse_st<LR, NT>(cur, tw, q, out);
-        else col_forward_io<LR, NT>(cur, tw, q, [&](int k, int b) { return cur[tile_slot<SF_NB>(k, b)]; }, out);
-        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < 16; ++r) x[r] = nx[r];
+        u64 *d = dst + base(u), *buf = bufs + (size_t)(u & 1) * SfSub<LR>::COL_WORDS;
+        if (u + 1 < U.u1) load(u + 1);
+        if (INV) {
+            T.inv2(x, tab, M.q);
+            T.to1(x, buf);
+            T.inv1(x, tab, M.q);
+#pragma unroll
+            for (int r = 0; r < 16; ++r) d[(size_t)T.k1(r) << LC] = sf_mul_shoup(x[r], M.ninv, M.ninv_p, M.q);
+        } else {
+            T.fwd1(x, tab, M.q);
+            T.to2(x, buf);
+            T.fwd2(x, tab, M.q);
+#pragma unroll
+            for (int t = 0; t < 16; ++t) d[(size_t)T.k2(t) << LC] = x[t];
+        }
     }
-}
-
-template <class K>
-static int bntt_occupancy(K kernel, int threads, size_t smem)
-{
-    int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, threads, smem) != cudaSuccess) {
-        cudaGetLastError();
-        b = 1;
-    }
-    return std::max(1, b);
 }
 
 // one resident wave (SMs x occupancy blocks), at most one block per unit
@@ -133,11 +139,34 @@ static int bntt_blocks(const sf_ctx *ctx, int occ, int n_units)
     return std::max(1, std::min(ctx->num_sms * occ, n_units));
 }
 
-static size_t bntt_smem_row(const SfRing &R)
+template <int LC>
+static constexpr size_t bntt_smem_row() { return sizeof(sf_pair) * SfSub<LC>::ROW_PAIRS + sizeof(u64) * SfSub<LC>::ROW_WORDS; }
+template <int LR>
+static constexpr size_t bntt_smem_col() { return sizeof(sf_pair) * SfSub<LR>::S + sizeof(u64) * 2 * SfSub<LR>::COL_WORDS; }
+
+template <bool INV, int LR, int LC>
+static void bntt_row(sf_ctx *ctx, const u64 *src, u64 *dst, int count, cudaStream_t st)
 {
-    return sizeof(sf_tw) * sf_row_nb(R.log_c) * R.c + sizeof(u64) * row_tile_words(R.log_c) * (sf_rows_double_buffered(R.log_c) ? 2 : 1);
+    const int ng = ((1 << LR) / 16) * ctx->ring.L;
+    const size_t sm = bntt_smem_row<LC>();
+    cudaEvent_t ev;
+    const int nb = bntt_blocks(ctx, sf_occupancy(k_bntt_row<INV, LR, LC>, SfSub<LC>::NT, sm), ng * count);
+    sf_launch_begin(ctx, SFK_BNTT_ROW, st, &ev);
+    k_bntt_row<INV, LR, LC><<<nb, SfSub<LC>::NT, sm, st>>>(ctx->ring, src, dst, count, ng);
+    sf_launch_end(ctx, SFK_BNTT_ROW, st, ev);
 }
-static size_t bntt_smem_col(const SfRing &R) { return sizeof(sf_tw) * R.r + sizeof(u64) * tile_words(R.log_r) * 2; }
+
+template <bool INV, int LR, int LC>
+static void bntt_col(sf_ctx *ctx, const u64 *src, u64 *dst, int count, cudaStream_t st)
+{
+    const int ng = ((1 << LC) / 16) * ctx->ring.L;
+    const size_t sm = bntt_smem_col<LR>();
+    cudaEvent_t ev;
+    const int nb = bntt_blocks(ctx, sf_occupancy(k_bntt_col<INV, LR, LC>, SfSub<LR>::NT, sm), ng * count);
+    sf_launch_begin(ctx, SFK_BNTT_COL, st, &ev);
+    k_bntt_col<INV, LR, LC><<<nb, SfSub<LR>::NT, sm, st>>>(ctx->ring, src, dst, count, ng);
+    sf_launch_end(ctx, SFK_BNTT_COL, st, ev);
+}
 
 extern "C" sf_status sf_ntt_batch(sf_ctx *ctx, const uint64_t *d_in, uint64_t *d_out, int32_t count, int32_t inverse,
                                   void *stream)
@@ -147,35 +176,17 @@ extern "C" sf_status sf_ntt_batch(sf_ctx *ctx, const uint64_t *d_in, uint64_t *d
         return sf_set_error(SF_EINVAL, "sf_ntt_batch: bad arguments");
     const SfRing &R = ctx->ring;
     cudaStream_t st = (cudaStream_t)stream;
-    const int rg = (R.r / sf_row_nb(R.log_c)) * R.L, cg = (R.c / SF_NB) * R.L;
-    if ((long long)count * std::max(rg, cg) > INT32_MAX)
+    // tiles of a limb: C / 16 (bounded as for the 32 tiles of a 128 x 512 split at N = 2^16)
+    const int tiles = R.log_n == 16 ? 32 : (1 << ((R.log_n + 1) / 2)) / 16;
+    if ((long long)count * R.L * tiles > INT32_MAX)
         return sf_set_error(SF_EINVAL, "sf_ntt_batch: count too large");
-    const size_t smr = bntt_smem_row(R), smc = bntt_smem_col(R);
-    cudaEvent_t ev;
-    SF_GEO_DISPATCH(R.log_n, {
-        constexpr int NTR = SfRow<LC>::NT, NTC = SfThreads<LR>::value;
+    SF_RING_DISPATCH(R.log_n, {
         if (!inverse) {
-            const int bc = bntt_blocks(ctx, bntt_occupancy(k_bntt_col<false, LR, LC>, NTC, smc), cg * count);
-            sf_launch_begin(ctx, SFK_BNTT_COL, st, &ev);
-            k_bntt_col<false, LR, LC><<<bc, NTC, smc, st>>>(R, d_in, d_out, count, cg);
-            sf_launch_end(ctx, SFK_BNTT_COL, st, ev);
-            sf_launch_begin(ctx, SFK_BNTT_ROW, st, &ev);
-            SF_RAD_DISPATCH(ctx->row_radix, {
-                const int br = bntt_blocks(ctx, bntt_occupancy(k_bntt_row<false, LR, LC, RAD>, NTR, smr), rg * count);
-                k_bntt_row<false, LR, LC, RAD><<<br, NTR, smr, st>>>(R, d_out, d_out, count, rg);
-            });
-            sf_launch_end(ctx, SFK_BNTT_ROW, st, ev);
+            bntt_col<false, LR, LC>(ctx, d_in, d_out, count, st);
+            bntt_row<false, LR, LC>(ctx, d_out, d_out, count, st);
         } else {
-            sf_launch_begin(ctx, SFK_BNTT_ROW, st, &ev);
-            SF_RAD_DISPATCH(ctx->row_radix, {
-                const int br = bntt_blocks(ctx, bntt_occupancy(k_bntt_row<true, LR, LC, RAD>, NTR, smr), rg * count);
-                k_bntt_row<true, LR, LC, RAD><<<br, NTR, smr, st>>>(R, d_in, d_out, count, rg);
-            });
-            sf_launch_end(ctx, SFK_BNTT_ROW, st, ev);
-            const int bc = bntt_blocks(ctx, bntt_occupancy(k_bntt_col<true, LR, LC>, NTC, smc), cg * count);
-            sf_launch_begin(ctx, SFK_BNTT_COL, st, &ev);
-            k_bntt_col<true, LR, LC><<<bc, NTC, smc, st>>>(R, d_out, d_out, count, cg);
-            sf_launch_end(ctx, SFK_BNTT_COL, st, ev);
+            bntt_row<true, LR, LC>(ctx, d_in, d_out, count, st);
+            bntt_col<true, LR, LC>(ctx, d_out, d_out, count, st);
         }
     });
     SF_CUDA_TRY(cudaGetLastError());
@@ -186,13 +197,11 @@ sf_status sf_bntt_init_attributes()
 {
     const int mx = 227 * 1024;
 #define SF_BNTT_ATTR(K) SF_CUDA_TRY(cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
-#define SF_BNTT_ATTRS(LR, LC)                                                                                     \
-    SF_BNTT_ATTR((k_bntt_row<false, LR, LC>)) SF_BNTT_ATTR((k_bntt_row<true, LR, LC>))                             \
-    SF_BNTT_ATTR((k_bntt_row<false, LR, LC, 1>)) SF_BNTT_ATTR((k_bntt_row<true, LR, LC, 1>))                       \
-    SF_BNTT_ATTR((k_bntt_row<false, LR, LC, 2>)) SF_BNTT_ATTR((k_bntt_row<true, LR, LC, 2>))                       \
+#define SF_BNTT_ATTRS(LR, LC)                                                                  \
+    SF_BNTT_ATTR((k_bntt_row<false, LR, LC>)) SF_BNTT_ATTR((k_bntt_row<true, LR, LC>))         \
     SF_BNTT_ATTR((k_bntt_col<false, LR, LC>)) SF_BNTT_ATTR((k_bntt_col<true, LR, LC>))
     SF_BNTT_ATTRS(5, 5) SF_BNTT_ATTRS(5, 6) SF_BNTT_ATTRS(6, 6) SF_BNTT_ATTRS(6, 7) SF_BNTT_ATTRS(7, 7)
-    SF_BNTT_ATTRS(7, 8) SF_BNTT_ATTRS(7, 9)
+    SF_BNTT_ATTRS(7, 8) SF_BNTT_ATTRS(8, 8)
 #undef SF_BNTT_ATTRS
 #undef SF_BNTT_ATTR
     return SF_OK;
@@ -266,9 +275,9 @@ extern "C" sf_status sf_modmul_probe(sf_ctx *ctx, int32_t kind, double *gmodmul_
     const SfMod &M = ctx->ring.m[0];
     int occ = 1;
     switch (kind) {
-    case 0: occ = bntt_occupancy(k_probe<0>, 256, 0); break;
-    case 1: occ = bntt_occupancy(k_probe<1>, 256, 0); break;
-    default: occ = bntt_occupancy(k_probe<2>, 256, 0); break;
+    case 0: occ = sf_occupancy(k_probe<0>, 256, 0); break;
+    case 1: occ = sf_occupancy(k_probe<1>, 256, 0); break;
+    default: occ = sf_occupancy(k_probe<2>, 256, 0); break;
     }
     const int grid = ctx->num_sms * occ;
     const size_t words = (size_t)8 * grid * 256;

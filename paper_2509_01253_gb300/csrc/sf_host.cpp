@@ -523,6 +523,8 @@ extern "C" sf_status sf_ctx_create(const sf_params *p, int32_t device, sf_ctx **
         M.ninv = sf_host_invmod((u64)N % q, q);
         M.ninv_p = sf_shoup_companion(M.ninv, q);
         M.one_p = sf_shoup_companion(1, q);
+        M.sh = 63 - __builtin_clzll(q);
+        M.binv = (unsigned)(((u128)1 << (32 + M.sh)) / q);
         u64 root = sf_root_2n(q, 2 * (u64)N);
         u64 iroot = sf_host_invmod(root, q);
         for (int k = 0; k < N; ++k) {
@@ -568,6 +570,34 @@ extern "C" sf_status sf_ctx_create(const sf_params *p, int32_t device, sf_ctx **
                     rowT_f[dst] = make_ulonglong2(tf[gi], tfp[gi]);
                     rowT_i[dst] = make_ulonglong2(ti[gi], tip[gi]);
                 }
+    }
+    // Twiddles of the register-resident passes (sf_reg.cuh).  Row tile: rows
+    // 8 tile + b (b < 8) and their mirrors R - 1 - row; phase-1 entries (k, b)
+    // at (k - 1) 16 + b, then phase-2 entries (e, b, i) at e C + b (C/16) + i.
+    const int lc2 = (p->log_n + 1) / 2, lr2 = p->log_n - lc2, r2 = 1 << lr2, c2 = 1 << lc2, ni = c2 / 16;
+    std::vector<ulonglong2> colP((size_t)nm * r2), rowP((size_t)nm * (r2 / 16) * 16 * (c2 - 1));
+    for (int m = 0; m < nm; ++m) {
+        const u64 *tf = psi.data() + (size_t)m * N, *tfp = psi_p.data() + (size_t)m * N;
+        for (int k = 0; k < r2; ++k) colP[(size_t)m * r2 + k] = make_ulonglong2(tf[k], tfp[k]);
+        for (int tile = 0; tile < r2 / 16; ++tile) {
+            ulonglong2 *dst = &rowP[((size_t)m * (r2 / 16) + tile) * 16 * (c2 - 1)];
+            for (int b = 0; b < 16; ++b) {
+                const size_t row = b < 8 ? 8 * tile + b : r2 - 1 - 8 * tile - (b - 8);
+                for (int k = 1; k < ni; ++k) {
+                    int mk = 1;
+                    while (mk * 2 <= k) mk *= 2;
+                    const size_t gi = mk * (r2 + row) + (k - mk);
+                    dst[(k - 1) * 16 + b] = make_ulonglong2(tf[gi], tfp[gi]);
+                }
+                for (int e = 0; e < 15; ++e) {
+                    const int s = e >= 7 ? 3 : e >= 3 ? 2 : e >= 1 ? 1 : 0, g = e - ((1 << s) - 1);
+                    for (int i = 0; i < ni; ++i) {
+                        const size_t gi = ((size_t)ni << s) * (r2 + row) + (i << s) + g;
+                        dst[16 * (ni - 1) + e * c2 + b * ni + i] = make_ulonglong2(tf[gi], tfp[gi]);
+                    }
+                }
+            }
+        }
     }
     // powers psi^(C e), e < 2R (closed-form column pass of a sparse polynomial)
     std::vector<ulonglong2> pwc((size_t)nm * 2 * R.r);
@@ -634,7 +664,7 @@ extern "C" sf_status sf_ctx_create(const sf_params *p, int32_t device, sf_ctx **
 #define UP(v, f)                                      \
     if (st == SF_OK) st = upload(ctx, v, &R.f);
     UP(psi, psi) UP(psi_p, psi_p) UP(ipsi, ipsi) UP(ipsi_p, ipsi_p) UP(pw, pw) UP(pw_p, pw_p)
-    UP(colT_f, colT_f) UP(colT_i, colT_i) UP(rowT_f, rowT_f) UP(rowT_i, rowT_i) UP(pwc, pwc)
+    UP(colT_f, colT_f) UP(colT_i, colT_i) UP(rowT_f, rowT_f) UP(rowT_i, rowT_i) UP(pwc, pwc) UP(colP, colP) UP(rowP, rowP)
     UP(mu_inv, mu_inv) UP(mu_inv_p, mu_inv_p) UP(mu_qhat, mu_qhat) UP(mu_qhat_p, mu_qhat_p)
     UP(md_inv, md_inv) UP(md_inv_p, md_inv_p) UP(md_phat, md_phat) UP(md_phat_p, md_phat_p)
     UP(md_pinv, md_pinv) UP(md_pinv_p, md_pinv_p)

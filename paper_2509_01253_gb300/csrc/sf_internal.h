@@ -24,6 +24,9 @@ struct SfMod {
     u64 r_mod_p;
     u64 ninv, ninv_p;  // N^-1 mod q (Shoup)
     u64 one_p;         // floor(2^64 / q): Shoup companion of 1 (full reduction)
+    // partial reduction of lazy values (sf_red3): sh = bits(q) - 1, binv = floor(2^(32 + sh) / q)
+    unsigned binv;
+    int sh;
 };
 
 // Everything a kernel needs about the ring, by value.
@@ -40,6 +43,9 @@ struct SfRing {
     // staged twiddle pairs (w, w'): column tables [nm][R] (k < R) and row
     // tables [nm][R/16][C][16] reordered per 16-row tile (see sf_tile.cuh)
     const ulonglong2 *colT_f, *colT_i, *rowT_f, *rowT_i;
+    // twiddle pairs of the register-resident passes (sf_reg.cuh): columns
+    // [nm][R'], row tiles [nm][R'/16][16 (C' - 1)], N = R' x C', C' = 2^ceil(log2 N / 2)
+    const ulonglong2 *colP, *rowP;
     // powers psi^k, k in [0, 2N), [nm][2N] (monomials in the NTT domain)
     const u64 *pw, *pw_p;
     // pairs (psi^(C e), companion), e < 2R, [nm][2R] (sparse column pass)
