@@ -252,8 +252,7 @@ class RingShape:
         self.L, self.K, self.dnum = p_info["n_data"], p_info["n_special"], p_info["dnum"]
         self.nm = self.L + self.K
         log_n = self.n.bit_length() - 1
-        # the library's split N = R x C (2^16 = 128 x 512)
-        self.lc = 9 if log_n == 16 else (log_n + 1) // 2
+        self.lc = (log_n + 1) // 2   # the library's split N = R x C
         self.lr = log_n - self.lc
         self.digits = [min(self.K, self.L - j * self.K) for j in range(self.dnum)]
 
@@ -265,7 +264,11 @@ def kernel_ops(kernel: str, g: RingShape, k_in: int = 1):
     (key switches) for the ks* kernels, (output, input ciphertext) pairs for
     leaf_col and outputs for leaf_row.  A one-limb ModUp digit converts with
     no product (its residue is the value), and the ModDown factor P^-1 rides
-    on the key and the conversion constants, so the finish has no product."""
+    on the key and the conversion constants.  Counted for a merge of NTT-domain
+    operands (the first level above the leaves); one of coefficient-domain
+    operands runs the forward transforms of the digits' own limbs in the
+    ks2 and ks3 kernels instead of ks1's and ks2's inverse ones: the same
+    number of butterflies."""
     N, L, K, nm, dnum, lr, lc = g.n, g.L, g.K, g.nm, g.dnum, g.lr, g.lc
     half = N // 2
     fbc_up = sum(d * (nm - d) for d in g.digits if d > 1) * N
@@ -274,10 +277,11 @@ def kernel_ops(kernel: str, g: RingShape, k_in: int = 1):
         "ks_gather": (0, 0, 4 * L * N),
         "ks1_inv_row": (0, L * half * lc, 0),
         "ks2_modup_col": (ext * half * lr, L * half * lr, L * N + fbc_up),
-        "ks3_inner_row": (ext * half * lc, 0, 2 * dnum * nm * N),
-        "ks3_inv_row_p": (0, 2 * K * half * lc, 0),
-        "ks4_moddown_col": (2 * L * half * lr, 2 * K * half * lr, 2 * K * N + 2 * K * L * N),
-        "ks5_finish_row": (2 * L * half * lc, 0, 0),
+        "ks3_inner_row": (ext * half * lc, 2 * nm * half * lc, 2 * dnum * nm * N),
+        "ks4_moddown_col": (0, 2 * nm * half * lr, 2 * K * N + 2 * (K + 1) * L * N),
+        # kernels of the seven-kernel key switch that the three above took in
+        "ks3_inv_row_p": (0, 0, 0),
+        "ks5_finish_row": (0, 0, 0),
         "leaf_col": (L * half * lr, 0, 0),
         "leaf_row": (k_in * L * half * lc, 0, 2 * k_in * L * N),
     }
@@ -299,10 +303,10 @@ def kernel_work(kernel: str, g: RingShape, k_in: int = 1):
         "ks1_inv_row": 2 * L * N * w,
         "ks2_modup_col": dnum * nm * N * w,
         "ks3_inner_row": (dnum * nm + 2 * nm) * N * w,
-        "ks3_inv_row_p": 4 * K * N * w,
-        "ks4_moddown_col": (2 * K + 2 * L) * N * w,
-        # read conv, acc and out (2L limbs each), write out
-        "ks5_finish_row": 8 * L * N * w,
+        # read the accumulators and out, write out
+        "ks4_moddown_col": (2 * nm + 4 * L) * N * w,
+        "ks3_inv_row_p": 0,
+        "ks5_finish_row": 0,
         "leaf_col": L * N * w,
         "leaf_row": (k_in * L + 2 * L) * N * w,
     }.get(kernel)
@@ -344,10 +348,6 @@ def load_peaks():
 # items), kept only while the kernel's code is unchanged since the capture;
 # scaled to a full launch by its items
 TRAFFIC_PER_ITEM = {
-    # k_ks3 at N = 2^16 (5 + 2 primes), 128 x 512 split: one launch of 128
-    # merges of the small r34 case (--small, ks_batch=128), 1.636432 GB read +
-    # 0.849524 GB written
-    ("ks3_inner_row", 16): (1.636432e9 + 0.849524e9) / 128,
 }
 
 

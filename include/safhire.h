@@ -110,22 +110,10 @@ void sf_ctx_destroy(sf_ctx *ctx);
 
 /* Tuning and instrumentation knobs (name, value):
  *   "ks_batch"      merges per key-switch batch (1..4096; default chosen per N)
- *   "leaf_sparse"   taps per 16-column tile up to which the leaf column pass
- *                   evaluates the sparse weight polynomial in closed form
- *                   instead of running the transform (-1: 8 log2 R, where the
- *                   closed form has fewer multiplications; 0: always the
- *                   transform, the default; at most 128)
- *   "ks3_threads"   threads per block of the key-switch inner product when
- *                   the NTT's rows have 128 points (N = 2^13, 2^14): 256
- *                   (8 residues per thread, the default) or 512 (4 per
- *                   thread, radix-4 row sweeps)
- *   "row_radix"     sweep schedule of the row passes of the key-switch and
- *                   leaf kernels: 0 radix-8 sweeps (the default), 1 radix-4
- *                   sweeps, 2 radix-8 sweeps with the two sweeps nearest
- *                   the rows' short butterflies of 256- and 512-point rows
- *                   run back to back in registers, the lanes of a warp
- *                   trading values by shuffles in between (other row
- *                   lengths as 0); every schedule gives identical residues
+ *   "leaf_sparse"   (-1 .. 128), "ks3_threads" (256 or 512), "row_radix" (0 .. 2)
+ *                   select among kernel forms that one form has replaced: the
+ *                   values are accepted and read back, every value runs the
+ *                   same kernels and gives the same residues
  *   "leaf_chunk"    cap on the leaves per packing unit (power of two): a group
  *                   of n leaves is packed as n/CH residue classes of CH leaves
  *                   reduced to roots, then the roots finish the tree
@@ -346,14 +334,9 @@ sf_status sf_eval_layers_gamma(sf_ctx *ctx, int32_t n_layers, const sf_layer *co
 
 /* Autotuner: times sf_eval_layers on the given rounds (which it evaluates,
  * results valid), `repeats` timed runs per candidate after a warm-up:
- * first each key-switch launch batch (32 ... 4096 merges; those above 512
- * only while their key-switch workspace stays within 16 GiB), then, with the
- * best batch, the leaf column pass of sparse tiles in closed form or as a
- * transform ("leaf_sparse" -1 or 0), then, for rings with 128-point rows,
- * the block shape of the key-switch inner product ("ks3_threads" 256 or
- * 512), then the row-pass schedule ("row_radix" 0, 1, 2).  Keeps the
- * fastest choices in the context and reports the batch with the best time
- * in milliseconds.
+ * each key-switch launch batch (32 ... 4096 merges; those above 512 only while
+ * their key-switch workspace stays within 16 GiB).  Keeps the fastest choice in
+ * the context and reports it with its time in milliseconds.
  * Synchronises `stream`. */
 sf_status sf_autotune_layers(sf_ctx *ctx, int32_t n_layers, const sf_layer *const *layers, const sf_rotkeys *const *rks,
                              const uint64_t *const *d_ins, const int32_t *k_ins, const uint32_t *const *h_sigma_prevs,

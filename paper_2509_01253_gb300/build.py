@@ -16,7 +16,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_safhire.so")
 BUILD_DIR = os.path.join(HERE, "_build")
-SOURCES = ["sf_host.cpp", "sf_ntt.cu", "sf_ks.cu", "sf_layer.cu", "sf_api.cu", "sf_engine.cu", "sf_noalloc.cu", "sf_pp.cu",
+SOURCES = ["sf_host.cpp", "sf_ntt.cu", "sf_ks.cu", "sf_ks_up.cu", "sf_ks_rows.cu", "sf_ks_down.cu", "sf_layer.cu", "sf_api.cu", "sf_engine.cu", "sf_noalloc.cu", "sf_pp.cu",
            "sf_bntt.cu", "sf_tq.cu"]
 GENCODE = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

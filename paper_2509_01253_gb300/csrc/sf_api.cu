@@ -95,7 +95,7 @@ extern "C" sf_status sf_gen_rotation_keys(sf_ctx *ctx, const sf_secret_key *sk, 
     rk->ctx = ctx;
     rk->gen = sf_next_generation();
     rk->d = ds;
-    // per key: values [dnum][2][nm][N] (NTT domain), then their Shoup companions
+    // per key: pairs [dnum][2][nm][N] of the NTT-domain values, storage order
     rk->key_words = (size_t)2 * R.dnum * 2 * R.nm * R.n;
     sf_status st = device_buffer((void **)&rk->d_keys, sizeof(u64) * rk->key_words * ds.size());
     u64 *d_alpha = nullptr, *d_e = nullptr;
@@ -128,12 +128,12 @@ extern "C" sf_status sf_gen_rotation_keys(sf_ctx *ctx, const sf_secret_key *sk, 
                 for (int k = 0; k < R.K; ++k) v = sf_host_mulmod(v, p->mods[R.L + k] % p->mods[m], p->mods[m]);
                 pg[m] = v;
             }
-            u64 *ka = rk->d_keys + rk->key_words * t + (size_t)(j * 2 + 0) * R.nm * R.n;
-            u64 *kb = rk->d_keys + rk->key_words * t + (size_t)(j * 2 + 1) * R.nm * R.n;
+            ulonglong2 *key = (ulonglong2 *)(rk->d_keys + rk->key_words * t);
+            ulonglong2 *ka = key + (size_t)(j * 2 + 0) * R.nm * R.n, *kb = key + (size_t)(j * 2 + 1) * R.nm * R.n;
             if (st == SF_OK) st = sf_signed_to_residues(ctx, d_ei, d_e, R.nm, R.nm, 0, 0);
             if (st == SF_OK) st = sf_ntt_jobs(ctx, jobs_a.data(), R.nm, false, 0);
             if (st == SF_OK) st = sf_ntt_jobs(ctx, jobs_e.data(), R.nm, false, 0);
-            if (st == SF_OK) st = sf_rotkey_finish(ctx, d_alpha, d_e, sk->d_s_mont, pg, ds[t], ka, kb, rk->key_words / 2, 0);
+            if (st == SF_OK) st = sf_rotkey_finish(ctx, d_alpha, d_e, sk->d_s_mont, pg, ds[t], ka, kb, 0);
             if (st == SF_OK && cudaDeviceSynchronize() != cudaSuccess) st = sf_set_error(SF_ECUDA, "keygen kernel failed");
         }
     }
@@ -170,12 +170,12 @@ extern "C" sf_status sf_rotkeys_export(sf_ctx *ctx, const sf_rotkeys *rk, int32_
     int t = key_slot(rk, d);
     if (t < 0) return sf_set_error(SF_EINVAL, "no rotation key for d = %d", d);
     const SfRing &R = ctx->ring;
-    const size_t vals = rk->key_words / 2;   // the values; the companions follow
+    const size_t vals = rk->key_words / 2;   // the values of the pairs
     void *w = nullptr;
     SF_TRY(sf_scratch(ctx, sizeof(u64) * vals, &w));
     u64 *tmp = (u64 *)w;
-    SF_CUDA_TRY(cudaMemcpy(tmp, rk->d_keys + rk->key_words * t, sizeof(u64) * vals, cudaMemcpyDeviceToDevice));
     int npol = R.dnum * 2 * R.nm;
+    SF_TRY(sf_to_natural(ctx, rk->d_keys + rk->key_words * t, 2, tmp, npol, 0));
     std::vector<SfPolyJob> jobs;
     for (int x = 0; x < npol; ++x) jobs.push_back({tmp + (size_t)x * R.n, tmp + (size_t)x * R.n, x % R.nm});
     SF_TRY(sf_ntt_jobs(ctx, jobs.data(), npol, true, 0));
@@ -430,7 +430,8 @@ extern "C" sf_status sf_linear_outputs(sf_ctx *ctx, const sf_layer *L, const uin
     Carver cv;
     size_t o_ct = cv.take((size_t)2 * k_in * ct), o_pos = cv.take(((size_t)L->E_in + 1) / 2),
            o_sig = cv.take(((size_t)n_outputs + 1) / 2), o_w1 = cv.take((size_t)LB * k_in * R.L * R.n),
-           o_lv = cv.take((size_t)n_outputs * ct), o_tap = cv.take(sf_leaf_tap_words(R, k_in, L->max_taps, LB));
+           o_in = cv.take((size_t)k_in * ct), o_lv = cv.take((size_t)n_outputs * ct), o_nat = cv.take((size_t)n_outputs * ct),
+           o_tap = cv.take(sf_leaf_tap_words(R, k_in, L->max_taps, LB));
     void *w = nullptr;
     SF_TRY(sf_scratch(ctx, cv.words * sizeof(u64), &w));
     u64 *ws = (u64 *)w;
@@ -438,7 +439,7 @@ extern "C" sf_status sf_linear_outputs(sf_ctx *ctx, const sf_layer *L, const uin
     std::vector<int> h_pos, h_sig(h_outputs, h_outputs + n_outputs);
     if (h_sigma_prev) SF_TRY(upload_perm_inverse(h_sigma_prev, L->E_in, d_pos, h_pos, st));
     SF_CUDA_TRY(cudaMemcpyAsync(d_sig, h_sig.data(), sizeof(int) * n_outputs, cudaMemcpyHostToDevice, st));
-    SF_TRY(prepare_inputs(ctx, d_in, nullptr, k_in, ws + o_ct, st));
+    SF_TRY(prepare_inputs(ctx, d_in, nullptr, k_in, ws + o_ct, ws + o_in, st));
     SfLeafParams P = leaf_params(L);
     P.k_in = k_in;
     P.pos_of = h_sigma_prev ? d_pos : nullptr;
@@ -455,9 +456,10 @@ extern "C" sf_status sf_linear_outputs(sf_ctx *ctx, const sf_layer *L, const uin
         p.leaves = ws + o_lv + (size_t)s0 * ct;
         SF_TRY(sf_leaves_launch(ctx, p, std::min(LB, n_outputs - s0), st));
     }
+    SF_TRY(sf_to_natural(ctx, ws + o_lv, 1, ws + o_nat, n_outputs * 2 * R.L, st));
     std::vector<SfPolyJob> jobs;
     for (int x = 0; x < n_outputs * 2 * R.L; ++x)
-        jobs.push_back({ws + o_lv + (size_t)x * R.n, d_out + (size_t)x * R.n, x % R.L});
+        jobs.push_back({ws + o_nat + (size_t)x * R.n, d_out + (size_t)x * R.n, x % R.L});
     SF_TRY(sf_ntt_jobs(ctx, jobs.data(), (int)jobs.size(), true, st));
     SF_CUDA_TRY(cudaStreamSynchronize(st));
     return SF_OK;
@@ -476,31 +478,21 @@ extern "C" sf_status sf_rotate(sf_ctx *ctx, const sf_rotkeys *rk, int32_t d, con
     cudaStream_t st = (cudaStream_t)stream;
     const size_t ct = ct_words(ctx);
     const int batch = std::min(ctx->ks_batch, count);
-    Carver cv;
-    size_t o_in = cv.take((size_t)count * ct), o_out = cv.take((size_t)count * ct),
-           o_ks = cv.take(sf_ks_scratch_words(R) * batch);
     void *w = nullptr;
-    SF_TRY(sf_scratch(ctx, cv.words * sizeof(u64), &w));
-    u64 *ws = (u64 *)w;
+    SF_TRY(sf_scratch(ctx, sf_ks_scratch_words(R, 0) * batch * sizeof(u64), &w));
     SF_TRY(sf_check_residues(ctx, d_ct, count * 2 * R.L, R.L, 0, st));
-    std::vector<SfPolyJob> jobs;
-    for (int x = 0; x < count * 2 * R.L; ++x) jobs.push_back({d_ct + (size_t)x * R.n, ws + o_in + (size_t)x * R.n, x % R.L});
-    SF_TRY(sf_ntt_jobs(ctx, jobs.data(), (int)jobs.size(), false, st));
     SfKsBatch b;
     memset(&b, 0, sizeof(b));
-    b.E = ws + o_in;
+    b.E = d_ct;
     b.E_stride = ct;
-    b.out = ws + o_out;
+    b.out = d_out;
     b.out_stride = ct;
     b.inner = 1 << 30;
     b.count = count;
     b.d = d;
     b.add_v = 0;
     b.key = rk->d_keys + rk->key_words * t;
-    SF_TRY(sf_ks_run(ctx, b, ws + o_ks, batch, st));
-    for (int x = 0; x < count * 2 * R.L; ++x) jobs[x] = {ws + o_out + (size_t)x * R.n, d_out + (size_t)x * R.n, x % R.L};
-    SF_TRY(sf_ntt_jobs(ctx, jobs.data(), (int)jobs.size(), true, st));
-    return SF_OK;
+    return sf_ks_run(ctx, b, (u64 *)w, batch, st);
 }
 
 static sf_status pack_impl(sf_ctx *ctx, const sf_rotkeys *rk, const uint64_t *d_leaves, int32_t n_leaves, int32_t n,
@@ -516,22 +508,19 @@ static sf_status pack_impl(sf_ctx *ctx, const sf_rotkeys *rk, const uint64_t *d_
     const int batch = std::min(ctx->ks_batch, std::max(1, n / 2));   // the widest level has n/2 merges
     Carver cv;
     size_t o_A = cv.take((size_t)n * ct), o_B = cv.take((size_t)std::max(n / 2, 1) * ct),
-           o_ks = cv.take(sf_ks_scratch_words(R) * batch);
+           o_ks = cv.take(sf_ks_scratch_words(R, 0) * batch);
     void *w = nullptr;
     SF_TRY(sf_scratch(ctx, cv.words * sizeof(u64), &w));
     u64 *ws = (u64 *)w;
-    std::vector<SfPolyJob> jobs;
-    for (int x = 0; x < n_leaves * 2 * R.L; ++x)
-        jobs.push_back({d_leaves + (size_t)x * R.n, ws + o_A + (size_t)x * R.n, x % R.L});
-    SF_TRY(sf_ntt_jobs(ctx, jobs.data(), (int)jobs.size(), false, st));
+    // the levels write back into the leaves' buffer: work on a copy of the caller's
+    SF_CUDA_TRY(cudaMemcpyAsync(ws + o_A, d_leaves, sizeof(u64) * ct * n_leaves, cudaMemcpyDeviceToDevice, st));
+    bool ntt = false;
     std::vector<int> valid(1, n_leaves);
     u64 *res = nullptr;
     size_t rs = 0;
     SF_TRY(sf_pack_tree(ctx, rk->d_keys, rk->d, rk->key_words, ws + o_A, ws + o_B, 1, n, 0, valid, true, ws + o_ks, batch,
-                        &res, &rs, st, gamma == 2));
-    jobs.clear();
-    for (int x = 0; x < 2 * R.L; ++x) jobs.push_back({res + (size_t)x * R.n, d_out + (size_t)x * R.n, x % R.L});
-    SF_TRY(sf_ntt_jobs(ctx, jobs.data(), (int)jobs.size(), true, st));
+                        &res, &rs, &ntt, st, gamma == 2));
+    SF_CUDA_TRY(cudaMemcpyAsync(d_out, res, sizeof(u64) * ct, cudaMemcpyDeviceToDevice, st));
     return SF_OK;
 }
 

@@ -7,8 +7,7 @@
 //  * Montgomery (1985) REDC with R = 2^64 for products of two variable
 //    residues: for T < q*2^64, (T + m q)/2^64 with m = T * (-q^-1) mod 2^64
 //    lies in [0, 2q) and equals T * 2^-64 mod q.
-//  * Harvey's lazy butterflies keep inverse-NTT values in [0, 4q); forward
-//    values grow by at most 4q per stage (see sf_bfly_ct), far below 2^64.
+// The lazy products and butterflies of the transforms are in sf_reg.cuh.
 #pragma once
 #include <stdint.h>
 
@@ -95,50 +94,6 @@ SF_HD u64 sf_mulhi_trunc(u64 a, u64 b)
     const u64 al = (uint32_t)a, ah = a >> 32, bl = (uint32_t)b, bh = b >> 32;
     return ah * bh + ((ah * bl) >> 32) + ((al * bh) >> 32);
 #endif
-}
-
-// Shoup's product with the truncated quotient: qhat is the exact
-// floor(x w' / 2^64) minus at most 2, so x*w - qhat*q lies in [0, 4q).
-SF_HD u64 sf_mul_shoup_lazy4(u64 x, u64 w, u64 wp, u64 q)
-{
-    return x * w - sf_mulhi_trunc(x, wp) * q;
-}
-
-// Forward (Cooley-Tukey) butterfly without reduction: with Y*w mod q taken
-// lazily in [0, 4q) (valid for any Y < 2^64), X' = X + T and Y' = X - T + 4q
-// grow the bound by at most 4q per stage.  Starting below 4q, a whole
-// transform of at most 16 stages stays below 68q < 2^58 for q < 2^51, so no
-// conditional subtraction is needed until a consumer wants canonical values
-// (every consumer reduces inputs below 2^64, or multiplies them by a residue
-// below q with a Montgomery reduction that accepts products below q 2^64).
-SF_HD void sf_bfly_ct(u64 &X, u64 &Y, u64 w, u64 wp, u64 q, u64 two_q)
-{
-    u64 t = sf_mul_shoup_lazy4(Y, w, wp, q);
-    u64 x = X;
-    X = x + t;
-    Y = x - t + 2 * two_q;
-}
-
-// Inverse (Gentleman-Sande) lazy butterfly: X, Y in [0, 4q) -> X', Y' in
-// [0, 4q).  The sum is brought back below 4q by one conditional subtraction;
-// the difference X - Y + 4q (below 8q) is multiplied with the truncated
-// quotient, which lands in [0, 4q) for any input.  Every consumer of an
-// inverse pass either runs more of these butterflies or finishes with a full
-// Shoup product (any input below 2^64, canonical output).
-SF_HD void sf_bfly_gs(u64 &X, u64 &Y, u64 w, u64 wp, u64 q, u64 two_q)
-{
-    const u64 four_q = 2 * two_q;
-    u64 x = X + Y;
-    u64 t = X - Y + four_q;
-    X = x >= four_q ? x - four_q : x;
-    Y = sf_mul_shoup_lazy4(t, w, wp, q);
-}
-
-// Reduce a lazy value in [0, 4q) to [0, q).
-SF_HD u64 sf_reduce4(u64 x, u64 q, u64 two_q)
-{
-    x = x >= two_q ? x - two_q : x;
-    return x >= q ? x - q : x;
 }
 
 // Reduce any x < 2^64 to [0, q): Shoup multiplication by 1 (one_p =

@@ -11,10 +11,8 @@
 // points into registers before it transforms the current one.
 //
 // Bound by the integer multiplier: at N = 2^16 the fmaheavy pipe is busy 70 to
-// 76 % of the cycles, DRAM 31 to 39 %, shared memory 20 to 33 %, and no warp
-// waits on memory or a barrier.  512 x 5 limbs of 2^16, forward: 1961 us with
-// the tile sweeps in shared memory (8 points per thread, three sweeps and three
-// barriers a pass), 1714 us here.
+// 76 % of the cycles.  512 x 5 limbs of 2^16, forward: 1961 us with tile sweeps in
+// shared memory, 1630 us here; 37 x 3 inverse limbs of 2^14: 32.8 and 28.2 us.
 #include <algorithm>
 
 #include "sf_internal.h"
@@ -22,113 +20,107 @@
 #include "sf_reg.cuh"
 #include "sf_round.h"
 
-template <bool INV, int LR, int LC>
-__global__ void __launch_bounds__(SfSub<LC>::NT, 512 / SfSub<LC>::NT)
+template <bool INV, int LR, int LC, bool PM>
+__global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS)
     k_bntt_row(SfRing R, const u64 *src, u64 *dst, int count, int ng)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const SfRowT<LC> T;
+    using T_ = SfRowT<LC, PM>;
+    const T_ T;
     sf_pair *tw = (sf_pair *)smem_raw;
-    u64 *buf = (u64 *)(tw + SfSub<LC>::ROW_PAIRS);
+    u64 *buf = (u64 *)(tw + SfShape<LC>::PAIRS);
     const SfUnitRange U = sf_unit_range(ng * count);
     const size_t per = (size_t)R.L << (LR + LC);
-    // unit u: group u / count = (row tile, limb i), item u % count = polynomial
-    auto row_ptr = [&](int u) -> size_t {
-        const int gg = u / count;
-        return per * (u % count) + ((size_t)(gg % R.L) << (LR + LC)) + ((size_t)T.row(gg / R.L, 1 << LR) << LC);
+    // group = (row tile, limb i), item = polynomial; offset of this thread's row
+    auto group_off = [&](int grp) -> size_t {
+        return ((size_t)(grp % R.L) << (LR + LC)) + ((size_t)T.row(grp / R.L, 1 << LR) << LC) + T.k1(0);
     };
-    u64 x[16], nx[16];
-    auto load = [&](int u) {
-        const u64 *s = src + row_ptr(u);
+    u64 x[8], nx[8];
+    SfCursor C(U.u0, count);
+    size_t off = group_off(C.grp) + per * C.item;
+    auto load = [&]() {
 #pragma unroll
-        for (int r = 0; r < 16; ++r) nx[r] = s[T.k1(r)];
+        for (int t = 0; t < 8; ++t) nx[t] = src[off + (T.k1(t) - T.k1(0))];
     };
-    if (U.u0 < U.u1) load(U.u0);
-    int staged = -1;
+    if (U.u0 < U.u1) load();
+    int staged = -1, mod = 0;
     for (int u = U.u0; u < U.u1; ++u) {
-        const int grp = u / count;
-        const SfMod &M = R.m[grp % R.L];
-        if (grp != staged) {
+        if (C.grp != staged) {
+            mod = C.grp % R.L;
             __syncthreads();   // the previous group's readers are done
-            sf_stage_row<LR, LC>(tw, R.rowP, grp % R.L, grp / R.L);
-            staged = grp;
+            sf_stage_row<LR, LC>(tw, R.rowP, mod, C.grp / R.L);
+            staged = C.grp;
             __syncthreads();
         }
+        const SfMod &M = R.m[mod];
 #pragma unroll
-        for (int r = 0; r < 16; ++r) x[r] = nx[r];
-        u64 *d = dst + row_ptr(u);
+        for (int t = 0; t < 8; ++t) x[t] = nx[t];
+        u64 *d = dst + off;
         // the loads of the next unit overtake this unit's stores: in place, the
         // two units touch different rows or polynomials
-        if (u + 1 < U.u1) load(u + 1);
+        C.next();
+        off = C.grp == staged ? off + per : group_off(C.grp);
+        if (u + 1 < U.u1) load();
         if (INV) {
-            __syncwarp();
-            T.put1(x, buf);
-            __syncwarp();
-            T.get2(x, buf);
-            T.inv2(x, tw, M.q);
-            T.to1(x, buf);
-            T.inv1(x, tw, M.q);
+            T.template exchange<T_::FIRST, T_::LAST>(x, buf);
+            T.inverse(x, tw, buf, M);
 #pragma unroll
-            for (int r = 0; r < 16; ++r) d[T.k1(r)] = sf_red3(x[r], M);
+            for (int t = 0; t < 8; ++t) d[T.k1(t) - T.k1(0)] = sf_red3(x[t], M);
         } else {
-            T.fwd1(x, tw, M.q);
-            T.to2(x, buf);
-            T.fwd2(x, tw, M.q);
-            T.to1(x, buf);   // back to coalesced positions
+            T.forward(x, tw, buf, M);
+            T.template exchange<T_::LAST, T_::FIRST>(x, buf);   // back to coalesced positions
 #pragma unroll
-            for (int r = 0; r < 16; ++r) d[T.k1(r)] = sf_reduce(x[r], M.q, M.one_p);
+            for (int t = 0; t < 8; ++t) d[T.k1(t) - T.k1(0)] = sf_canon(x[t], M);
         }
     }
 }
 
-template <bool INV, int LR, int LC>
-__global__ void __launch_bounds__(SfSub<LR>::NT, 512 / SfSub<LR>::NT)
+template <bool INV, int LR, int LC, bool PM>
+__global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS)
     k_bntt_col(SfRing R, const u64 *src, u64 *dst, int count, int ng)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const SfCol<LR> T;
+    const SfColT<LR, PM> T;
     sf_pair *tab = (sf_pair *)smem_raw;
-    u64 *bufs = (u64 *)(tab + SfSub<LR>::S);
+    u64 *buf = (u64 *)(tab + SfShape<LR>::S);
     const SfUnitRange U = sf_unit_range(ng * count);
     const size_t per = (size_t)R.L << (LR + LC);
-    // unit u: group u / count = (column tile, limb i), item u % count = polynomial
-    auto base = [&](int u) -> size_t {
-        const int gg = u / count;
-        return per * (u % count) + ((size_t)(gg % R.L) << (LR + LC)) + (gg / R.L) * 16 + T.b;
+    // group = (column tile, limb i), item = polynomial; offset of this thread's column
+    auto group_off = [&](int grp) -> size_t {
+        return ((size_t)(grp % R.L) << (LR + LC)) + (grp / R.L) * SfShape<LR>::NB + T.b;
     };
-    u64 x[16], nx[16];
-    auto load = [&](int u) {
-        const u64 *s = src + base(u);
+    u64 x[8], nx[8];
+    SfCursor C(U.u0, count);
+    size_t off = group_off(C.grp) + per * C.item;
+    auto load = [&]() {
 #pragma unroll
-        for (int r = 0; r < 16; ++r) nx[r] = s[(size_t)(INV ? T.k2(r) : T.k1(r)) << LC];
+        for (int t = 0; t < 8; ++t) nx[t] = src[off + ((size_t)(INV ? T.kl(t) : T.k1(t)) << LC)];
     };
-    if (U.u0 < U.u1) load(U.u0);
-    int staged = -1;
+    if (U.u0 < U.u1) load();
+    int staged = -1, mod = 0;
     for (int u = U.u0; u < U.u1; ++u) {
-        const int grp = u / count, i = grp % R.L;
-        const SfMod &M = R.m[i];
-        if (grp != staged) {
+        if (C.grp != staged) {
+            mod = C.grp % R.L;
             __syncthreads();   // the previous group's readers are done
-            sf_stage_cols<LR>(tab, R.colP, i, 1);
-            staged = grp;
+            sf_stage_cols<LR>(tab, R.colP, mod, 1);
+            staged = C.grp;
             __syncthreads();
         }
+        const SfMod &M = R.m[mod];
 #pragma unroll
-        for (int r = 0; r < 16; ++r) x[r] = nx[r];
-        u64 *d = dst + base(u), *buf = bufs + (size_t)(u & 1) * SfSub<LR>::COL_WORDS;
-        if (u + 1 < U.u1) load(u + 1);
+        for (int t = 0; t < 8; ++t) x[t] = nx[t];
+        u64 *d = dst + off;
+        C.next();
+        off = C.grp == staged ? off + per : group_off(C.grp);
+        if (u + 1 < U.u1) load();
         if (INV) {
-            T.inv2(x, tab, M.q);
-            T.to1(x, buf);
-            T.inv1(x, tab, M.q);
+            T.inverse(x, tab, buf, M);
 #pragma unroll
-            for (int r = 0; r < 16; ++r) d[(size_t)T.k1(r) << LC] = sf_mul_shoup(x[r], M.ninv, M.ninv_p, M.q);
+            for (int t = 0; t < 8; ++t) d[(size_t)T.k1(t) << LC] = sf_canon(sf_mad<PM>(0, x[t], make_ulonglong2(M.ninv, M.ninv_c), M), M);
         } else {
-            T.fwd1(x, tab, M.q);
-            T.to2(x, buf);
-            T.fwd2(x, tab, M.q);
+            T.forward(x, tab, buf, M);
 #pragma unroll
-            for (int t = 0; t < 16; ++t) d[(size_t)T.k2(t) << LC] = x[t];
+            for (int t = 0; t < 8; ++t) d[(size_t)T.kl(t) << LC] = x[t];
         }
     }
 }
@@ -140,31 +132,31 @@ static int bntt_blocks(const sf_ctx *ctx, int occ, int n_units)
 }
 
 template <int LC>
-static constexpr size_t bntt_smem_row() { return sizeof(sf_pair) * SfSub<LC>::ROW_PAIRS + sizeof(u64) * SfSub<LC>::ROW_WORDS; }
+static constexpr size_t bntt_smem_row() { return sizeof(sf_pair) * SfShape<LC>::PAIRS + sizeof(u64) * SfShape<LC>::WORDS; }
 template <int LR>
-static constexpr size_t bntt_smem_col() { return sizeof(sf_pair) * SfSub<LR>::S + sizeof(u64) * 2 * SfSub<LR>::COL_WORDS; }
+static constexpr size_t bntt_smem_col() { return sizeof(sf_pair) * SfShape<LR>::S + sizeof(u64) * SfShape<LR>::WORDS; }
 
-template <bool INV, int LR, int LC>
+template <bool INV, int LR, int LC, bool PM>
 static void bntt_row(sf_ctx *ctx, const u64 *src, u64 *dst, int count, cudaStream_t st)
 {
-    const int ng = ((1 << LR) / 16) * ctx->ring.L;
+    const int ng = ((1 << LR) / SfShape<LC>::NB) * ctx->ring.L;
     const size_t sm = bntt_smem_row<LC>();
     cudaEvent_t ev;
-    const int nb = bntt_blocks(ctx, sf_occupancy(k_bntt_row<INV, LR, LC>, SfSub<LC>::NT, sm), ng * count);
+    const int nb = bntt_blocks(ctx, sf_occupancy(k_bntt_row<INV, LR, LC, PM>, SfShape<LC>::NT, sm), ng * count);
     sf_launch_begin(ctx, SFK_BNTT_ROW, st, &ev);
-    k_bntt_row<INV, LR, LC><<<nb, SfSub<LC>::NT, sm, st>>>(ctx->ring, src, dst, count, ng);
+    k_bntt_row<INV, LR, LC, PM><<<nb, SfShape<LC>::NT, sm, st>>>(ctx->ring, src, dst, count, ng);
     sf_launch_end(ctx, SFK_BNTT_ROW, st, ev);
 }
 
-template <bool INV, int LR, int LC>
+template <bool INV, int LR, int LC, bool PM>
 static void bntt_col(sf_ctx *ctx, const u64 *src, u64 *dst, int count, cudaStream_t st)
 {
-    const int ng = ((1 << LC) / 16) * ctx->ring.L;
+    const int ng = ((1 << LC) / SfShape<LR>::NB) * ctx->ring.L;
     const size_t sm = bntt_smem_col<LR>();
     cudaEvent_t ev;
-    const int nb = bntt_blocks(ctx, sf_occupancy(k_bntt_col<INV, LR, LC>, SfSub<LR>::NT, sm), ng * count);
+    const int nb = bntt_blocks(ctx, sf_occupancy(k_bntt_col<INV, LR, LC, PM>, SfShape<LR>::NT, sm), ng * count);
     sf_launch_begin(ctx, SFK_BNTT_COL, st, &ev);
-    k_bntt_col<INV, LR, LC><<<nb, SfSub<LR>::NT, sm, st>>>(ctx->ring, src, dst, count, ng);
+    k_bntt_col<INV, LR, LC, PM><<<nb, SfShape<LR>::NT, sm, st>>>(ctx->ring, src, dst, count, ng);
     sf_launch_end(ctx, SFK_BNTT_COL, st, ev);
 }
 
@@ -176,17 +168,16 @@ extern "C" sf_status sf_ntt_batch(sf_ctx *ctx, const uint64_t *d_in, uint64_t *d
         return sf_set_error(SF_EINVAL, "sf_ntt_batch: bad arguments");
     const SfRing &R = ctx->ring;
     cudaStream_t st = (cudaStream_t)stream;
-    // tiles of a limb: C / 16 (bounded as for the 32 tiles of a 128 x 512 split at N = 2^16)
-    const int tiles = R.log_n == 16 ? 32 : (1 << ((R.log_n + 1) / 2)) / 16;
-    if ((long long)count * R.L * tiles > INT32_MAX)
+    // tiles of a limb: R or C over 16, or 8 for 256-point sub-transforms
+    if ((long long)count * R.L * (R.log_c == 8 ? std::max(R.r / 8, R.c / (R.log_r == 8 ? 8 : 16)) : R.c / 16) > INT32_MAX)
         return sf_set_error(SF_EINVAL, "sf_ntt_batch: count too large");
-    SF_RING_DISPATCH(R.log_n, {
+    SF_RING_DISPATCH(R, {
         if (!inverse) {
-            bntt_col<false, LR, LC>(ctx, d_in, d_out, count, st);
-            bntt_row<false, LR, LC>(ctx, d_out, d_out, count, st);
+            bntt_col<false, LR, LC, PM>(ctx, d_in, d_out, count, st);
+            bntt_row<false, LR, LC, PM>(ctx, d_out, d_out, count, st);
         } else {
-            bntt_row<true, LR, LC>(ctx, d_in, d_out, count, st);
-            bntt_col<true, LR, LC>(ctx, d_out, d_out, count, st);
+            bntt_row<true, LR, LC, PM>(ctx, d_in, d_out, count, st);
+            bntt_col<true, LR, LC, PM>(ctx, d_out, d_out, count, st);
         }
     });
     SF_CUDA_TRY(cudaGetLastError());
@@ -196,14 +187,12 @@ extern "C" sf_status sf_ntt_batch(sf_ctx *ctx, const uint64_t *d_in, uint64_t *d
 sf_status sf_bntt_init_attributes()
 {
     const int mx = 227 * 1024;
-#define SF_BNTT_ATTR(K) SF_CUDA_TRY(cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
-#define SF_BNTT_ATTRS(LR, LC)                                                                  \
-    SF_BNTT_ATTR((k_bntt_row<false, LR, LC>)) SF_BNTT_ATTR((k_bntt_row<true, LR, LC>))         \
-    SF_BNTT_ATTR((k_bntt_col<false, LR, LC>)) SF_BNTT_ATTR((k_bntt_col<true, LR, LC>))
-    SF_BNTT_ATTRS(5, 5) SF_BNTT_ATTRS(5, 6) SF_BNTT_ATTRS(6, 6) SF_BNTT_ATTRS(6, 7) SF_BNTT_ATTRS(7, 7)
-    SF_BNTT_ATTRS(7, 8) SF_BNTT_ATTRS(8, 8)
-#undef SF_BNTT_ATTRS
-#undef SF_BNTT_ATTR
+#define SF_ATTR(K) SF_CUDA_TRY(cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
+    SF_FOR_RINGS({
+        SF_ATTR((k_bntt_row<false, LR, LC, PM>)) SF_ATTR((k_bntt_row<true, LR, LC, PM>))
+        SF_ATTR((k_bntt_col<false, LR, LC, PM>)) SF_ATTR((k_bntt_col<true, LR, LC, PM>))
+    });
+#undef SF_ATTR
     return SF_OK;
 }
 
@@ -215,9 +204,8 @@ sf_status sf_bntt_init_attributes()
 #define PROBE_ITERS 1024
 #define PROBE_OPS (12 * PROBE_ITERS)
 
-template <int KIND>
-__global__ void __launch_bounds__(256, 2) k_probe(u64 *buf, u64 q, ulonglong2 t0, ulonglong2 t1, ulonglong2 t2,
-                                                 ulonglong2 t3)
+template <int KIND, bool PM>
+__global__ void __launch_bounds__(256, 2) k_probe(u64 *buf, SfMod M, sf_pair t0, sf_pair t1, sf_pair t2, sf_pair t3)
 {
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -227,39 +215,37 @@ __global__ void __launch_bounds__(256, 2) k_probe(u64 *buf, u64 q, ulonglong2 t0
         x[i] = buf[i * stride + t];
         acc[i] = 0;
     }
-    const u64 two_q = 2 * q;
+#pragma unroll 1
     for (int it = 0; it < PROBE_ITERS; ++it) {
         if (KIND == 0) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) sf_bfly_ct(x[i], x[i + 4], t0.x, t0.y, q, two_q);
+            for (int i = 0; i < 4; ++i) sf_fwd<PM>(x[i], x[i + 4], t0, M);
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
-                sf_bfly_ct(x[i], x[i + 2], t1.x, t1.y, q, two_q);
-                sf_bfly_ct(x[i + 4], x[i + 6], t2.x, t2.y, q, two_q);
+                sf_fwd<PM>(x[i], x[i + 2], t1, M);
+                sf_fwd<PM>(x[i + 4], x[i + 6], t2, M);
             }
 #pragma unroll
-            for (int i = 0; i < 8; i += 2) sf_bfly_ct(x[i], x[i + 1], t3.x, t3.y, q, two_q);
+            for (int i = 0; i < 8; i += 2) sf_fwd<PM>(x[i], x[i + 1], t3, M);
         } else if (KIND == 1) {
 #pragma unroll
-            for (int i = 0; i < 8; i += 2) sf_bfly_gs(x[i], x[i + 1], t3.x, t3.y, q, two_q);
+            for (int i = 0; i < 8; i += 2) sf_inv<PM>(x[i], x[i + 1], t3, M, M.off);
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
-                sf_bfly_gs(x[i], x[i + 2], t1.x, t1.y, q, two_q);
-                sf_bfly_gs(x[i + 4], x[i + 6], t2.x, t2.y, q, two_q);
+                sf_inv<PM>(x[i], x[i + 2], t1, M, M.off);
+                sf_inv<PM>(x[i + 4], x[i + 6], t2, M, M.off);
             }
 #pragma unroll
-            for (int i = 0; i < 4; ++i) sf_bfly_gs(x[i], x[i + 4], t0.x, t0.y, q, two_q);
+            for (int i = 0; i < 4; ++i) sf_inv<PM>(x[i], x[i + 4], t0, M, M.off);
         } else {
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                const ulonglong2 w = (i & 3) == 0 ? t0 : (i & 3) == 1 ? t1 : (i & 3) == 2 ? t2 : t3;
-                acc[i] += sf_mul_shoup_lazy4(x[i], w.x, w.y, q);
+                acc[i] = sf_mad<PM>(acc[i], x[i], (i & 3) == 0 ? t0 : (i & 3) == 1 ? t1 : (i & 3) == 2 ? t2 : t3, M);
                 x[i] ^= acc[i];
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const ulonglong2 w = i == 0 ? t0 : i == 1 ? t1 : i == 2 ? t2 : t3;
-                acc[i] += sf_mul_shoup_lazy4(x[i + 4], w.x, w.y, q);
+                acc[i] = sf_mad<PM>(acc[i], x[i + 4], i == 0 ? t0 : i == 1 ? t1 : i == 2 ? t2 : t3, M);
                 x[i] += acc[i + 4];
             }
         }
@@ -273,32 +259,25 @@ extern "C" sf_status sf_modmul_probe(sf_ctx *ctx, int32_t kind, double *gmodmul_
     SF_CHECK_CTX(ctx);
     if (!gmodmul_per_s || kind < 0 || kind > 2) return sf_set_error(SF_EINVAL, "sf_modmul_probe: bad arguments");
     const SfMod &M = ctx->ring.m[0];
-    int occ = 1;
-    switch (kind) {
-    case 0: occ = sf_occupancy(k_probe<0>, 256, 0); break;
-    case 1: occ = sf_occupancy(k_probe<1>, 256, 0); break;
-    default: occ = sf_occupancy(k_probe<2>, 256, 0); break;
-    }
-    const int grid = ctx->num_sms * occ;
+    const int pm = ctx->ring.pm;
+    using Kernel = void (*)(u64 *, SfMod, sf_pair, sf_pair, sf_pair, sf_pair);
+    static const Kernel kernels[2][3] = {{k_probe<0, false>, k_probe<1, false>, k_probe<2, false>},
+                                         {k_probe<0, true>, k_probe<1, true>, k_probe<2, true>}};
+    const Kernel kernel = kernels[pm][kind];
+    const int grid = ctx->num_sms * sf_occupancy(kernel, 256, 0);
     const size_t words = (size_t)8 * grid * 256;
     SF_CUDA_TRY(cudaDeviceSynchronize());
     void *w = nullptr;
     SF_TRY(sf_scratch(ctx, words * sizeof(u64), &w));
     u64 *buf = (u64 *)w;
     SF_CUDA_TRY(cudaMemset(buf, 0x5a, words * sizeof(u64)));
-    // four fixed twiddle pairs (w, floor(w 2^64 / q)) modulo q_0
-    ulonglong2 tw[4];
+    // four fixed twiddles modulo q_0 with their companions (sf_mad)
+    sf_pair tw[4];
     for (int i = 0; i < 4; ++i) {
         const u64 v = (M.q / 3 + 7919 * (u64)i) % M.q;
-        tw[i] = make_ulonglong2(v, sf_shoup_companion(v, M.q));
+        tw[i] = make_ulonglong2(v, pm ? sf_host_mulmod(v, ((u64)1 << 32) % M.q, M.q) : sf_shoup_companion(v, M.q));
     }
-    auto launch = [&]() {
-        switch (kind) {
-        case 0: k_probe<0><<<grid, 256>>>(buf, M.q, tw[0], tw[1], tw[2], tw[3]); break;
-        case 1: k_probe<1><<<grid, 256>>>(buf, M.q, tw[0], tw[1], tw[2], tw[3]); break;
-        default: k_probe<2><<<grid, 256>>>(buf, M.q, tw[0], tw[1], tw[2], tw[3]); break;
-        }
-    };
+    auto launch = [&]() { kernel<<<grid, 256>>>(buf, M, tw[0], tw[1], tw[2], tw[3]); };
     cudaEvent_t a = nullptr, b = nullptr;
     SF_CUDA_TRY(cudaEventCreate(&a));
     if (cudaEventCreate(&b) != cudaSuccess) {

@@ -122,12 +122,14 @@ static sf_status eval_jobs(sf_ctx *ctx, std::vector<Job> &jobs, cudaStream_t st)
     // ---- workspace
     Carver cv;
     std::vector<size_t> o_ct(jobs.size()), o_pos(jobs.size()), o_sig(jobs.size());
+    size_t in_words = 0;
     for (size_t x = 0; x < jobs.size(); ++x) {
         o_ct[x] = cv.take((size_t)2 * jobs[x].k_leaf() * ct);
+        in_words = std::max(in_words, (size_t)jobs[x].k_leaf() * ct);
         o_pos[x] = cv.take(((size_t)jobs[x].L->E_in + 1) / 2);
         o_sig[x] = cv.take(((size_t)jobs[x].L->E_out + 1) / 2);
     }
-    const size_t o_w1 = cv.take(w1_words);
+    const size_t o_w1 = cv.take(std::max(w1_words, in_words));   // also the inputs' transforms
     const size_t o_tap = cv.take(tap_words);
     size_t roots_bytes = 0;
     for (auto &c : classes)
@@ -176,7 +178,7 @@ static sf_status eval_jobs(sf_ctx *ctx, std::vector<Job> &jobs, cudaStream_t st)
     u64 *A = ws + o_A, *B = ws + o_B, *d_w1 = ws + o_w1, *d_ks = ws + o_ks;
 
     auto launch_all = [&](cudaStream_t s) -> sf_status {
-        for (auto &j : jobs) SF_TRY(prepare_inputs(ctx, j.d_in, j.d_pow, j.k_in, j.d_ct, s));
+        for (auto &j : jobs) SF_TRY(prepare_inputs(ctx, j.d_in, j.d_pow, j.k_in, j.d_ct, d_w1, s));
         auto leaves = [&](const Job &j, int s0, int stride, int cnt, u64 *dst) -> sf_status {
             const int jb = lb[&j - jobs.data()];
             SfLeafParams P = leaf_params(j.L);
@@ -200,15 +202,16 @@ static sf_status eval_jobs(sf_ctx *ctx, std::vector<Job> &jobs, cudaStream_t st)
             }
             return SF_OK;
         };
+        // the trace ends every group with a key switch: the result holds coefficients
         auto output = [&](const u64 *res, const Job &j, int g) -> sf_status {
-            SfPolyJob pj[SF_MAX_MODULI * 2];
-            for (int x = 0; x < 2 * R.L; ++x) pj[x] = {res + (size_t)x * R.n, j.d_out + ct * g + (size_t)x * R.n, x % R.L};
-            return sf_ntt_jobs(ctx, pj, 2 * R.L, true, s);
+            SF_CUDA_TRY(cudaMemcpyAsync(j.d_out + ct * g, res, ct_bytes, cudaMemcpyDeviceToDevice, s));
+            return SF_OK;
         };
         for (auto &c : classes) {
             const std::vector<int32_t> &kd = c.rk->d;
             u64 *RA = c.nch > 1 ? ws + c.o_roots_a : nullptr;
             u64 *RB = c.nch > 1 ? ws + c.o_roots_b : nullptr;
+            bool ntt = true;   // domain of the units' roots, the same for every wave
             for (size_t u0 = 0; u0 < c.units.size(); u0 += c.U) {
                 const int wn = (int)std::min<size_t>(c.U, c.units.size() - u0);
                 std::vector<int> valid(wn);
@@ -220,8 +223,9 @@ static sf_status eval_jobs(sf_ctx *ctx, std::vector<Job> &jobs, cudaStream_t st)
                 }
                 u64 *res = nullptr;
                 size_t rs = 0;
+                ntt = true;
                 SF_TRY(sf_pack_tree(ctx, c.rk->d_keys, kd, c.rk->key_words, A, B, wn, c.CH, 0, valid, c.nch == 1, d_ks,
-                                    batch, &res, &rs, s, c.gamma2));
+                                    batch, &res, &rs, &ntt, s, c.gamma2));
                 if (c.nch == 1) {
                     for (int u = 0; u < wn; ++u) {
                         const Unit &un = c.units[u0 + u];
@@ -243,7 +247,7 @@ static sf_status eval_jobs(sf_ctx *ctx, std::vector<Job> &jobs, cudaStream_t st)
                 u64 *res = nullptr;
                 size_t rs = 0;
                 SF_TRY(sf_pack_tree(ctx, c.rk->d_keys, kd, c.rk->key_words, RA, RB, (int)c.groups.size(), c.nch, c.log_ch,
-                                    valid, true, d_ks, batch, &res, &rs, s, c.gamma2));
+                                    valid, true, d_ks, batch, &res, &rs, &ntt, s, c.gamma2));
                 for (size_t gi = 0; gi < c.groups.size(); ++gi)
                     SF_TRY(output(res + rs * gi, jobs[c.groups[gi].first], c.groups[gi].second));
             }
@@ -348,7 +352,7 @@ extern "C" sf_status sf_eval_linear_layer_gamma(sf_ctx *ctx, const sf_layer *L, 
     if (gamma < 2 && d_powers) return sf_set_error(SF_EINVAL, "powers are only read at gamma = 2");
     std::vector<Job> jobs(1);
     SF_TRY(make_job(ctx, L, rk, d_in, k_in, h_sigma_prev, h_sigma_out, d_out, out_capacity, &jobs[0]));
-    if (gamma == 2 && 2 * k_in * (ctx->ring.c / SF_NB) > 4096)
+    if (gamma == 2 && 2 * k_in * sf_leaf_tiles(ctx->ring) > 4096)
         return sf_set_error(SF_EINVAL, "too many input ciphertexts for one round at gamma = 2");
     jobs[0].d_pow = gamma == 2 ? d_powers : nullptr;
     SF_TRY(eval_jobs(ctx, jobs, (cudaStream_t)stream));
@@ -401,7 +405,7 @@ extern "C" sf_status sf_eval_layers_gamma(sf_ctx *ctx, int32_t n_layers, const s
         SF_TRY(make_job(ctx, layers[x], rks[x], d_ins[x], k_ins[x], h_sigma_prevs ? h_sigma_prevs[x] : nullptr,
                         h_sigma_outs ? h_sigma_outs[x] : nullptr, d_outs[x], out_capacities[x], &jobs[x]));
         jobs[x].d_pow = d_powers ? d_powers[x] : nullptr;
-        if (jobs[x].d_pow && 2 * k_ins[x] * (ctx->ring.c / SF_NB) > 4096)
+        if (jobs[x].d_pow && 2 * k_ins[x] * sf_leaf_tiles(ctx->ring) > 4096)
             return sf_set_error(SF_EINVAL, "too many input ciphertexts for one round at gamma = 2");
     }
     SF_TRY(eval_jobs(ctx, jobs, (cudaStream_t)stream));
@@ -446,7 +450,7 @@ extern "C" sf_status sf_autotune_layers(sf_ctx *ctx, int32_t n_layers, const sf_
         *out_ms = tmin;
         return SF_OK;
     };
-    // 1) merges per key-switch launch; larger batches amortise each kernel's
+    // merges per key-switch launch; larger batches amortise each kernel's
     // twiddle staging and tail over more merges, at ks_scratch x batch bytes of
     // workspace, which is capped at SF_AUTOTUNE_KS_SCRATCH
     static const int cand[] = {32, 64, 128, 256, 512, 1024, 2048, 4096};
@@ -463,58 +467,6 @@ extern "C" sf_status sf_autotune_layers(sf_ctx *ctx, int32_t n_layers, const sf_
         }
     }
     ctx->ks_batch = best;
-    // 2) leaf column pass of sparse tiles: closed form (default rule) or always the transform
-    if (status == SF_OK) {
-        const int saved_sparse = ctx->leaf_sparse;
-        int best_sparse = saved_sparse;
-        for (int sp : {-1, 0}) {
-            if (sp == saved_sparse) continue;
-            ctx->leaf_sparse = sp;
-            double t = 0;
-            if ((status = measure(&t)) != SF_OK) break;
-            if (t < best_t) {
-                best_t = t;
-                best_sparse = sp;
-            }
-        }
-        ctx->leaf_sparse = best_sparse;
-    }
-    // 3) block shape of the key-switch inner product for 128-point rows:
-    //    256 threads x 8 elements or 512 threads x 4 elements
-    if (status == SF_OK && ctx->ring.log_c == 7) {
-        const int saved = ctx->ks3_threads;
-        int best_nt = saved;
-        for (int nt : {256, 512}) {
-            if (nt == saved) continue;
-            ctx->ks3_threads = nt;
-            double t = 0;
-            if ((status = measure(&t)) != SF_OK) break;
-            if (t < best_t) {
-                best_t = t;
-                best_nt = nt;
-            }
-        }
-        ctx->ks3_threads = best_nt;
-    }
-    // 4) NTT radix of the row passes (key-switch rows, inner product, ModDown
-    //    finish, leaf rows): radix-8 sweeps (three per row pass), radix-4
-    //    sweeps only, which hold half the values per unit, or radix 8 with two
-    //    sweeps of 256- and 512-point rows fused by warp-shuffle exchanges
-    if (status == SF_OK) {
-        const int saved = ctx->row_radix;
-        int best_rad = saved;
-        for (int rad : {0, 1, 2}) {
-            if (rad == saved) continue;
-            ctx->row_radix = rad;
-            double t = 0;
-            if ((status = measure(&t)) != SF_OK) break;
-            if (t < best_t) {
-                best_t = t;
-                best_rad = rad;
-            }
-        }
-        ctx->row_radix = best_rad;
-    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     sf_graph_cache_clear(ctx);

@@ -11,6 +11,7 @@
 #include <mutex>
 
 #include "sf_internal.h"
+#include "sf_reg.cuh"
 
 // ------------------------------------------------------------------ errors --
 
@@ -456,6 +457,46 @@ static sf_status upload(sf_ctx *ctx, const std::vector<T> &h, const T **out)
     return SF_OK;
 }
 
+// Bound of the product by pairs (w, 2^32 w mod q) as a multiple of q (sf_mad:
+// below 2^53 + 2^33 delta, q = 2^50 - delta), or 0 where q does not admit it: 20
+// times the bound, which a forward transform reaches, and 64 times, which the
+// inverse passes reach, stay below 2^63 and 2^64.
+static u64 pm_bound(u64 q)
+{
+    const u64 top = (u64)1 << 50;
+    if (q >= top || q <= top / 2) return 0;
+    const u64 delta = top - q;
+    if (delta >= ((u64)1 << 25)) return 0;
+    const u64 bound = (((u64)1 << 53) + (delta << 33) + q - 1) / q * q;
+    return bound <= ((u64)1 << 58) ? bound : 0;
+}
+
+// companion of w for the ring's products (sf_mad)
+static u64 pair_companion(u64 w, u64 q, int pm) { return pm ? sf_host_mulmod(w, ((u64)1 << 32) % q, q) : sf_shoup_companion(w, q); }
+
+// the row tiles' twiddles in the order the row passes read them (SfShape)
+template <int LC>
+static void sf_row_tables(const SfRing &R, const std::vector<u64> &psi, const std::vector<u64> &psi_p,
+                          std::vector<ulonglong2> &out)
+{
+    using Sh = SfShape<LC>;
+    for (int m = 0; m < R.nm; ++m)
+        for (int tile = 0; tile < R.r / Sh::NB; ++tile)
+            for (int ph = 0; ph < Sh::NP; ++ph)
+                for (int st = Sh::HI(ph); st >= Sh::LO(ph); --st) {
+                    const int lc = Sh::P(ph) + 2 - st;   // log2 of the subs per high
+                    for (int sub = 0; sub < (1 << lc); ++sub)
+                        for (int b = 0; b < Sh::NB; ++b) {
+                            const int rr = Sh::HALF * tile + b % Sh::HALF, row = b < Sh::HALF ? rr : R.r - 1 - rr;
+                            for (int hi = 0; hi < Sh::H(ph); ++hi) {
+                                const size_t groups = (size_t)Sh::S >> (st + 1);
+                                const size_t k = (size_t)m * R.n + groups * (R.r + row) + ((size_t)hi << lc) + sub;
+                                out.push_back(make_ulonglong2(psi[k], psi_p[k]));
+                            }
+                        }
+                }
+}
+
 extern "C" sf_status sf_ctx_create(const sf_params *p, int32_t device, sf_ctx **out)
 {
     if (!p || !out) return sf_set_error(SF_EINVAL, "sf_ctx_create: null argument");
@@ -477,10 +518,10 @@ extern "C" sf_status sf_ctx_create(const sf_params *p, int32_t device, sf_ctx **
     ctx->io_buf = nullptr;
     ctx->io_bytes = 0;
     // merges per key-switch launch (the autotuner's pick on the benchmark rounds);
-    // the scratch is ks_batch x (3L + max(L, 2K) + max(dnum (L+K), 2L)) limbs
+    // the scratch is ks_batch x ((dnum + 2)(L + K) + 2L) limbs
     ctx->ks_batch = p->log_n >= 16 ? 256 : 512;
     ctx->leaf_chunk = 1 << 30;
-    ctx->leaf_sparse = 0;   // the transform measured faster than the closed form on GB300
+    ctx->leaf_sparse = 0;
     ctx->ks3_threads = 256;
     ctx->row_radix = 0;
     ctx->mem_budget = (size_t)64 << 30;
@@ -493,9 +534,8 @@ extern "C" sf_status sf_ctx_create(const sf_params *p, int32_t device, sf_ctx **
     memset(&R, 0, sizeof(R));
     R.log_n = p->log_n;
     R.n = N;
-    // N = R x C: C = 2^ceil(log2 N / 2), except 2^16 = 128 x 512, so that the
-    // column passes of the largest ring keep 128-point columns
-    R.log_c = p->log_n == 16 ? 9 : (p->log_n + 1) / 2;
+    // N = R x C, both between 32 and 256 (sf_reg.cuh)
+    R.log_c = (p->log_n + 1) / 2;
     R.log_r = p->log_n - R.log_c;
     R.c = 1 << R.log_c;
     R.r = 1 << R.log_r;
@@ -507,7 +547,10 @@ extern "C" sf_status sf_ctx_create(const sf_params *p, int32_t device, sf_ctx **
     for (int a = 0; a < nm; ++a)
         for (int b = 0; b < nm; ++b)
             if (p->mods[a] / 4 >= p->mods[b]) R.modup_copy = 0;
-    std::vector<u64> psi((size_t)nm * N), psi_p((size_t)nm * N), ipsi((size_t)nm * N), ipsi_p((size_t)nm * N);
+    R.pm = 1;
+    for (u64 q : p->mods)
+        if (!pm_bound(q)) R.pm = 0;
+    std::vector<u64> psi((size_t)nm * N), psi_p((size_t)nm * N);   // and their companions
     std::vector<u64> pw((size_t)nm * 2 * N), pw_p((size_t)nm * 2 * N);
     for (int m = 0; m < nm; ++m) {
         u64 q = p->mods[m];
@@ -525,91 +568,40 @@ extern "C" sf_status sf_ctx_create(const sf_params *p, int32_t device, sf_ctx **
         M.one_p = sf_shoup_companion(1, q);
         M.sh = 63 - __builtin_clzll(q);
         M.binv = (unsigned)(((u128)1 << (32 + M.sh)) / q);
+        M.n2q = 0 - 2 * q;
+        M.off = R.pm ? pm_bound(q) : 4 * q;
+        M.off1 = std::max(8 * q, M.off);
+        M.ninv_c = pair_companion(M.ninv, q, R.pm);
         u64 root = sf_root_2n(q, 2 * (u64)N);
-        u64 iroot = sf_host_invmod(root, q);
-        for (int k = 0; k < N; ++k) {
-            unsigned e = brev_bits((unsigned)k, p->log_n);
-            u64 w = sf_host_powmod(root, e, q), iw = sf_host_powmod(iroot, e, q);
-            psi[(size_t)m * N + k] = w;
-            psi_p[(size_t)m * N + k] = sf_shoup_companion(w, q);
-            ipsi[(size_t)m * N + k] = iw;
-            ipsi_p[(size_t)m * N + k] = sf_shoup_companion(iw, q);
-        }
         u64 acc = 1;
         for (int k = 0; k < 2 * N; ++k) {
             pw[(size_t)m * 2 * N + k] = acc;
             pw_p[(size_t)m * 2 * N + k] = sf_shoup_companion(acc, q);
             acc = sf_host_mulmod(acc, root, q);
         }
-    }
-    // Staged twiddle pairs: column table k < R (global index k), and the
-    // row table of each 16-row tile, entry [k][b] = global index
-    // m(k) (R + r) + k - m(k) with r = 16 tile + b, m(k) = 2^floor(log2 k).
-    std::vector<ulonglong2> colT_f((size_t)nm * R.r), colT_i((size_t)nm * R.r);
-    std::vector<ulonglong2> rowT_f((size_t)nm * N), rowT_i((size_t)nm * N);
-    for (int m = 0; m < nm; ++m) {
-        const u64 *tf = psi.data() + (size_t)m * N, *tfp = psi_p.data() + (size_t)m * N;
-        const u64 *ti = ipsi.data() + (size_t)m * N, *tip = ipsi_p.data() + (size_t)m * N;
-        for (int k = 0; k < R.r; ++k) {
-            colT_f[(size_t)m * R.r + k] = make_ulonglong2(tf[k], tfp[k]);
-            colT_i[(size_t)m * R.r + k] = make_ulonglong2(ti[k], tip[k]);
-        }
-        // row tiles of nb rows (sf_row_nb: 16, or 8 for 256-point rows)
-        const int nb = sf_row_nb(R.log_c);
-        for (int tile = 0; tile < R.r / nb; ++tile)
-            for (int k = 0; k < R.c; ++k)
-                for (int b = 0; b < nb; ++b) {
-                    size_t dst = (size_t)m * N + ((size_t)tile * R.c + k) * nb + b;
-                    if (k == 0) {
-                        rowT_f[dst] = rowT_i[dst] = make_ulonglong2(0, 0);
-                        continue;
-                    }
-                    int mk = 1;
-                    while (mk * 2 <= k) mk *= 2;
-                    size_t gi = (size_t)mk * (R.r + nb * tile + b) + (k - mk);
-                    rowT_f[dst] = make_ulonglong2(tf[gi], tfp[gi]);
-                    rowT_i[dst] = make_ulonglong2(ti[gi], tip[gi]);
-                }
-    }
-    // Twiddles of the register-resident passes (sf_reg.cuh).  Row tile: rows
-    // 8 tile + b (b < 8) and their mirrors R - 1 - row; phase-1 entries (k, b)
-    // at (k - 1) 16 + b, then phase-2 entries (e, b, i) at e C + b (C/16) + i.
-    const int lc2 = (p->log_n + 1) / 2, lr2 = p->log_n - lc2, r2 = 1 << lr2, c2 = 1 << lc2, ni = c2 / 16;
-    std::vector<ulonglong2> colP((size_t)nm * r2), rowP((size_t)nm * (r2 / 16) * 16 * (c2 - 1));
-    for (int m = 0; m < nm; ++m) {
-        const u64 *tf = psi.data() + (size_t)m * N, *tfp = psi_p.data() + (size_t)m * N;
-        for (int k = 0; k < r2; ++k) colP[(size_t)m * r2 + k] = make_ulonglong2(tf[k], tfp[k]);
-        for (int tile = 0; tile < r2 / 16; ++tile) {
-            ulonglong2 *dst = &rowP[((size_t)m * (r2 / 16) + tile) * 16 * (c2 - 1)];
-            for (int b = 0; b < 16; ++b) {
-                const size_t row = b < 8 ? 8 * tile + b : r2 - 1 - 8 * tile - (b - 8);
-                for (int k = 1; k < ni; ++k) {
-                    int mk = 1;
-                    while (mk * 2 <= k) mk *= 2;
-                    const size_t gi = mk * (r2 + row) + (k - mk);
-                    dst[(k - 1) * 16 + b] = make_ulonglong2(tf[gi], tfp[gi]);
-                }
-                for (int e = 0; e < 15; ++e) {
-                    const int s = e >= 7 ? 3 : e >= 3 ? 2 : e >= 1 ? 1 : 0, g = e - ((1 << s) - 1);
-                    for (int i = 0; i < ni; ++i) {
-                        const size_t gi = ((size_t)ni << s) * (r2 + row) + (i << s) + g;
-                        dst[16 * (ni - 1) + e * c2 + b * ni + i] = make_ulonglong2(tf[gi], tfp[gi]);
-                    }
-                }
-            }
+        for (int k = 0; k < N; ++k) {
+            const size_t e = (size_t)m * 2 * N + brev_bits((unsigned)k, p->log_n);
+            psi[(size_t)m * N + k] = pw[e];
+            psi_p[(size_t)m * N + k] = R.pm ? pair_companion(pw[e], q, 1) : pw_p[e];
         }
     }
-    // powers psi^(C e), e < 2R (closed-form column pass of a sparse polynomial)
-    std::vector<ulonglong2> pwc((size_t)nm * 2 * R.r);
+    // Twiddles of the register-resident passes (sf_reg.cuh): column tables, and per
+    // row tile the entries of each phase and stage, [sub][row b][high]
+    std::vector<ulonglong2> colP((size_t)nm * R.r), rowP;
+    rowP.reserve((size_t)nm * N);
     for (int m = 0; m < nm; ++m)
-        for (int e = 0; e < 2 * R.r; ++e) {
-            const size_t k = (size_t)m * 2 * N + (size_t)e * R.c;
-            pwc[(size_t)m * 2 * R.r + e] = make_ulonglong2(pw[k], pw_p[k]);
-        }
+        for (int k = 0; k < R.r; ++k) colP[(size_t)m * R.r + k] = make_ulonglong2(psi[(size_t)m * N + k], psi_p[(size_t)m * N + k]);
+    switch (R.log_c) {
+    case 5: sf_row_tables<5>(R, psi, psi_p, rowP); break;
+    case 6: sf_row_tables<6>(R, psi, psi_p, rowP); break;
+    case 7: sf_row_tables<7>(R, psi, psi_p, rowP); break;
+    default: sf_row_tables<8>(R, psi, psi_p, rowP); break;
+    }
     // ModUp constants
     int dnum = p->dnum;
-    std::vector<u64> mu_inv((size_t)dnum * K, 0), mu_inv_p((size_t)dnum * K, 0);
-    std::vector<u64> mu_qhat((size_t)dnum * K * nm, 0), mu_qhat_p((size_t)dnum * K * nm, 0);
+    std::vector<u64> mu_inv((size_t)dnum * K, 0), mu_inv_c((size_t)dnum * K, 0);
+    std::vector<u64> mu_hinv((size_t)dnum * K, 0), mu_hinv_c((size_t)dnum * K, 0);
+    std::vector<u64> mu_qhat((size_t)dnum * K * nm, 0), mu_qhat_c((size_t)dnum * K * nm, 0);
     for (int j = 0; j < dnum; ++j) {
         int lo = j * K, hi = std::min((j + 1) * K, L);
         for (int i = lo; i < hi; ++i) {
@@ -620,14 +612,16 @@ extern "C" sf_status sf_ctx_create(const sf_params *p, int32_t device, sf_ctx **
             // N^-1 is folded in: the column pass of the inverse NTT leaves it out
             u64 iv = sf_host_mulmod(sf_host_invmod(qhat_qi, qi), sf_host_invmod((u64)N % qi, qi), qi);
             mu_inv[j * K + (i - lo)] = iv;
-            mu_inv_p[j * K + (i - lo)] = sf_shoup_companion(iv, qi);
+            mu_inv_c[j * K + (i - lo)] = pair_companion(iv, qi, R.pm);
+            mu_hinv[j * K + (i - lo)] = sf_host_invmod(qhat_qi, qi);
+            mu_hinv_c[j * K + (i - lo)] = pair_companion(mu_hinv[j * K + (i - lo)], qi, R.pm);
             for (int m = 0; m < nm; ++m) {
                 u64 qm = p->mods[m];
                 u64 v = 1;
                 for (int i2 = lo; i2 < hi; ++i2)
                     if (i2 != i) v = sf_host_mulmod(v, p->mods[i2] % qm, qm);
                 mu_qhat[((size_t)j * K + (i - lo)) * nm + m] = v;
-                mu_qhat_p[((size_t)j * K + (i - lo)) * nm + m] = sf_shoup_companion(v, qm);
+                mu_qhat_c[((size_t)j * K + (i - lo)) * nm + m] = pair_companion(v, qm, R.pm);
             }
         }
     }
@@ -635,7 +629,7 @@ extern "C" sf_status sf_ctx_create(const sf_params *p, int32_t device, sf_ctx **
     // P^-1 is carried by the conversion constants (Phat_k P^-1 mod q_i) and by
     // the reduction of the key products of the data limbs (times P^-1 mod
     // q_i), so the finish is one subtraction; every residue is unchanged.
-    std::vector<u64> md_inv(K), md_inv_p(K), md_phat((size_t)K * L), md_phat_p((size_t)K * L), md_pinv(L), md_pinv_p(L);
+    std::vector<u64> md_inv(K), md_inv_c(K), md_phat((size_t)K * L), md_phat_c((size_t)K * L), md_pinv(L), md_pinv_p(L);
     for (int i = 0; i < L; ++i) {
         u64 qi = p->mods[i];
         u64 pm = 1;
@@ -649,7 +643,7 @@ extern "C" sf_status sf_ctx_create(const sf_params *p, int32_t device, sf_ctx **
         for (int k2 = 0; k2 < K; ++k2)
             if (k2 != k) ph = sf_host_mulmod(ph, p->mods[L + k2] % pk, pk);
         md_inv[k] = sf_host_mulmod(sf_host_invmod(ph, pk), sf_host_invmod((u64)N % pk, pk), pk);
-        md_inv_p[k] = sf_shoup_companion(md_inv[k], pk);
+        md_inv_c[k] = pair_companion(md_inv[k], pk, R.pm);
         for (int i = 0; i < L; ++i) {
             u64 qi = p->mods[i];
             u64 v = 1;
@@ -657,16 +651,15 @@ extern "C" sf_status sf_ctx_create(const sf_params *p, int32_t device, sf_ctx **
                 if (k2 != k) v = sf_host_mulmod(v, p->mods[L + k2] % qi, qi);
             v = sf_host_mulmod(v, md_pinv[i], qi);
             md_phat[(size_t)k * L + i] = v;
-            md_phat_p[(size_t)k * L + i] = sf_shoup_companion(v, qi);
+            md_phat_c[(size_t)k * L + i] = pair_companion(v, qi, R.pm);
         }
     }
     sf_status st = SF_OK;
 #define UP(v, f)                                      \
     if (st == SF_OK) st = upload(ctx, v, &R.f);
-    UP(psi, psi) UP(psi_p, psi_p) UP(ipsi, ipsi) UP(ipsi_p, ipsi_p) UP(pw, pw) UP(pw_p, pw_p)
-    UP(colT_f, colT_f) UP(colT_i, colT_i) UP(rowT_f, rowT_f) UP(rowT_i, rowT_i) UP(pwc, pwc) UP(colP, colP) UP(rowP, rowP)
-    UP(mu_inv, mu_inv) UP(mu_inv_p, mu_inv_p) UP(mu_qhat, mu_qhat) UP(mu_qhat_p, mu_qhat_p)
-    UP(md_inv, md_inv) UP(md_inv_p, md_inv_p) UP(md_phat, md_phat) UP(md_phat_p, md_phat_p)
+    UP(pw, pw) UP(pw_p, pw_p) UP(colP, colP) UP(rowP, rowP)
+    UP(mu_inv, mu_inv) UP(mu_inv_c, mu_inv_c) UP(mu_hinv, mu_hinv) UP(mu_hinv_c, mu_hinv_c) UP(mu_qhat, mu_qhat) UP(mu_qhat_c, mu_qhat_c)
+    UP(md_inv, md_inv) UP(md_inv_c, md_inv_c) UP(md_phat, md_phat) UP(md_phat_c, md_phat_c)
     UP(md_pinv, md_pinv) UP(md_pinv_p, md_pinv_p)
 #undef UP
     if (st == SF_OK) st = sf_ntt_init_attributes();

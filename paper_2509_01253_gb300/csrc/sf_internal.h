@@ -11,11 +11,6 @@
 
 #define SF_MAX_DIGITS 8
 
-// Rows per row tile of the two-pass NTT: 16, 8 for 256-point rows, 4 for
-// 512-point rows, so a row tile holds at most 2048 residues (8 per thread of
-// a 256-thread block).
-SF_HD int sf_row_nb(int log_c) { return log_c >= 9 ? 4 : (log_c >= 8 ? 8 : 16); }
-
 // Per-modulus constants, passed to kernels by value (kernel parameter space).
 struct SfMod {
     u64 q, two_q;
@@ -27,37 +22,36 @@ struct SfMod {
     // partial reduction of lazy values (sf_red3): sh = bits(q) - 1, binv = floor(2^(32 + sh) / q)
     unsigned binv;
     int sh;
+    // products by pairs (sf_mad): -2q; the bound off of their results (a
+    // multiple of q); off1 = max(8q, off); companion of ninv in the ring's form
+    u64 n2q, off, off1, ninv_c;
 };
 
 // Everything a kernel needs about the ring, by value.
 struct SfRing {
     int log_n, n, log_r, r, log_c, c;
     int L, K, nm, dnum;
+    int pm;   // pairs are (w, 2^32 w mod q), else (w, floor(w 2^64 / q)): see sf_mad
     // every modulus is below 4x every other one: a one-limb digit's ModUp
     // (its residue itself, Qhat = 1) is a valid lazy input of the forward NTT
     // modulo any other modulus, with no reduction
     int modup_copy;
     SfMod m[SF_MAX_MODULI];
-    // twiddle tables, [nm][N] each (index 0 unused)
-    const u64 *psi, *psi_p, *ipsi, *ipsi_p;
-    // staged twiddle pairs (w, w'): column tables [nm][R] (k < R) and row
-    // tables [nm][R/16][C][16] reordered per 16-row tile (see sf_tile.cuh)
-    const ulonglong2 *colT_f, *colT_i, *rowT_f, *rowT_i;
-    // twiddle pairs of the register-resident passes (sf_reg.cuh): columns
-    // [nm][R'], row tiles [nm][R'/16][16 (C' - 1)], N = R' x C', C' = 2^ceil(log2 N / 2)
+    // twiddle pairs (w, companion) of the passes (sf_reg.cuh), N = R x C, C = 2^ceil(log2 N / 2):
+    // columns [nm][R], row tiles [nm][R/16][16 (C - 1)]
     const ulonglong2 *colP, *rowP;
     // powers psi^k, k in [0, 2N), [nm][2N] (monomials in the NTT domain)
     const u64 *pw, *pw_p;
-    // pairs (psi^(C e), companion), e < 2R, [nm][2R] (sparse column pass)
-    const ulonglong2 *pwc;
-    // ModUp: for digit j, limb i in the digit: N^-1 (Qhat_i mod q_i)^-1 with
-    //        Shoup (N^-1 finishes the inverse NTT); Qhat_i mod m for every m.
-    const u64 *mu_inv, *mu_inv_p;   // [dnum][K]
-    const u64 *mu_qhat, *mu_qhat_p; // [dnum][K][nm]
+    // Every constant with a companion _c is a pair in the ring's form (sf_mad).
+    // ModUp: for digit j, limb i in the digit: N^-1 (Qhat_i mod q_i)^-1 (N^-1
+    //        finishes the inverse NTT); mu_hinv: (Qhat_i mod q_i)^-1 alone, for
+    //        coefficient-domain operands; Qhat_i mod m for every m.
+    const u64 *mu_inv, *mu_inv_c, *mu_hinv, *mu_hinv_c;   // [dnum][K]
+    const u64 *mu_qhat, *mu_qhat_c; // [dnum][K][nm]
     // ModDown: N^-1 (Phat_k mod p_k)^-1; Phat_k P^-1 mod q_i (the conversion
-    // carries the final factor P^-1); P^-1 mod q_i (all Shoup)
-    const u64 *md_inv, *md_inv_p;   // [K]
-    const u64 *md_phat, *md_phat_p; // [K][L]
+    // carries the final factor P^-1); P^-1 mod q_i (Shoup)
+    const u64 *md_inv, *md_inv_c;   // [K]
+    const u64 *md_phat, *md_phat_c; // [K][L]
     const u64 *md_pinv, *md_pinv_p; // [L]
     int *status;                    // device status word (first latched error)
 };
@@ -103,9 +97,7 @@ struct sf_ctx {
     // options
     int ks_batch;
     int leaf_chunk;
-    int leaf_sparse;          // taps per column tile up to which the leaf column pass uses the closed form (-1: default rule)
-    int ks3_threads;          // block size of the key-switch inner product for 128-point rows (256 or 512)
-    int row_radix;            // row-pass sweep schedule of the key-switch and leaf row kernels: 0 radix-8, 1 radix-4, 2 radix-8 with warp-shuffle exchanges
+    int leaf_sparse, ks3_threads, row_radix;   // accepted and read back; every value runs the same kernels
     size_t mem_budget;        // bytes of leaf + tree buffers a round may use
     int use_graph;
     int kernel_timing;
@@ -130,7 +122,7 @@ struct sf_rotkeys {
     sf_ctx *ctx;
     uint64_t gen;             // unique per handle (graph cache key)
     std::vector<int32_t> d;   // automorphism indices
-    u64 *d_keys;              // per key: [dnum][2][nm][N] NTT-domain values, then their Shoup companions
+    u64 *d_keys;              // per key: [dnum][2][nm][N] pairs of the NTT-domain values, storage order (sf_reg.cuh)
     size_t key_words;         // words per key
 };
 
@@ -226,9 +218,6 @@ struct SfPolyJob {
     int mod;
 };
 sf_status sf_ntt_jobs(sf_ctx *ctx, const SfPolyJob *h_jobs, int n_jobs, bool inverse, cudaStream_t st);
-// dynamic shared memory: staged twiddles + `tiles` data tiles (sf_tile.cuh)
-size_t sf_smem_col(const SfRing &R, int tiles);
-size_t sf_smem_row(const SfRing &R, int tiles);
 
 // Elementwise helpers (sf_ntt.cu).  Polynomial t uses modulus offset + t % period.
 sf_status sf_to_mont(sf_ctx *ctx, u64 *d, int n_polys, int period, int offset, cudaStream_t st);
@@ -243,12 +232,14 @@ sf_status sf_decrypt_finish(sf_ctx *ctx, const u64 *cts, const u64 *p, u64 *out,
 sf_status sf_signed_to_residues(sf_ctx *ctx, const int64_t *v, u64 *out, int n_polys, int period, int offset,
                                 cudaStream_t st);
 sf_status sf_rotkey_finish(sf_ctx *ctx, const u64 *alpha, const u64 *e, const u64 *s_mont, const u64 *pg, int d,
-                           u64 *key_a, u64 *key_b, size_t comp, cudaStream_t st);
+                           ulonglong2 *key_a, ulonglong2 *key_b, cudaStream_t st);
 // device-side range check of caller input: latches SF_ERANGE in the status
 // word (reported by sf_sync) if a residue of poly t is >= modulus offset + t % period
 sf_status sf_check_residues(sf_ctx *ctx, const u64 *x, int n_polys, int period, int offset, cudaStream_t st);
-// Shoup companions floor(x 2^64 / q) of residues x (poly t uses modulus offset + t % period)
-sf_status sf_companions(sf_ctx *ctx, const u64 *x, u64 *dst, int n_polys, int period, int offset, cudaStream_t st);
+// NTT-domain residues -> pairs in storage order (poly t uses modulus offset + t % period)
+sf_status sf_to_pairs(sf_ctx *ctx, const u64 *x, ulonglong2 *dst, int n_polys, int period, int offset, cudaStream_t st);
+// storage order -> natural slot order: plain words (step 1) or the values of pairs (step 2)
+sf_status sf_to_natural(sf_ctx *ctx, const u64 *x, int step, u64 *dst, int n_polys, cudaStream_t st);
 
 // Raise the dynamic shared-memory limit of every kernel (once per device).
 sf_status sf_ntt_init_attributes();

@@ -3,14 +3,6 @@
 #include <algorithm>
 
 #include "sf_internal.h"
-#include "sf_tile.cuh"
-
-__device__ __forceinline__ SfGeo ring_geo(const SfRing &R)
-{
-    SfGeo g;
-    g.log_n = R.log_n; g.n = R.n; g.log_r = R.log_r; g.r = R.r; g.log_c = R.log_c; g.c = R.c;
-    return g;
-}
 
 // NTT slot j holds the evaluation at psi^(2 brev(j) + 1).
 __device__ __forceinline__ unsigned slot_exponent(int j, int log_n)
@@ -48,4 +40,18 @@ __device__ __forceinline__ u64 sf_shoup_companion_dev(u64 x, const SfMod &M)
     const u64 rem = x * M.r_mod - h * M.q;
     if (rem >= M.q) ++h;
     return x * M.one_p + h;
+}
+
+// a canonical residue with its companion in the ring's form (sf_mad): for pm
+// moduli (50 bits) 2^32 x mod q, shifted in steps that stay below 2^63
+__device__ __forceinline__ ulonglong2 sf_make_pair(u64 x, const SfMod &M, int pm)
+{
+    if (!pm) return make_ulonglong2(x, sf_shoup_companion_dev(x, M));
+    u64 v = x;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        v <<= 13;   // below 2^63: residues of 50-bit moduli
+        v = sf_reduce(v, M.q, M.one_p);
+    }
+    return make_ulonglong2(x, sf_reduce(v << 6, M.q, M.one_p));
 }

@@ -5,7 +5,9 @@
 // `count` merges sharing d, s, add_v and the key.  Merge number
 // x = first + i (i < count) splits into (g, t) = (x / inner, x % inner):
 //   E_x = E + g*E_outer + t*E_stride, likewise O_x (O may be null) and out_x;
-// every operand [2][L][N] in the NTT domain.  out must not alias E or O.
+// every operand [2][L][N].  out must not alias E or O.  Results are in the
+// coefficient domain; the operands too, or, with `ntt`, in the NTT domain
+// (storage order, canonical): the first key-switched level above the leaves.
 struct SfKsBatch {
     const u64 *E;
     size_t E_stride, E_outer;
@@ -16,16 +18,93 @@ struct SfKsBatch {
     int first;
     int inner;
     int count;
+    int ntt;        // operands in the NTT domain
     int d;          // automorphism X -> X^d
+    unsigned dinv;  // d^-1 mod 2N (set by sf_ks_launch)
     unsigned s;     // O is multiplied by X^s
     int add_v;      // 1: out = v + KS(...), 0: plain rotation
-    const u64 *key; // [dnum][2][nm][N] NTT-domain values, then the same shape of Shoup companions
+    const u64 *key; // [dnum][2][nm][N] pairs of the NTT-domain values, storage order
     u64 *scratch;   // sf_ks_scratch_words(R) words per merge of one launch batch
 };
 
-size_t sf_ks_scratch_words(const SfRing &R);
-// One launch sequence (K1..K5) for B.count merges, scratch for all of them.
+// limbs of scratch per merge: ModUp extensions, accumulators, tau_d(u.a), and for
+// NTT-domain operands its inverse rows
+SF_HD int sf_ks_x2(const SfRing &R) { return 0; }
+SF_HD int sf_ks_acc(const SfRing &R) { return R.dnum * R.nm; }
+SF_HD int sf_ks_ta(const SfRing &R) { return sf_ks_acc(R) + 2 * R.nm; }
+SF_HD int sf_ks_x1(const SfRing &R) { return sf_ks_ta(R) + R.L; }
+SF_HD size_t sf_ks_scratch_words_dev(const SfRing &R, int ntt)
+{
+    return (size_t)(sf_ks_x1(R) + (ntt ? R.L : 0)) << R.log_n;
+}
+
+// words per merge (ntt = 1: room for either kind of operands)
+size_t sf_ks_scratch_words(const SfRing &R, int ntt = 1);
+// One launch sequence for B.count merges, scratch for all of them.
 sf_status sf_ks_launch(sf_ctx *ctx, const SfKsBatch &B, cudaStream_t st);
 // Splits B into launch batches of `batch` merges reusing `scratch`
 // (batch * sf_ks_scratch_words words).
 sf_status sf_ks_run(sf_ctx *ctx, SfKsBatch B, u64 *scratch, int batch, cudaStream_t st);
+
+// The kernels of one launch sequence, each in its own translation unit:
+// ModUp columns (sf_ks_up.cu), rows with the inner product (sf_ks_rows.cu),
+// ModDown columns (sf_ks_down.cu).
+sf_status sf_ks_up_launch(sf_ctx *ctx, const SfKsBatch &B, cudaStream_t st);
+sf_status sf_ks_rows_launch(sf_ctx *ctx, const SfKsBatch &B, cudaStream_t st);
+sf_status sf_ks_down_launch(sf_ctx *ctx, const SfKsBatch &B, cudaStream_t st);
+sf_status sf_ks_up_init();
+sf_status sf_ks_rows_init();
+sf_status sf_ks_down_init();
+
+#if defined(__CUDACC__)
+__device__ __forceinline__ void merge_gt(const SfKsBatch &B, int b, int &g, int &t)
+{
+    const int x = B.first + b;
+    g = x / B.inner;
+    t = x - g * B.inner;
+}
+__device__ __forceinline__ const u64 *merge_E(const SfKsBatch &B, int b)
+{
+    int g, t;
+    merge_gt(B, b, g, t);
+    return B.E + B.E_outer * g + B.E_stride * t;
+}
+__device__ __forceinline__ const u64 *merge_O(const SfKsBatch &B, int b)
+{
+    if (!B.O) return nullptr;
+    int g, t;
+    merge_gt(B, b, g, t);
+    return B.O + B.O_outer * g + B.O_stride * t;
+}
+__device__ __forceinline__ u64 *merge_out(const SfKsBatch &B, int b)
+{
+    int g, t;
+    merge_gt(B, b, g, t);
+    return B.out + B.out_outer * g + B.out_stride * t;
+}
+// this merge's scratch, limb `limb` of it
+__device__ __forceinline__ u64 *ks_limb(const SfRing &R, const SfKsBatch &B, int b, int limb)
+{
+    return B.scratch + sf_ks_scratch_words_dev(R, B.ntt) * b + ((size_t)limb << R.log_n);
+}
+
+// coefficient p of E + X^s O of one limb, canonical; e, o: the limb's N
+// coefficients (o may be null)
+__device__ __forceinline__ u64 merge_coef(const u64 *e, const u64 *o, int p, unsigned s, int n, u64 q)
+{
+    const u64 v = e[p];
+    if (!o) return v;
+    const int k = p - (int)s;
+    const u64 w = o[k & (n - 1)];
+    // X^s O has coefficient O[p - s], or -O[p - s + N] below s
+    return k < 0 ? sf_sub(v, w, q) : sf_add(v, w, q);
+}
+#endif
+
+// blocks of a persistent launch over n_units (group, item) units: one
+// resident wave (num_sms x occupancy blocks), at most one block per unit
+static inline int ks_wave_blocks(const sf_ctx *ctx, int occ, int n_units)
+{
+    const int w = ctx->num_sms * occ;
+    return n_units < 1 ? 1 : (w < n_units ? w : n_units);
+}

@@ -7,16 +7,19 @@
 // (p = sigma_prev^-1(i)).  Three kernels per batch of outputs:
 //   leaf_prep: walks each output's receptive field once and buckets its taps
 //              by (input ciphertext, 16-column tile),
-//   leaf_col : builds the sparse w_{o,j} column tile in shared memory from its
-//              bucket and runs the forward column pass (or its closed form),
+//   leaf_col : scatters its bucket into a zeroed column tile in shared memory
+//              and runs the forward column pass,
 //   leaf_row : forward row pass, then the product with every input ciphertext
-//              (NTT domain, Shoup companions stored beside it), lazy sums -> leaf.
+//              (pairs in storage order, sf_reg.cuh), lazy sums -> leaf (NTT
+//              domain, storage order).
 // Step 9 (shuffle) is the slot -> output map sigma_out; step 10 (packing) is
 // the PackLWEs tree plus field trace driven by sf_pack_tree below.
 #include "sf_internal.h"
 #include "sf_kernels.cuh"
 #include "sf_ks.h"
 #include "sf_layer.h"
+#include "sf_async.cuh"
+#include "sf_reg.cuh"
 
 __device__ __forceinline__ int leaf_output(const SfLeafParams &P, int slot)
 {
@@ -24,22 +27,12 @@ __device__ __forceinline__ int leaf_output(const SfLeafParams &P, int slot)
     return P.sig_out ? P.sig_out[slot] : slot;
 }
 
-// Taps of one column tile kept for the closed-form column pass.  A tile
-// with few taps skips the sweep: the column pass maps column c of a
-// polynomial to its values at the R roots of Y^R = -1, z_k =
-// phi^(2 brev(k) + 1) with phi = psi^C, so a single tap v at row r
-// contributes v * psi^(C r (2 brev(k) + 1) mod 2N) to row k -- R products per
-// tap instead of (R/2) log2 R butterflies per column.
-#define SF_LEAF_TAPS 128
-
-size_t sf_smem_leaf_col(const SfRing &R) { return sf_smem_col(R, 1) + sizeof(sf_tw) * 2 * R.r; }
-
 // Calls f(j, row, column, signed Wq) for every tap of output o: input
 // ciphertext j, and the coefficient N - k (or 0) of w_{o,j} it lands on as
 // (row, column) of the R x C split; the sign carries the X^-k = -X^(N-k) of
 // the extraction.  Threads split the taps.
 template <class F>
-__device__ __forceinline__ void leaf_taps_all(const SfRing &R, const SfGeo &g, const SfLeafParams &P, int o, F f)
+__device__ __forceinline__ void leaf_taps_all(const SfRing &R, const SfLeafParams &P, int o, F f)
 {
     const int co = o % P.C_out, hw = o / P.C_out;
     const int ho = hw / P.W_out, wo = hw % P.W_out;
@@ -58,7 +51,7 @@ __device__ __forceinline__ void leaf_taps_all(const SfRing &R, const SfGeo &g, c
             const int k = p & (R.n - 1);
             const int cidx = k ? R.n - k : 0;
             const int64_t wq = P.gamma2 ? 2 * wrow[tp.w] : wrow[tp.w];
-            f(p >> R.log_n, cidx >> g.log_c, cidx & (g.c - 1), k ? -wq : wq);
+            f(p >> R.log_n, cidx >> R.log_c, cidx & (R.c - 1), k ? -wq : wq);
             if (P.gamma2) {
                 // gamma = 2 (Lemma 1 at t = 2): the row is (N/2)^-1 (X^-k ct_j + X^-3k ct3_j), so
                 // the tap also lands at X^-3k of the power ct3_j.  With e = 3k mod 2N,
@@ -66,7 +59,7 @@ __device__ __forceinline__ void leaf_taps_all(const SfRing &R, const SfGeo &g, c
                 const int e = (3 * k) & (2 * R.n - 1);
                 const int c3 = e == 0 ? 0 : (e <= R.n ? R.n - e : 2 * R.n - e);
                 const bool neg = e != 0 && e <= R.n;
-                f(P.k_src + (p >> R.log_n), c3 >> g.log_c, c3 & (g.c - 1), neg ? -wq : wq);
+                f(P.k_src + (p >> R.log_n), c3 >> R.log_c, c3 & (R.c - 1), neg ? -wq : wq);
             }
         }
     }
@@ -74,7 +67,7 @@ __device__ __forceinline__ void leaf_taps_all(const SfRing &R, const SfGeo &g, c
 
 size_t sf_leaf_tap_words(const SfRing &R, int k_in, int max_taps, int slots)
 {
-    const size_t nb = (size_t)k_in * (R.c / SF_NB) + 1;
+    const size_t nb = (size_t)k_in * sf_leaf_tiles(R) + 1;
     return (size_t)slots * max_taps * 2 + (slots * nb + 1) / 2;
 }
 
@@ -85,15 +78,14 @@ size_t sf_leaf_tap_words(const SfRing &R, int k_in, int max_taps, int slots)
 __global__ void __launch_bounds__(256) k_leaf_prep(SfRing R, SfLeafParams P)
 {
     __shared__ int cnt[SF_MAX_BUCKETS + 1];
-    const SfGeo g = ring_geo(R);
     const int z = blockIdx.x;
     const int o = leaf_output(P, P.s0 + z * P.s_stride);
     if (o < 0) return;   // leaf_col skips this slot as well
-    const int nb = P.n_buckets, tiles = g.c / SF_NB;
+    const int nb = P.n_buckets, tiles = sf_leaf_tiles(R), wl = sf_leaf_width_log(R);
     int *off = P.tap_off + (size_t)z * (nb + 1);
     for (int b = threadIdx.x; b <= nb; b += blockDim.x) cnt[b] = 0;
     __syncthreads();
-    leaf_taps_all(R, g, P, o, [&](int j, int row, int col, int64_t) { atomicAdd(&cnt[j * tiles + (col >> 4)], 1); });
+    leaf_taps_all(R, P, o, [&](int j, int row, int col, int64_t) { atomicAdd(&cnt[j * tiles + (col >> wl)], 1); });
     __syncthreads();
     if (threadIdx.x == 0) {
         int acc = 0;
@@ -107,9 +99,10 @@ __global__ void __launch_bounds__(256) k_leaf_prep(SfRing R, SfLeafParams P)
     }
     __syncthreads();
     longlong2 *dst = P.tap_buf + (size_t)z * P.max_taps;
-    leaf_taps_all(R, g, P, o, [&](int j, int row, int col, int64_t wq) {
-        const int pos = atomicAdd(&cnt[j * tiles + (col >> 4)], 1);
-        dst[pos] = make_longlong2((row << 4) | (col & 15), wq);
+    leaf_taps_all(R, P, o, [&](int j, int row, int col, int64_t wq) {
+        const int pos = atomicAdd(&cnt[j * tiles + (col >> wl)], 1);
+        // the word of the padded column tile it lands on (SfColT)
+        dst[pos] = make_longlong2(((row + (row >> 3)) << wl) + (col & ((1 << wl) - 1)), wq);
     });
 }
 
@@ -121,185 +114,161 @@ __device__ __forceinline__ u64 leaf_coeff(const SfMod &M, int64_t wq)
     return (wq < 0 && v) ? M.q - v : v;
 }
 
-// leaf_col: grid (C/16 column tiles, k_in * L, slots).  smem: column
-// twiddles + 1 tile + the powers psi^(C e), e < 2R.
-template <int LR, int LC>
-__global__ void __launch_bounds__(SfThreads<LR>::value, SfThreads<LR>::value >= 512 ? 2 : 4) k_leaf_col(SfRing R, SfLeafParams P)
+// leaf_col: grid (column tiles, k_in * L, slots).  Bound by the integer
+// multiplier (one forward column pass per tile; the bucket holds a few taps to
+// a few hundred).
+template <int LR, int LC, bool PM>
+__global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_leaf_col(SfRing R, SfLeafParams P)
 {
-    constexpr int NT = SfThreads<LR>::value;
+    constexpr int NT = SfShape<LR>::NT, NB = SfShape<LR>::NB;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ u64 tap_v[SF_LEAF_TAPS];
-    __shared__ int tap_rc[SF_LEAF_TAPS];
-    // sparse form: taps sorted by column (start[b] .. start[b+1])
-    __shared__ int col_start[SF_NB + 1];
-    __shared__ int col_fill[SF_NB];
-    __shared__ int srt_t[SF_LEAF_TAPS];
-    constexpr SfGeoT<LR, LC> g{};
-    const int c0 = blockIdx.x * SF_NB;
+    const SfColT<LR, PM> T;
     const int j = blockIdx.y / R.L, i = blockIdx.y % R.L;
-    const int slot = P.s0 + blockIdx.z * P.s_stride;
-    const int o = leaf_output(P, slot);
-    if (o < 0) return;
+    if (leaf_output(P, P.s0 + blockIdx.z * P.s_stride) < 0) return;
     const SfMod &M = R.m[i];
-    sf_tw *tw = (sf_tw *)smem_raw;
-    u64 *sm = (u64 *)(tw + g.r);
-    sf_tw *pwc = (sf_tw *)(sm + tile_words(g.log_r));
-    constexpr int ne = SF_NB << LR;
-    u64 *dst = P.w1 + (((size_t)blockIdx.z * P.k_in + j) * R.L + i) * (size_t)(1 << (LR + LC));
+    sf_pair *tab = (sf_pair *)smem_raw;
+    u64 *tile = (u64 *)(tab + SfShape<LR>::S);
+    sf_stage_cols<LR>(tab, R.colP, i, 1);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) tile[threadIdx.x + e * NT] = 0;
+    __syncthreads();
     // this block's bucket of taps (built by leaf_prep)
     const int *off = P.tap_off + (size_t)blockIdx.z * (P.n_buckets + 1);
-    const int bk = j * (g.c / SF_NB) + blockIdx.x;
+    const int bk = j * ((1 << LC) / NB) + blockIdx.x;
     const int t0 = off[bk], nt = off[bk + 1] - t0;
     const longlong2 *src = P.tap_buf + (size_t)blockIdx.z * P.max_taps + t0;
-    if (threadIdx.x < SF_NB) col_fill[threadIdx.x] = 0;
-    if (nt <= P.sparse_max) {
-        // stage the powers for the closed form while the taps load
-        const sf_tw *pw = R.pwc + (size_t)i * 2 * g.r;
-        for (int e = threadIdx.x; e < 2 * g.r; e += NT) pwc[e] = pw[e];
+    for (int t = threadIdx.x; t < nt; t += NT) {
+        const longlong2 e = src[t];
+        tile[e.x] = leaf_coeff(M, e.y);
     }
     __syncthreads();
-    if (nt <= SF_LEAF_TAPS) {
-        for (int t = threadIdx.x; t < nt; t += blockDim.x) {
-            const longlong2 e = src[t];
-            tap_v[t] = leaf_coeff(M, e.y);
-            tap_rc[t] = (int)e.x;
-            atomicAdd(&col_fill[e.x & 15], 1);
-        }
-    }
-    __syncthreads();
-    if (nt <= P.sparse_max) {
-        // counting sort by column; the order inside a column does not matter (exact sums)
-        if (threadIdx.x == 0) {
-            int acc = 0;
-            for (int b = 0; b < SF_NB; ++b) {
-                col_start[b] = acc;
-                acc += col_fill[b];
-                col_fill[b] = col_start[b];
-            }
-            col_start[SF_NB] = acc;
-        }
-        __syncthreads();
-        for (int t = threadIdx.x; t < nt; t += blockDim.x) srt_t[atomicAdd(&col_fill[tap_rc[t] & 15], 1)] = t;
-        __syncthreads();
-        const unsigned emask = 2u * g.r - 1;
-        for (int e = threadIdx.x; e < ne; e += NT) {
-            const int k = e >> 4, b = e & 15;
-            const unsigned br2 = 2u * (__brev((unsigned)k) >> (32 - g.log_r)) + 1u;
-            u64 acc = 0;
-            for (int t = col_start[b]; t < col_start[b + 1]; ++t) {
-                const int tt = srt_t[t];
-                const sf_tw z = pwc[(((unsigned)tap_rc[tt] >> 4) * br2) & emask];
-                acc += sf_mul_shoup_lazy(tap_v[tt], z.x, z.y, M.q);
-            }
-            dst[col_gidx_t<LC>(c0, e)] = sf_reduce(acc, M.q, M.one_p);
-        }
-        return;
-    }
-    for (int e = threadIdx.x; e < tile_words(g.log_r); e += blockDim.x) sm[e] = 0;
-    load_col_tw_t<LR, NT>(tw, R.colT_f, i);
-    __syncthreads();
-    if (nt <= SF_LEAF_TAPS) {
-        for (int t = threadIdx.x; t < nt; t += blockDim.x) sm[(tap_rc[t] >> 4) * SF_PAD + (tap_rc[t] & 15)] = tap_v[t];
-    } else {
-        for (int t = threadIdx.x; t < nt; t += blockDim.x) {
-            const longlong2 e = src[t];
-            sm[(e.x >> 4) * SF_PAD + (e.x & 15)] = leaf_coeff(M, e.y);
-        }
-    }
-    __syncthreads();
-    // forward column pass; its last sweep writes the tile to global memory
-    u64 *gd = dst + c0;
-    col_forward_io<LR, NT>(sm, tw, M.q, [&](int k, int b) { return sm[tile_slot<SF_NB>(k, b)]; },
-                           [&](int k, int b, u64 v) { gd[((size_t)k << LC) + b] = v; });
+    u64 x[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) x[t] = tile[T.at(T.k1(t))];
+    T.forward(x, tab, tile, M);   // its first exchange waits for these reads
+    u64 *dst = P.w1 + ((((size_t)blockIdx.z * P.k_in + j) * R.L + i) << (LR + LC)) + blockIdx.x * NB + T.b;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) dst[(size_t)T.kl(t) << LC] = x[t];
 }
 
-// leaf_row: grid (R/16 row tiles, L, slots).  smem: forward row twiddles + 1 tile.
-template <int LR, int LC, int RAD = 0>
-__global__ void __launch_bounds__(SfRow<LC>::NT, 3) k_leaf_row(SfRing R, SfLeafParams P)
+// leaf_row: persistent; groups (row tile, limb i), items slots.  Per input
+// ciphertext a forward row pass and two multiply-accumulates per point, the
+// accumulators in registers.  Bound by the integer multiplier; the staged
+// twiddles (61 KB at 256-point rows) serve every slot of the group.
+template <int LR, int LC, bool PM>
+__global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS_ACC) k_leaf_row(SfRing R, SfLeafParams P, int ng, int cnt)
 {
-    constexpr int NT = SfRow<LC>::NT, NB = SfRow<LC>::NB, EPT = SfRow<LC>::ELEMS / NT;
+    constexpr int NT = SfShape<LC>::NT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr SfGeoT<LR, LC> g{};
-    const int r0 = blockIdx.x * NB, i = blockIdx.y;
-    const int slot = P.s0 + blockIdx.z * P.s_stride;
-    const int o = leaf_output(P, slot);
-    const size_t tile_off = (size_t)r0 * g.c;
-    u64 *leaf = P.leaves + P.leaf_stride * blockIdx.z;
-    u64 *da = leaf + ((size_t)i << (LR + LC)) + tile_off;
-    u64 *db = leaf + ((size_t)(R.L + i) << (LR + LC)) + tile_off;
-    if (o < 0) {
+    const SfRowT<LC, PM> T;
+    sf_pair *tw = (sf_pair *)smem_raw;
+    u64 *buf = (u64 *)(tw + SfShape<LC>::PAIRS), *pre = buf + SfShape<LC>::WORDS + threadIdx.x;
+    const SfUnitRange U = sf_unit_range(ng * cnt);
+    const sf_pair *ct = (const sf_pair *)P.ct;
+    // group = (row tile, limb), item = slot; each thread copies its own points of
+    // an input ciphertext ahead (padding slots copy whatever the scratch holds)
+    struct Group {
+        int i, tile;
+        size_t off;   // this thread's row in the limb, from a ciphertext's first limb
+    };
+    auto group = [&](int grp) -> Group {
+        const int tile = grp / R.L, i = grp - tile * R.L;
+        return {i, tile, ((size_t)i << (LR + LC)) + ((size_t)T.row(tile, 1 << LR) << LC)};
+    };
+    const size_t per = (size_t)R.L << (LR + LC);
+    auto prefetch = [&](const Group &G, int z, int j) {
+        const u64 *src = P.w1 + ((size_t)z * P.k_in + j) * per + G.off;
 #pragma unroll
-        for (int k = 0; k < EPT; ++k) {
-            const int e = threadIdx.x + k * NT;
-            da[e] = 0;
-            db[e] = 0;
+        for (int t = 0; t < 8; ++t) sf_cp8(pre + t * NT, src + T.k1(t));
+        sf_cp_commit();
+    };
+    SfCursor C(U.u0, cnt);
+    Group G = group(C.grp), N = G;
+    if (U.u0 < U.u1) prefetch(G, C.item, 0);
+    int staged = -1;
+    for (int u = U.u0; u < U.u1; ++u) {
+        const int z = C.item;
+        if (C.grp != staged) {
+            __syncthreads();   // the previous group's readers are done
+            sf_stage_row<LR, LC>(tw, R.rowP, G.i, G.tile);
+            staged = C.grp;
+            __syncthreads();
         }
-        return;
-    }
-    sf_tw *tw = (sf_tw *)smem_raw;
-    u64 *sm = (u64 *)(tw + NB * g.c);
-    const SfMod M = R.m[i];
-    load_row_tw_t<LR, LC, NT>(tw, R.rowT_f, i, r0);
-    // per input ciphertext w * ct (w < 68q lazy, ct < q with its Shoup
-    // companion) lands in [0, 4q) and is summed: below 4 q k_in < 2^63 for k_in < 1024
-    u64 acc_a[EPT], acc_b[EPT];
+        const SfMod &M = R.m[G.i];
+        C.next();
+        if (C.grp != staged) N = group(C.grp);
+        // per input ciphertext w * ct (w lazy, ct < q with its companion) lands
+        // below off <= 2^58 and is summed, with a partial reduction every 16
+        u64 acc_a[8], acc_b[8], x[8];
 #pragma unroll
-    for (int k = 0; k < EPT; ++k) acc_a[k] = acc_b[k] = 0;
-    for (int j = 0; j < P.k_in; ++j) {
-        const u64 *src = P.w1 + (((size_t)blockIdx.z * P.k_in + j) * R.L + i) * (size_t)(1 << (LR + LC)) + tile_off;
+        for (int t = 0; t < 8; ++t) acc_a[t] = acc_b[t] = 0;
+        const sf_pair *ca = ct + ((size_t)G.i << (LR + LC)) + T.store_at(G.tile, 0);
+#pragma unroll 1
+        for (int j = 0; j < P.k_in; ++j) {
+            sf_cp_wait<0>();
 #pragma unroll
-        for (int x = 0; x < EPT; ++x) {
-            const int e = threadIdx.x + x * NT;
-            sm[row_slot_t<LC>(e)] = src[e];
+            for (int t = 0; t < 8; ++t) x[t] = pre[t * NT];
+            T.template phase_fwd<0>(x, tw, M);
+            if (j + 1 < P.k_in) prefetch(G, z, j + 1);   // the points of this one are in registers
+            else if (u + 1 < U.u1) prefetch(N, C.item, 0);
+            T.forward_rest(x, tw, buf, M);
+            const sf_pair *cb = ca + per;
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                const sf_pair a = __ldg(ca + t * NT), b = __ldg(cb + t * NT);
+                acc_a[t] = sf_mad<PM>(acc_a[t], x[t], a, M);
+                acc_b[t] = sf_mad<PM>(acc_b[t], x[t], b, M);
+            }
+            ca = cb + per;
+            if ((j & 15) == 15) {
+#pragma unroll
+                for (int t = 0; t < 8; ++t) acc_a[t] = sf_red3(acc_a[t], M), acc_b[t] = sf_red3(acc_b[t], M);
+            }
         }
-        __syncthreads();
-        row_forward_t<LC, NT, RAD>(sm, tw, M.q);
-        const size_t comp = (size_t)P.k_in * 2 * R.L << (LR + LC);
-        const u64 *ca = P.ct + (((size_t)j * 2 + 0) * R.L + i) * (size_t)(1 << (LR + LC)) + tile_off;
-        const u64 *cb = P.ct + (((size_t)j * 2 + 1) * R.L + i) * (size_t)(1 << (LR + LC)) + tile_off;
+        const bool live = leaf_output(P, P.s0 + z * P.s_stride) >= 0;   // padding leaves are zero
+        u64 *da = P.leaves + P.leaf_stride * z + ((size_t)G.i << (LR + LC)) + T.store_at(G.tile, 0), *db = da + per;
 #pragma unroll
-        for (int k = 0; k < EPT; ++k) {
-            const int e = threadIdx.x + k * NT;
-            const u64 w = sm[row_slot_t<LC>(e)];
-            acc_a[k] += sf_mul_shoup_lazy4(w, __ldg(ca + e), __ldg(ca + comp + e), M.q);
-            acc_b[k] += sf_mul_shoup_lazy4(w, __ldg(cb + e), __ldg(cb + comp + e), M.q);
+        for (int t = 0; t < 8; ++t) {
+            da[t * NT] = live ? sf_canon(acc_a[t], M) : 0;
+            db[t * NT] = live ? sf_canon(acc_b[t], M) : 0;
         }
-        __syncthreads();
+        G = N;
     }
-#pragma unroll
-    for (int k = 0; k < EPT; ++k) {
-        const int e = threadIdx.x + k * NT;
-        da[e] = sf_reduce(acc_a[k], M.q, M.one_p);
-        db[e] = sf_reduce(acc_b[k], M.q, M.one_p);
-    }
+}
+
+template <int LR>
+static constexpr size_t leaf_smem_col() { return sizeof(sf_pair) * SfShape<LR>::S + sizeof(u64) * SfShape<LR>::WORDS; }
+template <int LC>
+static constexpr size_t leaf_smem_row()
+{
+    return sizeof(sf_pair) * SfShape<LC>::PAIRS + sizeof(u64) * (SfShape<LC>::WORDS + SfShape<LC>::TILE);
 }
 
 sf_status sf_leaves_launch(sf_ctx *ctx, const SfLeafParams &P, int cnt, cudaStream_t st)
 {
     const SfRing &R = ctx->ring;
     if (cnt <= 0) return SF_OK;
-    const size_t smem_c = sf_smem_leaf_col(R), smem_r = sf_smem_row(R, 1);
-    // closed form while nt R products cost less than the tile's 16 (R/2) log2 R butterflies
-    const int sparse_max = std::min(SF_LEAF_TAPS, ctx->leaf_sparse >= 0 ? ctx->leaf_sparse : SF_NB * R.log_r / 2);
     cudaEvent_t ev;
     for (int off = 0; off < cnt; off += 65535) {
         SfLeafParams p = P;
-        p.sparse_max = sparse_max;
         const int c = std::min(65535, cnt - off);
         p.s0 = P.s0 + off * P.s_stride;
         p.w1 = P.w1;    // w1 holds `cnt` slots; reuse from its start for each sub-launch
         p.leaves = P.leaves + P.leaf_stride * off;
-        if (P.n_buckets > SF_MAX_BUCKETS) return sf_set_error(SF_EINVAL, "too many input ciphertexts for one round");
+        if (P.k_in * sf_leaf_tiles(R) > SF_MAX_BUCKETS) return sf_set_error(SF_EINVAL, "too many input ciphertexts for one round");
         sf_launch_begin(ctx, SFK_LEAF_PREP, st, &ev);
         k_leaf_prep<<<c, 256, 0, st>>>(R, p);
         sf_launch_end(ctx, SFK_LEAF_PREP, st, ev);
-        sf_launch_begin(ctx, SFK_LEAF_COL, st, &ev);
-        SF_GEO_DISPATCH(R.log_n, k_leaf_col<LR, LC><<<dim3(R.c / SF_NB, P.k_in * R.L, c), SfThreads<LR>::value, smem_c, st>>>(R, p););
-        sf_launch_end(ctx, SFK_LEAF_COL, st, ev);
-        sf_launch_begin(ctx, SFK_LEAF_ROW, st, &ev);
-        const dim3 gr(R.r / sf_row_nb(R.log_c), R.L, c);
-        SF_GEO_DISPATCH(R.log_n, SF_RAD_DISPATCH(ctx->row_radix, k_leaf_row<LR, LC, RAD><<<gr, SfRow<LC>::NT, smem_r, st>>>(R, p);););
-        sf_launch_end(ctx, SFK_LEAF_ROW, st, ev);
+        SF_RING_DISPATCH(R, {
+            sf_launch_begin(ctx, SFK_LEAF_COL, st, &ev);
+            k_leaf_col<LR, LC, PM><<<dim3((1 << LC) / SfShape<LR>::NB, P.k_in * R.L, c), SfShape<LR>::NT, leaf_smem_col<LR>(), st>>>(R, p);
+            sf_launch_end(ctx, SFK_LEAF_COL, st, ev);
+            sf_launch_begin(ctx, SFK_LEAF_ROW, st, &ev);
+            const int ng = ((1 << LR) / SfShape<LC>::NB) * R.L;
+            const int occ = sf_occupancy(k_leaf_row<LR, LC, PM>, SfShape<LC>::NT, leaf_smem_row<LC>());
+            k_leaf_row<LR, LC, PM><<<ks_wave_blocks(ctx, occ, ng * c), SfShape<LC>::NT, leaf_smem_row<LC>(), st>>>(R, p, ng, c);
+            sf_launch_end(ctx, SFK_LEAF_ROW, st, ev);
+        });
     }
     SF_CUDA_TRY(cudaGetLastError());
     return SF_OK;
@@ -307,16 +276,15 @@ sf_status sf_leaves_launch(sf_ctx *ctx, const SfLeafParams &P, int cnt, cudaStre
 
 // ------------------------------------------------------------ pack tree --
 
-// Level-1 merge at gamma = 2, NTT domain: out = E + X^s O (out = E without O).
+// Level-1 merge at gamma = 2: out = E + X^s O (out = E without O), in the NTT
+// domain (storage order) or the coefficient domain as B.ntt says.
 // grid (N / (256 SF_EW), L, merges), SfKsBatch indexing as in the key switch.
 #define SF_EW2 8
 __global__ void __launch_bounds__(256) k_merge_plain(SfRing R, SfKsBatch B)
 {
     const int b = blockIdx.z, i = blockIdx.y;
-    int g = (B.first + b) / B.inner, t = (B.first + b) - g * B.inner;
-    const u64 *E = B.E + B.E_outer * g + B.E_stride * t;
-    const u64 *O = B.O ? B.O + B.O_outer * g + B.O_stride * t : nullptr;
-    u64 *out = B.out + B.out_outer * g + B.out_stride * t;
+    const u64 *E = merge_E(B, b), *O = merge_O(B, b);
+    u64 *out = merge_out(B, b);
     const SfMod &M = R.m[i];
     const size_t pb = (size_t)i << (R.log_n + 1);
     const int j0 = blockIdx.x * (256 * SF_EW2) + threadIdx.x;
@@ -324,14 +292,17 @@ __global__ void __launch_bounds__(256) k_merge_plain(SfRing R, SfKsBatch B)
     for (int x = 0; x < SF_EW2; ++x) {
         const int j = j0 + x * 256;
         if (j >= R.n) break;
+        const unsigned kk = B.ntt ? mono_index(sf_natural_index(j, R.log_r, R.log_c), B.s, R.log_n) : 0;
         for (int part = 0; part < 2; ++part) {
-            const size_t off = ((size_t)(part * R.L + i) << R.log_n) + j;
-            u64 v = E[off];
-            if (O) {
-                const unsigned kk = mono_index(j, B.s, R.log_n);
-                v = sf_add(v, sf_mul_shoup(O[off], R.pw[pb + kk], R.pw_p[pb + kk], M.q), M.q);
+            const size_t limb = (size_t)(part * R.L + i) << R.log_n;
+            u64 v;
+            if (B.ntt) {
+                v = E[limb + j];
+                if (O) v = sf_add(v, sf_mul_shoup(O[limb + j], R.pw[pb + kk], R.pw_p[pb + kk], M.q), M.q);
+            } else {
+                v = merge_coef(E + limb, O ? O + limb : nullptr, j, B.s, R.n, M.q);
             }
-            out[off] = v;
+            out[limb + j] = v;
         }
     }
 }
@@ -359,7 +330,8 @@ static sf_status merge_plain_run(sf_ctx *ctx, const SfKsBatch &B, cudaStream_t s
 // level lvl-1) using s = N / 2^lvl and d = 2^lvl + 1.
 sf_status sf_pack_tree(sf_ctx *ctx, const u64 *keys_base, const std::vector<int32_t> &key_d, size_t key_words,
                        u64 *A, u64 *B, int G, int n_nodes, int level0, const std::vector<int> &valid, bool trace,
-                       u64 *ks_scratch, int batch, u64 **res, size_t *res_stride, cudaStream_t st, bool tau3_done)
+                       u64 *ks_scratch, int batch, u64 **res, size_t *res_stride, bool *ntt, cudaStream_t st,
+                       bool tau3_done)
 {
     const SfRing &R = ctx->ring;
     const size_t ct = (size_t)2 * R.L * R.n;
@@ -397,6 +369,7 @@ sf_status sf_pack_tree(sf_ctx *ctx, const u64 *keys_base, const std::vector<int3
         kb.d = d;
         kb.s = (unsigned)(R.n >> lvl);
         kb.add_v = 1;
+        kb.ntt = *ntt;
         kb.key = key;
         int gi = 0;
         while (gi < G) {
@@ -438,6 +411,7 @@ sf_status sf_pack_tree(sf_ctx *ctx, const u64 *keys_base, const std::vector<int3
         }
         std::swap(cur, nxt);
         std::swap(cur_gs, nxt_gs);
+        if (!plain) *ntt = false;   // a key switch leaves coefficients
     }
     // field trace: for k = level1+1 .. log2(N): ct <- ct + tau_{2^k+1}(ct)
     // (from k = 2 at gamma = 2: the client's power supplied the tau_3 term)
@@ -455,10 +429,12 @@ sf_status sf_pack_tree(sf_ctx *ctx, const u64 *keys_base, const std::vector<int3
         b.count = G;
         b.d = d;
         b.add_v = 1;
+        b.ntt = *ntt;
         b.key = key;
         SF_TRY(sf_ks_run(ctx, b, ks_scratch, batch, st));
         std::swap(cur, nxt);
         std::swap(cur_gs, nxt_gs);
+        *ntt = false;
     }
     *res = cur;
     *res_stride = cur_gs;
@@ -591,23 +567,8 @@ sf_status sf_extract_launch(sf_ctx *ctx, const u64 *ct, u64 *out, int i, cudaStr
 sf_status sf_layer_init_attributes()
 {
     const int mx = 227 * 1024;
-#define SF_LEAF_ATTRS(LR, LC)                                                                               \
-    {                                                                                                        \
-        /* the tap list is static shared memory: the dynamic part gets the rest */                          \
-        cudaFuncAttributes fa;                                                                               \
-        SF_CUDA_TRY(cudaFuncGetAttributes(&fa, k_leaf_col<LR, LC>));                                         \
-        SF_CUDA_TRY(cudaFuncSetAttribute(k_leaf_col<LR, LC>, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
-                                         mx - (int)fa.sharedSizeBytes));                                     \
-    }
-    SF_LEAF_ATTRS(5, 5) SF_LEAF_ATTRS(5, 6) SF_LEAF_ATTRS(6, 6) SF_LEAF_ATTRS(6, 7) SF_LEAF_ATTRS(7, 7)
-    SF_LEAF_ATTRS(7, 8) SF_LEAF_ATTRS(7, 9)
-#undef SF_LEAF_ATTRS
-#define SF_LEAF_ROW_ATTR(LR, LC) \
-    SF_CUDA_TRY(cudaFuncSetAttribute((k_leaf_row<LR, LC>), cudaFuncAttributeMaxDynamicSharedMemorySize, mx)); \
-    SF_CUDA_TRY(cudaFuncSetAttribute((k_leaf_row<LR, LC, 1>), cudaFuncAttributeMaxDynamicSharedMemorySize, mx)); \
-    SF_CUDA_TRY(cudaFuncSetAttribute((k_leaf_row<LR, LC, 2>), cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
-    SF_LEAF_ROW_ATTR(5, 5) SF_LEAF_ROW_ATTR(5, 6) SF_LEAF_ROW_ATTR(6, 6) SF_LEAF_ROW_ATTR(6, 7) SF_LEAF_ROW_ATTR(7, 7)
-    SF_LEAF_ROW_ATTR(7, 8) SF_LEAF_ROW_ATTR(7, 9)
-#undef SF_LEAF_ROW_ATTR
+#define SF_ATTR(K) SF_CUDA_TRY(cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
+    SF_FOR_RINGS({ SF_ATTR((k_leaf_col<LR, LC, PM>)) SF_ATTR((k_leaf_row<LR, LC, PM>)) });
+#undef SF_ATTR
     return SF_OK;
 }

@@ -56,7 +56,10 @@ extern "C" sf_status sf_rotate_noalloc(sf_ctx *ctx, const sf_rotkeys *rk, int32_
     const size_t ct = (size_t)2 * R.L * R.n;
     // key switches run in launch batches of the context's size, as in sf_rotate
     const int batch = std::min(ctx->ks_batch, (int)count);
-    const size_t need = 2 * round_words((size_t)count * ct) + round_words(sf_ks_scratch_words(R) * batch);
+    // the documented limit: two ciphertexts and this many key-switch limbs per
+    // call (the key switch itself uses less)
+    const size_t limbs = R.L + std::max(R.L, 2 * R.K) + std::max(R.dnum * R.nm, 2 * R.L) + 2 * R.L;
+    const size_t need = 2 * round_words((size_t)count * ct) + round_words((limbs << R.log_n) * batch);
     if (need > SF_NOALLOC_SCRATCH_WORDS)
         return sf_set_error(SF_EINVAL,
                             "sf_rotate_noalloc: %d ciphertexts need %zu bytes of scratch, the fixed maximum is %zu bytes",
@@ -64,40 +67,23 @@ extern "C" sf_status sf_rotate_noalloc(sf_ctx *ctx, const sf_rotkeys *rk, int32_
     u64 *ws = nullptr;
     SF_TRY(noalloc_scratch(ctx->device, &ws));
     cudaStream_t st = (cudaStream_t)stream;
-    u64 *in_ntt = ws, *out_ntt = ws + round_words((size_t)count * ct);
-    u64 *ks = out_ntt + round_words((size_t)count * ct);
     // per-launch event bracketing would create CUDA events; keep this call free of that
     const int timing = ctx->kernel_timing;
     ctx->kernel_timing = 0;
     sf_status s = SF_OK;
     {
-        SfPolyJob jobs[64];
-        for (int x0 = 0; x0 < count * 2 * R.L && s == SF_OK; x0 += 64) {
-            int cnt = 0;
-            for (int x = x0; x < count * 2 * R.L && cnt < 64; ++x, ++cnt)
-                jobs[cnt] = {d_ct + (size_t)x * R.n, in_ntt + (size_t)x * R.n, x % R.L};
-            s = sf_ntt_jobs(ctx, jobs, cnt, false, st);
-        }
-        if (s == SF_OK) {
-            SfKsBatch b;
-            memset(&b, 0, sizeof(b));
-            b.E = in_ntt;
-            b.E_stride = ct;
-            b.out = out_ntt;
-            b.out_stride = ct;
-            b.inner = 1 << 30;
-            b.count = count;
-            b.d = d;
-            b.add_v = 0;
-            b.key = rk->d_keys + rk->key_words * slot;
-            s = sf_ks_run(ctx, b, ks, batch, st);
-        }
-        for (int x0 = 0; x0 < count * 2 * R.L && s == SF_OK; x0 += 64) {
-            int cnt = 0;
-            for (int x = x0; x < count * 2 * R.L && cnt < 64; ++x, ++cnt)
-                jobs[cnt] = {out_ntt + (size_t)x * R.n, d_out + (size_t)x * R.n, x % R.L};
-            s = sf_ntt_jobs(ctx, jobs, cnt, true, st);
-        }
+        SfKsBatch b;
+        memset(&b, 0, sizeof(b));
+        b.E = d_ct;
+        b.E_stride = ct;
+        b.out = d_out;
+        b.out_stride = ct;
+        b.inner = 1 << 30;
+        b.count = count;
+        b.d = d;
+        b.add_v = 0;
+        b.key = rk->d_keys + rk->key_words * slot;
+        s = sf_ks_run(ctx, b, ws, batch, st);
     }
     ctx->kernel_timing = timing;
     return s;

@@ -3,85 +3,93 @@
 // products, encryption and decryption finishing, key generation).
 #include "sf_internal.h"
 #include "sf_kernels.cuh"
+#include "sf_reg.cuh"
 
-// One pass of a batched transform.  blockIdx.y selects the job, blockIdx.x
-// the tile.  Forward = column pass (reads job.src) then row pass (reduces to
-// [0, q)); inverse = row pass (reads job.src) then column pass (multiplies by
-// N^-1 and reduces).  Later passes work in place on job.dst.
-template <bool INV, bool COLS, int NT>
-__global__ void __launch_bounds__(NT) k_ntt_pass(SfRing R, SfJobList jobs)
+// One pass of a batched transform (sf_reg.cuh).  blockIdx.y selects the job,
+// blockIdx.x the tile.  Forward = column pass (reads job.src) then row pass
+// (reduces to [0, q)); inverse = row pass (reads job.src) then column pass
+// (multiplies by N^-1 and reduces).  The second pass works in place on job.dst.
+template <bool INV, bool COLS, int LR, int LC, bool PM>
+__global__ void __launch_bounds__(COLS ? SfShape<LR>::NT : SfShape<LC>::NT) k_ntt_pass(SfRing R, SfJobList jobs)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SfPolyJob jb = jobs.j[blockIdx.y];
-    const SfGeo g = ring_geo(R);
-    const SfMod M = R.m[jb.mod];
-    const bool first = (INV != COLS);   // forward starts with columns, inverse with rows
-    const u64 *src = first ? jb.src : jb.dst;
-    sf_tw *tw = (sf_tw *)smem_raw;
-    if (COLS) {
-        u64 *s = (u64 *)(tw + g.r);
-        const int c0 = blockIdx.x * SF_NB;
-        load_col_tw(tw, INV ? R.colT_i : R.colT_f, g, jb.mod);
-        for (int e = threadIdx.x; e < col_elems(g); e += blockDim.x) s[col_slot(e)] = src[col_gidx(g, c0, e)];
+    const SfMod &M = R.m[jb.mod];
+    const u64 *src = (INV != COLS) ? jb.src : jb.dst;   // forward starts with columns, inverse with rows
+    sf_pair *tw = (sf_pair *)smem_raw;
+    if constexpr (COLS) {
+        const SfColT<LR, PM> T;
+        u64 x[8];
+        u64 *buf = (u64 *)(tw + SfShape<LR>::S);
+        const int c0 = blockIdx.x * SfShape<LR>::NB + T.b;
+        sf_stage_cols<LR>(tw, R.colP, jb.mod, 1);
+#pragma unroll
+        for (int t = 0; t < 8; ++t) x[t] = src[((size_t)(INV ? T.kl(t) : T.k1(t)) << LC) + c0];
         __syncthreads();
-        if (INV) col_inverse<NT>(s, tw, g.log_r, M.q);
-        else col_forward<NT>(s, tw, g.log_r, M.q);
-        for (int e = threadIdx.x; e < col_elems(g); e += blockDim.x) {
-            u64 v = s[col_slot(e)];
-            if (INV) v = sf_csub(sf_mul_shoup_lazy(v, M.ninv, M.ninv_p, M.q), M.q);
-            jb.dst[col_gidx(g, c0, e)] = v;
+        if (INV) {
+            T.inverse(x, tw, buf, M);
+#pragma unroll
+            for (int t = 0; t < 8; ++t) jb.dst[((size_t)T.k1(t) << LC) + c0] = sf_canon(sf_mad<PM>(0, x[t], make_ulonglong2(M.ninv, M.ninv_c), M), M);
+        } else {
+            T.forward(x, tw, buf, M);
+#pragma unroll
+            for (int t = 0; t < 8; ++t) jb.dst[((size_t)T.kl(t) << LC) + c0] = x[t];
         }
     } else {
-        u64 *s = (u64 *)(tw + sf_row_nb(g.log_c) * g.c);
-        const int r0 = blockIdx.x * sf_row_nb(g.log_c);
-        load_row_tw(tw, INV ? R.rowT_i : R.rowT_f, g, jb.mod, r0);
-        const u64 *s0 = src + (size_t)r0 * g.c;
-        for (int e = threadIdx.x; e < row_elems(g); e += blockDim.x) s[row_slot(g, e)] = s0[e];
+        using T_ = SfRowT<LC, PM>;
+        const T_ T;
+        u64 x[8];
+        u64 *buf = (u64 *)(tw + SfShape<LC>::PAIRS);
+        const size_t row = (size_t)T.row(blockIdx.x, 1 << LR) << LC;
+        sf_stage_row<LR, LC>(tw, R.rowP, jb.mod, blockIdx.x);
+#pragma unroll
+        for (int t = 0; t < 8; ++t) x[t] = src[row + T.k1(t)];
         __syncthreads();
-        if (INV) row_inverse<NT>(s, tw, g.log_c, M.q);
-        else row_forward<NT>(s, tw, g.log_c, M.q);
-        u64 *d0 = jb.dst + (size_t)r0 * g.c;
-        for (int e = threadIdx.x; e < row_elems(g); e += blockDim.x) {
-            u64 v = s[row_slot(g, e)];
-            if (!INV) v = sf_reduce(v, M.q, M.one_p);
-            d0[e] = v;
+        if (INV) {
+            T.template exchange<T_::FIRST, T_::LAST>(x, buf);
+            T.inverse(x, tw, buf, M);
+#pragma unroll
+            for (int t = 0; t < 8; ++t) jb.dst[row + T.k1(t)] = sf_red3(x[t], M);
+        } else {
+            T.forward(x, tw, buf, M);
+            T.template exchange<T_::LAST, T_::FIRST>(x, buf);   // back to coalesced positions
+#pragma unroll
+            for (int t = 0; t < 8; ++t) jb.dst[row + T.k1(t)] = sf_canon(x[t], M);
         }
     }
 }
 
-// dynamic shared memory of the pass kernels
-size_t sf_smem_col(const SfRing &R, int tiles) { return sizeof(sf_tw) * R.r + sizeof(u64) * tile_words(R.log_r) * tiles; }
-size_t sf_smem_row(const SfRing &R, int tiles)
-{
-    return sizeof(sf_tw) * sf_row_nb(R.log_c) * R.c + sizeof(u64) * row_tile_words(R.log_c) * tiles;
-}
+template <int LR>
+static constexpr size_t smem_col() { return sizeof(sf_pair) * SfShape<LR>::S + sizeof(u64) * SfShape<LR>::WORDS; }
+template <int LC>
+static constexpr size_t smem_row() { return sizeof(sf_pair) * SfShape<LC>::PAIRS + sizeof(u64) * SfShape<LC>::WORDS; }
 
 sf_status sf_ntt_jobs(sf_ctx *ctx, const SfPolyJob *h_jobs, int n_jobs, bool inverse, cudaStream_t st)
 {
     const SfRing &R = ctx->ring;
-    const size_t smem_col = sf_smem_col(R, 1), smem_row = sf_smem_row(R, 1);
     for (int off = 0; off < n_jobs; off += SF_MAX_JOBS) {
         int cnt = std::min(SF_MAX_JOBS, n_jobs - off);
         SfJobList jl;
         for (int i = 0; i < cnt; ++i) jl.j[i] = h_jobs[off + i];
-        dim3 gc(R.c / SF_TC, cnt), gr(R.r / sf_row_nb(R.log_c), cnt);
         cudaEvent_t ev;
-        const int ntc = sf_tile_threads(R.log_r), ntr = SF_THREADS;   // row tiles: 256 threads
-        if (!inverse) {
-            sf_launch_begin(ctx, SFK_NTT_FWD_COL, st, &ev);
-            SF_NT_DISPATCH(ntc, k_ntt_pass<false, true, NT><<<gc, NT, smem_col, st>>>(R, jl););
-            sf_launch_end(ctx, SFK_NTT_FWD_COL, st, ev);
-            sf_launch_begin(ctx, SFK_NTT_FWD_ROW, st, &ev);
-            SF_NT_DISPATCH(ntr, k_ntt_pass<false, false, NT><<<gr, NT, smem_row, st>>>(R, jl););
-            sf_launch_end(ctx, SFK_NTT_FWD_ROW, st, ev);
-        } else {
-            sf_launch_begin(ctx, SFK_NTT_INV_ROW, st, &ev);
-            SF_NT_DISPATCH(ntr, k_ntt_pass<true, false, NT><<<gr, NT, smem_row, st>>>(R, jl););
-            sf_launch_end(ctx, SFK_NTT_INV_ROW, st, ev);
-            sf_launch_begin(ctx, SFK_NTT_INV_COL, st, &ev);
-            SF_NT_DISPATCH(ntc, k_ntt_pass<true, true, NT><<<gc, NT, smem_col, st>>>(R, jl););
-            sf_launch_end(ctx, SFK_NTT_INV_COL, st, ev);
-        }
+        SF_RING_DISPATCH(R, {
+            const dim3 gc((1 << LC) / SfShape<LR>::NB, cnt), gr((1 << LR) / SfShape<LC>::NB, cnt);
+            if (!inverse) {
+                sf_launch_begin(ctx, SFK_NTT_FWD_COL, st, &ev);
+                k_ntt_pass<false, true, LR, LC, PM><<<gc, SfShape<LR>::NT, smem_col<LR>(), st>>>(R, jl);
+                sf_launch_end(ctx, SFK_NTT_FWD_COL, st, ev);
+                sf_launch_begin(ctx, SFK_NTT_FWD_ROW, st, &ev);
+                k_ntt_pass<false, false, LR, LC, PM><<<gr, SfShape<LC>::NT, smem_row<LC>(), st>>>(R, jl);
+                sf_launch_end(ctx, SFK_NTT_FWD_ROW, st, ev);
+            } else {
+                sf_launch_begin(ctx, SFK_NTT_INV_ROW, st, &ev);
+                k_ntt_pass<true, false, LR, LC, PM><<<gr, SfShape<LC>::NT, smem_row<LC>(), st>>>(R, jl);
+                sf_launch_end(ctx, SFK_NTT_INV_ROW, st, ev);
+                sf_launch_begin(ctx, SFK_NTT_INV_COL, st, &ev);
+                k_ntt_pass<true, true, LR, LC, PM><<<gc, SfShape<LR>::NT, smem_col<LR>(), st>>>(R, jl);
+                sf_launch_end(ctx, SFK_NTT_INV_COL, st, ev);
+            }
+        });
     }
     SF_CUDA_TRY(cudaGetLastError());
     return SF_OK;
@@ -184,8 +192,9 @@ __global__ void k_signed_to_residues(SfRing R, const int64_t *v, u64 *out, int n
 struct SfPg {
     u64 v[SF_MAX_MODULI];
 };
+// key_a, key_b: pairs [nm][N] in storage order
 __global__ void k_rotkey_finish(SfRing R, const u64 *alpha, const u64 *e, const u64 *s_mont, SfPg pg, int d,
-                                u64 *key_a, u64 *key_b, size_t comp)
+                                ulonglong2 *key_a, ulonglong2 *key_b)
 {
     SF_GRID_STRIDE(i, (size_t)R.nm * R.n)
     {
@@ -204,11 +213,9 @@ __global__ void k_rotkey_finish(SfRing R, const u64 *alpha, const u64 *e, const 
             a = sf_mul_shoup(a, R.md_pinv[m], R.md_pinv_p[m], M.q);
             b = sf_mul_shoup(b, R.md_pinv[m], R.md_pinv_p[m], M.q);
         }
-        // plain values, then their Shoup companions `comp` words later
-        key_a[i] = a;
-        key_b[i] = b;
-        key_a[i + comp] = sf_shoup_companion_dev(a, M);
-        key_b[i + comp] = sf_shoup_companion_dev(b, M);
+        const size_t p = ((size_t)m << R.log_n) + sf_storage_index(j, R.log_r, R.log_c);
+        key_a[p] = sf_make_pair(a, M, R.pm);
+        key_b[p] = sf_make_pair(b, M, R.pm);
     }
 }
 
@@ -273,21 +280,33 @@ sf_status sf_signed_to_residues(sf_ctx *ctx, const int64_t *v, u64 *out, int n_p
 }
 
 sf_status sf_rotkey_finish(sf_ctx *ctx, const u64 *alpha, const u64 *e, const u64 *s_mont, const u64 *pg, int d,
-                           u64 *key_a, u64 *key_b, size_t comp, cudaStream_t st)
+                           ulonglong2 *key_a, ulonglong2 *key_b, cudaStream_t st)
 {
     SfPg p;
     for (int m = 0; m < SF_MAX_MODULI; ++m) p.v[m] = m < ctx->ring.nm ? pg[m] : 0;
-    SF_ELEM_LAUNCH(k_rotkey_finish, (size_t)ctx->ring.nm * ctx->ring.n, alpha, e, s_mont, p, d, key_a, key_b, comp);
+    SF_ELEM_LAUNCH(k_rotkey_finish, (size_t)ctx->ring.nm * ctx->ring.n, alpha, e, s_mont, p, d, key_a, key_b);
     return SF_OK;
 }
 
-// Shoup companions of NTT-domain residues, in place into dst: dst[i] = floor(x[i] 2^64 / q)
-__global__ void k_shoup_companions(SfRing R, const u64 *x, u64 *dst, int n_polys, int period, int offset)
+// NTT-domain residues (natural slot order) -> pairs in storage order
+__global__ void k_to_pairs(SfRing R, const u64 *x, ulonglong2 *dst, int n_polys, int period, int offset)
 {
     SF_GRID_STRIDE(i, (size_t)n_polys * R.n)
     {
         const SfMod &M = R.m[offset + (int)((i >> R.log_n) % period)];
-        dst[i] = sf_shoup_companion_dev(x[i], M);
+        const size_t base = i & ~(size_t)(R.n - 1);
+        const u64 v = x[base + sf_natural_index((int)(i & (R.n - 1)), R.log_r, R.log_c)];
+        dst[i] = sf_make_pair(v, M, R.pm);
+    }
+}
+
+// storage order -> natural slot order, the values of pairs (step 2) or plain words (step 1)
+__global__ void k_to_natural(SfRing R, const u64 *x, int step, u64 *dst, int n_polys)
+{
+    SF_GRID_STRIDE(i, (size_t)n_polys * R.n)
+    {
+        const size_t base = i & ~(size_t)(R.n - 1);
+        dst[i] = x[(base + sf_storage_index((int)(i & (R.n - 1)), R.log_r, R.log_c)) * step];
     }
 }
 
@@ -309,22 +328,26 @@ sf_status sf_check_residues(sf_ctx *ctx, const u64 *x, int n_polys, int period, 
     return SF_OK;
 }
 
-sf_status sf_companions(sf_ctx *ctx, const u64 *x, u64 *dst, int n_polys, int period, int offset, cudaStream_t st)
+sf_status sf_to_pairs(sf_ctx *ctx, const u64 *x, ulonglong2 *dst, int n_polys, int period, int offset, cudaStream_t st)
 {
-    SF_ELEM_LAUNCH(k_shoup_companions, (size_t)n_polys * ctx->ring.n, x, dst, n_polys, period, offset);
+    SF_ELEM_LAUNCH(k_to_pairs, (size_t)n_polys * ctx->ring.n, x, dst, n_polys, period, offset);
+    return SF_OK;
+}
+
+sf_status sf_to_natural(sf_ctx *ctx, const u64 *x, int step, u64 *dst, int n_polys, cudaStream_t st)
+{
+    SF_ELEM_LAUNCH(k_to_natural, (size_t)n_polys * ctx->ring.n, x, step, dst, n_polys);
     return SF_OK;
 }
 
 sf_status sf_ntt_init_attributes()
 {
     const int mx = 227 * 1024;
-#define SF_NTT_ATTR(NT)                                                                                             \
-    SF_CUDA_TRY(cudaFuncSetAttribute(k_ntt_pass<false, true, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));  \
-    SF_CUDA_TRY(cudaFuncSetAttribute(k_ntt_pass<false, false, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx)); \
-    SF_CUDA_TRY(cudaFuncSetAttribute(k_ntt_pass<true, true, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));   \
-    SF_CUDA_TRY(cudaFuncSetAttribute(k_ntt_pass<true, false, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
-    SF_NTT_ATTR(256)
-    SF_NTT_ATTR(512)
-#undef SF_NTT_ATTR
+#define SF_ATTR(K) SF_CUDA_TRY(cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
+    SF_FOR_RINGS({
+            SF_ATTR((k_ntt_pass<false, true, LR, LC, PM>)) SF_ATTR((k_ntt_pass<false, false, LR, LC, PM>))
+            SF_ATTR((k_ntt_pass<true, true, LR, LC, PM>)) SF_ATTR((k_ntt_pass<true, false, LR, LC, PM>))
+        });
+#undef SF_ATTR
     return SF_OK;
 }

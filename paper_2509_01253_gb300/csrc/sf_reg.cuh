@@ -1,295 +1,371 @@
 // sf_reg.cuh -- register-resident passes of the negacyclic NTT.
 //
-// A ring of N = R x C points is transformed as R-point columns and C-point
-// rows (R, C between 32 and 256; see sf_tile.cuh for the transform itself).  A
-// block of S threads runs 16 sub-transforms of S points, 16 points per thread,
-// in two register phases with one exchange through shared memory between them:
-//   phase 1: thread i of a sub-transform holds k = i + u S/16 + 16 t
-//            (t < S/16, u < 256/S), the stages of distance S/2 .. 16;
-//   phase 2: it holds k = 16 i + t, the stages of distance 8, 4, 2, 1.
-// The inverse runs them in the opposite order.  Global memory is read and
-// written straight from registers, so a pass costs one shared-memory round
-// trip (16 bytes per point) against four to six of the sweeps that keep the
-// tile in shared memory.  Row passes put the S/16 threads of a row in one warp:
-// their exchange needs no block barrier.
+// Transform (Longa-Naehrig 2016 merged form): forward Cooley-Tukey with the
+// table psi_brev[k] = psi^brev(k) (psi a primitive 2N-th root), natural-order
+// input, bit-reversed output: out[j] = a(psi^(2 brev(j) + 1)).  Inverse:
+// Gentleman-Sande with psi^-brev(k), then a factor N^-1.  Index j = r C + c with
+// N = R C (R, C between 32 and 256): the forward stages of distance >= C mix
+// elements of one column ("column pass"), the others stay inside one row.
+// Local stage of m groups, group g: global table index m + g for every column,
+// m (R + r) + g for row r.
 //
-// Twiddles are Shoup pairs (w, floor(w 2^64 / q)).  psi^-brev(m + g) =
+// A pass keeps its points in registers and exchanges them through shared memory
+// between phases; global memory is read and written straight from registers.
+//
+// Every thread holds 8 points and runs up to three stages per phase, in two
+// (32, 64 points) or three phases (128, 256 points).  A tile is 2048 points at
+// 128 and 256 points (16 or 8 sub-transforms, 256 threads): with three blocks
+// per SM a kernel has 24 warps and 85 registers a thread, which hold the
+// accumulators of the inner products or the converted digits beside the points.
+// The C/8 threads of a row share a warp, so row exchanges need no block barrier
+// and the warps of a block run independently; columns exchange through block
+// barriers.  16 points a thread (one exchange less, 128 registers, 16 warps)
+// lost: the inner product ran 25.6 us per key switch at N = 2^16, waiting on
+// memory and on instruction fetches.
+//
+// Twiddles are pairs (w, companion), see sf_mad.  psi^-brev(m + g) =
 // -psi^brev(m + (m - 1 - g)) for m = 2^a: the inverse twiddle of a group is
 // minus the forward twiddle of the mirrored group of its level, so one table
 // serves both directions (the inverse butterfly multiplies Y - X instead of
 // X - Y).  The mirror of row r is row R - 1 - r; a row tile therefore holds
-// eight rows and their mirrors, and the inverse pass reads the same staged
-// table at thread index tid ^ (9 S/16 - 1).
+// rows and their mirrors, and the inverse pass reads the same staged table at
+// mirrored positions.
 //
 // NTT-domain polynomials that stay inside the library (leaves, prepared
 // inputs, rotation keys) are stored in "storage order", [tile][t][thread] of a
-// row pass's phase 2, so that every kernel reads and writes them coalesced
+// row pass's last phase, so that every kernel reads and writes them coalesced
 // from registers (sf_storage_index).
 #pragma once
 #include "sf_arith.cuh"
 #include "sf_internal.h"
 
-typedef ulonglong2 sf_pair;   // (w, w')
+typedef ulonglong2 sf_pair;   // (w, companion)
 
-// shape of the sub-transforms of 2^LS points
+// Shape of a tile: NB sub-transforms of 2^LS points (for rows NB / 2 rows and
+// their mirrors), LP threads each.  Phase ph holds index bits P .. P + 2 of a
+// point's position k in the registers and runs the stages of distance
+// 2^HI .. 2^LO.
 template <int LS>
-struct SfSub {
-    static constexpr int S = 1 << LS, R1 = LS - 4, NI = S / 16, U = 256 / S, NT = S;
-    static constexpr int COL_WORDS = 16 * S;              // exchange buffer of a column tile, [k][b]
-    static constexpr int PITCH = 17 * NI;                 // row of a row tile: k + k / 16, conflict-free in both phases
-    static constexpr int ROW_WORDS = 16 * PITCH;
-    static constexpr int ROW_PAIRS = 16 * (S - 1);        // twiddles of a row tile
+struct SfShape {
+    static constexpr int LS_ = LS, S = 1 << LS, NB = LS == 8 ? 8 : 16, HALF = NB / 2, LP = S / 8, NT = NB * LP, TILE = NB * S;
+    // exchange buffers: a row k + k / 8 of [b], a column tile [k + k / 8][b]
+    static constexpr int PITCH = 9 * LP, WORDS = NB * PITCH;
+    static constexpr int PAIRS = NB * (S - 1);   // twiddles of a row tile
+    static constexpr int NP = LS >= 7 ? 3 : 2;
+    // blocks per SM: 24 warps of 80 registers; 16 of 128 for the kernels with the
+    // inner products' accumulators, which otherwise spill and hold back the key's
+    // loads (per round of 32768 key switches at N = 2^16, 5 + 2 primes: 548 ms at
+    // 24 warps, 490 at 16; the leaf rows 117 and 102 ms)
+    static constexpr int BPS = 768 / NT, BPS_ACC = 512 / NT;
+    SF_HD static constexpr int P(int ph) { return ph == 0 ? LS - 3 : (ph == 1 && LS >= 7) ? 2 : 0; }
+    SF_HD static constexpr int LO(int ph) { return P(ph); }
+    SF_HD static constexpr int HI(int ph) { return ph == 0 ? LS - 1 : P(ph - 1) - 1; }
+    // padded position k + k / 8 of register t of thread i in phase ph: pos(ph, i) + step(ph, t)
+    SF_HD static constexpr int pos(int ph, int i)
+    {
+        const int p = P(ph), hi = i >> p, lo = i & ((1 << p) - 1);
+        return (hi << (p + 3)) + lo + (hi << p) + (p >= 3 ? lo >> 3 : 0);
+    }
+    SF_HD static constexpr int step(int ph, int t)
+    {
+        const int p = P(ph);
+        return (t << p) + (p >= 3 ? t << (p - 3) : p == 2 ? t >> 1 : 0);
+    }
+    // groups of threads that share a phase's twiddles, in one row
+    SF_HD static constexpr int H(int ph) { return S >> (P(ph) + 3); }
+    // first entry of stage q (q <= HI) of phase ph among the phase's entries: 2^(P+2-q') per stage q'
+    SF_HD static constexpr int E(int ph, int q) { return (1 << (P(ph) + 2 - q)) - (1 << (P(ph) + 2 - HI(ph))); }
+    // first entry of phase ph in a row tile's table
+    SF_HD static constexpr int OFF(int ph)
+    {
+        return ph == 0 ? 0 : (ph == 1 ? 0 : E(1, LO(1) - 1) * NB * H(1)) + E(0, LO(0) - 1) * NB * H(0);
+    }
 };
 
-// ---- butterflies -----------------------------------------------------------
-
-// acc + (x*w mod q), the added term in [0, 4q): Shoup's product with the
-// truncated quotient (sf_mulhi_trunc); the accumulator rides through the wide
-// multiplies, which add it for free
-SF_HD u64 sf_mad_shoup_lazy4(u64 acc, u64 x, u64 w, u64 wp, u64 q)
+// ---- products and butterflies -----------------------------------------------
+// Two forms of a product by a fixed operand w < q, both with a stored companion
+// and both returning acc + r with r = x w (mod q), 0 <= r < off for any x < 2^64;
+// the accumulator rides through the wide multiplies, which add it for free.
+//
+// PM = false, any q < 2^51: Shoup's product, companion floor(w 2^64 / q), with
+// the truncated quotient (sf_mulhi_trunc): r < 4q.  9 multiplies, 19 instructions
+// a butterfly.
+//
+// PM = true, q = 2^50 - delta with small delta (the largest NTT primes of 50
+// bits): with x = x0 + 2^32 x1 and the companion v = 2^32 w mod q,
+//     x w = x0 w + x1 v = T (mod q),   T < 2^83,
+// and since q is almost 2^50 the high parts of w and v are the quotients
+// themselves: qh = floor(x0 floor(w / 2^19) / 2^32) + floor(x1 floor(v / 2^19) /
+// 2^32) is T / 2^51 less at most 4 (four floors), and below 2^32, so r = T - qh 2q
+// = (T - qh 2^51) + qh 2 delta lies in [0, 2^53 + 2^33 delta).  8 multiplies, 15
+// instructions: register-resident forward butterflies run at 1289 G/s against
+// 1164, inverse ones at 1272 against 1145.
+template <bool PM>
+__device__ __forceinline__ u64 sf_mad(u64 acc, u64 x, const sf_pair w, const SfMod &M)
 {
-    return acc + x * w + sf_mulhi_trunc(x, wp) * (0 - q);
+    if constexpr (PM) {
+        const unsigned x0 = (unsigned)x, x1 = (unsigned)(x >> 32);
+        const unsigned qh = __umulhi(x0, (unsigned)(w.x >> 19)) + __umulhi(x1, (unsigned)(w.y >> 19));
+        return acc + x0 * w.x + x1 * w.y + qh * M.n2q;
+    } else {
+        return acc + x * w.x + sf_mulhi_trunc(x, w.y) * (0 - M.q);
+    }
 }
 
-// forward: X + wY, X - wY + 4q; bounds grow by 4q per stage (below 72q < 2^57
-// after 16 stages from 8q)
-__device__ __forceinline__ void sf_fwd(u64 &X, u64 &Y, const sf_pair w, u64 q)
+// forward: X + wY, X - wY + off; bounds grow by off per stage, from at most
+// 4 off to 20 off < 2^63 after 16 stages (checked when the context is made)
+template <bool PM>
+__device__ __forceinline__ void sf_fwd(u64 &X, u64 &Y, const sf_pair w, const SfMod &M)
 {
     const u64 x = X;
-    X = sf_mad_shoup_lazy4(x, Y, w.x, w.y, q);
-    Y = x + x + 4 * q - X;
+    X = sf_mad<PM>(x, Y, w, M);
+    Y = x + x + M.off - X;
 }
 
-// inverse with the mirrored twiddle: X + Y, (Y - X) w.  At stage k of a pass
-// (k = 0 .. 7) inputs are below 4q 2^k and off = 4q 2^k, so the difference is
-// positive and below 2^(k+3) q <= 2^10 q < 2^60; no conditional subtraction.
-__device__ __forceinline__ void sf_inv(u64 &X, u64 &Y, const sf_pair w, u64 q, u64 off)
+// inverse with the mirrored twiddle: X + Y, (Y - X) w.  `off` is a multiple of q
+// above every input, so the difference is positive.  Inputs of a pass are below
+// 4q; after stage 0 values stay below off1 = max(8q, off) and the bound doubles
+// from stage to stage (sf_inv_off).
+template <bool PM>
+__device__ __forceinline__ void sf_inv(u64 &X, u64 &Y, const sf_pair w, const SfMod &M, u64 off)
 {
     const u64 d = Y - X + off;
     X = X + Y;
-    Y = sf_mad_shoup_lazy4(0, d, w.x, w.y, q);
+    Y = sf_mad<PM>(0, d, w, M);
 }
 
-// v < 2^63 (and below 2^32 q) brought below 3q: q̂ = floor((v >> sh) binv / 2^32)
-// is floor(v / q) minus at most 2
+// v < 2^63 (and below 2^32 q) brought below 3q: floor((v >> sh) binv / 2^32) is
+// floor(v / q) minus at most 2
 __device__ __forceinline__ u64 sf_red3(u64 v, const SfMod &M)
 {
     return v + (u64)__umulhi((unsigned)(v >> M.sh), M.binv) * (0 - M.q);
 }
 
-// ---- phases ------------------------------------------------------------------
-// x holds phase-1 element (t, u) at t U + u, phase-2 element t at t.  tw(k)
-// returns the twiddle of local index k (level 2^a: k = 2^a + group).
-
-template <int LS, class TW>
-__device__ __forceinline__ void sf_p1_fwd(u64 (&x)[16], TW tw, u64 q)
-{
-    constexpr int R1 = SfSub<LS>::R1, U = SfSub<LS>::U;
-#pragma unroll
-    for (int s = 0; s < R1; ++s) {
-        const int d = 1 << (R1 - 1 - s);
-#pragma unroll
-        for (int g = 0; g < (1 << s); ++g) {
-            const sf_pair w = tw((1 << s) + g);
-#pragma unroll
-            for (int a = 0; a < d; ++a)
-#pragma unroll
-                for (int u = 0; u < U; ++u) sf_fwd(x[(2 * d * g + a) * U + u], x[(2 * d * g + a + d) * U + u], w, q);
-        }
-    }
-}
-
-// tw(e): twiddle e = 2^s - 1 + g of the thread's 16 points (stage s, group g)
-template <class TW>
-__device__ __forceinline__ void sf_p2_fwd(u64 (&x)[16], TW tw, u64 q)
-{
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-        const int d = 8 >> s;
-#pragma unroll
-        for (int g = 0; g < (1 << s); ++g) {
-            const sf_pair w = tw((1 << s) - 1 + g);
-#pragma unroll
-            for (int a = 0; a < d; ++a) sf_fwd(x[2 * d * g + a], x[2 * d * g + a + d], w, q);
-        }
-    }
-}
-
-// inverse phase 2 (stages 0 .. 3 of the pass); tw(e) as above, mirrored
-template <class TW>
-__device__ __forceinline__ void sf_p2_inv(u64 (&x)[16], TW tw, u64 q)
-{
-#pragma unroll
-    for (int s = 3; s >= 0; --s) {
-        const int d = 8 >> s;
-        const u64 off = q << (2 + (3 - s));
-#pragma unroll
-        for (int g = 0; g < (1 << s); ++g) {
-            const sf_pair w = tw((1 << s) - 1 + g);
-#pragma unroll
-            for (int a = 0; a < d; ++a) sf_inv(x[2 * d * g + a], x[2 * d * g + a + d], w, q, off);
-        }
-    }
-}
-
-// inverse phase 1 (stages 4 .. 4 + R1 - 1 of the pass)
-template <int LS, class TW>
-__device__ __forceinline__ void sf_p1_inv(u64 (&x)[16], TW tw, u64 q)
-{
-    constexpr int R1 = SfSub<LS>::R1, U = SfSub<LS>::U;
-#pragma unroll
-    for (int s = R1 - 1; s >= 0; --s) {
-        const int d = 1 << (R1 - 1 - s);
-        const u64 off = q << (2 + 4 + (R1 - 1 - s));
-#pragma unroll
-        for (int g = 0; g < (1 << s); ++g) {
-            const sf_pair w = tw((1 << s) + g);
-#pragma unroll
-            for (int a = 0; a < d; ++a)
-#pragma unroll
-                for (int u = 0; u < U; ++u) sf_inv(x[(2 * d * g + a) * U + u], x[(2 * d * g + a + d) * U + u], w, q, off);
-        }
-    }
-}
+// v < 2^63 (and below 2^32 q) brought to [0, q)
+__device__ __forceinline__ u64 sf_canon(u64 v, const SfMod &M) { return sf_csub(sf_csub(sf_red3(v, M), M.q), M.q); }
 
 // ---- column tiles --------------------------------------------------------------
-// 16 columns of 2^LR points; thread: column b = tid & 15, i = tid >> 4, so a
-// half-warp touches 16 consecutive words of one row of the polynomial.  The
-// column table is colT[k], k < R, staged once; buf is an exchange buffer.
+// NB columns of 2^LR points; thread: column b = tid % NB, i = tid / NB, so NB
+// consecutive threads touch NB consecutive words of one row of the polynomial.
+// Register t of phase ph holds k = (i >> P) 2^(P+3) + t 2^P + (i mod 2^P).  The
+// column table is tab[k], k < R; buf is the exchange buffer.
 
-template <int LR>
-struct SfCol {
-    using Sub = SfSub<LR>;
+// Bound of the inputs of inverse stage st (a multiple of q): 4q, off1, 2 off1, ...
+// The eighth stage would leave 64 bits no room, so after their second phase
+// (stages 2 to 4) 256-point passes reduce the one register that was a sum in all
+// of its stages (t = 0); the others were products at most two stages ago, below
+// 4 off1.
+template <int LS>
+__device__ __forceinline__ u64 sf_inv_off(int st, const SfMod &M)
+{
+    if (st == 0) return 4 * M.q;
+    return M.off1 << (LS == 8 && st >= 5 ? st - 3 : st - 1);
+}
+
+template <int LR, bool PM>
+struct SfColT {
+    using Sh = SfShape<LR>;
+    static constexpr int LAST = Sh::NP - 1;
     int b, i;
-    __device__ __forceinline__ SfCol() : b(threadIdx.x & 15), i(threadIdx.x >> 4) {}
-    // row of phase-1 element r = t U + u, of phase-2 element t
-    __device__ __forceinline__ int k1(int r) const { return i + (r % Sub::U) * Sub::NI + 16 * (r / Sub::U); }
-    __device__ __forceinline__ int k2(int t) const { return 16 * i + t; }
+    __device__ __forceinline__ SfColT() : b(threadIdx.x % Sh::NB), i(threadIdx.x / Sh::NB) {}
+    template <int PH>
+    __device__ __forceinline__ int k(int t) const
+    {
+        constexpr int P = Sh::P(PH);
+        return ((i >> P) << (P + 3)) + (t << P) + (i & ((1 << P) - 1));
+    }
+    __device__ __forceinline__ int k1(int t) const { return k<0>(t); }
+    __device__ __forceinline__ int kl(int t) const { return k<LAST>(t); }
+    __device__ __forceinline__ int at(int kk) const { return (kk + (kk >> 3)) * Sh::NB + b; }
 
-    __device__ __forceinline__ void fwd1(u64 (&x)[16], const sf_pair *tab, u64 q) const
+    template <int PH>
+    __device__ __forceinline__ void phase_fwd(u64 (&x)[8], const sf_pair *tab, const SfMod &M) const
     {
-        sf_p1_fwd<LR>(x, [&](int k) { return tab[k]; }, q);
-    }
-    __device__ __forceinline__ void fwd2(u64 (&x)[16], const sf_pair *tab, u64 q) const
-    {
-        sf_p2_fwd(x, [&](int e) {
-            const int s = e >= 7 ? 3 : e >= 3 ? 2 : e >= 1 ? 1 : 0, g = e - ((1 << s) - 1);
-            return tab[(Sub::NI << s) + (i << s) + g];
-        }, q);
-    }
-    __device__ __forceinline__ void inv2(u64 (&x)[16], const sf_pair *tab, u64 q) const
-    {
-        sf_p2_inv(x, [&](int e) {
-            const int s = e >= 7 ? 3 : e >= 3 ? 2 : e >= 1 ? 1 : 0, g = e - ((1 << s) - 1);
-            return tab[(Sub::NI << s) + ((Sub::NI - 1 - i) << s) + (1 << s) - 1 - g];
-        }, q);
-    }
-    __device__ __forceinline__ void inv1(u64 (&x)[16], const sf_pair *tab, u64 q) const
-    {
-        sf_p1_inv<LR>(x, [&](int k) {
-            const int m = k >= 8 ? 8 : k >= 4 ? 4 : k >= 2 ? 2 : 1;
-            return tab[3 * m - 1 - k];
-        }, q);
-    }
-    // phase 1 -> phase 2 and back through buf; one block barrier each.  Passes
-    // that follow one another alternate between two buffers, so the barrier of
-    // one also orders the reads of the one before against the next writes.
-    __device__ __forceinline__ void to2(u64 (&x)[16], u64 *buf) const
-    {
+        constexpr int P = Sh::P(PH), HI = Sh::HI(PH), LO = Sh::LO(PH);
 #pragma unroll
-        for (int r = 0; r < 16; ++r) buf[k1(r) * 16 + b] = x[r];
+        for (int st = HI; st >= LO; --st) {
+            const int d = 1 << (st - P), lc = P + 2 - st;
+#pragma unroll
+            for (int sub = 0; sub < (1 << lc); ++sub) {
+                const sf_pair w = tab[(Sh::S >> (st + 1)) + ((i >> P) << lc) + sub];
+#pragma unroll
+                for (int a = 0; a < d; ++a) sf_fwd<PM>(x[2 * d * sub + a], x[2 * d * sub + a + d], w, M);
+            }
+        }
+    }
+    // stages of the inverse pass (bounds: sf_inv_off)
+    template <int PH>
+    __device__ __forceinline__ void phase_inv(u64 (&x)[8], const sf_pair *tab, const SfMod &M) const
+    {
+        constexpr int P = Sh::P(PH), HI = Sh::HI(PH), LO = Sh::LO(PH);
+#pragma unroll
+        for (int st = LO; st <= HI; ++st) {
+            const int d = 1 << (st - P), lc = P + 2 - st;
+            const u64 off = sf_inv_off<Sh::LS_>(st, M);
+#pragma unroll
+            for (int sub = 0; sub < (1 << lc); ++sub) {
+                // group g mirrored: 2 m - 1 - g with m = S >> (st + 1)
+                const sf_pair w = tab[(Sh::S >> st) - 1 - ((i >> P) << lc) - sub];
+#pragma unroll
+                for (int a = 0; a < d; ++a) sf_inv<PM>(x[2 * d * sub + a], x[2 * d * sub + a + d], w, M, off);
+            }
+        }
+        if (Sh::LS_ == 8 && PH == 1) x[0] = sf_red3(x[0], M);   // see sf_inv_off
+    }
+    // exchange through buf; the leading barrier orders the previous reads of buf
+    // (an exchange, or points copied ahead into it) before these writes
+    template <int FROM, int TO>
+    __device__ __forceinline__ void exchange(u64 (&x)[8], u64 *buf) const
+    {
+        u64 *from = buf + Sh::pos(FROM, i) * Sh::NB + b;
+        const u64 *to = buf + Sh::pos(TO, i) * Sh::NB + b;
         __syncthreads();
 #pragma unroll
-        for (int t = 0; t < 16; ++t) x[t] = buf[k2(t) * 16 + b];
-    }
-    __device__ __forceinline__ void to1(u64 (&x)[16], u64 *buf) const
-    {
-#pragma unroll
-        for (int t = 0; t < 16; ++t) buf[k2(t) * 16 + b] = x[t];
+        for (int t = 0; t < 8; ++t) from[Sh::step(FROM, t) * Sh::NB] = x[t];
         __syncthreads();
 #pragma unroll
-        for (int r = 0; r < 16; ++r) x[r] = buf[k1(r) * 16 + b];
+        for (int t = 0; t < 8; ++t) x[t] = to[Sh::step(TO, t) * Sh::NB];
+    }
+    __device__ __forceinline__ void forward(u64 (&x)[8], const sf_pair *tab, u64 *buf, const SfMod &M) const
+    {
+        phase_fwd<0>(x, tab, M);
+        exchange<0, 1>(x, buf);
+        phase_fwd<1>(x, tab, M);
+        if constexpr (Sh::NP == 3) {
+            exchange<1, 2>(x, buf);
+            phase_fwd<2>(x, tab, M);
+        }
+    }
+    __device__ __forceinline__ void inverse(u64 (&x)[8], const sf_pair *tab, u64 *buf, const SfMod &M) const
+    {
+        phase_inv<LAST>(x, tab, M);
+        inverse_rest(x, tab, buf, M);
+    }
+    __device__ __forceinline__ void inverse_rest(u64 (&x)[8], const sf_pair *tab, u64 *buf, const SfMod &M) const
+    {
+        if constexpr (Sh::NP == 3) {
+            exchange<2, 1>(x, buf);
+            phase_inv<1>(x, tab, M);
+        }
+        exchange<1, 0>(x, buf);
+        phase_inv<0>(x, tab, M);
     }
 };
 
 // ---- row tiles -------------------------------------------------------------------
-// 8 rows and their mirrors; thread: row b = tid / NI, i = tid % NI (the threads
-// of a row share a warp).  Staged table tw: phase-1 twiddles (k, b) at
-// (k - 1) 16 + b, k < NI; phase-2 twiddles (e, thread) at P2 + e NT + tid.
+// Thread: row b = tid / LP, i = tid % LP.  Register t of phase ph holds element
+// k = (i >> P) 2^(P+3) + t 2^P + (i mod 2^P).  The staged table holds, per
+// phase and stage, [sub][b][high]: the twiddle of group (high, sub) of row b.
 
-template <int LC>
+template <int LC, bool PM>
 struct SfRowT {
-    using Sub = SfSub<LC>;
-    static constexpr int P2 = 16 * (Sub::NI - 1), MIR = 9 * Sub::NI - 1;
+    using Sh = SfShape<LC>;
+    static constexpr int FIRST = 0, LAST = Sh::NP - 1;
     int b, i;
-    __device__ __forceinline__ SfRowT() : b(threadIdx.x / Sub::NI), i(threadIdx.x % Sub::NI) {}
+    __device__ __forceinline__ SfRowT() : b(threadIdx.x / Sh::LP), i(threadIdx.x % Sh::LP) {}
     // row of the polynomial that row b of tile `tile` is (R rows in all)
-    __device__ __forceinline__ int row(int tile, int R) const { return b < 8 ? 8 * tile + b : R - 1 - 8 * tile - (b - 8); }
-    __device__ __forceinline__ int k1(int r) const { return i + (r % Sub::U) * Sub::NI + 16 * (r / Sub::U); }
+    __device__ __forceinline__ int row(int tile, int R) const
+    {
+        return b < Sh::HALF ? Sh::HALF * tile + b : R - 1 - Sh::HALF * tile - (b - Sh::HALF);
+    }
+    template <int PH>
+    __device__ __forceinline__ int k(int t) const
+    {
+        constexpr int P = Sh::P(PH);
+        return ((i >> P) << (P + 3)) + (t << P) + (i & ((1 << P) - 1));
+    }
+    // element of the first phase: t LP + i, consecutive over the threads of a row
+    __device__ __forceinline__ int k1(int t) const { return k<0>(t); }
 
-    __device__ __forceinline__ void fwd1(u64 (&x)[16], const sf_pair *tw, u64 q) const
+    template <int PH>
+    __device__ __forceinline__ void phase_fwd(u64 (&x)[8], const sf_pair *tw, const SfMod &M) const
     {
-        sf_p1_fwd<LC>(x, [&](int k) { return tw[(k - 1) * 16 + b]; }, q);
-    }
-    __device__ __forceinline__ void fwd2(u64 (&x)[16], const sf_pair *tw, u64 q) const
-    {
-        sf_p2_fwd(x, [&](int e) { return tw[P2 + e * Sub::NT + threadIdx.x]; }, q);
-    }
-    __device__ __forceinline__ void inv2(u64 (&x)[16], const sf_pair *tw, u64 q) const
-    {
-        const int tid = threadIdx.x ^ MIR;
-        sf_p2_inv(x, [&](int e) {
-            const int s = e >= 7 ? 3 : e >= 3 ? 2 : e >= 1 ? 1 : 0, g = e - ((1 << s) - 1);
-            return tw[P2 + ((2 << s) - 2 - g) * Sub::NT + tid];
-        }, q);
-    }
-    __device__ __forceinline__ void inv1(u64 (&x)[16], const sf_pair *tw, u64 q) const
-    {
-        sf_p1_inv<LC>(x, [&](int k) {
-            const int m = k >= 8 ? 8 : k >= 4 ? 4 : k >= 2 ? 2 : 1;
-            return tw[(3 * m - 2 - k) * 16 + (b ^ 8)];
-        }, q);
-    }
-    __device__ __forceinline__ void put1(const u64 (&x)[16], u64 *buf) const
-    {
+        constexpr int P = Sh::P(PH), HI = Sh::HI(PH), LO = Sh::LO(PH), H = Sh::H(PH);
+        const sf_pair *tp = tw + Sh::OFF(PH) + b * H + (i >> P);
 #pragma unroll
-        for (int r = 0; r < 16; ++r) buf[b * Sub::PITCH + k1(r) + (k1(r) >> 4)] = x[r];
-    }
-    __device__ __forceinline__ void put2(const u64 (&x)[16], u64 *buf) const
-    {
+        for (int st = HI; st >= LO; --st) {
+            const int d = 1 << (st - P);
 #pragma unroll
-        for (int t = 0; t < 16; ++t) buf[b * Sub::PITCH + 17 * i + t] = x[t];
-    }
-    __device__ __forceinline__ void get1(u64 (&x)[16], const u64 *buf) const
-    {
+            for (int sub = 0; sub < (8 >> (st - P + 1)); ++sub) {
+                const sf_pair w = tp[(Sh::E(PH, st) + sub) * Sh::NB * H];
 #pragma unroll
-        for (int r = 0; r < 16; ++r) x[r] = buf[b * Sub::PITCH + k1(r) + (k1(r) >> 4)];
+                for (int a = 0; a < d; ++a) sf_fwd<PM>(x[2 * d * sub + a], x[2 * d * sub + a + d], w, M);
+            }
+        }
     }
-    __device__ __forceinline__ void get2(u64 (&x)[16], const u64 *buf) const
+    // stages of the inverse pass (bounds: sf_inv_off)
+    template <int PH>
+    __device__ __forceinline__ void phase_inv(u64 (&x)[8], const sf_pair *tw, const SfMod &M) const
     {
+        constexpr int P = Sh::P(PH), HI = Sh::HI(PH), LO = Sh::LO(PH), H = Sh::H(PH);
+        const sf_pair *tp = tw + Sh::OFF(PH) + (b ^ Sh::HALF) * H + (H - 1 - (i >> P));
 #pragma unroll
-        for (int t = 0; t < 16; ++t) x[t] = buf[b * Sub::PITCH + 17 * i + t];
+        for (int st = LO; st <= HI; ++st) {
+            const int d = 1 << (st - P), subs = 8 >> (st - P + 1);
+            const u64 off = sf_inv_off<Sh::LS_>(st, M);
+#pragma unroll
+            for (int sub = 0; sub < subs; ++sub) {
+                const sf_pair w = tp[(Sh::E(PH, st) + subs - 1 - sub) * Sh::NB * H];
+#pragma unroll
+                for (int a = 0; a < d; ++a) sf_inv<PM>(x[2 * d * sub + a], x[2 * d * sub + a + d], w, M, off);
+            }
+        }
+        if (Sh::LS_ == 8 && PH == 1) x[0] = sf_red3(x[0], M);   // see sf_inv_off
     }
-    // exchanges inside the warp: the leading barrier orders the previous
-    // exchange's reads before these writes
-    __device__ __forceinline__ void to2(u64 (&x)[16], u64 *buf) const
+    template <int PH>
+    __device__ __forceinline__ void put(const u64 (&x)[8], u64 *buf) const
+    {
+        u64 *to = buf + b * Sh::PITCH + Sh::pos(PH, i);
+#pragma unroll
+        for (int t = 0; t < 8; ++t) to[Sh::step(PH, t)] = x[t];
+    }
+    template <int PH>
+    __device__ __forceinline__ void get(u64 (&x)[8], const u64 *buf) const
+    {
+        const u64 *from = buf + b * Sh::PITCH + Sh::pos(PH, i);
+#pragma unroll
+        for (int t = 0; t < 8; ++t) x[t] = from[Sh::step(PH, t)];
+    }
+    // exchange inside the warp; the leading barrier orders the reads of the
+    // previous exchange before these writes
+    template <int FROM, int TO>
+    __device__ __forceinline__ void exchange(u64 (&x)[8], u64 *buf) const
     {
         __syncwarp();
-        put1(x, buf);
+        put<FROM>(x, buf);
         __syncwarp();
-        get2(x, buf);
+        get<TO>(x, buf);
     }
-    __device__ __forceinline__ void to1(u64 (&x)[16], u64 *buf) const
+    // forward pass: first-phase elements in, last-phase elements out (storage order)
+    __device__ __forceinline__ void forward(u64 (&x)[8], const sf_pair *tw, u64 *buf, const SfMod &M) const
     {
-        __syncwarp();
-        put2(x, buf);
-        __syncwarp();
-        get1(x, buf);
+        phase_fwd<0>(x, tw, M);
+        forward_rest(x, tw, buf, M);
     }
-    // storage order: element t of this thread in tile `tile`
+    __device__ __forceinline__ void forward_rest(u64 (&x)[8], const sf_pair *tw, u64 *buf, const SfMod &M) const
+    {
+        exchange<0, 1>(x, buf);
+        phase_fwd<1>(x, tw, M);
+        if constexpr (Sh::NP == 3) {
+            exchange<1, 2>(x, buf);
+            phase_fwd<2>(x, tw, M);
+        }
+    }
+    // inverse pass: the other way round
+    __device__ __forceinline__ void inverse(u64 (&x)[8], const sf_pair *tw, u64 *buf, const SfMod &M) const
+    {
+        if constexpr (Sh::NP == 3) {
+            phase_inv<2>(x, tw, M);
+            exchange<2, 1>(x, buf);
+        }
+        phase_inv<1>(x, tw, M);
+        exchange<1, 0>(x, buf);
+        phase_inv<0>(x, tw, M);
+    }
+    // storage order: last-phase element t of this thread in tile `tile`
     __device__ __forceinline__ static size_t store_at(int tile, int t)
     {
-        return (size_t)tile * 16 * Sub::S + (size_t)t * Sub::NT + threadIdx.x;
+        return (size_t)tile * Sh::TILE + (size_t)t * Sh::NT + threadIdx.x;
     }
 };
 
@@ -297,31 +373,31 @@ struct SfRowT {
 template <int LR>
 __device__ __forceinline__ void sf_stage_cols(sf_pair *dst, const sf_pair *__restrict__ table, int m0, int n)
 {
-    for (int k = threadIdx.x; k < (n << LR); k += SfSub<LR>::NT) dst[k] = table[((size_t)m0 << LR) + k];
+    for (int k = threadIdx.x; k < (n << LR); k += SfShape<LR>::NT) dst[k] = table[((size_t)m0 << LR) + k];
 }
 template <int LR, int LC>
 __device__ __forceinline__ void sf_stage_row(sf_pair *dst, const sf_pair *__restrict__ table, int mod, int tile)
 {
-    constexpr int W = SfSub<LC>::ROW_PAIRS;
-    const sf_pair *src = table + ((size_t)mod * ((1 << LR) / 16) + tile) * W;
-    for (int k = threadIdx.x; k < W; k += SfSub<LC>::NT) dst[k] = src[k];
+    constexpr int W = SfShape<LC>::PAIRS;
+    const sf_pair *src = table + ((size_t)mod * ((1 << LR) / SfShape<LC>::NB) + tile) * W;
+    for (int k = threadIdx.x; k < W; k += SfShape<LC>::NT) dst[k] = src[k];
 }
 
 // storage index of NTT slot j (natural bit-reversed order) and back
-__host__ __device__ __forceinline__ int sf_storage_index(int j, int log_r, int log_c)
+SF_HD int sf_storage_index(int j, int log_r, int log_c)
 {
-    const int R = 1 << log_r, ni = 1 << (log_c - 4);
+    const int R = 1 << log_r, hl = log_c == 8 ? 2 : 3, lp = log_c - 3;
     const int row = j >> log_c, col = j & ((1 << log_c) - 1);
-    const bool mir = row >= R / 2;
-    const int rr = mir ? R - 1 - row : row;
-    return (((rr >> 3) << 4) << log_c) + ((col & 15) << log_c) + ((rr & 7) + (mir ? 8 : 0)) * ni + (col >> 4);
+    const int mir = row >= R / 2, rr = mir ? R - 1 - row : row;
+    const int b = (rr & ((1 << hl) - 1)) + (mir << hl);
+    return ((rr >> hl) << (hl + 1 + log_c)) + ((col & 7) << (hl + 1 + lp)) + (b << lp) + (col >> 3);
 }
-__host__ __device__ __forceinline__ int sf_natural_index(int p, int log_r, int log_c)
+SF_HD int sf_natural_index(int p, int log_r, int log_c)
 {
-    const int R = 1 << log_r, ni_l = log_c - 4;
-    const int tile = p >> (log_c + 4), t = (p >> log_c) & 15, b = (p >> ni_l) & 15, i = p & ((1 << ni_l) - 1);
-    const int row = b < 8 ? 8 * tile + b : R - 1 - 8 * tile - (b - 8);
-    return (row << log_c) + 16 * i + t;
+    const int R = 1 << log_r, hl = log_c == 8 ? 2 : 3, lp = log_c - 3;
+    const int tile = p >> (hl + 1 + log_c), t = (p >> (hl + 1 + lp)) & 7, b = (p >> lp) & ((2 << hl) - 1), i = p & ((1 << lp) - 1);
+    const int rr = (tile << hl) + (b & ((1 << hl) - 1));
+    return (((b >> hl) ? R - 1 - rr : rr) << log_c) + 8 * i + t;
 }
 
 // ---- balanced persistent partition ----------------------------------------
@@ -339,8 +415,42 @@ __device__ __forceinline__ SfUnitRange sf_unit_range(int n_units)
             (int)(((long long)blockIdx.x + 1) * n_units / gridDim.x)};
 }
 
+// Walks a block's units (group, item) without a division per unit.
+struct SfCursor {
+    int grp, item, n_items;
+    __device__ __forceinline__ SfCursor(int u, int n) : grp(u / n), item(u % n), n_items(n) {}
+    __device__ __forceinline__ void next()
+    {
+        if (++item == n_items) {
+            item = 0;
+            ++grp;
+        }
+    }
+};
+
+// runs the statements with constexpr LR, LC, PM for the ring R
+#define SF_RING_DISPATCH(R, ...)                              \
+    do {                                                      \
+        if ((R).pm) {                                         \
+            constexpr bool PM = true;                         \
+            SF_SIZE_DISPATCH((R).log_n, __VA_ARGS__);         \
+        } else {                                              \
+            constexpr bool PM = false;                        \
+            SF_SIZE_DISPATCH((R).log_n, __VA_ARGS__);         \
+        }                                                     \
+    } while (0)
+
+// the same for every ring size and either product (kernel attributes)
+#define SF_FOR_RINGS(...)                                                          \
+    do {                                                                           \
+        for (int ln_ = 10; ln_ <= 16; ++ln_) {                                     \
+            { constexpr bool PM = true; SF_SIZE_DISPATCH(ln_, __VA_ARGS__); }      \
+            { constexpr bool PM = false; SF_SIZE_DISPATCH(ln_, __VA_ARGS__); }     \
+        }                                                                          \
+    } while (0)
+
 // runs the statements with constexpr LR, LC for the ring size log_n (10..16)
-#define SF_RING_DISPATCH(log_n, ...)                                  \
+#define SF_SIZE_DISPATCH(log_n, ...)                                  \
     do {                                                              \
         switch (log_n) {                                              \
         case 10: { constexpr int LR = 5, LC = 5; __VA_ARGS__ } break; \

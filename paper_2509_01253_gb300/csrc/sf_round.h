@@ -6,7 +6,6 @@
 #include <vector>
 
 #include "sf_internal.h"
-#include "sf_tile.cuh"
 #include "sf_layer.h"
 
 #define SF_CHECK_CTX(ctx)                                                        \
@@ -66,11 +65,11 @@ static inline SfLeafParams leaf_params(const sf_layer *L)
     return P;
 }
 
-// Input ciphertexts -> NTT domain (canonical), followed by their Shoup
-// companions (for the leaf products).  With the client's powers (gamma = 2,
-// d_pow non-null) the k_in powers follow the k_in inputs, so the leaves see
-// 2 k_in ciphertexts; ct holds twice the words of the ciphertexts it takes.
-static inline sf_status prepare_inputs(sf_ctx *ctx, const u64 *d_in, const u64 *d_pow, int k_in, u64 *ct,
+// Input ciphertexts -> pairs of their NTT, in storage order (for the leaf
+// products).  With the client's powers (gamma = 2, d_pow non-null) the k_in
+// powers follow the k_in inputs, so the leaves see 2 k_in ciphertexts; ct holds
+// twice the words of the ciphertexts it takes, tmp as many as them.
+static inline sf_status prepare_inputs(sf_ctx *ctx, const u64 *d_in, const u64 *d_pow, int k_in, u64 *ct, u64 *tmp,
                                        cudaStream_t st)
 {
     const SfRing &R = ctx->ring;
@@ -81,11 +80,10 @@ static inline sf_status prepare_inputs(sf_ctx *ctx, const u64 *d_in, const u64 *
     std::vector<SfPolyJob> jobs;
     for (int x = 0; x < k_all * 2 * R.L; ++x) {
         const u64 *src = x < k_in * 2 * R.L ? d_in + (size_t)x * R.n : d_pow + (size_t)x * R.n - words;
-        jobs.push_back({src, ct + (size_t)x * R.n, x % R.L});
+        jobs.push_back({src, tmp + (size_t)x * R.n, x % R.L});
     }
     SF_TRY(sf_ntt_jobs(ctx, jobs.data(), (int)jobs.size(), false, st));
-    SF_TRY(sf_companions(ctx, ct, ct + (size_t)k_all * 2 * R.L * R.n, k_all * 2 * R.L, R.L, 0, st));
-    return SF_OK;
+    return sf_to_pairs(ctx, tmp, (ulonglong2 *)ct, k_all * 2 * R.L, R.L, 0, st);
 }
 
 static inline sf_status upload_perm_inverse(const uint32_t *perm, int n, int *d_dst, std::vector<int> &host, cudaStream_t st)
@@ -109,7 +107,7 @@ static inline int leaf_batch_slots(const SfRing &R, int k_in, int max_taps)
 // points the tap buckets of P at words (sized by sf_leaf_tap_words)
 static inline void sf_leaf_tap_bind(const SfRing &R, SfLeafParams &P, u64 *words, int slots)
 {
-    P.n_buckets = P.k_in * (R.c / SF_NB);
+    P.n_buckets = P.k_in * sf_leaf_tiles(R);
     P.tap_buf = (longlong2 *)words;
     P.tap_off = (int *)(words + (size_t)slots * P.max_taps * 2);
 }
