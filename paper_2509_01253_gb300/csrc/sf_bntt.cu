@@ -4,19 +4,22 @@
 // The batch is [count][L][N]: limb i of polynomial p is reduced modulo q_i.
 // A transform is the two register-resident passes of sf_reg.cuh (forward:
 // column pass, then row pass; inverse: row pass, then column pass with the
-// factor N^-1).  Each pass is one persistent launch of one resident wave over
-// the units (group, polynomial), a group being a column or row tile position
+// factor N^-1).  Each pass is one launch over the units (group,
+// polynomial), several waves of blocks with even shares (ks_wave_blocks), a group being a column or row tile position
 // and a limb: a block takes an equal range of units (sf_unit_range), stages a
-// group's twiddles when its range enters the group, and loads the next unit's
-// points into registers before it transforms the current one.
+// group's twiddles when its range enters the group, and copies the next unit's
+// points ahead with cp.async while it transforms the current one (loads into
+// registers sank behind the transform: the column pass waited on memory).
 //
 // Bound by the integer multiplier: at N = 2^16 the fmaheavy pipe is busy 70 to
 // 76 % of the cycles.  512 x 5 limbs of 2^16, forward: 1961 us with tile sweeps in
-// shared memory, 1630 us here; 37 x 3 inverse limbs of 2^14: 32.8 and 28.2 us.
+// shared memory, 1550 us here; 37 x 3 inverse limbs of 2^14: 32.8 and 28.5 us.
 #include <algorithm>
 
+#include "sf_async.cuh"
 #include "sf_internal.h"
 #include "sf_kernels.cuh"
+#include "sf_ks.h"
 #include "sf_reg.cuh"
 #include "sf_round.h"
 
@@ -28,21 +31,23 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS)
     using T_ = SfRowT<LC, PM>;
     const T_ T;
     sf_pair *tw = (sf_pair *)smem_raw;
-    u64 *buf = (u64 *)(tw + SfShape<LC>::PAIRS);
+    constexpr int NT = SfShape<LC>::NT;
+    u64 *buf = (u64 *)(tw + SfShape<LC>::PAIRS), *pre = buf + SfShape<LC>::WORDS + threadIdx.x;
     const SfUnitRange U = sf_unit_range(ng * count);
     const size_t per = (size_t)R.L << (LR + LC);
     // group = (row tile, limb i), item = polynomial; offset of this thread's row
     auto group_off = [&](int grp) -> size_t {
         return ((size_t)(grp % R.L) << (LR + LC)) + ((size_t)T.row(grp / R.L, 1 << LR) << LC) + T.k1(0);
     };
-    u64 x[8], nx[8];
     SfCursor C(U.u0, count);
     size_t off = group_off(C.grp) + per * C.item;
-    auto load = [&]() {
+    // each thread copies its own points of the next unit ahead
+    auto prefetch = [&]() {
 #pragma unroll
-        for (int t = 0; t < 8; ++t) nx[t] = src[off + (T.k1(t) - T.k1(0))];
+        for (int t = 0; t < 8; ++t) sf_cp8(pre + t * NT, src + off + (T.k1(t) - T.k1(0)));
+        sf_cp_commit();
     };
-    if (U.u0 < U.u1) load();
+    if (U.u0 < U.u1) prefetch();
     int staged = -1, mod = 0;
     for (int u = U.u0; u < U.u1; ++u) {
         if (C.grp != staged) {
@@ -53,21 +58,26 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS)
             __syncthreads();
         }
         const SfMod &M = R.m[mod];
+        u64 x[8];
+        sf_cp_wait<0>();
 #pragma unroll
-        for (int t = 0; t < 8; ++t) x[t] = nx[t];
+        for (int t = 0; t < 8; ++t) x[t] = pre[t * NT];
         u64 *d = dst + off;
-        // the loads of the next unit overtake this unit's stores: in place, the
-        // two units touch different rows or polynomials
+        // the next unit's copy overtakes this unit's stores: in place, the two units
+        // touch different rows or polynomials
         C.next();
         off = C.grp == staged ? off + per : group_off(C.grp);
-        if (u + 1 < U.u1) load();
         if (INV) {
             T.template exchange<T_::FIRST, T_::LAST>(x, buf);
+            if (u + 1 < U.u1) prefetch();
             T.inverse(x, tw, buf, M);
+            sf_inv_rows_out(x, M);
 #pragma unroll
-            for (int t = 0; t < 8; ++t) d[T.k1(t) - T.k1(0)] = sf_red3(x[t], M);
+            for (int t = 0; t < 8; ++t) d[T.k1(t) - T.k1(0)] = x[t];
         } else {
-            T.forward(x, tw, buf, M);
+            T.template phase_fwd<0>(x, tw, M);
+            if (u + 1 < U.u1) prefetch();
+            T.forward_rest(x, tw, buf, M);
             T.template exchange<T_::LAST, T_::FIRST>(x, buf);   // back to coalesced positions
 #pragma unroll
             for (int t = 0; t < 8; ++t) d[T.k1(t) - T.k1(0)] = sf_canon(x[t], M);
@@ -82,21 +92,23 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SfColT<LR, PM> T;
     sf_pair *tab = (sf_pair *)smem_raw;
-    u64 *buf = (u64 *)(tab + SfShape<LR>::S);
+    constexpr int NT = SfShape<LR>::NT;
+    u64 *buf = (u64 *)(tab + SfShape<LR>::S), *pre = buf + SfShape<LR>::WORDS + threadIdx.x;
     const SfUnitRange U = sf_unit_range(ng * count);
     const size_t per = (size_t)R.L << (LR + LC);
     // group = (column tile, limb i), item = polynomial; offset of this thread's column
     auto group_off = [&](int grp) -> size_t {
         return ((size_t)(grp % R.L) << (LR + LC)) + (grp / R.L) * SfShape<LR>::NB + T.b;
     };
-    u64 x[8], nx[8];
     SfCursor C(U.u0, count);
     size_t off = group_off(C.grp) + per * C.item;
-    auto load = [&]() {
+    // each thread copies its own points of the next unit ahead
+    auto prefetch = [&]() {
 #pragma unroll
-        for (int t = 0; t < 8; ++t) nx[t] = src[off + ((size_t)(INV ? T.kl(t) : T.k1(t)) << LC)];
+        for (int t = 0; t < 8; ++t) sf_cp8(pre + t * NT, src + off + ((size_t)(INV ? T.kl(t) : T.k1(t)) << LC));
+        sf_cp_commit();
     };
-    if (U.u0 < U.u1) load();
+    if (U.u0 < U.u1) prefetch();
     int staged = -1, mod = 0;
     for (int u = U.u0; u < U.u1; ++u) {
         if (C.grp != staged) {
@@ -107,34 +119,33 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS)
             __syncthreads();
         }
         const SfMod &M = R.m[mod];
+        u64 x[8];
+        sf_cp_wait<0>();
 #pragma unroll
-        for (int t = 0; t < 8; ++t) x[t] = nx[t];
+        for (int t = 0; t < 8; ++t) x[t] = pre[t * NT];
         u64 *d = dst + off;
         C.next();
         off = C.grp == staged ? off + per : group_off(C.grp);
-        if (u + 1 < U.u1) load();
         if (INV) {
-            T.inverse(x, tab, buf, M);
+            T.template phase_inv<SfColT<LR, PM>::LAST>(x, tab, M);
+            if (u + 1 < U.u1) prefetch();   // this unit's points are in registers
+            T.inverse_rest(x, tab, buf, M);
 #pragma unroll
             for (int t = 0; t < 8; ++t) d[(size_t)T.k1(t) << LC] = sf_canon(sf_mad<PM>(0, x[t], make_ulonglong2(M.ninv, M.ninv_c), M), M);
         } else {
-            T.forward(x, tab, buf, M);
+            T.template phase_fwd<0>(x, tab, M);
+            if (u + 1 < U.u1) prefetch();
+            T.forward_rest(x, tab, buf, M);
 #pragma unroll
             for (int t = 0; t < 8; ++t) d[(size_t)T.kl(t) << LC] = x[t];
         }
     }
 }
 
-// one resident wave (SMs x occupancy blocks), at most one block per unit
-static int bntt_blocks(const sf_ctx *ctx, int occ, int n_units)
-{
-    return std::max(1, std::min(ctx->num_sms * occ, n_units));
-}
-
 template <int LC>
-static constexpr size_t bntt_smem_row() { return sizeof(sf_pair) * SfShape<LC>::PAIRS + sizeof(u64) * SfShape<LC>::WORDS; }
+static constexpr size_t bntt_smem_row() { return sizeof(sf_pair) * SfShape<LC>::PAIRS + sizeof(u64) * (SfShape<LC>::WORDS + SfShape<LC>::TILE); }
 template <int LR>
-static constexpr size_t bntt_smem_col() { return sizeof(sf_pair) * SfShape<LR>::S + sizeof(u64) * SfShape<LR>::WORDS; }
+static constexpr size_t bntt_smem_col() { return sizeof(sf_pair) * SfShape<LR>::S + sizeof(u64) * (SfShape<LR>::WORDS + SfShape<LR>::TILE); }
 
 template <bool INV, int LR, int LC, bool PM>
 static void bntt_row(sf_ctx *ctx, const u64 *src, u64 *dst, int count, cudaStream_t st)
@@ -142,7 +153,7 @@ static void bntt_row(sf_ctx *ctx, const u64 *src, u64 *dst, int count, cudaStrea
     const int ng = ((1 << LR) / SfShape<LC>::NB) * ctx->ring.L;
     const size_t sm = bntt_smem_row<LC>();
     cudaEvent_t ev;
-    const int nb = bntt_blocks(ctx, sf_occupancy(k_bntt_row<INV, LR, LC, PM>, SfShape<LC>::NT, sm), ng * count);
+    const int nb = ks_wave_blocks(ctx, sf_occupancy(k_bntt_row<INV, LR, LC, PM>, SfShape<LC>::NT, sm), ng * count, 8);
     sf_launch_begin(ctx, SFK_BNTT_ROW, st, &ev);
     k_bntt_row<INV, LR, LC, PM><<<nb, SfShape<LC>::NT, sm, st>>>(ctx->ring, src, dst, count, ng);
     sf_launch_end(ctx, SFK_BNTT_ROW, st, ev);
@@ -154,7 +165,7 @@ static void bntt_col(sf_ctx *ctx, const u64 *src, u64 *dst, int count, cudaStrea
     const int ng = ((1 << LC) / SfShape<LR>::NB) * ctx->ring.L;
     const size_t sm = bntt_smem_col<LR>();
     cudaEvent_t ev;
-    const int nb = bntt_blocks(ctx, sf_occupancy(k_bntt_col<INV, LR, LC, PM>, SfShape<LR>::NT, sm), ng * count);
+    const int nb = ks_wave_blocks(ctx, sf_occupancy(k_bntt_col<INV, LR, LC, PM>, SfShape<LR>::NT, sm), ng * count, 8);
     sf_launch_begin(ctx, SFK_BNTT_COL, st, &ev);
     k_bntt_col<INV, LR, LC, PM><<<nb, SfShape<LR>::NT, sm, st>>>(ctx->ring, src, dst, count, ng);
     sf_launch_end(ctx, SFK_BNTT_COL, st, ev);

@@ -219,7 +219,8 @@ static sf_status eval_jobs(sf_ctx *ctx, std::vector<Job> &jobs, cudaStream_t st)
                     const Unit &un = c.units[u0 + u];
                     const Job &j = jobs[un.job];
                     valid[u] = un.va;
-                    if (un.va > 0) SF_TRY(leaves(j, un.g * j.n + un.a, c.nch, c.CH, A + (size_t)u * c.CH * ct));
+                    // padding leaves are never read (sf_pack_tree's valid counts)
+                    if (un.va > 0) SF_TRY(leaves(j, un.g * j.n + un.a, c.nch, un.va, A + (size_t)u * c.CH * ct));
                 }
                 u64 *res = nullptr;
                 size_t rs = 0;

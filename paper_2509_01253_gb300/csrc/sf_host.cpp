@@ -458,9 +458,9 @@ static sf_status upload(sf_ctx *ctx, const std::vector<T> &h, const T **out)
 }
 
 // Bound of the product by pairs (w, 2^32 w mod q) as a multiple of q (sf_mad:
-// below 2^53 + 2^33 delta, q = 2^50 - delta), or 0 where q does not admit it: 20
-// times the bound, which a forward transform reaches, and 64 times, which the
-// inverse passes reach, stay below 2^63 and 2^64.
+// below 2^53 + 2^33 delta, q = 2^50 - delta), or 0 where q does not admit it: 24
+// times the bound, which a forward transform reaches, and 32 times, which the
+// inverse passes reach, stay within 2^63.
 static u64 pm_bound(u64 q)
 {
     const u64 top = (u64)1 << 50;

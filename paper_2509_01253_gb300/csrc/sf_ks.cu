@@ -33,7 +33,8 @@ size_t sf_ks_scratch_words(const SfRing &R, int ntt) { return sf_ks_scratch_word
 //   out.a[p] = v.a[p]                      (0 for a plain rotation)
 //   out.b[p] = v.b[p] + tau_d(u.b)[p],     v = E + X^s O
 // Coefficient-domain operands: tau_d and X^s are signed index maps.  NTT-domain
-// operands (storage order): a slot permutation and monomial products.
+// operands (storage order): a slot permutation and monomial products, and out
+// times N^-1.
 // grid (N / (256 SF_EW), L, merges): each thread does SF_EW points, so the
 // per-merge pointers are set up once per thread.  Bound by HBM (0.89 of the
 // copy bandwidth at N = 2^16): 3.0 us per merge there.  Done inside k_ks2 and
@@ -97,13 +98,15 @@ __global__ void __launch_bounds__(256) k_ks_gather(SfRing R, SfKsBatch B)
             const u64 xas = sf_mul_shoup(Oas, ws, wsp, q), xbs = sf_mul_shoup(Obs, ws, wsp, q);
             ta[p] = sf_sub(Eas, xas, q);
             const u64 ub = sf_sub(Ebs, xbs, q);
-            oa[p] = sf_add(Eaj, xaj, q);
-            ob[p] = sf_add(sf_add(Ebj, xbj, q), ub, q);
+            Eaj = sf_add(Eaj, xaj, q);
+            Ebj = sf_add(sf_add(Ebj, xbj, q), ub, q);
         } else {
             ta[p] = Eas;
-            oa[p] = Eaj;
-            ob[p] = sf_add(Ebj, Ebs, q);
+            Ebj = sf_add(Ebj, Ebs, q);
         }
+        // joins accumulators that carry N^-1
+        oa[p] = sf_mul_shoup(Eaj, M.ninv, M.ninv_p, q);
+        ob[p] = sf_mul_shoup(Ebj, M.ninv, M.ninv_p, q);
     }
 }
 

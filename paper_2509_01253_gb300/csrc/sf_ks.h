@@ -1,5 +1,7 @@
 // sf_ks.h -- batched automorphism + key switching (see sf_ks.cu).
 #pragma once
+#include <algorithm>
+
 #include "sf_internal.h"
 
 // `count` merges sharing d, s, add_v and the key.  Merge number
@@ -101,10 +103,16 @@ __device__ __forceinline__ u64 merge_coef(const u64 *e, const u64 *o, int p, uns
 }
 #endif
 
-// blocks of a persistent launch over n_units (group, item) units: one
-// resident wave (num_sms x occupancy blocks), at most one block per unit
-static inline int ks_wave_blocks(const sf_ctx *ctx, int occ, int n_units)
+// Blocks of a launch over n_units (group, item) units, split evenly
+// (sf_unit_range): as many waves of num_sms x occupancy blocks as leave a block
+// `per_block` units for the tables it stages.  One wave of equal shares lost: the
+// warps of an SM's blocks are not served evenly, so that one block ends early and
+// leaves the others fewer warps to hide latency with (512 x 5 limbs of 2^16: 1779
+// us with one wave, 1550 us with 8 units a block; the key-switch rows 418 and 392
+// ms per 32768 at N = 2^16).
+static inline int ks_wave_blocks(const sf_ctx *ctx, int occ, int n_units, int per_block)
 {
     const int w = ctx->num_sms * occ;
-    return n_units < 1 ? 1 : (w < n_units ? w : n_units);
+    const int waves = std::max(1, std::min(32, n_units / (w * per_block)));
+    return std::max(1, std::min(w * waves, n_units));
 }

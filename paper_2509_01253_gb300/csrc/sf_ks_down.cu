@@ -5,7 +5,7 @@
 // accumulators, scales them to y_k = [x_k Phat_k^-1]_{p_k} (canonical) and keeps
 // them in registers; for each data limb it runs the inverse column pass,
 // subtracts the base conversion (constants Phat_k P^-1 mod q_i; the
-// accumulators carry P^-1 already) and adds what k_ks_gather left in `out` (for
+// accumulators carry P^-1 N^-1 already) and adds what k_ks_gather left in `out` (for
 // NTT-domain operands the accumulators hold it).  The result is canonical, in the
 // coefficient domain, with no forward transform after ModDown.
 //
@@ -88,15 +88,23 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_ks4(SfRin
                     }
                 continue;
             }
-            // x N^-1 + out - conv, products below off: the sum stays below (2 + KT) off
+            // x + out - conv, x below 4 off once x[0] is reduced, a pair of products
+            // below 4 off: the sum stays below (5 + 2 KT) off < 2^62
+            x[0] = sf_red3(x[0], M);
 #pragma unroll
-            for (int r = 0; r < 8; ++r) x[r] = sf_mad<PM>(o[r] + KT * M.off, x[r], make_ulonglong2(M.ninv, M.ninv_c), M);
+            for (int r = 0; r < 8; ++r) x[r] += o[r] + 2 * KT * M.off;
 #pragma unroll
-            for (int k = 0; k < KT; ++k) {
+            for (int k = 0; k < KT; k += 2) {
                 if (k >= R.K) break;
                 const sf_pair w = make_ulonglong2(R.md_phat[(size_t)k * R.L + m], R.md_phat_c[(size_t)k * R.L + m]);
+                if (k + 1 < KT && k + 1 < R.K) {
+                    const sf_pair z = make_ulonglong2(R.md_phat[(size_t)(k + 1) * R.L + m], R.md_phat_c[(size_t)(k + 1) * R.L + m]);
 #pragma unroll
-                for (int r = 0; r < 8; ++r) x[r] -= sf_mad<PM>(0, y[k][r], w, M);
+                    for (int r = 0; r < 8; ++r) x[r] -= sf_mad2<PM>(0, y[k][r], w, y[k + 1 < KT ? k + 1 : 0][r], z, M);
+                } else {
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) x[r] -= sf_mad<PM>(0, y[k][r], w, M);
+                }
             }
 #pragma unroll
             for (int r = 0; r < 8; ++r) out[(size_t)T.k1(r) << LC] = sf_canon(x[r], M);
@@ -120,7 +128,7 @@ static void down_launch(sf_ctx *ctx, const SfKsBatch &b, cudaStream_t st)
     const int g0 = ((1 << LC) / SfShape<LR>::NB) * 2;
     const int nsplit = (int)std::max<long long>(1, std::min<long long>(R.L, (long long)ctx->num_sms * occ / ((long long)g0 * b.count)));
     const int ng = g0 * nsplit;
-    k_ks4<LR, LC, KT, PM><<<ks_wave_blocks(ctx, occ, ng * b.count), SfShape<LR>::NT, sm, st>>>(R, b, ng, nsplit);
+    k_ks4<LR, LC, KT, PM><<<ks_wave_blocks(ctx, occ, ng * b.count, 2), SfShape<LR>::NT, sm, st>>>(R, b, ng, nsplit);
 }
 
 sf_status sf_ks_down_launch(sf_ctx *ctx, const SfKsBatch &b, cudaStream_t st)

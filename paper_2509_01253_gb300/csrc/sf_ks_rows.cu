@@ -6,7 +6,7 @@
 // NTT-domain operands) and the product with the key, whose pairs are
 // stored in the order the registers hold the values; then the inverse row pass
 // of both accumulators, the rows that the ModDown columns read.  The key's data
-// limbs carry P^-1, so those accumulators are ACC P^-1; for NTT-domain operands
+// limbs carry P^-1 N^-1, so those become ACC P^-1; for NTT-domain operands
 // v (+ tau_d(u.b) on the b part), which k_ks_gather left in `out`, is added
 // here, so that it rides through the inverse transform.
 //
@@ -27,21 +27,22 @@
 template <int LR, int LC, bool PM>
 __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS) k_ks1(SfRing R, SfKsBatch B, int ng)
 {
+    constexpr int NT = SfShape<LC>::NT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SfRowT<LC, PM> T;
     sf_pair *tw = (sf_pair *)smem_raw;
-    u64 *buf = (u64 *)(tw + SfShape<LC>::PAIRS);
+    u64 *buf = (u64 *)(tw + SfShape<LC>::PAIRS), *pre = buf + SfShape<LC>::WORDS + threadIdx.x;
     const SfUnitRange U = sf_unit_range(ng * B.count);
     const size_t per = sf_ks_scratch_words_dev(R, B.ntt);
-    u64 x[8], nx[8];
     SfCursor C(U.u0, B.count);
-    // group = (row tile, limb i), item = merge
-    auto load = [&]() {
-        const u64 *src = B.scratch + per * C.item + ((size_t)(sf_ks_ta(R) + C.grp % R.L) << (LR + LC));
+    // group = (row tile, limb i), item = merge; each thread copies its own points ahead
+    auto prefetch = [&]() {
+        const u64 *src = B.scratch + per * C.item + ((size_t)(sf_ks_ta(R) + C.grp % R.L) << (LR + LC)) + T.store_at(C.grp / R.L, 0);
 #pragma unroll
-        for (int t = 0; t < 8; ++t) nx[t] = src[T.store_at(C.grp / R.L, t)];
+        for (int t = 0; t < 8; ++t) sf_cp8(pre + t * NT, src + t * NT);
+        sf_cp_commit();
     };
-    if (U.u0 < U.u1) load();
+    if (U.u0 < U.u1) prefetch();
     int staged = -1, i = 0;
     size_t off = 0;
     for (int u = U.u0; u < U.u1; ++u) {
@@ -55,13 +56,17 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS) k_ks1(SfRin
         }
         const SfMod &M = R.m[i];
         u64 *dst = B.scratch + per * C.item + off;
+        u64 x[8];
+        sf_cp_wait<0>();
 #pragma unroll
-        for (int t = 0; t < 8; ++t) x[t] = nx[t];
+        for (int t = 0; t < 8; ++t) x[t] = pre[t * NT];
+        T.template phase_inv<SfRowT<LC, PM>::LAST>(x, tw, M);
         C.next();
-        if (u + 1 < U.u1) load();
-        T.inverse(x, tw, buf, M);
+        if (u + 1 < U.u1) prefetch();   // this unit's points are in registers
+        T.inverse_rest(x, tw, buf, M);
+        sf_inv_rows_out(x, M);
 #pragma unroll
-        for (int t = 0; t < 8; ++t) dst[T.k1(t)] = sf_red3(x[t], M);
+        for (int t = 0; t < 8; ++t) dst[T.k1(t)] = x[t];
     }
 }
 
@@ -116,9 +121,10 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS_ACC) k_ks3(S
         const SfMod &M = R.m[G.m];
         C.next();
         if (C.grp != staged) N = group(C.grp);
-        u64 acc_a[8], acc_b[8], x[8];
+        SfAcc<PM> acc_a[8], acc_b[8];
+        u64 x[8];
 #pragma unroll
-        for (int t = 0; t < 8; ++t) acc_a[t] = acc_b[t] = 0;
+        for (int t = 0; t < 8; ++t) acc_a[t] = acc_b[t] = {0, 0};
         const sf_pair *ka = key + ((size_t)G.m << (LR + LC)) + T.store_at(G.tile, 0);
 #pragma unroll 1
         for (int j = 0; j < R.dnum; ++j) {
@@ -137,13 +143,16 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS_ACC) k_ks3(S
                 ahead();
                 T.forward_rest(x, tw, buf, M);
             }
-            // x lazy, key < q with its companion: each product below off, 8 of them below 2^61
             const sf_pair *kb = ka + ((size_t)R.nm << (LR + LC));
 #pragma unroll
             for (int t = 0; t < 8; ++t) {
                 const sf_pair a = __ldg(ka + t * NT), c = __ldg(kb + t * NT);
-                acc_a[t] = sf_mad<PM>(acc_a[t], x[t], a, M);
-                acc_b[t] = sf_mad<PM>(acc_b[t], x[t], c, M);
+                sf_acc_add<PM>(acc_a[t], x[t], a, M);
+                sf_acc_add<PM>(acc_b[t], x[t], c, M);
+            }
+            if (j % SF_ACC_TERMS == SF_ACC_TERMS - 1 && j + 1 < R.dnum) {
+#pragma unroll
+                for (int t = 0; t < 8; ++t) sf_acc_close<PM>(acc_a[t], M), sf_acc_close<PM>(acc_b[t], M);
             }
             ka = kb + ((size_t)R.nm << (LR + LC));
         }
@@ -153,17 +162,21 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS_ACC) k_ks3(S
         // instruction cache
 #pragma unroll 1
         for (int part = 0; part < 2; ++part) {
-            // 3q after the partial reduction, 4q with v
+            // below 3q, 4q with v
 #pragma unroll
-            for (int t = 0; t < 8; ++t) x[t] = sf_red3(part ? acc_b[t] : acc_a[t], M);
+            for (int t = 0; t < 8; ++t) {
+                SfAcc<PM> a = part ? acc_b[t] : acc_a[t];
+                x[t] = sf_acc_close<PM>(a, M);
+            }
             if (add) {
 #pragma unroll
                 for (int t = 0; t < 8; ++t) x[t] += add[t * NT];
                 add += (size_t)R.L << (LR + LC);
             }
             T.inverse(x, tw, buf, M);
+            sf_inv_rows_out(x, M);
 #pragma unroll
-            for (int t = 0; t < 8; ++t) dst[T.k1(t)] = sf_red3(x[t], M);
+            for (int t = 0; t < 8; ++t) dst[T.k1(t)] = x[t];
             dst += (size_t)R.nm << (LR + LC);
         }
         G = N;
@@ -171,9 +184,9 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS_ACC) k_ks3(S
 }
 
 template <int LC>
-static constexpr size_t rows_smem(bool pre)
+static constexpr size_t rows_smem()
 {
-    return sizeof(sf_pair) * SfShape<LC>::PAIRS + sizeof(u64) * (SfShape<LC>::WORDS + (pre ? SfShape<LC>::TILE : 0));
+    return sizeof(sf_pair) * SfShape<LC>::PAIRS + sizeof(u64) * (SfShape<LC>::WORDS + SfShape<LC>::TILE);
 }
 
 sf_status sf_ks_rows_launch(sf_ctx *ctx, const SfKsBatch &b, cudaStream_t st)
@@ -182,10 +195,10 @@ sf_status sf_ks_rows_launch(sf_ctx *ctx, const SfKsBatch &b, cudaStream_t st)
     cudaEvent_t ev;
     SF_RING_DISPATCH(R, {
         constexpr int NT = SfShape<LC>::NT;
-        constexpr size_t sm = rows_smem<LC>(true);
+        constexpr size_t sm = rows_smem<LC>();
         const int ng = ((1 << LR) / SfShape<LC>::NB) * R.nm;
         sf_launch_begin(ctx, SFK_KS3_INNER_ROW, st, &ev);
-        k_ks3<LR, LC, PM><<<ks_wave_blocks(ctx, sf_occupancy(k_ks3<LR, LC, PM>, NT, sm), ng * b.count), NT, sm, st>>>(R, b, ng);
+        k_ks3<LR, LC, PM><<<ks_wave_blocks(ctx, sf_occupancy(k_ks3<LR, LC, PM>, NT, sm), ng * b.count, 8), NT, sm, st>>>(R, b, ng);
         sf_launch_end(ctx, SFK_KS3_INNER_ROW, st, ev);
     });
     SF_CUDA_TRY(cudaGetLastError());
@@ -198,10 +211,10 @@ sf_status sf_ks_inv_rows_launch(sf_ctx *ctx, const SfKsBatch &b, cudaStream_t st
     cudaEvent_t ev;
     SF_RING_DISPATCH(R, {
         constexpr int NT = SfShape<LC>::NT;
-        constexpr size_t sm = rows_smem<LC>(false);
+        constexpr size_t sm = rows_smem<LC>();
         const int ng = ((1 << LR) / SfShape<LC>::NB) * R.L;
         sf_launch_begin(ctx, SFK_KS1_INV_ROW, st, &ev);
-        k_ks1<LR, LC, PM><<<ks_wave_blocks(ctx, sf_occupancy(k_ks1<LR, LC, PM>, NT, sm), ng * b.count), NT, sm, st>>>(R, b, ng);
+        k_ks1<LR, LC, PM><<<ks_wave_blocks(ctx, sf_occupancy(k_ks1<LR, LC, PM>, NT, sm), ng * b.count, 8), NT, sm, st>>>(R, b, ng);
         sf_launch_end(ctx, SFK_KS1_INV_ROW, st, ev);
     });
     SF_CUDA_TRY(cudaGetLastError());

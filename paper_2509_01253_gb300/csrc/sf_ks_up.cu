@@ -79,16 +79,22 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_ks2(SfRin
 #pragma unroll
                 for (int r = 0; r < 8; ++r) x[r] = y[0][r];
             } else {
-                // base conversion, lazy: each term below off, the sum below nd off
+                // base conversion, lazy: each pair of terms below 4 off
 #pragma unroll
                 for (int r = 0; r < 8; ++r) x[r] = 0;
 #pragma unroll
-                for (int t = 0; t < ND; ++t) {
+                for (int t = 0; t < ND; t += 2) {
                     if (t >= nd) break;
                     const size_t ci = ((size_t)(j * R.K + t)) * R.nm + m;
                     const sf_pair w = make_ulonglong2(R.mu_qhat[ci], R.mu_qhat_c[ci]);
+                    if (t + 1 < ND && t + 1 < nd) {
+                        const sf_pair z = make_ulonglong2(R.mu_qhat[ci + R.nm], R.mu_qhat_c[ci + R.nm]);
 #pragma unroll
-                    for (int r = 0; r < 8; ++r) x[r] = sf_mad<PM>(x[r], y[t][r], w, M);
+                        for (int r = 0; r < 8; ++r) x[r] = sf_mad2<PM>(x[r], y[t][r], w, y[t + 1 < ND ? t + 1 : 0][r], z, M);
+                    } else {
+#pragma unroll
+                        for (int r = 0; r < 8; ++r) x[r] = sf_mad<PM>(x[r], y[t][r], w, M);
+                    }
                 }
             }
             T.forward(x, tab + (size_t)m * SfShape<LR>::S, buf, M);
@@ -115,7 +121,7 @@ static void up_launch(sf_ctx *ctx, const SfKsBatch &b, cudaStream_t st)
     // split the moduli only while the launch does not fill one wave
     const int nsplit = (int)std::max<long long>(1, std::min<long long>(R.nm, (long long)ctx->num_sms * occ / ((long long)g0 * b.count)));
     const int ng = g0 * nsplit;
-    k_ks2<LR, LC, ND, PM><<<ks_wave_blocks(ctx, occ, ng * b.count), SfShape<LR>::NT, sm, st>>>(R, b, ng, nsplit);
+    k_ks2<LR, LC, ND, PM><<<ks_wave_blocks(ctx, occ, ng * b.count, 2), SfShape<LR>::NT, sm, st>>>(R, b, ng, nsplit);
 }
 
 sf_status sf_ks_up_launch(sf_ctx *ctx, const SfKsBatch &b, cudaStream_t st)

@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_leaf_col(
     for (int t = 0; t < 8; ++t) dst[(size_t)T.kl(t) << LC] = x[t];
 }
 
-// leaf_row: persistent; groups (row tile, limb i), items slots.  Per input
+// leaf_row: groups (row tile, limb i), items slots.  Per input
 // ciphertext a forward row pass and two multiply-accumulates per point, the
 // accumulators in registers.  Bound by the integer multiplier; the staged
 // twiddles (61 KB at 256-point rows) serve every slot of the group.
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS_ACC) k_leaf_
     const SfUnitRange U = sf_unit_range(ng * cnt);
     const sf_pair *ct = (const sf_pair *)P.ct;
     // group = (row tile, limb), item = slot; each thread copies its own points of
-    // an input ciphertext ahead (padding slots copy whatever the scratch holds)
+    // an input ciphertext ahead
     struct Group {
         int i, tile;
         size_t off;   // this thread's row in the limb, from a ciphertext's first limb
@@ -197,11 +197,10 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS_ACC) k_leaf_
         const SfMod &M = R.m[G.i];
         C.next();
         if (C.grp != staged) N = group(C.grp);
-        // per input ciphertext w * ct (w lazy, ct < q with its companion) lands
-        // below off <= 2^58 and is summed, with a partial reduction every 16
-        u64 acc_a[8], acc_b[8], x[8];
+        SfAcc<PM> acc_a[8], acc_b[8];
+        u64 x[8];
 #pragma unroll
-        for (int t = 0; t < 8; ++t) acc_a[t] = acc_b[t] = 0;
+        for (int t = 0; t < 8; ++t) acc_a[t] = acc_b[t] = {0, 0};
         const sf_pair *ca = ct + ((size_t)G.i << (LR + LC)) + T.store_at(G.tile, 0);
 #pragma unroll 1
         for (int j = 0; j < P.k_in; ++j) {
@@ -216,21 +215,20 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS_ACC) k_leaf_
 #pragma unroll
             for (int t = 0; t < 8; ++t) {
                 const sf_pair a = __ldg(ca + t * NT), b = __ldg(cb + t * NT);
-                acc_a[t] = sf_mad<PM>(acc_a[t], x[t], a, M);
-                acc_b[t] = sf_mad<PM>(acc_b[t], x[t], b, M);
+                sf_acc_add<PM>(acc_a[t], x[t], a, M);
+                sf_acc_add<PM>(acc_b[t], x[t], b, M);
             }
             ca = cb + per;
-            if ((j & 15) == 15) {
+            if (j % SF_ACC_TERMS == SF_ACC_TERMS - 1 && j + 1 < P.k_in) {
 #pragma unroll
-                for (int t = 0; t < 8; ++t) acc_a[t] = sf_red3(acc_a[t], M), acc_b[t] = sf_red3(acc_b[t], M);
+                for (int t = 0; t < 8; ++t) sf_acc_close<PM>(acc_a[t], M), sf_acc_close<PM>(acc_b[t], M);
             }
         }
-        const bool live = leaf_output(P, P.s0 + z * P.s_stride) >= 0;   // padding leaves are zero
         u64 *da = P.leaves + P.leaf_stride * z + ((size_t)G.i << (LR + LC)) + T.store_at(G.tile, 0), *db = da + per;
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
-            da[t * NT] = live ? sf_canon(acc_a[t], M) : 0;
-            db[t * NT] = live ? sf_canon(acc_b[t], M) : 0;
+            da[t * NT] = sf_csub3(sf_acc_close<PM>(acc_a[t], M), M);
+            db[t * NT] = sf_csub3(sf_acc_close<PM>(acc_b[t], M), M);
         }
         G = N;
     }
@@ -266,7 +264,7 @@ sf_status sf_leaves_launch(sf_ctx *ctx, const SfLeafParams &P, int cnt, cudaStre
             sf_launch_begin(ctx, SFK_LEAF_ROW, st, &ev);
             const int ng = ((1 << LR) / SfShape<LC>::NB) * R.L;
             const int occ = sf_occupancy(k_leaf_row<LR, LC, PM>, SfShape<LC>::NT, leaf_smem_row<LC>());
-            k_leaf_row<LR, LC, PM><<<ks_wave_blocks(ctx, occ, ng * c), SfShape<LC>::NT, leaf_smem_row<LC>(), st>>>(R, p, ng, c);
+            k_leaf_row<LR, LC, PM><<<ks_wave_blocks(ctx, occ, ng * c, 8), SfShape<LC>::NT, leaf_smem_row<LC>(), st>>>(R, p, ng, c);
             sf_launch_end(ctx, SFK_LEAF_ROW, st, ev);
         });
     }

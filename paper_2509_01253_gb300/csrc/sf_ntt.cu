@@ -48,8 +48,9 @@ __global__ void __launch_bounds__(COLS ? SfShape<LR>::NT : SfShape<LC>::NT) k_nt
         if (INV) {
             T.template exchange<T_::FIRST, T_::LAST>(x, buf);
             T.inverse(x, tw, buf, M);
+            sf_inv_rows_out(x, M);
 #pragma unroll
-            for (int t = 0; t < 8; ++t) jb.dst[row + T.k1(t)] = sf_red3(x[t], M);
+            for (int t = 0; t < 8; ++t) jb.dst[row + T.k1(t)] = x[t];
         } else {
             T.forward(x, tw, buf, M);
             T.template exchange<T_::LAST, T_::FIRST>(x, buf);   // back to coalesced positions
@@ -206,12 +207,12 @@ __global__ void k_rotkey_finish(SfRing R, const u64 *alpha, const u64 *e, const 
         u64 sd = sf_mul_mont(pg.v[m], s_mont[((size_t)m << R.log_n) + js], M.q, M.qinv_neg);
         u64 b = sf_sub(sf_add(as, e[i], M.q), sd, M.q);
         u64 a = alpha[i];
-        // The data limbs are stored times P^-1 mod q_m: the inner product
-        // then yields ACC_Q P^-1, the term ModDown needs, with no product of
-        // its own (sf_rotkeys_export multiplies the factor back out).
+        // The data limbs are stored times P^-1 N^-1 mod q_m: the inverse transform
+        // of the inner product then is ACC_Q P^-1, the term ModDown needs, with no
+        // product of its own (sf_rotkeys_export multiplies the factor back out).
         if (m < R.L) {
-            a = sf_mul_shoup(a, R.md_pinv[m], R.md_pinv_p[m], M.q);
-            b = sf_mul_shoup(b, R.md_pinv[m], R.md_pinv_p[m], M.q);
+            a = sf_mul_shoup(sf_mul_shoup(a, R.md_pinv[m], R.md_pinv_p[m], M.q), M.ninv, M.ninv_p, M.q);
+            b = sf_mul_shoup(sf_mul_shoup(b, R.md_pinv[m], R.md_pinv_p[m], M.q), M.ninv, M.ninv_p, M.q);
         }
         const size_t p = ((size_t)m << R.log_n) + sf_storage_index(j, R.log_r, R.log_c);
         key_a[p] = sf_make_pair(a, M, R.pm);

@@ -83,6 +83,14 @@ struct SfShape {
 };
 
 // ---- products and butterflies -----------------------------------------------
+
+// v (below 2^32 q) brought below 3q: floor((v >> sh) binv / 2^32) is floor(v / q)
+// minus at most 2
+__device__ __forceinline__ u64 sf_red3(u64 v, const SfMod &M)
+{
+    return v + (u64)__umulhi((unsigned)(v >> M.sh), M.binv) * (0 - M.q);
+}
+
 // Two forms of a product by a fixed operand w < q, both with a stored companion
 // and both returning acc + r with r = x w (mod q), 0 <= r < off for any x < 2^64;
 // the accumulator rides through the wide multiplies, which add it for free.
@@ -112,8 +120,57 @@ __device__ __forceinline__ u64 sf_mad(u64 acc, u64 x, const sf_pair w, const SfM
     }
 }
 
+// acc + x w + y z (mod q) for canonical x, y, the added part below 4 off; with PM
+// the two products share the last multiply: 4q times the sum of their quotients
+// by 2^52, each below 2^30 + 2^17 and short by less than 4, so the rest is below
+// 8 2^52 + 2^33 delta
+template <bool PM>
+__device__ __forceinline__ u64 sf_mad2(u64 acc, u64 x, const sf_pair w, u64 y, const sf_pair z, const SfMod &M)
+{
+    if constexpr (PM) {
+        const unsigned x0 = (unsigned)x, x1 = (unsigned)(x >> 32), y0 = (unsigned)y, y1 = (unsigned)(y >> 32);
+        const unsigned qh = __umulhi(x0, (unsigned)(w.x >> 20)) + __umulhi(x1, (unsigned)(w.y >> 20)) +
+                            __umulhi(y0, (unsigned)(z.x >> 20)) + __umulhi(y1, (unsigned)(z.y >> 20));
+        return acc + x0 * w.x + x1 * w.y + y0 * z.x + y1 * z.y + qh * (2 * M.n2q);
+    } else {
+        return sf_mad<PM>(sf_mad<PM>(acc, x, w, M), y, z, M);
+    }
+}
+
+// Inner products: acc.s + sum of x_j w_j, canonical w_j, closed by sf_acc_close.
+// With PM the quotients of all terms are summed and multiplied once; by 2^53 each
+// is below 2^30 (x < 2^64), so a sum holds 4 terms (SF_ACC_TERMS) between closes.
+#define SF_ACC_TERMS 4
+template <bool PM>
+struct SfAcc {
+    u64 s;
+    unsigned qh;
+};
+template <bool PM>
+__device__ __forceinline__ void sf_acc_add(SfAcc<PM> &a, u64 x, const sf_pair w, const SfMod &M)
+{
+    if constexpr (PM) {
+        const unsigned x0 = (unsigned)x, x1 = (unsigned)(x >> 32);
+        a.s = a.s + x0 * w.x + x1 * w.y;
+        a.qh += __umulhi(x0, (unsigned)(w.x >> 21)) + __umulhi(x1, (unsigned)(w.y >> 21));
+    } else {
+        a.s = sf_mad<PM>(a.s, x, w, M);
+    }
+}
+// the sum below 3q; the accumulator goes on from it.  Before: per term
+// T - qh 2^53 < 4 2^53 and qh 8 delta < 2^33 delta, so four terms stay below
+// 2^57 + 2^35 delta <= 4 off + 2^57 < 2^61.
+template <bool PM>
+__device__ __forceinline__ u64 sf_acc_close(SfAcc<PM> &a, const SfMod &M)
+{
+    if constexpr (PM) a.s = a.s + a.qh * (4 * M.n2q);
+    a.s = sf_red3(a.s, M);
+    a.qh = 0;
+    return a.s;
+}
+
 // forward: X + wY, X - wY + off; bounds grow by off per stage, from at most
-// 4 off to 20 off < 2^63 after 16 stages (checked when the context is made)
+// 8 off to 24 off < 2^63 after 16 stages (checked when the context is made)
 template <bool PM>
 __device__ __forceinline__ void sf_fwd(u64 &X, u64 &Y, const sf_pair w, const SfMod &M)
 {
@@ -123,9 +180,7 @@ __device__ __forceinline__ void sf_fwd(u64 &X, u64 &Y, const sf_pair w, const Sf
 }
 
 // inverse with the mirrored twiddle: X + Y, (Y - X) w.  `off` is a multiple of q
-// above every input, so the difference is positive.  Inputs of a pass are below
-// 4q; after stage 0 values stay below off1 = max(8q, off) and the bound doubles
-// from stage to stage (sf_inv_off).
+// above every input (sf_inv_off), so the difference is positive.
 template <bool PM>
 __device__ __forceinline__ void sf_inv(u64 &X, u64 &Y, const sf_pair w, const SfMod &M, u64 off)
 {
@@ -134,15 +189,9 @@ __device__ __forceinline__ void sf_inv(u64 &X, u64 &Y, const sf_pair w, const Sf
     Y = sf_mad<PM>(0, d, w, M);
 }
 
-// v < 2^63 (and below 2^32 q) brought below 3q: floor((v >> sh) binv / 2^32) is
-// floor(v / q) minus at most 2
-__device__ __forceinline__ u64 sf_red3(u64 v, const SfMod &M)
-{
-    return v + (u64)__umulhi((unsigned)(v >> M.sh), M.binv) * (0 - M.q);
-}
-
-// v < 2^63 (and below 2^32 q) brought to [0, q)
-__device__ __forceinline__ u64 sf_canon(u64 v, const SfMod &M) { return sf_csub(sf_csub(sf_red3(v, M), M.q), M.q); }
+// v (below 2^32 q) brought to [0, q)
+__device__ __forceinline__ u64 sf_csub3(u64 v, const SfMod &M) { return sf_csub(sf_csub(v, M.q), M.q); }   // v < 3q
+__device__ __forceinline__ u64 sf_canon(u64 v, const SfMod &M) { return sf_csub3(sf_red3(v, M), M); }
 
 // ---- column tiles --------------------------------------------------------------
 // NB columns of 2^LR points; thread: column b = tid % NB, i = tid / NB, so NB
@@ -150,16 +199,30 @@ __device__ __forceinline__ u64 sf_canon(u64 v, const SfMod &M) { return sf_csub(
 // Register t of phase ph holds k = (i >> P) 2^(P+3) + t 2^P + (i mod 2^P).  The
 // column table is tab[k], k < R; buf is the exchange buffer.
 
-// Bound of the inputs of inverse stage st (a multiple of q): 4q, off1, 2 off1, ...
-// The eighth stage would leave 64 bits no room, so after their second phase
-// (stages 2 to 4) 256-point passes reduce the one register that was a sum in all
-// of its stages (t = 0); the others were products at most two stages ago, below
-// 4 off1.
+// Bounds of an inverse pass (multiples of q, off1 = max(8q, off) <= 2^58).  Its
+// inputs are below off1; a product stays below off and the bound of a sum doubles.
+// Before the last phase (three stages) the registers that were sums in three
+// stages of the phase before, or in two after two others, are reduced
+// (sf_inv_fold), so that its inputs are below 4 off1 and every value stays below
+// 2^63.  After the last phase x[4 .. 7] are products, below off, x[2], x[3] below
+// 2 off and x[1] below 4 off; x[0] is below 32 off1.
 template <int LS>
 __device__ __forceinline__ u64 sf_inv_off(int st, const SfMod &M)
 {
-    if (st == 0) return 4 * M.q;
-    return M.off1 << (LS == 8 && st >= 5 ? st - 3 : st - 1);
+    return M.off1 << (st < LS - 3 ? st : st - (LS - 3) + 2);
+}
+template <int LS>
+__device__ __forceinline__ void sf_inv_fold(u64 (&x)[8], const SfMod &M)
+{
+    if (LS >= 6) x[0] = sf_red3(x[0], M);
+    if (LS == 7) x[4] = sf_red3(x[4], M);
+}
+
+// rows of an inverse pass handed to its columns: below off again
+__device__ __forceinline__ void sf_inv_rows_out(u64 (&x)[8], const SfMod &M)
+{
+#pragma unroll
+    for (int t = 0; t < 4; ++t) x[t] = sf_red3(x[t], M);
 }
 
 template <int LR, bool PM>
@@ -210,7 +273,7 @@ struct SfColT {
                 for (int a = 0; a < d; ++a) sf_inv<PM>(x[2 * d * sub + a], x[2 * d * sub + a + d], w, M, off);
             }
         }
-        if (Sh::LS_ == 8 && PH == 1) x[0] = sf_red3(x[0], M);   // see sf_inv_off
+        if (PH == 1) sf_inv_fold<Sh::LS_>(x, M);
     }
     // exchange through buf; the leading barrier orders the previous reads of buf
     // (an exchange, or points copied ahead into it) before these writes
@@ -229,6 +292,10 @@ struct SfColT {
     __device__ __forceinline__ void forward(u64 (&x)[8], const sf_pair *tab, u64 *buf, const SfMod &M) const
     {
         phase_fwd<0>(x, tab, M);
+        forward_rest(x, tab, buf, M);
+    }
+    __device__ __forceinline__ void forward_rest(u64 (&x)[8], const sf_pair *tab, u64 *buf, const SfMod &M) const
+    {
         exchange<0, 1>(x, buf);
         phase_fwd<1>(x, tab, M);
         if constexpr (Sh::NP == 3) {
@@ -310,7 +377,7 @@ struct SfRowT {
                 for (int a = 0; a < d; ++a) sf_inv<PM>(x[2 * d * sub + a], x[2 * d * sub + a + d], w, M, off);
             }
         }
-        if (Sh::LS_ == 8 && PH == 1) x[0] = sf_red3(x[0], M);   // see sf_inv_off
+        if (PH == 1) sf_inv_fold<Sh::LS_>(x, M);
     }
     template <int PH>
     __device__ __forceinline__ void put(const u64 (&x)[8], u64 *buf) const
@@ -354,11 +421,15 @@ struct SfRowT {
     // inverse pass: the other way round
     __device__ __forceinline__ void inverse(u64 (&x)[8], const sf_pair *tw, u64 *buf, const SfMod &M) const
     {
+        phase_inv<LAST>(x, tw, M);
+        inverse_rest(x, tw, buf, M);
+    }
+    __device__ __forceinline__ void inverse_rest(u64 (&x)[8], const sf_pair *tw, u64 *buf, const SfMod &M) const
+    {
         if constexpr (Sh::NP == 3) {
-            phase_inv<2>(x, tw, M);
             exchange<2, 1>(x, buf);
+            phase_inv<1>(x, tw, M);
         }
-        phase_inv<1>(x, tw, M);
         exchange<1, 0>(x, buf);
         phase_inv<0>(x, tw, M);
     }
@@ -400,8 +471,8 @@ SF_HD int sf_natural_index(int p, int log_r, int log_c)
     return (((b >> hl) ? R - 1 - rr : rr) << log_c) + 8 * i + t;
 }
 
-// ---- balanced persistent partition ----------------------------------------
-// A persistent launch of gridDim.x blocks over n_units work units numbered
+// ---- balanced partition ----------------------------------------
+// A launch of gridDim.x blocks over n_units work units numbered
 // group-major (u = group * n_items + item) gives block x the units
 // [x n / grid, (x + 1) n / grid): every block the floor or the ceiling of the
 // mean, whatever the group count, and a block restages tables only where its
