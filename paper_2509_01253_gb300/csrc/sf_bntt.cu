@@ -13,7 +13,7 @@
 //
 // Bound by the integer multiplier: at N = 2^16 the fmaheavy pipe is busy 70 to
 // 76 % of the cycles.  512 x 5 limbs of 2^16, forward: 1961 us with tile sweeps in
-// shared memory, 1550 us here; 37 x 3 inverse limbs of 2^14: 32.8 and 28.5 us.
+// shared memory, 1515 us here; 37 x 3 inverse limbs of 2^14: 32.8 and 26.6 us.
 #include <algorithm>
 
 #include "sf_async.cuh"
@@ -31,8 +31,7 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS)
     using T_ = SfRowT<LC, PM>;
     const T_ T;
     sf_pair *tw = (sf_pair *)smem_raw;
-    constexpr int NT = SfShape<LC>::NT;
-    u64 *buf = (u64 *)(tw + SfShape<LC>::PAIRS), *pre = buf + SfShape<LC>::WORDS + threadIdx.x;
+    u64 *buf = (u64 *)(tw + SfShape<LC>::PAIRS), *ahead = buf + SfShape<LC>::WORDS;
     const SfUnitRange U = sf_unit_range(ng * count);
     const size_t per = (size_t)R.L << (LR + LC);
     // group = (row tile, limb i), item = polynomial; offset of this thread's row
@@ -44,7 +43,7 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS)
     // each thread copies its own points of the next unit ahead
     auto prefetch = [&]() {
 #pragma unroll
-        for (int t = 0; t < 8; ++t) sf_cp8(pre + t * NT, src + off + (T.k1(t) - T.k1(0)));
+        for (int t = 0; t < 8; ++t) sf_cp8(T.template mine<0>(ahead) + SfShape<LC>::step(0, t), src + off + (T.k1(t) - T.k1(0)));
         sf_cp_commit();
     };
     if (U.u0 < U.u1) prefetch();
@@ -60,17 +59,18 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS)
         const SfMod &M = R.m[mod];
         u64 x[8];
         sf_cp_wait<0>();
-#pragma unroll
-        for (int t = 0; t < 8; ++t) x[t] = pre[t * NT];
+        if (INV) __syncwarp();   // the last phase's points lie among the row's threads
+        T.template get<INV ? T_::LAST : 0>(x, ahead);
         u64 *d = dst + off;
         // the next unit's copy overtakes this unit's stores: in place, the two units
         // touch different rows or polynomials
         C.next();
         off = C.grp == staged ? off + per : group_off(C.grp);
         if (INV) {
-            T.template exchange<T_::FIRST, T_::LAST>(x, buf);
+            T.template phase_inv<T_::LAST>(x, tw, M);
+            __syncwarp();
             if (u + 1 < U.u1) prefetch();
-            T.inverse(x, tw, buf, M);
+            T.inverse_rest(x, tw, buf, M);
             sf_inv_rows_out(x, M);
 #pragma unroll
             for (int t = 0; t < 8; ++t) d[T.k1(t) - T.k1(0)] = x[t];
@@ -92,8 +92,8 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SfColT<LR, PM> T;
     sf_pair *tab = (sf_pair *)smem_raw;
-    constexpr int NT = SfShape<LR>::NT;
-    u64 *buf = (u64 *)(tab + SfShape<LR>::S), *pre = buf + SfShape<LR>::WORDS + threadIdx.x;
+    // two buffers: points ahead and exchanges by turns
+    u64 *buf = (u64 *)(tab + SfShape<LR>::S), *ahead = buf + SfShape<LR>::WORDS;
     const SfUnitRange U = sf_unit_range(ng * count);
     const size_t per = (size_t)R.L << (LR + LC);
     // group = (column tile, limb i), item = polynomial; offset of this thread's column
@@ -103,12 +103,13 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS)
     SfCursor C(U.u0, count);
     size_t off = group_off(C.grp) + per * C.item;
     // each thread copies its own points of the next unit ahead
-    auto prefetch = [&]() {
+    constexpr int PH = INV ? SfColT<LR, PM>::LAST : 0;
+    auto prefetch = [&](u64 *to) {
 #pragma unroll
-        for (int t = 0; t < 8; ++t) sf_cp8(pre + t * NT, src + off + ((size_t)(INV ? T.kl(t) : T.k1(t)) << LC));
+        for (int t = 0; t < 8; ++t) sf_cp8(T.template mine<PH>(to) + SfShape<LR>::step(PH, t) * SfShape<LR>::NB, src + off + ((size_t)T.template k<PH>(t) << LC));
         sf_cp_commit();
     };
-    if (U.u0 < U.u1) prefetch();
+    if (U.u0 < U.u1) prefetch(buf);
     int staged = -1, mod = 0;
     for (int u = U.u0; u < U.u1; ++u) {
         if (C.grp != staged) {
@@ -121,31 +122,32 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS)
         const SfMod &M = R.m[mod];
         u64 x[8];
         sf_cp_wait<0>();
-#pragma unroll
-        for (int t = 0; t < 8; ++t) x[t] = pre[t * NT];
+        T.template get<PH>(x, buf);
         u64 *d = dst + off;
         C.next();
         off = C.grp == staged ? off + per : group_off(C.grp);
+        auto next = [&] {
+            if (u + 1 < U.u1) prefetch(ahead);
+        };
         if (INV) {
-            T.template phase_inv<SfColT<LR, PM>::LAST>(x, tab, M);
-            if (u + 1 < U.u1) prefetch();   // this unit's points are in registers
-            T.inverse_rest(x, tab, buf, M);
+            T.inverse(x, tab, buf, M, next);
 #pragma unroll
             for (int t = 0; t < 8; ++t) d[(size_t)T.k1(t) << LC] = sf_canon(sf_mad<PM>(0, x[t], make_ulonglong2(M.ninv, M.ninv_c), M), M);
         } else {
-            T.template phase_fwd<0>(x, tab, M);
-            if (u + 1 < U.u1) prefetch();
-            T.forward_rest(x, tab, buf, M);
+            T.forward(x, tab, buf, M, next);
 #pragma unroll
             for (int t = 0; t < 8; ++t) d[(size_t)T.kl(t) << LC] = x[t];
         }
+        u64 *used = buf;
+        buf = ahead;
+        ahead = used;
     }
 }
 
 template <int LC>
-static constexpr size_t bntt_smem_row() { return sizeof(sf_pair) * SfShape<LC>::PAIRS + sizeof(u64) * (SfShape<LC>::WORDS + SfShape<LC>::TILE); }
+static constexpr size_t bntt_smem_row() { return sizeof(sf_pair) * SfShape<LC>::PAIRS + sizeof(u64) * 2 * SfShape<LC>::WORDS; }
 template <int LR>
-static constexpr size_t bntt_smem_col() { return sizeof(sf_pair) * SfShape<LR>::S + sizeof(u64) * (SfShape<LR>::WORDS + SfShape<LR>::TILE); }
+static constexpr size_t bntt_smem_col() { return sizeof(sf_pair) * SfShape<LR>::S + sizeof(u64) * 2 * SfShape<LR>::WORDS; }
 
 template <bool INV, int LR, int LC, bool PM>
 static void bntt_row(sf_ctx *ctx, const u64 *src, u64 *dst, int count, cudaStream_t st)

@@ -22,11 +22,10 @@
 template <int LR, int LC, int KT, bool PM>
 __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_ks4(SfRing R, SfKsBatch B, int ng, int nsplit)
 {
-    constexpr int NT = SfShape<LR>::NT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SfColT<LR, PM> T;
-    sf_pair *tab = (sf_pair *)smem_raw;   // [nm][R], the exchange buffer, points ahead
-    u64 *buf = (u64 *)(tab + (size_t)R.nm * SfShape<LR>::S), *pre = buf + SfShape<LR>::WORDS + threadIdx.x;
+    sf_pair *tab = (sf_pair *)smem_raw;   // [nm][R], two buffers: points ahead and exchanges by turns
+    u64 *buf = (u64 *)(tab + (size_t)R.nm * SfShape<LR>::S), *ahead = buf + SfShape<LR>::WORDS;
     sf_stage_cols<LR>(tab, R.colP, 0, R.nm);
     __syncthreads();
     const SfUnitRange U = sf_unit_range(ng * B.count);
@@ -45,15 +44,16 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_ks4(SfRin
     };
     // modulus of step s of a unit; each thread copies its own points of a step ahead
     auto step_mod = [&](const Unit &V, int s) { return s < R.K ? R.L + s : V.lo + s - R.K; };
-    auto prefetch = [&](const Unit &V, int s) {
+    constexpr int LAST = SfColT<LR, PM>::LAST;
+    auto prefetch = [&](const Unit &V, int s, u64 *to) {
         const u64 *src = V.acc + ((size_t)step_mod(V, s) << (LR + LC));
 #pragma unroll
-        for (int t = 0; t < 8; ++t) sf_cp8(pre + t * NT, src + ((size_t)T.kl(t) << LC));
+        for (int t = 0; t < 8; ++t) sf_cp8(T.template mine<LAST>(to) + SfShape<LR>::step(LAST, t) * SfShape<LR>::NB, src + ((size_t)T.kl(t) << LC));
         sf_cp_commit();
     };
     SfCursor C(U.u0, ng);
     Unit V = unit(C), N = V;
-    if (U.u0 < U.u1) prefetch(V, 0);
+    if (U.u0 < U.u1) prefetch(V, 0, buf);
     for (int u = U.u0; u < U.u1; ++u) {
         u64 *out0 = merge_out(B, C.grp) + ((size_t)(V.part * R.L) << (LR + LC)) + V.col;
         // `out` holds v (+ tau_d(u.b)) of coefficient-domain operands; a plain
@@ -70,14 +70,16 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_ks4(SfRin
             u64 *out = out0 + ((size_t)m << (LR + LC));
             u64 x[8], o[8];
             sf_cp_wait<0>();
+            T.template get<LAST>(x, buf);
+            T.inverse(x, tab + (size_t)m * SfShape<LR>::S, buf, M, [&] {
+                if (s + 1 < V.steps) prefetch(V, s + 1, ahead);
+                else if (u + 1 < U.u1) prefetch(N, 0, ahead);
 #pragma unroll
-            for (int t = 0; t < 8; ++t) x[t] = pre[t * NT];
-            T.template phase_inv<SfColT<LR, PM>::LAST>(x, tab + (size_t)m * SfShape<LR>::S, M);
-            if (s + 1 < V.steps) prefetch(V, s + 1);   // the points of this step are in registers
-            else if (u + 1 < U.u1) prefetch(N, 0);
-#pragma unroll
-            for (int t = 0; t < 8; ++t) o[t] = add && s >= R.K ? out[(size_t)T.k1(t) << LC] : 0;
-            T.inverse_rest(x, tab + (size_t)m * SfShape<LR>::S, buf, M);
+                for (int t = 0; t < 8; ++t) o[t] = add && s >= R.K ? out[(size_t)T.k1(t) << LC] : 0;
+            });
+            u64 *used = buf;
+            buf = ahead;
+            ahead = used;
             if (s < R.K) {
                 const sf_pair w = make_ulonglong2(R.md_inv[s], R.md_inv_c[s]);
 #pragma unroll
@@ -116,7 +118,7 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_ks4(SfRin
 template <int LR>
 static size_t down_smem(const SfRing &R)
 {
-    return sizeof(sf_pair) * R.nm * SfShape<LR>::S + sizeof(u64) * (SfShape<LR>::WORDS + SfShape<LR>::TILE);
+    return sizeof(sf_pair) * R.nm * SfShape<LR>::S + sizeof(u64) * 2 * SfShape<LR>::WORDS;
 }
 
 template <int LR, int LC, int KT, bool PM>

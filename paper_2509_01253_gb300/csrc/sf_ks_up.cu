@@ -25,7 +25,13 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_ks2(SfRin
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SfColT<LR, PM> T;
     sf_pair *tab = (sf_pair *)smem_raw;                   // [nm][R]
-    u64 *buf = (u64 *)(tab + (size_t)R.nm * SfShape<LR>::S);
+    // two exchange buffers, by turns
+    u64 *buf = (u64 *)(tab + (size_t)R.nm * SfShape<LR>::S), *other = buf + SfShape<LR>::WORDS;
+    auto turn = [&] {
+        u64 *used = buf;
+        buf = other;
+        other = used;
+    };
     sf_stage_cols<LR>(tab, R.colP, 0, R.nm);
     __syncthreads();
     const SfUnitRange U = sf_unit_range(ng * B.count);
@@ -52,6 +58,7 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_ks2(SfRin
             if (B.ntt) {
                 // NTT-domain operands: TA's rows are inverse transformed, N^-1 rides on the scaling
                 T.inverse(y[t], tab + (size_t)(lo + t) * SfShape<LR>::S, buf, M);
+                turn();
                 w = make_ulonglong2(R.mu_inv[j * R.K + t], R.mu_inv_c[j * R.K + t]);
             }
             if (B.ntt || nd > 1) {
@@ -98,6 +105,7 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_ks2(SfRin
                 }
             }
             T.forward(x, tab + (size_t)m * SfShape<LR>::S, buf, M);
+            turn();
             u64 *dst = B.scratch + per * b + ((size_t)(sf_ks_x2(R) + j * R.nm + m) << (LR + LC)) + col;
 #pragma unroll
             for (int t = 0; t < 8; ++t) dst[(size_t)T.kl(t) << LC] = x[t];
@@ -108,7 +116,7 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_ks2(SfRin
 template <int LR>
 static size_t up_smem(const SfRing &R)
 {
-    return sizeof(sf_pair) * R.nm * SfShape<LR>::S + sizeof(u64) * SfShape<LR>::WORDS;
+    return sizeof(sf_pair) * R.nm * SfShape<LR>::S + sizeof(u64) * 2 * SfShape<LR>::WORDS;
 }
 
 template <int LR, int LC, int ND, bool PM>

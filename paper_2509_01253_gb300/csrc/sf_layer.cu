@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_leaf_col(
     u64 x[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) x[t] = tile[T.at(T.k1(t))];
-    T.forward(x, tab, tile, M);   // its first exchange waits for these reads
+    T.forward(x, tab, tile, M);
     u64 *dst = P.w1 + ((((size_t)blockIdx.z * P.k_in + j) * R.L + i) << (LR + LC)) + blockIdx.x * NB + T.b;
 #pragma unroll
     for (int t = 0; t < 8; ++t) dst[(size_t)T.kl(t) << LC] = x[t];

@@ -275,47 +275,73 @@ struct SfColT {
         }
         if (PH == 1) sf_inv_fold<Sh::LS_>(x, M);
     }
-    // exchange through buf; the leading barrier orders the previous reads of buf
-    // (an exchange, or points copied ahead into it) before these writes
-    template <int FROM, int TO>
-    __device__ __forceinline__ void exchange(u64 (&x)[8], u64 *buf) const
+    // The first of the two exchanges (last of an inverse pass) crosses the block;
+    // the other one stays among the threads that hold one 32-point stretch of every
+    // column: a warp at 256 points, two at 128.  A thread overwrites only the words
+    // it read last, so an exchange takes one barrier, and a transform one block
+    // barrier, if a block's consecutive transforms alternate between two buffers:
+    // a thread past that barrier of one transform has all threads past their reads
+    // of the other buffer (`after` may then copy points into this thread's words of
+    // it).  With four block barriers a transform, 512 x 5 limbs of 2^16 took 1550 us
+    // against 1515 and the ModDown 228 ms against 222 per 32768 key switches.
+    template <int PH>
+    __device__ __forceinline__ u64 *mine(u64 *buf) const { return buf + Sh::pos(PH, i) * Sh::NB + b; }
+    template <int PH>
+    __device__ __forceinline__ void put(const u64 (&x)[8], u64 *buf) const
     {
-        u64 *from = buf + Sh::pos(FROM, i) * Sh::NB + b;
-        const u64 *to = buf + Sh::pos(TO, i) * Sh::NB + b;
-        __syncthreads();
 #pragma unroll
-        for (int t = 0; t < 8; ++t) from[Sh::step(FROM, t) * Sh::NB] = x[t];
-        __syncthreads();
-#pragma unroll
-        for (int t = 0; t < 8; ++t) x[t] = to[Sh::step(TO, t) * Sh::NB];
+        for (int t = 0; t < 8; ++t) mine<PH>(buf)[Sh::step(PH, t) * Sh::NB] = x[t];
     }
-    __device__ __forceinline__ void forward(u64 (&x)[8], const sf_pair *tab, u64 *buf, const SfMod &M) const
+    template <int PH>
+    __device__ __forceinline__ void get(u64 (&x)[8], u64 *buf) const
+    {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) x[t] = mine<PH>(buf)[Sh::step(PH, t) * Sh::NB];
+    }
+    __device__ __forceinline__ static void stretch_sync()
+    {
+        if constexpr (4 * Sh::NB == 32) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(1 + threadIdx.x / (4 * Sh::NB)), "n"(4 * Sh::NB) : "memory");
+    }
+    template <class F>
+    __device__ __forceinline__ void forward(u64 (&x)[8], const sf_pair *tab, u64 *buf, const SfMod &M, F after) const
     {
         phase_fwd<0>(x, tab, M);
-        forward_rest(x, tab, buf, M);
-    }
-    __device__ __forceinline__ void forward_rest(u64 (&x)[8], const sf_pair *tab, u64 *buf, const SfMod &M) const
-    {
-        exchange<0, 1>(x, buf);
+        put<0>(x, buf);
+        __syncthreads();
+        after();
+        get<1>(x, buf);
         phase_fwd<1>(x, tab, M);
         if constexpr (Sh::NP == 3) {
-            exchange<1, 2>(x, buf);
+            put<1>(x, buf);
+            stretch_sync();
+            get<2>(x, buf);
             phase_fwd<2>(x, tab, M);
         }
     }
-    __device__ __forceinline__ void inverse(u64 (&x)[8], const sf_pair *tab, u64 *buf, const SfMod &M) const
+    template <class F>
+    __device__ __forceinline__ void inverse(u64 (&x)[8], const sf_pair *tab, u64 *buf, const SfMod &M, F after) const
     {
         phase_inv<LAST>(x, tab, M);
-        inverse_rest(x, tab, buf, M);
-    }
-    __device__ __forceinline__ void inverse_rest(u64 (&x)[8], const sf_pair *tab, u64 *buf, const SfMod &M) const
-    {
+        put<LAST>(x, buf);
         if constexpr (Sh::NP == 3) {
-            exchange<2, 1>(x, buf);
+            stretch_sync();
+            get<1>(x, buf);
             phase_inv<1>(x, tab, M);
+            put<1>(x, buf);
         }
-        exchange<1, 0>(x, buf);
+        __syncthreads();
+        after();
+        get<0>(x, buf);
         phase_inv<0>(x, tab, M);
+    }
+    __device__ __forceinline__ void forward(u64 (&x)[8], const sf_pair *tab, u64 *buf, const SfMod &M) const
+    {
+        forward(x, tab, buf, M, [] {});
+    }
+    __device__ __forceinline__ void inverse(u64 (&x)[8], const sf_pair *tab, u64 *buf, const SfMod &M) const
+    {
+        inverse(x, tab, buf, M, [] {});
     }
 };
 
@@ -380,18 +406,18 @@ struct SfRowT {
         if (PH == 1) sf_inv_fold<Sh::LS_>(x, M);
     }
     template <int PH>
+    __device__ __forceinline__ u64 *mine(u64 *buf) const { return buf + b * Sh::PITCH + Sh::pos(PH, i); }
+    template <int PH>
     __device__ __forceinline__ void put(const u64 (&x)[8], u64 *buf) const
     {
-        u64 *to = buf + b * Sh::PITCH + Sh::pos(PH, i);
 #pragma unroll
-        for (int t = 0; t < 8; ++t) to[Sh::step(PH, t)] = x[t];
+        for (int t = 0; t < 8; ++t) mine<PH>(buf)[Sh::step(PH, t)] = x[t];
     }
     template <int PH>
-    __device__ __forceinline__ void get(u64 (&x)[8], const u64 *buf) const
+    __device__ __forceinline__ void get(u64 (&x)[8], u64 *buf) const
     {
-        const u64 *from = buf + b * Sh::PITCH + Sh::pos(PH, i);
 #pragma unroll
-        for (int t = 0; t < 8; ++t) x[t] = from[Sh::step(PH, t)];
+        for (int t = 0; t < 8; ++t) x[t] = mine<PH>(buf)[Sh::step(PH, t)];
     }
     // exchange inside the warp; the leading barrier orders the reads of the
     // previous exchange before these writes
@@ -399,6 +425,12 @@ struct SfRowT {
     __device__ __forceinline__ void exchange(u64 (&x)[8], u64 *buf) const
     {
         __syncwarp();
+        exchange_on<FROM, TO>(x, buf);
+    }
+    // the same where this thread read the words it writes last
+    template <int FROM, int TO>
+    __device__ __forceinline__ void exchange_on(u64 (&x)[8], u64 *buf) const
+    {
         put<FROM>(x, buf);
         __syncwarp();
         get<TO>(x, buf);
@@ -414,7 +446,7 @@ struct SfRowT {
         exchange<0, 1>(x, buf);
         phase_fwd<1>(x, tw, M);
         if constexpr (Sh::NP == 3) {
-            exchange<1, 2>(x, buf);
+            exchange_on<1, 2>(x, buf);
             phase_fwd<2>(x, tw, M);
         }
     }
@@ -429,8 +461,10 @@ struct SfRowT {
         if constexpr (Sh::NP == 3) {
             exchange<2, 1>(x, buf);
             phase_inv<1>(x, tw, M);
+            exchange_on<1, 0>(x, buf);
+        } else {
+            exchange<1, 0>(x, buf);
         }
-        exchange<1, 0>(x, buf);
         phase_inv<0>(x, tw, M);
     }
     // storage order: last-phase element t of this thread in tile `tile`
