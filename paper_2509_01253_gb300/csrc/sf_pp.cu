@@ -20,35 +20,39 @@
 // products, ppt_dft_pairs; two at t = 3, ppt_dft3);
 // twiddles and t-th roots come from a per-limb table of omega^e.  Table 2's
 // rings and the small test rings are compiled with t and alpha as constants
-// (k_ppt_ntt); other rings run the generic kernel (k_pp_ntt).
+// (k_ppt_ntt), without reductions inside a transform where the primes have at
+// most 50 bits; other rings run the generic kernel (k_pp_ntt).
 #include <algorithm>
 #include <vector>
 
 #include "sf_pp.cuh"
 
-template <int T, int ALPHA>
-__global__ void __launch_bounds__(SfPpT<T, ALPHA>::THREADS) k_ppt_ntt(SfPpRing R, const u64 *in, u64 *out, int inverse)
+template <int T, int ALPHA, bool LZ, bool INV>
+__global__ void __launch_bounds__(SfPpT<T, ALPHA>::THREADS) k_ppt_ntt(SfPpRing R, const u64 *in, u64 *out)
 {
     constexpr int M = SfPpT<T, ALPHA>::M, NT = SfPpT<T, ALPHA>::THREADS;
     __shared__ u64 s[M];
     const int i = blockIdx.x;
-    const SfPpMod &P = R.mod[i];
     const size_t off = ((size_t)blockIdx.y * R.L + i) * M;
-    if (inverse) {
+    if (INV) {
         for (int e = threadIdx.x; e < M; e += NT) s[e] = in[off + e];
         __syncthreads();
-        constexpr int H = (T - 1) / 2;
-        ppt_inverse<T, M, T>(s, R.iw + (size_t)i * M, R.iw_p + (size_t)i * M, R.dftc + (size_t)i * H * H * 4, P.q,
-                             P.one_p, P);
-        for (int e = threadIdx.x; e < M; e += NT) out[off + e] = sf_mul_shoup(s[e], P.minv, P.minv_p, P.q);
+        pp_block_inverse<T, ALPHA, LZ>(s, R, i);
+        for (int e = threadIdx.x; e < M; e += NT) out[off + e] = s[e];
     } else {
-        constexpr int H = (T - 1) / 2;
         // the first stage reads the input straight from global memory
         const u64 *src = in + off;
-        ppt_forward_ld<T, M>(s, [src](int e) { return src[e]; }, R.w + (size_t)i * M, R.w_p + (size_t)i * M,
-                             R.dftc + (size_t)i * H * H * 4, P.q, P.one_p, P);
-        for (int e = threadIdx.x; e < M; e += NT) out[off + e] = s[e];
+        pp_block_forward_ld<T, ALPHA, LZ>(s, [src](int e) { return src[e]; }, R, i);
+        for (int e = threadIdx.x; e < M; e += NT) out[off + e] = LZ ? pp_canon(s[e], R.mod[i]) : s[e];
     }
+}
+
+template <int T, int ALPHA, bool LZ>
+static void ppt_ntt(const SfPpRing &R, const u64 *in, u64 *out, int count, bool inverse, cudaStream_t st)
+{
+    const dim3 grid(R.L, count);
+    if (inverse) k_ppt_ntt<T, ALPHA, LZ, true><<<grid, SfPpT<T, ALPHA>::THREADS, 0, st>>>(R, in, out);
+    else k_ppt_ntt<T, ALPHA, LZ, false><<<grid, SfPpT<T, ALPHA>::THREADS, 0, st>>>(R, in, out);
 }
 
 // Batched length-M transform: grid (L, count); [count][L][M] in and out.
@@ -162,7 +166,11 @@ extern "C" sf_status sf_pp_ring_create(int32_t t, int32_t alpha, int32_t L, int3
     }
     const int H = (t - 1) / 2;
     const size_t o_qhat = (size_t)4 * L * R.M, o_dftc = o_qhat + (size_t)2 * L * L;
-    std::vector<u64> tab(o_dftc + (size_t)4 * L * H * H);
+    const size_t o_tw = (o_dftc + (size_t)4 * L * H * H + 1) & ~(size_t)1;   // pairs: 16-byte aligned
+    const int nd = t == 3 ? 2 : t == 5 ? 5 : 2 * H * H;   // SfPpDft<t>::N
+    const size_t o_dftl = o_tw + (size_t)4 * L * R.M;
+    std::vector<u64> tab(o_dftl + (size_t)2 * L * nd);
+    R.lazy = bits <= 50;
     for (int i = 0; i < L; ++i) {
         const u64 q = r->q[i];
         const u64 w = pp_root(q, R.M, t), iw = sf_host_invmod(w, q);
@@ -189,6 +197,18 @@ extern "C" sf_status sf_pp_ring_create(int32_t t, int32_t alpha, int32_t L, int3
         P.minv_p = sf_shoup_companion(P.minv, q);
         P.h2 = sf_host_invmod(2, q);
         P.h2_p = sf_shoup_companion(P.h2, q);
+        P.sh = 63 - __builtin_clzll(q);
+        P.binv = (unsigned)(((unsigned __int128)1 << (32 + P.sh)) / q);
+        // twiddles by stage: entry M - len + (k - 1) len / t + j is omega_len^(+- j k)
+        for (int dir = 0; dir < 2; ++dir)
+            for (int len = R.M; len > t; len /= t)
+                for (int k = 1; k < t; ++k)
+                    for (int j = 0; j < len / t; ++j) {
+                        const size_t e = (size_t)i * R.M + (size_t)(R.M / len) * j * k;
+                        u64 *d = &tab[o_tw + 2 * ((size_t)(2 * i + dir) * R.M + R.M - len + (k - 1) * (len / t) + j)];
+                        d[0] = tab[(size_t)(2 * dir) * L * R.M + e];
+                        d[1] = tab[(size_t)(2 * dir + 1) * L * R.M + e];
+                    }
         // zeta = omega^(M/3): c = (zeta - zeta^2) / 2 (used at t = 3 only)
         const u64 z = sf_host_powmod(w, (u64)(R.M / t), q), z2 = sf_host_mulmod(z, z, q);
         P.c3 = sf_host_mulmod((z + q - z2) % q, P.h2, q);
@@ -205,6 +225,21 @@ extern "C" sf_status sf_pp_ring_create(int32_t t, int32_t alpha, int32_t L, int3
                 d[2] = S;
                 d[3] = sf_shoup_companion(S, q);
             }
+    }
+    // constants of the lazy DFTs from C, S (r = 1: c_k, s_k)
+    for (int i = 0; i < L; ++i) {
+        const u64 q = r->q[i];
+        const u64 *cs = &tab[o_dftc + 4 * (size_t)i * H * H];
+        std::vector<u64> v;
+        const auto half = [&](u64 x) { return sf_host_mulmod(x % q, R.mod[i].h2, q); };
+        if (t == 3) v = {q - R.mod[i].h2, R.mod[i].c3};
+        else if (t == 5) v = {half(q - R.mod[i].h2), half(cs[0] + q - cs[4]), cs[6], (cs[2] + q - cs[6]) % q, (2 * q - cs[2] - cs[6]) % q};
+        else
+            for (int k = 0; k < H * H; ++k) v.push_back(cs[4 * k]), v.push_back(cs[4 * k + 2]);
+        for (int k = 0; k < nd; ++k) {
+            tab[o_dftl + 2 * ((size_t)i * nd + k)] = v[k];
+            tab[o_dftl + 2 * ((size_t)i * nd + k) + 1] = sf_shoup_companion(v[k], q);
+        }
     }
     // RNS digits: (Q / q_i) mod q_j and (Q / q_i)^-1 mod q_i
     for (int i = 0; i < L; ++i) {
@@ -237,6 +272,8 @@ extern "C" sf_status sf_pp_ring_create(int32_t t, int32_t alpha, int32_t L, int3
     R.iw_p = R.iw + (size_t)L * R.M;
     R.qhat = R.iw_p + (size_t)L * R.M;
     R.dftc = R.qhat + (size_t)2 * L * L;
+    R.tw = (const pp_pair *)(r->d_tables + o_tw);
+    R.dftl = (const pp_pair *)(r->d_tables + o_dftl);
     *out = r;
     return SF_OK;
 }
@@ -277,8 +314,8 @@ extern "C" sf_status sf_pp_ntt(sf_pp_ring *r, const uint64_t *d_in, uint64_t *d_
     const SfPpRing &R = r->R;
     bool done = false;
     SF_PPT_DISPATCH(R.t, R.alpha, done, {
-        k_ppt_ntt<T, ALPHA><<<dim3(R.L, count), SfPpT<T, ALPHA>::THREADS, 0, (cudaStream_t)stream>>>(R, d_in, d_out,
-                                                                                                    inverse);
+        if (R.lazy) ppt_ntt<T, ALPHA, true>(R, d_in, d_out, count, inverse, (cudaStream_t)stream);
+        else ppt_ntt<T, ALPHA, false>(R, d_in, d_out, count, inverse, (cudaStream_t)stream);
     });
     if (!done)
         k_pp_ntt<<<dim3(R.L, count), SF_PP_THREADS, sizeof(u64) * R.M, (cudaStream_t)stream>>>(R, d_in, d_out, inverse);
@@ -454,22 +491,24 @@ __global__ void k_pp_ksk_finish(SfPpRing R, const u64 *prod, const u64 *e_res, c
 // registers, and the two inverse transforms write the result.  The launches
 // this replaces ran five kernels per ciphertext, each on L^2 blocks or fewer,
 // and transformed the key again for every ciphertext: M = 5^5, 3 limbs, 333
-// ciphertexts took 170 ms.
+// ciphertexts took 171 ms; 0.52 ms fused, 0.27 ms with the lazy transforms.
 
 // coefficient e of tau_h(x) mod Phi_M gathered from x (length N, canonical):
 // x_k sits at k h mod M of the unreduced image, and position e < N receives the
 // image at e minus the image at N + (e mod m); hinv = h^-1 mod M
+// (e, hinv < M <= 4096)
+template <int T, int ALPHA>
 __device__ __forceinline__ u64 pp_auto_at(const u64 *x, int e, const SfPpRing &R, int hinv, u64 q)
 {
-    const int k0 = (int)(((long long)e * hinv) % R.M);
-    const int k1 = (int)(((long long)(R.N + e % R.m) * hinv) % R.M);
-    return sf_sub(k0 < R.N ? x[k0] : 0, k1 < R.N ? x[k1] : 0, q);
+    const unsigned M = pp_len<T, ALPHA>(R), N = pp_deg<T, ALPHA>(R), m = pp_fold<T, ALPHA>(R);
+    const unsigned k0 = (unsigned)e * hinv % M, k1 = (N + e % m) * hinv % M;
+    return sf_sub(k0 < N ? x[k0] : 0, k1 < N ? x[k1] : 0, q);
 }
 
 // The key in the form the key switch reads: polynomial p = 2 i + part (digit
 // i, ka or kb) modulo limb j, transformed: key[p][j][M], then the Shoup
 // companions in the same order.  grid (L, 2 L).
-template <int T, int ALPHA>
+template <int T, int ALPHA, bool LZ>
 __global__ void __launch_bounds__(SfPpShape<T, ALPHA>::NT) k_pp_key_ntt(SfPpRing R, const u64 *ka, const u64 *kb, u64 *key)
 {
     constexpr int NT = SfPpShape<T, ALPHA>::NT;
@@ -477,25 +516,26 @@ __global__ void __launch_bounds__(SfPpShape<T, ALPHA>::NT) k_pp_key_ntt(SfPpRing
     u64 *s = (u64 *)smem_raw;
     const int j = blockIdx.x, p = blockIdx.y, N = R.N;
     const u64 *x = ((p & 1) ? kb : ka) + ((size_t)(p >> 1) * R.L + j) * N;
-    pp_block_forward_ld<T, ALPHA>(s, [x, N](int e) -> u64 { return e < N ? x[e] : 0; }, R, j);
+    pp_block_forward_ld<T, ALPHA, LZ>(s, [x, N](int e) -> u64 { return e < N ? x[e] : 0; }, R, j);
     u64 *dst = key + ((size_t)p * R.L + j) * R.M;
     const size_t comp = (size_t)2 * R.L * R.L * R.M;
     for (int e = threadIdx.x; e < R.M; e += NT) {
-        dst[e] = s[e];
-        dst[comp + e] = pp_companion(s[e], R.mod[j]);
+        const u64 v = LZ ? pp_canon(s[e], R.mod[j]) : s[e];
+        dst[e] = v;
+        dst[comp + e] = pp_companion(v, R.mod[j]);
     }
 }
 
 // out = (-sum_i d_i ka_i, tau_h(b) - sum_i d_i kb_i), d_i = [tau_h(a)_i
 // (Q/q_i)^-1]_{q_i} read as an integer; grid (L, count), key from k_pp_key_ntt.
-template <int T, int ALPHA>
+template <int T, int ALPHA, bool LZ>
 __global__ void __launch_bounds__(SfPpShape<T, ALPHA>::NT, SfPpShape<T, ALPHA>::MINB)
     k_pp_ks(SfPpRing R, const u64 *in, u64 *out, int hinv, const u64 *key)
 {
     constexpr int NT = SfPpShape<T, ALPHA>::NT, EPT = (SfPpShape<T, ALPHA>::MMAX + NT - 1) / NT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     u64 *s = (u64 *)smem_raw;
-    const int j = blockIdx.x, N = R.N, M = R.M, L = R.L;
+    const int j = blockIdx.x, N = pp_deg<T, ALPHA>(R), M = pp_len<T, ALPHA>(R), L = R.L;
     const SfPpMod &P = R.mod[j];
     const size_t per = (size_t)L * N;
     const u64 *a = in + (size_t)blockIdx.y * 2 * per, *b = a + per + (size_t)j * N;
@@ -506,12 +546,12 @@ __global__ void __launch_bounds__(SfPpShape<T, ALPHA>::NT, SfPpShape<T, ALPHA>::
     for (int i = 0; i < L; ++i) {
         const SfPpMod &Pi = R.mod[i];
         const u64 *ai = a + (size_t)i * N;
-        pp_block_forward_ld<T, ALPHA>(
+        pp_block_forward_ld<T, ALPHA, LZ>(
             s,
             [&](int e) -> u64 {
                 if (e >= N) return 0;
-                const u64 d = sf_mul_shoup(pp_auto_at(ai, e, R, hinv, Pi.q), Pi.qh_inv, Pi.qh_inv_p, Pi.q);
-                return i == j ? d : sf_reduce(d, P.q, P.one_p);
+                const u64 d = sf_mul_shoup(pp_auto_at<T, ALPHA>(ai, e, R, hinv, Pi.q), Pi.qh_inv, Pi.qh_inv_p, Pi.q);
+                return i == j ? d : LZ ? pp_canon(d, P) : sf_reduce(d, P.q, P.one_p);
             },
             R, j);
         const u64 *ka = key + ((size_t)(2 * i) * L + j) * M, *kb = key + ((size_t)(2 * i + 1) * L + j) * M;
@@ -519,10 +559,14 @@ __global__ void __launch_bounds__(SfPpShape<T, ALPHA>::NT, SfPpShape<T, ALPHA>::
         for (int x = 0; x < EPT; ++x) {
             const int e = threadIdx.x + x * NT;
             if (e < M) {
-                // canonical sums: L products of up to 61-bit residues leave no lazy room
                 const u64 v = s[e];
-                acc_a[x] = sf_add(acc_a[x], sf_mul_shoup(v, __ldg(ka + e), __ldg(ka + comp + e), P.q), P.q);
-                acc_b[x] = sf_add(acc_b[x], sf_mul_shoup(v, __ldg(kb + e), __ldg(kb + comp + e), P.q), P.q);
+                if constexpr (LZ) {   // L products below 4q
+                    acc_a[x] = pp_mad(acc_a[x], v, make_ulonglong2(__ldg(ka + e), __ldg(ka + comp + e)), P.q);
+                    acc_b[x] = pp_mad(acc_b[x], v, make_ulonglong2(__ldg(kb + e), __ldg(kb + comp + e)), P.q);
+                } else {   // products of up to 61-bit residues leave no lazy room
+                    acc_a[x] = sf_add(acc_a[x], sf_mul_shoup(v, __ldg(ka + e), __ldg(ka + comp + e), P.q), P.q);
+                    acc_b[x] = sf_add(acc_b[x], sf_mul_shoup(v, __ldg(kb + e), __ldg(kb + comp + e), P.q), P.q);
+                }
             }
         }
         __syncthreads();
@@ -531,14 +575,15 @@ __global__ void __launch_bounds__(SfPpShape<T, ALPHA>::NT, SfPpShape<T, ALPHA>::
 #pragma unroll
         for (int x = 0; x < EPT; ++x) {
             const int e = threadIdx.x + x * NT;
-            if (e < M) s[e] = part ? acc_b[x] : acc_a[x];
+            const u64 v = part ? acc_b[x] : acc_a[x];
+            if (e < M) s[e] = LZ ? pp_red3(v, P) : v;
         }
         __syncthreads();
-        pp_block_inverse<T, ALPHA>(s, R, j);
+        pp_block_inverse<T, ALPHA, LZ>(s, R, j);
         u64 *o = out + (size_t)blockIdx.y * 2 * per + (size_t)part * per + (size_t)j * N;
         for (int e = threadIdx.x; e < N; e += NT) {
-            const u64 v = sf_sub(s[e], s[N + e % R.m], P.q);   // the Phi_M fold
-            o[e] = sf_sub(part ? pp_auto_at(b, e, R, hinv, P.q) : 0, v, P.q);
+            const u64 v = sf_sub(s[e], s[N + e % pp_fold<T, ALPHA>(R)], P.q);   // the Phi_M fold
+            o[e] = sf_sub(part ? pp_auto_at<T, ALPHA>(b, e, R, hinv, P.q) : 0, v, P.q);
         }
         __syncthreads();
     }
@@ -633,7 +678,7 @@ static size_t pp_key_words(const SfPpRing &R) { return (size_t)4 * R.L * R.L * R
 static sf_status pp_key_ntt(const SfPpRing &R, const u64 *ka, const u64 *kb, u64 *key, cudaStream_t st)
 {
     SF_PP_DISPATCH_ANY(R, {
-        k_pp_key_ntt<T, ALPHA><<<dim3(R.L, 2 * R.L), SfPpShape<T, ALPHA>::NT, sizeof(u64) * R.M, st>>>(R, ka, kb, key);
+        k_pp_key_ntt<T, ALPHA, LZ><<<dim3(R.L, 2 * R.L), SfPpShape<T, ALPHA>::NT, sizeof(u64) * R.M, st>>>(R, ka, kb, key);
     });
     SF_CUDA_TRY(cudaGetLastError());
     return SF_OK;
@@ -646,7 +691,7 @@ static sf_status pp_keyswitch(const SfPpRing &R, const u64 *in, u64 *out, int co
 {
     const int hinv = pp_inverse_index(((h % R.M) + R.M) % R.M, R.M);
     SF_PP_DISPATCH_ANY(R, {
-        k_pp_ks<T, ALPHA><<<dim3(R.L, count), SfPpShape<T, ALPHA>::NT, sizeof(u64) * R.M, st>>>(R, in, out, hinv, key);
+        k_pp_ks<T, ALPHA, LZ><<<dim3(R.L, count), SfPpShape<T, ALPHA>::NT, sizeof(u64) * R.M, st>>>(R, in, out, hinv, key);
     });
     SF_CUDA_TRY(cudaGetLastError());
     return SF_OK;

@@ -115,14 +115,21 @@ __device__ __forceinline__ u64 tq_crt(u64 x0, u64 x1, const SfPpRing &R, const S
 // coefficient i of tau_h(x) mod Phi_M read from x (length N) by gathering:
 // the unreduced image has x_k at k h mod M, and position i < N receives the
 // image at i minus the image at N + (i mod m); hinv = h^-1 mod M
+// (i, hinv < M <= 4096)
+template <int T, int ALPHA>
 __device__ __forceinline__ u64 tq_auto_at(const u64 *x, int i, const SfPpRing &R, int hinv)
 {
-    const int k0 = (int)(((long long)i * hinv) % R.M);
-    const int k1 = (int)(((long long)(R.N + i % R.m) * hinv) % R.M);
-    const u64 v0 = k0 < R.N ? x[k0] & SF_TQ_MASK : 0;
-    const u64 v1 = k1 < R.N ? x[k1] & SF_TQ_MASK : 0;
+    const unsigned M = pp_len<T, ALPHA>(R), N = pp_deg<T, ALPHA>(R), m = pp_fold<T, ALPHA>(R);
+    const unsigned k0 = (unsigned)i * hinv % M, k1 = (N + i % m) * hinv % M;
+    const u64 v0 = k0 < N ? x[k0] & SF_TQ_MASK : 0;
+    const u64 v1 = k1 < N ? x[k1] & SF_TQ_MASK : 0;
     return (v0 - v1) & SF_TQ_MASK;
 }
+
+// The two primes have 50 bits: compiled rings run the lazy transforms; v as they
+// leave it, made canonical
+template <int T>
+__device__ __forceinline__ u64 tq_canon(u64 v, const SfPpMod &P) { return T ? pp_canon(v, P) : v; }
 
 // ------------------------------------------------------------- kernels ----
 
@@ -144,14 +151,14 @@ __global__ void __launch_bounds__(SfPpShape<T, ALPHA>::NT, SfPpShape<T, ALPHA>::
     extern __shared__ __align__(16) unsigned char smem_raw[];
     u64 *vec = (u64 *)smem_raw;
     u64 *res0 = vec + R.M;                      // [2][N]
-    int16_t *dig = (int16_t *)(res0 + 2 * R.N);  // [l][N]
-    const int M = R.M, N = R.N, m = R.m;
+    const int M = pp_len<T, ALPHA>(R), N = pp_deg<T, ALPHA>(R), m = pp_fold<T, ALPHA>(R);
+    int16_t *dig = (int16_t *)(res0 + 2 * N);   // [l][N]
     const size_t c = blockIdx.x;
     const u64 *a = ct + c * 2 * N, *b = a + N;
     // tau_h(a): permute, then X^(N + e) = -sum_{k < t-1} X^(e + k m)
     for (int e = threadIdx.x; e < M; e += NT) vec[e] = 0;
     __syncthreads();
-    for (int e = threadIdx.x; e < N; e += NT) vec[(int)(((long long)e * h) % M)] = a[e] & SF_TQ_MASK;
+    for (int e = threadIdx.x; e < N; e += NT) vec[(unsigned)e * h % (unsigned)M] = a[e] & SF_TQ_MASK;
     __syncthreads();
     for (int e = threadIdx.x; e < m; e += NT) {
         const u64 v = vec[N + e];
@@ -173,7 +180,7 @@ __global__ void __launch_bounds__(SfPpShape<T, ALPHA>::NT, SfPpShape<T, ALPHA>::
             // digit i lifted mod p_j as the first stage reads it
             const int16_t *di = dig + (size_t)i * N;
             const u64 pq = P.q;
-            pp_block_forward_ld<T, ALPHA>(
+            pp_block_forward_ld<T, ALPHA, (T != 0)>(
                 vec,
                 [di, N, pq](int e) -> u64 {
                     const int d = e < N ? di[e] : 0;
@@ -187,8 +194,8 @@ __global__ void __launch_bounds__(SfPpShape<T, ALPHA>::NT, SfPpShape<T, ALPHA>::
                 const int e = threadIdx.x + x * NT;
                 if (e < M) {
                     const u64 v = vec[e];
-                    acc_a[x] += sf_mul_shoup_lazy(v, __ldg(ka + e), __ldg(ka + kw + e), P.q);
-                    acc_b[x] += sf_mul_shoup_lazy(v, __ldg(kb + e), __ldg(kb + kw + e), P.q);
+                    acc_a[x] = pp_mad(acc_a[x], v, make_ulonglong2(__ldg(ka + e), __ldg(ka + kw + e)), P.q);
+                    acc_b[x] = pp_mad(acc_b[x], v, make_ulonglong2(__ldg(kb + e), __ldg(kb + kw + e)), P.q);
                 }
             }
             __syncthreads();
@@ -197,10 +204,10 @@ __global__ void __launch_bounds__(SfPpShape<T, ALPHA>::NT, SfPpShape<T, ALPHA>::
 #pragma unroll
             for (int x = 0; x < EPT; ++x) {
                 const int e = threadIdx.x + x * NT;
-                if (e < M) vec[e] = sf_reduce(part ? acc_b[x] : acc_a[x], P.q, P.one_p);
+                if (e < M) vec[e] = T ? pp_red3(part ? acc_b[x] : acc_a[x], P) : pp_canon(part ? acc_b[x] : acc_a[x], P);
             }
             __syncthreads();
-            pp_block_inverse<T, ALPHA>(vec, R, j);
+            pp_block_inverse<T, ALPHA, (T != 0)>(vec, R, j);
             for (int e = threadIdx.x; e < m; e += NT) {
                 const u64 v = vec[N + e];
                 for (int k = 0; k < R.t - 1; ++k) vec[e + k * m] = sf_sub(vec[e + k * m], v, P.q);
@@ -212,7 +219,7 @@ __global__ void __launch_bounds__(SfPpShape<T, ALPHA>::NT, SfPpShape<T, ALPHA>::
                 u64 *o = out + c * 2 * N + (size_t)part * N;
                 for (int e = threadIdx.x; e < N; e += NT) {
                     const u64 X = tq_crt(res0[(size_t)part * N + e], vec[e], R, G);
-                    o[e] = ((part ? tq_auto_at(b, e, R, hinv) : 0) - X) & SF_TQ_MASK;
+                    o[e] = ((part ? tq_auto_at<T, ALPHA>(b, e, R, hinv) : 0) - X) & SF_TQ_MASK;
                 }
             }
             __syncthreads();
@@ -233,12 +240,12 @@ __global__ void __launch_bounds__(SfPpShape<T, ALPHA>::NT)
     const u64 *x = a + blockIdx.x * sa;
     for (int j = 0; j < 2; ++j) {
         const SfPpMod &P = R.mod[j];
-        pp_block_forward_ld<T, ALPHA>(
+        pp_block_forward_ld<T, ALPHA, (T != 0)>(
             va, [x, N, &P](int e) -> u64 { return e < N ? sf_reduce(x[e] & SF_TQ_MASK, P.q, P.one_p) : 0; }, R, j);
-        pp_block_forward_ld<T, ALPHA>(vs, [s, N, &P](int e) -> u64 { return e < N ? tq_lift_signed(s[e], P) : 0; }, R, j);
-        for (int e = threadIdx.x; e < M; e += NT) va[e] = pp_mulmod(va[e], vs[e], P);
+        pp_block_forward_ld<T, ALPHA, (T != 0)>(vs, [s, N, &P](int e) -> u64 { return e < N ? tq_lift_signed(s[e], P) : 0; }, R, j);
+        for (int e = threadIdx.x; e < M; e += NT) va[e] = pp_mulmod(tq_canon<T>(va[e], P), tq_canon<T>(vs[e], P), P);
         __syncthreads();
-        pp_block_inverse<T, ALPHA>(va, R, j);
+        pp_block_inverse<T, ALPHA, (T != 0)>(va, R, j);
         for (int e = threadIdx.x; e < m; e += NT) {
             const u64 v = va[N + e];
             for (int k = 0; k < R.t - 1; ++k) va[e + k * m] = sf_sub(va[e + k * m], v, P.q);
@@ -265,13 +272,14 @@ __global__ void __launch_bounds__(SfPpShape<T, ALPHA>::NT)
     const SfPpMod &P = R.mod[j];
     const u64 *x = (part ? kb : ka) + (size_t)i * R.N;
     const int N = R.N;
-    pp_block_forward_ld<T, ALPHA>(
+    pp_block_forward_ld<T, ALPHA, (T != 0)>(
         vec, [x, N, &P](int e) -> u64 { return e < N ? sf_reduce(x[e] & SF_TQ_MASK, P.q, P.one_p) : 0; }, R, j);
     u64 *dst = key + ((size_t)(i * 2 + part) * 2 + j) * R.M;
     const size_t kw = (size_t)4 * l * R.M;
     for (int e = threadIdx.x; e < R.M; e += NT) {
-        dst[e] = vec[e];
-        dst[kw + e] = pp_companion(vec[e], P);
+        const u64 v = tq_canon<T>(vec[e], P);
+        dst[e] = v;
+        dst[kw + e] = pp_companion(v, P);
     }
 }
 
