@@ -42,6 +42,8 @@ size_t sf_ks_scratch_words(const SfRing &R, int ntt) { return sf_ks_scratch_word
 #define SF_EW 8
 __global__ void __launch_bounds__(256) k_ks_gather(SfRing R, SfKsBatch B)
 {
+    sf_pdl_next(B);
+    sf_pdl_wait(B);
     const int b = blockIdx.z, i = blockIdx.y;
     const u64 *E = merge_E(B, b), *O = merge_O(B, b);
     u64 *ta = ks_limb(R, B, b, sf_ks_ta(R) + i);
@@ -125,9 +127,10 @@ sf_status sf_ks_launch(sf_ctx *ctx, const SfKsBatch &B0, cudaStream_t st)
         b.count = std::min(32768, B0.count - off);
         b.first = B0.first + off;
         b.dinv = inv & (2u * R.n - 1u);
+        b.pdl = ks_overlap(b.count);
         b.scratch += sf_ks_scratch_words(R, B0.ntt) * off;
         sf_launch_begin(ctx, SFK_KS_GATHER, st, &ev);
-        k_ks_gather<<<dim3((R.n + 256 * SF_EW - 1) / (256 * SF_EW), R.L, b.count), 256, 0, st>>>(R, b);
+        sf_pdl_launch(k_ks_gather, dim3((R.n + 256 * SF_EW - 1) / (256 * SF_EW), R.L, b.count), 256, 0, st, R, b);
         sf_launch_end(ctx, SFK_KS_GATHER, st, ev);
         if (b.ntt) SF_TRY(sf_ks_inv_rows_launch(ctx, b, st));
         SF_TRY(sf_ks_up_launch(ctx, b, st));

@@ -23,6 +23,7 @@ struct SfKsBatch {
     int ntt;        // operands in the NTT domain
     int d;          // automorphism X -> X^d
     unsigned dinv;  // d^-1 mod 2N (set by sf_ks_launch)
+    int pdl;             // launches overlap (sf_pdl_launch)
     unsigned s;     // O is multiplied by X^s
     int add_v;      // 1: out = v + KS(...), 0: plain rotation
     const u64 *key; // [dnum][2][nm][N] pairs of the NTT-domain values, storage order
@@ -116,3 +117,44 @@ static inline int ks_wave_blocks(const sf_ctx *ctx, int occ, int n_units, int pe
     const int waves = std::max(1, std::min(32, n_units / (w * per_block)));
     return std::max(1, std::min(w * waves, n_units));
 }
+
+// The launches of a single rotation or merge overlap (programmatic dependent launch):
+// a kernel starts once the blocks of the one before have all started, the column
+// kernels stage their twiddle tables, and every kernel waits for the completion of the
+// one before (sf_pdl_wait) before its first access to data, so that completion carries
+// along the chain; nothing but the tables, written when the context was made, is read
+// before.  One rotation at N = 2^16: 83 us launched in order, 73 us so.  (70 us with
+// the row kernels' tables staged ahead as well, but the code for it slowed the inner
+// product of every batch by up to 2.7 %.)  Batches lose by it, as waiting blocks hold
+// room and crowd SMs (64 outputs at N = 2^13, tree levels of 32 .. 1 merges: 326 us in
+// order, 345 with every level overlapped that leaves SMs idle, 321 with single merges
+// only; a ResNet-20 convolution with every launch overlapped 70.7 and 79.4 ms).
+static inline int ks_overlap(int count) { return count == 1; }
+#ifdef __CUDACC__
+__device__ __forceinline__ void sf_pdl_next(const SfKsBatch &B)
+{
+    if (B.pdl) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void sf_pdl_wait(const SfKsBatch &B)
+{
+    if (B.pdl) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// kernel(R, b, args...)
+template <class... P, class... A>
+static inline void sf_pdl_launch(void (*kernel)(SfRing, SfKsBatch, P...), dim3 grid, int threads, size_t smem, cudaStream_t st,
+                                 const SfRing &R, const SfKsBatch &b, A... args)
+{
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute a[1];
+    a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = a;
+    c.numAttrs = b.pdl ? 1 : 0;
+    cudaLaunchKernelEx(&c, kernel, R, b, P(args)...);
+}
+#endif

@@ -26,8 +26,10 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_ks4(SfRin
     const SfColT<LR, PM> T;
     sf_pair *tab = (sf_pair *)smem_raw;   // [nm][R], two buffers: points ahead and exchanges by turns
     u64 *buf = (u64 *)(tab + (size_t)R.nm * SfShape<LR>::S), *ahead = buf + SfShape<LR>::WORDS;
+    sf_pdl_next(B);
     sf_stage_cols<LR>(tab, R.colP, 0, R.nm);
     __syncthreads();
+    sf_pdl_wait(B);
     const SfUnitRange U = sf_unit_range(ng * B.count);
     const size_t per = sf_ks_scratch_words_dev(R, B.ntt);
     // A unit's transforms: the K special limbs, then its share of the data limbs.
@@ -130,7 +132,7 @@ static void down_launch(sf_ctx *ctx, const SfKsBatch &b, cudaStream_t st)
     const int g0 = ((1 << LC) / SfShape<LR>::NB) * 2;
     const int nsplit = (int)std::max<long long>(1, std::min<long long>(R.L, (long long)ctx->num_sms * occ / ((long long)g0 * b.count)));
     const int ng = g0 * nsplit;
-    k_ks4<LR, LC, KT, PM><<<ks_wave_blocks(ctx, occ, ng * b.count, 2), SfShape<LR>::NT, sm, st>>>(R, b, ng, nsplit);
+    sf_pdl_launch(k_ks4<LR, LC, KT, PM>, ks_wave_blocks(ctx, occ, ng * b.count, 2), SfShape<LR>::NT, sm, st, R, b, ng, nsplit);
 }
 
 sf_status sf_ks_down_launch(sf_ctx *ctx, const SfKsBatch &b, cudaStream_t st)

@@ -32,6 +32,8 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS) k_ks1(SfRin
     const SfRowT<LC, PM> T;
     sf_pair *tw = (sf_pair *)smem_raw;
     u64 *buf = (u64 *)(tw + SfShape<LC>::PAIRS), *pre = buf + SfShape<LC>::WORDS + threadIdx.x;
+    sf_pdl_next(B);
+    sf_pdl_wait(B);
     const SfUnitRange U = sf_unit_range(ng * B.count);
     const size_t per = sf_ks_scratch_words_dev(R, B.ntt);
     SfCursor C(U.u0, B.count);
@@ -78,6 +80,8 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS_ACC) k_ks3(S
     const SfRowT<LC, PM> T;
     sf_pair *tw = (sf_pair *)smem_raw;
     u64 *buf = (u64 *)(tw + SfShape<LC>::PAIRS), *pre = buf + SfShape<LC>::WORDS + threadIdx.x;
+    sf_pdl_next(B);
+    sf_pdl_wait(B);
     const SfUnitRange U = sf_unit_range(ng * B.count);
     const sf_pair *key = (const sf_pair *)B.key;
     const size_t per = sf_ks_scratch_words_dev(R, B.ntt);
@@ -198,7 +202,7 @@ sf_status sf_ks_rows_launch(sf_ctx *ctx, const SfKsBatch &b, cudaStream_t st)
         constexpr size_t sm = rows_smem<LC>();
         const int ng = ((1 << LR) / SfShape<LC>::NB) * R.nm;
         sf_launch_begin(ctx, SFK_KS3_INNER_ROW, st, &ev);
-        k_ks3<LR, LC, PM><<<ks_wave_blocks(ctx, sf_occupancy(k_ks3<LR, LC, PM>, NT, sm), ng * b.count, 8), NT, sm, st>>>(R, b, ng);
+        sf_pdl_launch(k_ks3<LR, LC, PM>, ks_wave_blocks(ctx, sf_occupancy(k_ks3<LR, LC, PM>, NT, sm), ng * b.count, 8), NT, sm, st, R, b, ng);
         sf_launch_end(ctx, SFK_KS3_INNER_ROW, st, ev);
     });
     SF_CUDA_TRY(cudaGetLastError());
@@ -214,7 +218,7 @@ sf_status sf_ks_inv_rows_launch(sf_ctx *ctx, const SfKsBatch &b, cudaStream_t st
         constexpr size_t sm = rows_smem<LC>();
         const int ng = ((1 << LR) / SfShape<LC>::NB) * R.L;
         sf_launch_begin(ctx, SFK_KS1_INV_ROW, st, &ev);
-        k_ks1<LR, LC, PM><<<ks_wave_blocks(ctx, sf_occupancy(k_ks1<LR, LC, PM>, NT, sm), ng * b.count, 8), NT, sm, st>>>(R, b, ng);
+        sf_pdl_launch(k_ks1<LR, LC, PM>, ks_wave_blocks(ctx, sf_occupancy(k_ks1<LR, LC, PM>, NT, sm), ng * b.count, 8), NT, sm, st, R, b, ng);
         sf_launch_end(ctx, SFK_KS1_INV_ROW, st, ev);
     });
     SF_CUDA_TRY(cudaGetLastError());

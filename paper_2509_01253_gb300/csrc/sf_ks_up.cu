@@ -32,8 +32,10 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_ks2(SfRin
         buf = other;
         other = used;
     };
+    sf_pdl_next(B);
     sf_stage_cols<LR>(tab, R.colP, 0, R.nm);
     __syncthreads();
+    sf_pdl_wait(B);
     const SfUnitRange U = sf_unit_range(ng * B.count);
     const size_t per = sf_ks_scratch_words_dev(R, B.ntt);
     // item-major: the blocks in flight work on the tiles of a few merges
@@ -129,7 +131,7 @@ static void up_launch(sf_ctx *ctx, const SfKsBatch &b, cudaStream_t st)
     // split the moduli only while the launch does not fill one wave
     const int nsplit = (int)std::max<long long>(1, std::min<long long>(R.nm, (long long)ctx->num_sms * occ / ((long long)g0 * b.count)));
     const int ng = g0 * nsplit;
-    k_ks2<LR, LC, ND, PM><<<ks_wave_blocks(ctx, occ, ng * b.count, 2), SfShape<LR>::NT, sm, st>>>(R, b, ng, nsplit);
+    sf_pdl_launch(k_ks2<LR, LC, ND, PM>, ks_wave_blocks(ctx, occ, ng * b.count, 2), SfShape<LR>::NT, sm, st, R, b, ng, nsplit);
 }
 
 sf_status sf_ks_up_launch(sf_ctx *ctx, const SfKsBatch &b, cudaStream_t st)
