@@ -443,7 +443,7 @@ def ntt_record(sf, torch, wl_, p_info: dict, probe: dict, flush) -> dict:
     hbm_peak, kind = load_peaks()
     gbs = nbytes / (ms * 1e-3) / 1e9
     gmm = bfly / (ms * 1e-3) / 1e9
-    return {"what": f"forward NTT of {count} x {L} limbs of N = {n} (sf_ntt_batch, two persistent passes)",
+    return {"what": f"forward NTT of {count} x {L} limbs of N = {n} (sf_ntt_batch, two passes)",
             "ms_per_call": ms, "algorithmic_bytes": nbytes, "gbs": gbs, "hbm_peak": hbm_peak, "peak_source": kind,
             "frac_hbm": gbs / hbm_peak, "gmodmul_s": gmm, "frac_of_probe": gmm / probe["fwd_bfly"]}
 
