@@ -358,8 +358,10 @@ sf_status sf_linear_outputs(sf_ctx *ctx, const sf_layer *layer, const uint64_t *
 /* Sec. 2.2: for each of `count` ciphertexts, apply X -> X^d to a and b
  * (RLWE under s(X^d)) and key-switch back to s(X) with the hybrid gadget:
  * out = (ModDown(sum_j c_j alpha_j), tau_d(b) + ModDown(sum_j c_j b_j)),
- * c_j = ModUp of digit j of tau_d(a).  d_ct, d_out: uint64[count][2][L][N]
- * (may not overlap).  Errors: SF_EINVAL if rk holds no key for d. */
+ * c_j = ModUp of digit j of tau_d(a).  d_ct, d_out: uint64[count][2][L][N];
+ * they may overlap or be the same buffer, in which case the call works from a
+ * copy of d_ct in the context's workspace.  Errors: SF_EINVAL if rk holds no
+ * key for d. */
 sf_status sf_rotate(sf_ctx *ctx, const sf_rotkeys *rk, int32_t d, const uint64_t *d_ct, uint64_t *d_out,
                     int32_t count, void *stream);
 

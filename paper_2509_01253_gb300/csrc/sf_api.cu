@@ -478,12 +478,17 @@ extern "C" sf_status sf_rotate(sf_ctx *ctx, const sf_rotkeys *rk, int32_t d, con
     cudaStream_t st = (cudaStream_t)stream;
     const size_t ct = ct_words(ctx);
     const int batch = std::min(ctx->ks_batch, count);
+    const bool copy = sf_words_overlap(d_ct, d_out, ct * count);
+    Carver cv;
+    size_t o_ks = cv.take(sf_ks_scratch_words(R, 0) * batch), o_in = cv.take(copy ? ct * count : 0);
     void *w = nullptr;
-    SF_TRY(sf_scratch(ctx, sf_ks_scratch_words(R, 0) * batch * sizeof(u64), &w));
+    SF_TRY(sf_scratch(ctx, cv.words * sizeof(u64), &w));
+    u64 *ws = (u64 *)w;
     SF_TRY(sf_check_residues(ctx, d_ct, count * 2 * R.L, R.L, 0, st));
+    if (copy) SF_CUDA_TRY(cudaMemcpyAsync(ws + o_in, d_ct, sizeof(u64) * ct * count, cudaMemcpyDeviceToDevice, st));
     SfKsBatch b;
     memset(&b, 0, sizeof(b));
-    b.E = d_ct;
+    b.E = copy ? ws + o_in : d_ct;
     b.E_stride = ct;
     b.out = d_out;
     b.out_stride = ct;
@@ -492,7 +497,7 @@ extern "C" sf_status sf_rotate(sf_ctx *ctx, const sf_rotkeys *rk, int32_t d, con
     b.d = d;
     b.add_v = 0;
     b.key = rk->d_keys + rk->key_words * t;
-    return sf_ks_run(ctx, b, (u64 *)w, batch, st);
+    return sf_ks_run(ctx, b, ws + o_ks, batch, st);
 }
 
 static sf_status pack_impl(sf_ctx *ctx, const sf_rotkeys *rk, const uint64_t *d_leaves, int32_t n_leaves, int32_t n,

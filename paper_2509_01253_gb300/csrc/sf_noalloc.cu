@@ -71,10 +71,15 @@ extern "C" sf_status sf_rotate_noalloc(sf_ctx *ctx, const sf_rotkeys *rk, int32_
     const int timing = ctx->kernel_timing;
     ctx->kernel_timing = 0;
     sf_status s = SF_OK;
-    {
+    // the workspaces of one launch batch, then room for a copy of the input
+    const bool copy = sf_words_overlap(d_ct, d_out, ct * count);
+    u64 *in = ws + round_words(sf_ks_scratch_words(R, 0) * batch);
+    if (copy && cudaMemcpyAsync(in, d_ct, sizeof(u64) * ct * count, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+        s = sf_set_error(SF_ECUDA, "sf_rotate_noalloc: copying the input failed: %s", cudaGetErrorString(cudaGetLastError()));
+    if (s == SF_OK) {
         SfKsBatch b;
         memset(&b, 0, sizeof(b));
-        b.E = d_ct;
+        b.E = copy ? in : d_ct;
         b.E_stride = ct;
         b.out = d_out;
         b.out_stride = ct;
