@@ -369,7 +369,8 @@ sf_status sf_rotate(sf_ctx *ctx, const sf_rotkeys *rk, int32_t d, const uint64_t
  * (zero-padded to n, a power of two with n_leaves <= n <= N/2) into one
  * ciphertext whose coefficient l*N/n is N times coefficient 0 of leaf l; all
  * other coefficients are cleared by the field trace.  Uses (n - 1) + log2(N/n)
- * key switches.  d_leaves: uint64[n_leaves][2][L][N]; d_out: uint64[2][L][N]. */
+ * key switches.  d_leaves: uint64[n_leaves][2][L][N] (residues modulo q_i, any
+ * representative below 2^64); d_out: uint64[2][L][N]. */
 sf_status sf_pack(sf_ctx *ctx, const sf_rotkeys *rk, const uint64_t *d_leaves, int32_t n_leaves, int32_t n,
                   uint64_t *d_out, void *stream);
 
@@ -426,7 +427,9 @@ sf_status sf_shuffle_cts(sf_ctx *ctx, const uint32_t *h_perm, const uint64_t *d_
  *    (different streams, or other threads) race and corrupt each other's
  *    results; issue them on one stream or wait in between.  Each call writes
  *    every scratch word before reading it, so nothing needs to start at zero.
- * Arguments, layout and results are those of sf_rotate (bit-identical). */
+ * Arguments, layout and results are those of sf_rotate (bit-identical); the
+ * residues are not checked: any representative below 2^64 stands for its
+ * residue. */
 sf_status sf_rotate_noalloc(sf_ctx *ctx, const sf_rotkeys *rk, int32_t d, const uint64_t *d_ct, uint64_t *d_out,
                             int32_t count, void *stream);
 

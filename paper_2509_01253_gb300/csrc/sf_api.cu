@@ -517,8 +517,9 @@ static sf_status pack_impl(sf_ctx *ctx, const sf_rotkeys *rk, const uint64_t *d_
     void *w = nullptr;
     SF_TRY(sf_scratch(ctx, cv.words * sizeof(u64), &w));
     u64 *ws = (u64 *)w;
-    // the levels write back into the leaves' buffer: work on a copy of the caller's
-    SF_CUDA_TRY(cudaMemcpyAsync(ws + o_A, d_leaves, sizeof(u64) * ct * n_leaves, cudaMemcpyDeviceToDevice, st));
+    // the levels write back into the leaves' buffer, and merge canonical residues: work
+    // on a canonical copy of the caller's
+    SF_TRY(sf_canonical_copy(ctx, d_leaves, ws + o_A, n_leaves * 2 * R.L, R.L, 0, st));
     bool ntt = false;
     std::vector<int> valid(1, n_leaves);
     u64 *res = nullptr;

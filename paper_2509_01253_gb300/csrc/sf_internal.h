@@ -236,6 +236,8 @@ sf_status sf_rotkey_finish(sf_ctx *ctx, const u64 *alpha, const u64 *e, const u6
 // device-side range check of caller input: latches SF_ERANGE in the status
 // word (reported by sf_sync) if a residue of poly t is >= modulus offset + t % period
 sf_status sf_check_residues(sf_ctx *ctx, const u64 *x, int n_polys, int period, int offset, cudaStream_t st);
+// dst = x with every residue brought to [0, q) (poly t uses modulus offset + t % period)
+sf_status sf_canonical_copy(sf_ctx *ctx, const u64 *x, u64 *dst, int n_polys, int period, int offset, cudaStream_t st);
 // NTT-domain residues -> pairs in storage order (poly t uses modulus offset + t % period)
 sf_status sf_to_pairs(sf_ctx *ctx, const u64 *x, ulonglong2 *dst, int n_polys, int period, int offset, cudaStream_t st);
 // storage order -> natural slot order: plain words (step 1) or the values of pairs (step 2)

@@ -64,6 +64,10 @@ __global__ void __launch_bounds__(256) k_ks_gather(SfRing R, SfKsBatch B)
             // p receives index e = p d^-1 mod 2N of u, negated when e >= N
             const unsigned e = (p * B.dinv) & (2 * n - 1), src = e & mask;
             u64 ua = Ea[src], ub = Eb[src], va = 0, vb = 0;
+            if (B.unreduced) {
+                ua = sf_reduce(ua, q, M.one_p);
+                ub = sf_reduce(ub, q, M.one_p);
+            }
             if (B.add_v) {
                 va = Ea[p];
                 vb = Eb[p];

@@ -21,6 +21,7 @@ struct SfKsBatch {
     int inner;
     int count;
     int ntt;        // operands in the NTT domain
+    int unreduced;  // plain rotation of residues that nothing has checked: brought to [0, q) as they are read
     int d;          // automorphism X -> X^d
     unsigned dinv;  // d^-1 mod 2N (set by sf_ks_launch)
     int pdl;             // launches overlap (sf_pdl_launch)

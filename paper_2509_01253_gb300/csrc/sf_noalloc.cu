@@ -87,6 +87,7 @@ extern "C" sf_status sf_rotate_noalloc(sf_ctx *ctx, const sf_rotkeys *rk, int32_
         b.count = count;
         b.d = d;
         b.add_v = 0;
+        b.unreduced = 1;   // no sf_check_residues here
         b.key = rk->d_keys + rk->key_words * slot;
         s = sf_ks_run(ctx, b, ws, batch, st);
     }

@@ -329,6 +329,22 @@ sf_status sf_check_residues(sf_ctx *ctx, const u64 *x, int n_polys, int period, 
     return SF_OK;
 }
 
+// copy of caller polynomials whose residues nothing has checked, made canonical
+__global__ void k_canonical_copy(SfRing R, const u64 *x, u64 *dst, int n_polys, int period, int offset)
+{
+    SF_GRID_STRIDE(i, (size_t)n_polys * R.n)
+    {
+        const SfMod &M = R.m[offset + (int)((i >> R.log_n) % period)];
+        dst[i] = sf_reduce(x[i], M.q, M.one_p);
+    }
+}
+
+sf_status sf_canonical_copy(sf_ctx *ctx, const u64 *x, u64 *dst, int n_polys, int period, int offset, cudaStream_t st)
+{
+    SF_ELEM_LAUNCH(k_canonical_copy, (size_t)n_polys * ctx->ring.n, x, dst, n_polys, period, offset);
+    return SF_OK;
+}
+
 sf_status sf_to_pairs(sf_ctx *ctx, const u64 *x, ulonglong2 *dst, int n_polys, int period, int offset, cudaStream_t st)
 {
     SF_ELEM_LAUNCH(k_to_pairs, (size_t)n_polys * ctx->ring.n, x, dst, n_polys, period, offset);
