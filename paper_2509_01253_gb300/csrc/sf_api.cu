@@ -429,9 +429,9 @@ extern "C" sf_status sf_linear_outputs(sf_ctx *ctx, const sf_layer *L, const uin
     const int LB = std::min(leaf_batch_slots(R, k_in, L->max_taps), n_outputs);
     Carver cv;
     size_t o_ct = cv.take((size_t)2 * k_in * ct), o_pos = cv.take(((size_t)L->E_in + 1) / 2),
-           o_sig = cv.take(((size_t)n_outputs + 1) / 2), o_w1 = cv.take((size_t)LB * k_in * R.L * R.n),
-           o_in = cv.take((size_t)k_in * ct), o_lv = cv.take((size_t)n_outputs * ct), o_nat = cv.take((size_t)n_outputs * ct),
-           o_tap = cv.take(sf_leaf_tap_words(R, k_in, L->max_taps, LB));
+           o_sig = cv.take(((size_t)n_outputs + 1) / 2),
+           o_w1 = cv.take(std::max((size_t)LB * k_in * R.L * R.n, (size_t)k_in * ct)),   // also the inputs' transforms
+           o_lv = cv.take((size_t)n_outputs * ct), o_tap = cv.take(sf_leaf_tap_words(R, k_in, L->max_taps, LB));
     void *w = nullptr;
     SF_TRY(sf_scratch(ctx, cv.words * sizeof(u64), &w));
     u64 *ws = (u64 *)w;
@@ -439,7 +439,7 @@ extern "C" sf_status sf_linear_outputs(sf_ctx *ctx, const sf_layer *L, const uin
     std::vector<int> h_pos, h_sig(h_outputs, h_outputs + n_outputs);
     if (h_sigma_prev) SF_TRY(upload_perm_inverse(h_sigma_prev, L->E_in, d_pos, h_pos, st));
     SF_CUDA_TRY(cudaMemcpyAsync(d_sig, h_sig.data(), sizeof(int) * n_outputs, cudaMemcpyHostToDevice, st));
-    SF_TRY(prepare_inputs(ctx, d_in, nullptr, k_in, ws + o_ct, ws + o_in, st));
+    SF_TRY(prepare_inputs(ctx, d_in, nullptr, k_in, ws + o_ct, ws + o_w1, st));
     SfLeafParams P = leaf_params(L);
     P.k_in = k_in;
     P.pos_of = h_sigma_prev ? d_pos : nullptr;
@@ -456,10 +456,11 @@ extern "C" sf_status sf_linear_outputs(sf_ctx *ctx, const sf_layer *L, const uin
         p.leaves = ws + o_lv + (size_t)s0 * ct;
         SF_TRY(sf_leaves_launch(ctx, p, std::min(LB, n_outputs - s0), st));
     }
-    SF_TRY(sf_to_natural(ctx, ws + o_lv, 1, ws + o_nat, n_outputs * 2 * R.L, st));
+    // natural order in the caller's buffer, transformed there
+    SF_TRY(sf_to_natural(ctx, ws + o_lv, 1, d_out, n_outputs * 2 * R.L, st));
     std::vector<SfPolyJob> jobs;
     for (int x = 0; x < n_outputs * 2 * R.L; ++x)
-        jobs.push_back({ws + o_nat + (size_t)x * R.n, d_out + (size_t)x * R.n, x % R.L});
+        jobs.push_back({d_out + (size_t)x * R.n, d_out + (size_t)x * R.n, x % R.L});
     SF_TRY(sf_ntt_jobs(ctx, jobs.data(), (int)jobs.size(), true, st));
     SF_CUDA_TRY(cudaStreamSynchronize(st));
     return SF_OK;
