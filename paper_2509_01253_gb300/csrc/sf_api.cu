@@ -188,7 +188,8 @@ extern "C" sf_status sf_rotkeys_export(sf_ctx *ctx, const sf_rotkeys *rk, int32_
         u64 pm = R.n % p->mods[m];
         for (int k = 0; k < R.K; ++k) pm = sf_host_mulmod(pm, p->mods[R.L + k] % p->mods[m], p->mods[m]);
         u64 *row = h_key + (size_t)x * R.n;
-        for (int k = 0; k < R.n; ++k) row[k] = sf_host_mulmod(row[k], pm, p->mods[m]);
+        const u64 pm_p = sf_shoup_companion(pm, p->mods[m]);
+        for (int k = 0; k < R.n; ++k) row[k] = sf_mul_shoup(row[k], pm, pm_p, p->mods[m]);
     }
     return SF_OK;
 }
