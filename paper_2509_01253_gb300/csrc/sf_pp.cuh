@@ -167,6 +167,7 @@ struct SfPpT {
                            : T == 5 ? (ALPHA == 2 ? 25 : ALPHA == 3 ? 125 : ALPHA == 4 ? 625 : 3125)
                                     : (ALPHA == 2 ? 49 : ALPHA == 3 ? 343 : 2401);
     static constexpr int THREADS = ppt_threads(T, M);
+    static constexpr int WIDE = (M / T + 31) / 32 * 32;   // k_ppt_ntt_wide: one butterfly a thread and stage
 };
 
 // the 3-point DFT with two products: with zeta + zeta^2 = -1,
@@ -221,16 +222,16 @@ __device__ __forceinline__ void ppt_dft_pairs(u64 *x, const u64 *dc, u64 q, u64 
     for (int k = 0; k < T; ++k) x[k] = y[k];
 }
 
-// one forward stage reading its inputs through ld(index) (the block's vector
+// NT: the block's threads.  One forward stage reading its inputs through ld(index) (the block's vector
 // itself, or a producer for the first stage) and writing them to s
-template <int T, int M, int LEN, class LD>
+template <int T, int M, int LEN, int NT, class LD>
 __device__ __forceinline__ void ppt_stage_fwd_ld(u64 *s, LD ld, const u64 *w, const u64 *wp, const u64 *dc, u64 q,
                                                  u64 one_p, const SfPpMod &P)
 {
     static_assert(T >= 3 && (T & 1), "compiled rings have an odd prime t");
     constexpr int THIRD = LEN / T, STRIDE = M / LEN;
 #pragma unroll 1
-    for (int g0 = 0; g0 < M / T; g0 += ppt_threads(T, M)) {
+    for (int g0 = 0; g0 < M / T; g0 += NT) {
         const int idx = g0 + threadIdx.x;
         if (idx >= M / T) break;
         const int blk = idx / THIRD, j = idx - blk * THIRD;
@@ -256,21 +257,21 @@ __device__ __forceinline__ void ppt_stage_fwd_ld(u64 *s, LD ld, const u64 *w, co
     }
 }
 
-template <int T, int M, int LEN>
+template <int T, int M, int LEN, int NT>
 __device__ __forceinline__ void ppt_stage_fwd(u64 *s, const u64 *w, const u64 *wp, const u64 *dc, u64 q, u64 one_p,
                                               const SfPpMod &P)
 {
-    ppt_stage_fwd_ld<T, M, LEN>(s, [s](int i) { return s[i]; }, w, wp, dc, q, one_p, P);
+    ppt_stage_fwd_ld<T, M, LEN, NT>(s, [s](int i) { return s[i]; }, w, wp, dc, q, one_p, P);
 }
 
-template <int T, int M, int LEN>
+template <int T, int M, int LEN, int NT>
 __device__ __forceinline__ void ppt_stage_inv(u64 *s, const u64 *iw, const u64 *iwp, const u64 *dc, u64 q, u64 one_p,
                                               const SfPpMod &P)
 {
     static_assert(T >= 3 && (T & 1), "compiled rings have an odd prime t");
     constexpr int THIRD = LEN / T, STRIDE = M / LEN;
 #pragma unroll 1
-    for (int g0 = 0; g0 < M / T; g0 += ppt_threads(T, M)) {
+    for (int g0 = 0; g0 < M / T; g0 += NT) {
         const int idx = g0 + threadIdx.x;
         if (idx >= M / T) break;
         const int blk = idx / THIRD, j = idx - blk * THIRD;
@@ -294,33 +295,33 @@ __device__ __forceinline__ void ppt_stage_inv(u64 *s, const u64 *iw, const u64 *
     }
 }
 
-template <int T, int M, int LEN>
+template <int T, int M, int LEN, int NT>
 __device__ __forceinline__ void ppt_forward(u64 *s, const u64 *w, const u64 *wp, const u64 *dc, u64 q, u64 one_p,
                                             const SfPpMod &P)
 {
-    ppt_stage_fwd<T, M, LEN>(s, w, wp, dc, q, one_p, P);
+    ppt_stage_fwd<T, M, LEN, NT>(s, w, wp, dc, q, one_p, P);
     __syncthreads();
-    if constexpr (LEN / T >= T) ppt_forward<T, M, LEN / T>(s, w, wp, dc, q, one_p, P);
+    if constexpr (LEN / T >= T) ppt_forward<T, M, LEN / T, NT>(s, w, wp, dc, q, one_p, P);
 }
 
 // the whole forward transform with the first stage's inputs read through
 // ld(index), index < M (each read once), e.g. straight from global memory
-template <int T, int M, class LD>
+template <int T, int M, int NT, class LD>
 __device__ __forceinline__ void ppt_forward_ld(u64 *s, LD ld, const u64 *w, const u64 *wp, const u64 *dc, u64 q,
                                                u64 one_p, const SfPpMod &P)
 {
-    ppt_stage_fwd_ld<T, M, M>(s, ld, w, wp, dc, q, one_p, P);
+    ppt_stage_fwd_ld<T, M, M, NT>(s, ld, w, wp, dc, q, one_p, P);
     __syncthreads();
-    if constexpr (M / T >= T) ppt_forward<T, M, M / T>(s, w, wp, dc, q, one_p, P);
+    if constexpr (M / T >= T) ppt_forward<T, M, M / T, NT>(s, w, wp, dc, q, one_p, P);
 }
 
-template <int T, int M, int LEN>
+template <int T, int M, int LEN, int NT>
 __device__ __forceinline__ void ppt_inverse(u64 *s, const u64 *iw, const u64 *iwp, const u64 *dc, u64 q, u64 one_p,
                                             const SfPpMod &P)
 {
-    ppt_stage_inv<T, M, LEN>(s, iw, iwp, dc, q, one_p, P);
+    ppt_stage_inv<T, M, LEN, NT>(s, iw, iwp, dc, q, one_p, P);
     __syncthreads();
-    if constexpr (LEN * T <= M) ppt_inverse<T, M, LEN * T>(s, iw, iwp, dc, q, one_p, P);
+    if constexpr (LEN * T <= M) ppt_inverse<T, M, LEN * T, NT>(s, iw, iwp, dc, q, one_p, P);
 }
 
 // ---- lazy stages --------------------------------------------------------------
@@ -553,7 +554,7 @@ __device__ __forceinline__ void pp_block_forward_ld(u64 *s, LD ld, const SfPpRin
     } else {
         constexpr int M = SfPpT<T, ALPHA>::M, H = (T - 1) / 2;
         const SfPpMod &P = R.mod[j];
-        ppt_forward_ld<T, M>(s, ld, R.w + (size_t)j * M, R.w_p + (size_t)j * M, R.dftc + (size_t)j * H * H * 4, P.q,
+        ppt_forward_ld<T, M, SfPpT<T, ALPHA>::THREADS>(s, ld, R.w + (size_t)j * M, R.w_p + (size_t)j * M, R.dftc + (size_t)j * H * H * 4, P.q,
                              P.one_p, P);
     }
 }
@@ -572,7 +573,7 @@ __device__ __forceinline__ void pp_block_inverse(u64 *s, const SfPpRing &R, int 
     } else {
         constexpr int M = SfPpT<T, ALPHA>::M, H = (T - 1) / 2, NT = SfPpT<T, ALPHA>::THREADS;
         const SfPpMod &P = R.mod[j];
-        ppt_inverse<T, M, T>(s, R.iw + (size_t)j * M, R.iw_p + (size_t)j * M, R.dftc + (size_t)j * H * H * 4, P.q,
+        ppt_inverse<T, M, T, NT>(s, R.iw + (size_t)j * M, R.iw_p + (size_t)j * M, R.dftc + (size_t)j * H * H * 4, P.q,
                              P.one_p, P);
         for (int e = threadIdx.x; e < M; e += NT) s[e] = sf_mul_shoup(s[e], P.minv, P.minv_p, P.q);
         __syncthreads();
