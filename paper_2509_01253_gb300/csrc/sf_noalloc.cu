@@ -56,14 +56,18 @@ extern "C" sf_status sf_rotate_noalloc(sf_ctx *ctx, const sf_rotkeys *rk, int32_
     const size_t ct = (size_t)2 * R.L * R.n;
     // key switches run in launch batches of the context's size, as in sf_rotate
     const int batch = std::min(ctx->ks_batch, (int)count);
-    // the documented limit: two ciphertexts and this many key-switch limbs per
-    // call (the key switch itself uses less)
+    // what the call uses: the workspaces of one launch batch, then room for a copy of
+    // the input (buffers that share words)
+    const size_t ks_words = round_words(sf_ks_scratch_words(R, 0) * batch), used = ks_words + round_words((size_t)count * ct);
+    // the documented limit, which stays as it is: two ciphertexts and this many
+    // key-switch limbs per call
     const size_t limbs = R.L + std::max(R.L, 2 * R.K) + std::max(R.dnum * R.nm, 2 * R.L) + 2 * R.L;
-    const size_t need = 2 * round_words((size_t)count * ct) + round_words((limbs << R.log_n) * batch);
-    if (need > SF_NOALLOC_SCRATCH_WORDS)
+    const size_t limit = 2 * round_words((size_t)count * ct) + round_words((limbs << R.log_n) * batch);
+    if (std::max(used, limit) > SF_NOALLOC_SCRATCH_WORDS)
         return sf_set_error(SF_EINVAL,
-                            "sf_rotate_noalloc: %d ciphertexts need %zu bytes of scratch, the fixed maximum is %zu bytes",
-                            count, need * sizeof(u64), SF_NOALLOC_SCRATCH_WORDS * sizeof(u64));
+                            "sf_rotate_noalloc: %d ciphertexts are beyond the documented limit: two ciphertexts each and their "
+                            "key-switch workspaces are %zu bytes, the fixed maximum is %zu bytes",
+                            count, std::max(used, limit) * sizeof(u64), SF_NOALLOC_SCRATCH_WORDS * sizeof(u64));
     u64 *ws = nullptr;
     SF_TRY(noalloc_scratch(ctx->device, &ws));
     cudaStream_t st = (cudaStream_t)stream;
@@ -71,9 +75,8 @@ extern "C" sf_status sf_rotate_noalloc(sf_ctx *ctx, const sf_rotkeys *rk, int32_
     const int timing = ctx->kernel_timing;
     ctx->kernel_timing = 0;
     sf_status s = SF_OK;
-    // the workspaces of one launch batch, then room for a copy of the input
     const bool copy = sf_words_overlap(d_ct, d_out, ct * count);
-    u64 *in = ws + round_words(sf_ks_scratch_words(R, 0) * batch);
+    u64 *in = ws + ks_words;
     if (copy && cudaMemcpyAsync(in, d_ct, sizeof(u64) * ct * count, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
         s = sf_set_error(SF_ECUDA, "sf_rotate_noalloc: copying the input failed: %s", cudaGetErrorString(cudaGetLastError()));
     if (s == SF_OK) {
