@@ -530,7 +530,7 @@ sf_status sf_pp_decrypt(sf_pp_ring *ring, const int64_t *d_s, const uint64_t *d_
  * d_e int64[L][N], d_kb[i] = ka_i s + e_i + (Q/q_i) tau_h(s) (mod Q).
  * sf_pp_keyswitch: d_out[c] = (-sum_i d_i ka_i, tau_h(b) - sum_i d_i kb_i),
  * which decrypts under s to tau_h(m + e) - sum_i d_i e_i; d_out must not
- * alias d_ct. */
+ * equal d_ct (a shifted overlap is served from a copy of d_ct). */
 sf_status sf_pp_ksk(sf_pp_ring *ring, const int64_t *d_s, int32_t h, const uint64_t *d_ka, const int64_t *d_e,
                     uint64_t *d_kb, void *stream);
 sf_status sf_pp_keyswitch(sf_pp_ring *ring, const uint64_t *d_ct, uint64_t *d_out, int32_t count, int32_t h,

@@ -162,6 +162,13 @@ sf_status sf_set_error(sf_status st, const char *fmt, ...);
 
 // --------------------------------------------------------- host utilities --
 
+// Key switches read an input at permuted positions while other threads write the
+// output: a call whose buffers share words works from a copy of its input.
+static inline bool sf_words_overlap(const u64 *a, const u64 *b, size_t words)
+{
+    const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b, n = words * sizeof(u64);
+    return x < y + n && y < x + n;
+}
 u64 sf_host_powmod(u64 a, u64 e, u64 q);
 u64 sf_host_invmod(u64 a, u64 q);
 u64 sf_host_mulmod(u64 a, u64 b, u64 q);

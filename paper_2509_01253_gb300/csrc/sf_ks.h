@@ -50,14 +50,6 @@ sf_status sf_ks_launch(sf_ctx *ctx, const SfKsBatch &B, cudaStream_t st);
 // (batch * sf_ks_scratch_words words).
 sf_status sf_ks_run(sf_ctx *ctx, SfKsBatch B, u64 *scratch, int batch, cudaStream_t st);
 
-// The gather reads E at permuted positions while other threads write `out`, so a
-// call whose buffers share words key-switches from a copy of its input.
-static inline bool sf_words_overlap(const u64 *a, const u64 *b, size_t words)
-{
-    const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b, n = words * sizeof(u64);
-    return x < y + n && y < x + n;
-}
-
 // The kernels of one launch sequence, each in its own translation unit:
 // ModUp columns (sf_ks_up.cu), rows with the inner product (sf_ks_rows.cu),
 // ModDown columns (sf_ks_down.cu).

@@ -744,10 +744,15 @@ extern "C" sf_status sf_pp_keyswitch(sf_pp_ring *r, const uint64_t *d_ct, uint64
     const SfPpRing &R = r->R;
     if (h % R.t == 0) return sf_set_error(SF_EINVAL, "automorphism index %d not coprime to M = %d", h, R.M);
     cudaStream_t st = (cudaStream_t)stream;
+    // blocks read whole ciphertexts while others write theirs: an output that shares
+    // words with the input is written from a copy of it, kept behind the key
+    const size_t words = (size_t)count * 2 * R.L * R.N, key_words = pp_key_words(R);
+    const bool copy = sf_words_overlap(d_ct, d_out, words);
     u64 *key;
-    SF_TRY(pp_ks_buffer(r, pp_key_words(R), &key));
+    SF_TRY(pp_ks_buffer(r, key_words + (copy ? words : 0), &key));
     SF_TRY(pp_key_ntt(R, d_ka, d_kb, key, st));
-    return pp_keyswitch(R, d_ct, d_out, count, h, key, st);
+    if (copy) SF_CUDA_TRY(cudaMemcpyAsync(key + key_words, d_ct, sizeof(u64) * words, cudaMemcpyDeviceToDevice, st));
+    return pp_keyswitch(R, copy ? key + key_words : d_ct, d_out, count, h, key, st);
 }
 
 extern "C" sf_status sf_pp_hom_trace(sf_pp_ring *r, const uint64_t *d_ct, uint64_t *d_out, int32_t count,
