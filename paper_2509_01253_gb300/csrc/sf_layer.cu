@@ -23,7 +23,6 @@
 
 __device__ __forceinline__ int leaf_output(const SfLeafParams &P, int slot)
 {
-    if (slot >= P.n_slots_valid) return -1;
     return P.sig_out ? P.sig_out[slot] : slot;
 }
 
@@ -80,7 +79,6 @@ __global__ void __launch_bounds__(256) k_leaf_prep(SfRing R, SfLeafParams P)
     __shared__ int cnt[SF_MAX_BUCKETS + 1];
     const int z = blockIdx.x;
     const int o = leaf_output(P, P.s0 + z * P.s_stride);
-    if (o < 0) return;   // leaf_col skips this slot as well
     const int nb = P.n_buckets, tiles = sf_leaf_tiles(R), wl = sf_leaf_width_log(R);
     int *off = P.tap_off + (size_t)z * (nb + 1);
     for (int b = threadIdx.x; b <= nb; b += blockDim.x) cnt[b] = 0;
@@ -124,7 +122,6 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_leaf_col(
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SfColT<LR, PM> T;
     const int j = blockIdx.y / R.L, i = blockIdx.y % R.L;
-    if (leaf_output(P, P.s0 + blockIdx.z * P.s_stride) < 0) return;
     const SfMod &M = R.m[i];
     sf_pair *tab = (sf_pair *)smem_raw;
     u64 *tile = (u64 *)(tab + SfShape<LR>::S);
@@ -246,6 +243,7 @@ sf_status sf_leaves_launch(sf_ctx *ctx, const SfLeafParams &P, int cnt, cudaStre
 {
     const SfRing &R = ctx->ring;
     if (cnt <= 0) return SF_OK;
+    if (P.s0 + (cnt - 1) * P.s_stride >= P.n_slots_valid) return sf_set_error(SF_EINVAL, "leaf slot without an output");
     cudaEvent_t ev;
     for (int off = 0; off < cnt; off += 65535) {
         SfLeafParams p = P;

@@ -9,7 +9,8 @@ struct SfTermDev {
 };
 
 // Launch slot z computes slot s = s0 + z * s_stride, i.e. output sig_out[s]
-// (or s when sig_out is null); slots >= n_slots_valid are zero padding leaves.
+// (or s when sig_out is null).  Every launched slot is below n_slots_valid
+// (sf_leaves_launch refuses others): padding leaves are neither computed nor read.
 struct SfLeafParams {
     SfTermDev t[2];
     int n_terms;
