@@ -482,7 +482,7 @@ extern "C" sf_status sf_rotate(sf_ctx *ctx, const sf_rotkeys *rk, int32_t d, con
     const int batch = std::min(ctx->ks_batch, count);
     const bool copy = sf_words_overlap(d_ct, d_out, ct * count);
     Carver cv;
-    size_t o_ks = cv.take(sf_ks_scratch_words(R, 0) * batch), o_in = cv.take(copy ? ct * count : 0);
+    size_t o_ks = cv.take(sf_ks_scratch_words(R) * batch), o_in = cv.take(copy ? ct * count : 0);
     void *w = nullptr;
     SF_TRY(sf_scratch(ctx, cv.words * sizeof(u64), &w));
     u64 *ws = (u64 *)w;
@@ -515,7 +515,7 @@ static sf_status pack_impl(sf_ctx *ctx, const sf_rotkeys *rk, const uint64_t *d_
     const int batch = std::min(ctx->ks_batch, std::max(1, n / 2));   // the widest level has n/2 merges
     Carver cv;
     size_t o_A = cv.take((size_t)n * ct), o_B = cv.take((size_t)std::max(n / 2, 1) * ct),
-           o_ks = cv.take(sf_ks_scratch_words(R, 0) * batch);
+           o_ks = cv.take(sf_ks_scratch_words(R) * batch);
     void *w = nullptr;
     SF_TRY(sf_scratch(ctx, cv.words * sizeof(u64), &w));
     u64 *ws = (u64 *)w;

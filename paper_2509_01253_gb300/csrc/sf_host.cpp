@@ -518,7 +518,7 @@ extern "C" sf_status sf_ctx_create(const sf_params *p, int32_t device, sf_ctx **
     ctx->io_buf = nullptr;
     ctx->io_bytes = 0;
     // merges per key-switch launch (the autotuner's pick on the benchmark rounds);
-    // the scratch is ks_batch x ((dnum + 2)(L + K) + 2L) limbs
+    // the scratch is ks_batch x ((dnum + 2)(L + K) + L) limbs
     ctx->ks_batch = p->log_n >= 16 ? 256 : 512;
     ctx->leaf_chunk = 1 << 30;
     ctx->leaf_sparse = 0;

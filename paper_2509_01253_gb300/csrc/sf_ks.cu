@@ -26,8 +26,6 @@
 #include "sf_kernels.cuh"
 #include "sf_reg.cuh"
 
-size_t sf_ks_scratch_words(const SfRing &R, int ntt) { return sf_ks_scratch_words_dev(R, ntt); }
-
 // Elementwise, one pass over E and O per merge:
 //   TA[i][p] = tau_d(u.a)[p],  u = E - X^s O
 //   out.a[p] = v.a[p]                      (0 for a plain rotation)
@@ -132,7 +130,7 @@ sf_status sf_ks_launch(sf_ctx *ctx, const SfKsBatch &B0, cudaStream_t st)
         b.first = B0.first + off;
         b.dinv = inv & (2u * R.n - 1u);
         b.pdl = ks_overlap(b.count);
-        b.scratch += sf_ks_scratch_words(R, B0.ntt) * off;
+        b.scratch += sf_ks_scratch_words(R) * off;
         sf_launch_begin(ctx, SFK_KS_GATHER, st, &ev);
         sf_pdl_launch(k_ks_gather, dim3((R.n + 256 * SF_EW - 1) / (256 * SF_EW), R.L, b.count), 256, 0, st, R, b);
         sf_launch_end(ctx, SFK_KS_GATHER, st, ev);

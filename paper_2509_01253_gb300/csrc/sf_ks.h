@@ -31,19 +31,15 @@ struct SfKsBatch {
     u64 *scratch;   // sf_ks_scratch_words(R) words per merge of one launch batch
 };
 
-// limbs of scratch per merge: ModUp extensions, accumulators, tau_d(u.a), and for
-// NTT-domain operands its inverse rows
-SF_HD int sf_ks_x2(const SfRing &R) { return 0; }
+// Scratch of a merge, in limbs: the ModUp extensions [dnum][nm] from limb 0,
+// accumulators, tau_d(u.a).  The inverse rows of NTT-domain operands (x1) lie where
+// the accumulators go: k_ks2 has read them before k_ks3 writes there.
 SF_HD int sf_ks_acc(const SfRing &R) { return R.dnum * R.nm; }
+SF_HD int sf_ks_x1(const SfRing &R) { return sf_ks_acc(R); }
 SF_HD int sf_ks_ta(const SfRing &R) { return sf_ks_acc(R) + 2 * R.nm; }
-SF_HD int sf_ks_x1(const SfRing &R) { return sf_ks_ta(R) + R.L; }
-SF_HD size_t sf_ks_scratch_words_dev(const SfRing &R, int ntt)
-{
-    return (size_t)(sf_ks_x1(R) + (ntt ? R.L : 0)) << R.log_n;
-}
 
-// words per merge (ntt = 1: room for either kind of operands)
-size_t sf_ks_scratch_words(const SfRing &R, int ntt = 1);
+// words per merge
+SF_HD size_t sf_ks_scratch_words(const SfRing &R) { return (size_t)(sf_ks_ta(R) + R.L) << R.log_n; }
 // One launch sequence for B.count merges, scratch for all of them.
 sf_status sf_ks_launch(sf_ctx *ctx, const SfKsBatch &B, cudaStream_t st);
 // Splits B into launch batches of `batch` merges reusing `scratch`
@@ -89,7 +85,7 @@ __device__ __forceinline__ u64 *merge_out(const SfKsBatch &B, int b)
 // this merge's scratch, limb `limb` of it
 __device__ __forceinline__ u64 *ks_limb(const SfRing &R, const SfKsBatch &B, int b, int limb)
 {
-    return B.scratch + sf_ks_scratch_words_dev(R, B.ntt) * b + ((size_t)limb << R.log_n);
+    return B.scratch + sf_ks_scratch_words(R) * b + ((size_t)limb << R.log_n);
 }
 
 // coefficient p of E + X^s O of one limb, canonical; e, o: the limb's N

@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_ks4(SfRin
     __syncthreads();
     sf_pdl_wait(B);
     const SfUnitRange U = sf_unit_range(ng * B.count);
-    const size_t per = sf_ks_scratch_words_dev(R, B.ntt);
+    const size_t per = sf_ks_scratch_words(R);
     // A unit's transforms: the K special limbs, then its share of the data limbs.
     // item-major: the blocks in flight work on the tiles of a few merges.
     struct Unit {

@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS) k_ks1(SfRin
     sf_pdl_next(B);
     sf_pdl_wait(B);
     const SfUnitRange U = sf_unit_range(ng * B.count);
-    const size_t per = sf_ks_scratch_words_dev(R, B.ntt);
+    const size_t per = sf_ks_scratch_words(R);
     SfCursor C(U.u0, B.count);
     // group = (row tile, limb i), item = merge; each thread copies its own points ahead
     auto prefetch = [&]() {
@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS_ACC) k_ks3(S
     sf_pdl_wait(B);
     const SfUnitRange U = sf_unit_range(ng * B.count);
     const sf_pair *key = (const sf_pair *)B.key;
-    const size_t per = sf_ks_scratch_words_dev(R, B.ntt);
+    const size_t per = sf_ks_scratch_words(R);
     // group = (row tile, modulus m), item = merge; the digit's own limbs of
     // NTT-domain operands are tau_d(u.a) itself, already transformed
     struct Group {
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS_ACC) k_ks3(S
 #pragma unroll
             for (int t = 0; t < 8; ++t) sf_cp8(pre + t * NT, src + T.store_at(G.tile, t));
         } else {
-            const u64 *src = base + ((size_t)(sf_ks_x2(R) + j * R.nm + G.m) << (LR + LC)) + G.row;
+            const u64 *src = base + ((size_t)(j * R.nm + G.m) << (LR + LC)) + G.row;
 #pragma unroll
             for (int t = 0; t < 8; ++t) sf_cp8(pre + t * NT, src + T.k1(t));
         }

@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_ks2(SfRin
     __syncthreads();
     sf_pdl_wait(B);
     const SfUnitRange U = sf_unit_range(ng * B.count);
-    const size_t per = sf_ks_scratch_words_dev(R, B.ntt);
+    const size_t per = sf_ks_scratch_words(R);
     // item-major: the blocks in flight work on the tiles of a few merges
     SfCursor C(U.u0, ng);   // C.grp: merge, C.item: group
     for (int u = U.u0; u < U.u1; ++u, C.next()) {
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_ks2(SfRin
             }
             T.forward(x, tab + (size_t)m * SfShape<LR>::S, buf, M);
             turn();
-            u64 *dst = B.scratch + per * b + ((size_t)(sf_ks_x2(R) + j * R.nm + m) << (LR + LC)) + col;
+            u64 *dst = B.scratch + per * b + ((size_t)(j * R.nm + m) << (LR + LC)) + col;
 #pragma unroll
             for (int t = 0; t < 8; ++t) dst[(size_t)T.kl(t) << LC] = x[t];
         }

@@ -58,7 +58,7 @@ extern "C" sf_status sf_rotate_noalloc(sf_ctx *ctx, const sf_rotkeys *rk, int32_
     const int batch = std::min(ctx->ks_batch, (int)count);
     // what the call uses: the workspaces of one launch batch, then room for a copy of
     // the input (buffers that share words)
-    const size_t ks_words = round_words(sf_ks_scratch_words(R, 0) * batch), used = ks_words + round_words((size_t)count * ct);
+    const size_t ks_words = round_words(sf_ks_scratch_words(R) * batch), used = ks_words + round_words((size_t)count * ct);
     // the documented limit, which stays as it is: two ciphertexts and this many
     // key-switch limbs per call
     const size_t limbs = R.L + std::max(R.L, 2 * R.K) + std::max(R.dnum * R.nm, 2 * R.L) + 2 * R.L;
