@@ -37,7 +37,10 @@
 // per-merge pointers are set up once per thread.  Bound by HBM (0.89 of the
 // copy bandwidth at N = 2^16): 3.0 us per merge there.  Done inside k_ks2 and
 // k_ks4 instead, the gathers' latency cost those kernels 9 us more per merge.
+// UNREDUCED (B.unreduced) is an instance of its own: the same test at run time cost
+// every other call 0.5 to 1.5 % (a rotation at N = 2^16 73.8 us, 72.7 without).
 #define SF_EW 8
+template <bool UNREDUCED>
 __global__ void __launch_bounds__(256) k_ks_gather(SfRing R, SfKsBatch B)
 {
     sf_pdl_next(B);
@@ -62,7 +65,7 @@ __global__ void __launch_bounds__(256) k_ks_gather(SfRing R, SfKsBatch B)
             // p receives index e = p d^-1 mod 2N of u, negated when e >= N
             const unsigned e = (p * B.dinv) & (2 * n - 1), src = e & mask;
             u64 ua = Ea[src], ub = Eb[src], va = 0, vb = 0;
-            if (B.unreduced) {
+            if (UNREDUCED) {
                 ua = sf_reduce(ua, q, M.one_p);
                 ub = sf_reduce(ub, q, M.one_p);
             }
@@ -132,7 +135,7 @@ sf_status sf_ks_launch(sf_ctx *ctx, const SfKsBatch &B0, cudaStream_t st)
         b.pdl = ks_overlap(b.count);
         b.scratch += sf_ks_scratch_words(R) * off;
         sf_launch_begin(ctx, SFK_KS_GATHER, st, &ev);
-        sf_pdl_launch(k_ks_gather, dim3((R.n + 256 * SF_EW - 1) / (256 * SF_EW), R.L, b.count), 256, 0, st, R, b);
+        sf_pdl_launch(b.unreduced ? k_ks_gather<true> : k_ks_gather<false>, dim3((R.n + 256 * SF_EW - 1) / (256 * SF_EW), R.L, b.count), 256, 0, st, R, b);
         sf_launch_end(ctx, SFK_KS_GATHER, st, ev);
         if (b.ntt) SF_TRY(sf_ks_inv_rows_launch(ctx, b, st));
         SF_TRY(sf_ks_up_launch(ctx, b, st));
