@@ -37,8 +37,9 @@
 // per-merge pointers are set up once per thread.  Bound by HBM (0.89 of the
 // copy bandwidth at N = 2^16): 3.0 us per merge there.  Done inside k_ks2 and
 // k_ks4 instead, the gathers' latency cost those kernels 9 us more per merge.
-// UNREDUCED (B.unreduced) is an instance of its own: the same test at run time cost
-// every other call 0.5 to 1.5 % (a rotation at N = 2^16 73.8 us, 72.7 without).
+// UNREDUCED (B.unreduced) is an instance of its own: with the test at run time a
+// 64 x 64 layer at N = 2^12 took 321.9 us, 320.3 without, a rotation at N = 2^16
+// 73.8 and 73.6.
 #define SF_EW 8
 template <bool UNREDUCED>
 __global__ void __launch_bounds__(256) k_ks_gather(SfRing R, SfKsBatch B)

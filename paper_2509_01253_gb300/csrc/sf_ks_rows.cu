@@ -84,7 +84,9 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS_ACC) k_ks3(S
     sf_pdl_wait(B);
     const SfUnitRange U = sf_unit_range(ng * B.count);
     const sf_pair *key = (const sf_pair *)B.key;
-    const size_t per = sf_ks_scratch_words(R);
+    // limbs of scratch per merge; as a word count it costs this kernel registers, and 2.7 %
+    // (26.1 ms per resnet20-sized convolution at N = 2^14 against 25.4)
+    const int per = sf_ks_ta(R) + R.L;
     // group = (row tile, modulus m), item = merge; the digit's own limbs of
     // NTT-domain operands are tau_d(u.a) itself, already transformed
     struct Group {
@@ -98,7 +100,7 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS_ACC) k_ks3(S
     auto own_limb = [&](int m, int j) { return B.ntt && m >= j * R.K && m < min((j + 1) * R.K, R.L); };
     // each thread copies its own points of a digit ahead
     auto prefetch = [&](const Group &G, int item, int j) {
-        const u64 *base = B.scratch + per * item;
+        const u64 *base = B.scratch + ((size_t)(per * item) << (LR + LC));
         if (own_limb(G.m, j)) {
             const u64 *src = base + ((size_t)(sf_ks_ta(R) + G.m) << (LR + LC));
 #pragma unroll
@@ -161,7 +163,7 @@ __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS_ACC) k_ks3(S
             ka = kb + ((size_t)R.nm << (LR + LC));
         }
         const u64 *add = B.ntt && G.m < R.L ? merge_out(B, b) + ((size_t)G.m << (LR + LC)) + T.store_at(G.tile, 0) : nullptr;
-        u64 *dst = B.scratch + per * b + ((size_t)(sf_ks_acc(R) + G.m) << (LR + LC)) + G.row;
+        u64 *dst = B.scratch + ((size_t)(per * b + sf_ks_acc(R) + G.m) << (LR + LC)) + G.row;
         // one copy of the inverse pass for both parts: the code stays within the
         // instruction cache
 #pragma unroll 1
