@@ -268,7 +268,7 @@ def kernel_ops(kernel: str, g: RingShape, k_in: int = 1):
     operands (the first level above the leaves); one of coefficient-domain
     operands runs the forward transforms of the digits' own limbs in the
     ks2 and ks3 kernels instead of ks1's and ks2's inverse ones: the same
-    number of butterflies."""
+    number of butterflies; its gather has no products."""
     N, L, K, nm, dnum, lr, lc = g.n, g.L, g.K, g.nm, g.dnum, g.lr, g.lc
     half = N // 2
     fbc_up = sum(d * (nm - d) for d in g.digits if d > 1) * N

@@ -440,7 +440,7 @@ sf_status sf_rotate_noalloc(sf_ctx *ctx, const sf_rotkeys *rk, int32_t d, const 
  * inverse = 0: coefficients (each residue below 4 q_i) -> NTT domain,
  * canonical, slot j holding the evaluation at psi^(2 brev(j) + 1) with psi a
  * primitive 2N-th root modulo q_i; inverse = 1: NTT-domain values (below
- * 4 q_i) -> canonical coefficients.  Two persistent launches on `stream`.
+ * 4 q_i) -> canonical coefficients.  Two launches on `stream`.
  * Errors: SF_EINVAL for null buffers, count < 1, inverse not 0/1, or a batch
  * whose count x L x (tiles per limb) exceeds 2^31 - 1 (larger than any
  * device memory). */

@@ -47,20 +47,6 @@ SF_HD u64 sf_add(u64 a, u64 b, u64 q) { return sf_csub(a + b, q); }
 
 SF_HD u64 sf_sub(u64 a, u64 b, u64 q) { return a >= b ? a - b : a + q - b; }
 
-// 128-bit accumulator for sums of products (hi, lo).
-struct sf_u128 {
-    u64 lo, hi;
-};
-
-SF_HD void sf_mac128(sf_u128 &acc, u64 a, u64 b)
-{
-    u64 lo = a * b;
-    u64 hi = sf_mulhi(a, b);
-    u64 nlo = acc.lo + lo;
-    acc.hi += hi + (nlo < lo ? 1 : 0);
-    acc.lo = nlo;
-}
-
 // Montgomery REDC: returns T * 2^-64 mod q in [0, 2q) for T = hi*2^64 + lo < q*2^64.
 // qinv_neg = -q^-1 mod 2^64.
 SF_HD u64 sf_redc_lazy(u64 hi, u64 lo, u64 q, u64 qinv_neg)

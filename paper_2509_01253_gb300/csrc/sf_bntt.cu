@@ -11,9 +11,9 @@
 // points ahead with cp.async while it transforms the current one (loads into
 // registers sank behind the transform: the column pass waited on memory).
 //
-// Bound by the integer multiplier: at N = 2^16 the fmaheavy pipe is busy 70 to
-// 76 % of the cycles.  512 x 5 limbs of 2^16, forward: 1961 us with tile sweeps in
-// shared memory, 1515 us here; 37 x 3 inverse limbs of 2^14: 32.8 and 26.6 us.
+// Bound by the integer multiplier: at N = 2^16 the fmaheavy pipe is busy 57 to
+// 70 % of the cycles.  512 x 5 limbs of 2^16, forward: 1961 us with tile sweeps in
+// shared memory, 1543 us here; 37 x 3 inverse limbs of 2^14: 32.8 and 26.6 us.
 #include <algorithm>
 
 #include "sf_async.cuh"

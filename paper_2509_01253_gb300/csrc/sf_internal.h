@@ -38,7 +38,7 @@ struct SfRing {
     int modup_copy;
     SfMod m[SF_MAX_MODULI];
     // twiddle pairs (w, companion) of the passes (sf_reg.cuh), N = R x C, C = 2^ceil(log2 N / 2):
-    // columns [nm][R], row tiles [nm][R/16][16 (C - 1)]
+    // columns [nm][R], row tiles [nm][R/NB][NB (C - 1)], NB = 16 rows a tile, 8 of 256 points
     const ulonglong2 *colP, *rowP;
     // powers psi^k, k in [0, 2N), [nm][2N] (monomials in the NTT domain)
     const u64 *pw, *pw_p;
@@ -197,9 +197,9 @@ enum SfKernelKind {
     SFK_KS1_INV_ROW,
     SFK_KS2_MODUP_COL,
     SFK_KS3_INNER_ROW,
-    SFK_KS3_INV_ROW_P,
+    SFK_KS3_INV_ROW_P,    // no kernel any more: kept so that the list of families stays as it was
     SFK_KS4_MODDOWN_COL,
-    SFK_KS5_FINISH_ROW,
+    SFK_KS5_FINISH_ROW,   // likewise
     SFK_LEAF_COL,
     SFK_LEAF_ROW,
     SFK_SHUFFLE,

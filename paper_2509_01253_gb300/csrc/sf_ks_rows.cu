@@ -14,9 +14,9 @@
 // multiply-accumulates, plus 8 butterflies for the two inverse passes, against
 // 8 bytes read and 16/dnum written.  Every exchange stays inside a warp, so the
 // loop over the items has no block barrier; the next digit's points arrive by
-// cp.async while this one is transformed.  Three blocks of 256 threads per SM at
-// 256-point rows: 32 KB of staged twiddles, an 18 KB exchange buffer and 16 KB of
-// points ahead each.
+// cp.async while this one is transformed.  At 256-point rows a block of 256 threads
+// has 32 KB of staged twiddles, an 18 KB exchange buffer and 16 KB of points ahead;
+// three blocks per SM for k_ks1, two of 128 registers for k_ks3.
 #include <algorithm>
 
 #include "sf_async.cuh"

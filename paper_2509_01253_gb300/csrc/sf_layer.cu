@@ -6,7 +6,7 @@
 // with k(i) the in-ciphertext position of input i after unshuffling
 // (p = sigma_prev^-1(i)).  Three kernels per batch of outputs:
 //   leaf_prep: walks each output's receptive field once and buckets its taps
-//              by (input ciphertext, 16-column tile),
+//              by (input ciphertext, column tile: 16 columns, 8 at N = 2^16),
 //   leaf_col : scatters its bucket into a zeroed column tile in shared memory
 //              and runs the forward column pass,
 //   leaf_row : forward row pass, then the product with every input ciphertext
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(SfShape<LR>::NT, SfShape<LR>::BPS) k_leaf_col(
 // leaf_row: groups (row tile, limb i), items slots.  Per input
 // ciphertext a forward row pass and two multiply-accumulates per point, the
 // accumulators in registers.  Bound by the integer multiplier; the staged
-// twiddles (61 KB at 256-point rows) serve every slot of the group.
+// twiddles (32 KB at 256-point rows) serve every slot of the group.
 template <int LR, int LC, bool PM>
 __global__ void __launch_bounds__(SfShape<LC>::NT, SfShape<LC>::BPS_ACC) k_leaf_row(SfRing R, SfLeafParams P, int ng, int cnt)
 {

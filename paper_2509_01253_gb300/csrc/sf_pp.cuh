@@ -520,7 +520,11 @@ __host__ __device__ constexpr int ppt_first() { return ppt_radix(T, SfPpT<T, ALP
 // whose blocks are smaller): at M = 5^5 that caps the torus kernel's registers at 48,
 // with a few spilled words.  Torus key switch of 4096 ciphertexts, 5 digits: 2423 us
 // at 5^5, 1631 us at 3^7 (1709 with two blocks); 4852 and 2747 us with the canonical
-// stages.
+// stages.  k_pp_ks spills 248 bytes a thread at 5^5 and 292 at 3^7 under the same
+// bounds and still gains by them: 2000 ciphertexts of 3 limbs take 1400 us at 5^5
+// (1 block 1690, 3 blocks 1518), 1391 at 7^4 (1853, 1385) and 899 at 3^7 (1 block
+// 1323, 2 blocks 958); 30 ciphertexts 56.1 (54.0, 64.4), 58.1 (58.3, 62.3) and
+// 55.9 us (47.7, 47.7).
 template <int T, int ALPHA>
 struct SfPpShape {
     static constexpr int NT = SfPpT<T, ALPHA>::THREADS, MMAX = SfPpT<T, ALPHA>::M, MINB = T == 3 ? 3 : 2;

@@ -15,13 +15,13 @@
 // Every thread holds 8 points and runs up to three stages per phase, in two
 // (32, 64 points) or three phases (128, 256 points).  A tile is 2048 points at
 // 128 and 256 points (16 or 8 sub-transforms, 256 threads): with three blocks
-// per SM a kernel has 24 warps and 85 registers a thread, which hold the
-// accumulators of the inner products or the converted digits beside the points.
-// The C/8 threads of a row share a warp, so row exchanges need no block barrier
-// and the warps of a block run independently; columns exchange through block
-// barriers.  16 points a thread (one exchange less, 128 registers, 16 warps)
-// lost: the inner product ran 25.6 us per key switch at N = 2^16, waiting on
-// memory and on instruction fetches.
+// per SM a kernel has 24 warps and 80 registers a thread; the kernels that hold
+// the accumulators of inner products beside the points run two blocks of 128
+// registers (SfShape::BPS_ACC).  The C/8 threads of a row share a warp, so row
+// exchanges need no block barrier and the warps of a block run independently;
+// columns take one block barrier a transform (SfColT).  16 points a thread (one
+// exchange less, 128 registers, 16 warps) lost: the inner product ran 25.6 us
+// per key switch at N = 2^16, waiting on memory and on instruction fetches.
 //
 // Twiddles are pairs (w, companion), see sf_mad.  psi^-brev(m + g) =
 // -psi^brev(m + (m - 1 - g)) for m = 2^a: the inverse twiddle of a group is

@@ -307,10 +307,10 @@ def plan_gammas(net: EncodedNetwork, split: list, margin: float = 0.02, leaf_fac
     (1 - margin) total_r.  The leaves alone would double; the default 2.2
     also carries the powers' input transforms and the plain bottom-level
     merges that the gamma = 2 rounds add (fitted on GB300 over the ResNet-34
-    rounds: 2.11 to 2.24).  Early, wide layers keep gamma = 0; the late
-    rounds, where key switches dominate, take gamma = 2.  The choice is the
-    server's alone: the client sends the powers for exactly the rounds that
-    take gamma = 2."""
+    rounds, 2.11 to 2.24, with earlier leaf kernels; not fitted again since).
+    Early, wide layers keep gamma = 0; the late rounds, where key switches
+    dominate, take gamma = 2.  The choice is the server's alone: the client
+    sends the powers for exactly the rounds that take gamma = 2."""
     assert len(split) == len(net.rounds)
     plan = []
     for r, (leaf, total) in enumerate(split):
